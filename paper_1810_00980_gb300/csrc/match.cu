@@ -25,6 +25,7 @@
 #include <chrono>
 #include <cmath>
 #include <cstring>
+#include <map>
 #include <mutex>
 #include <vector>
 
@@ -371,7 +372,49 @@ __device__ __forceinline__ void acc_switch(Acc& a, int64_t win, unsigned long lo
     }
 }
 
-// c delta / (c delta - dur) in Q64 by long division (64 fraction bits, rounded down)
+// N / D in Q64: the integer part, and floor((N mod D) 2^64 / D).  The fraction is two digits of
+// the schoolbook division in base 2^32 (Knuth, TAOCP vol. 2, 4.3.1, Algorithm D), instead of 64
+// shift-and-subtract steps.  Below 2^32 (spans c delta of a graph in seconds) each digit is one
+// plain 64-bit division; above, the divisor is normalised and each digit's estimate from its
+// upper half is corrected at most twice.
+__host__ __device__ __forceinline__ uint64_t q64_digit(uint64_t r, uint64_t D) {
+    // floor(r 2^32 / D) for r < D, D's top bit set
+    const uint64_t v1 = D >> 32, v0 = D & 0xffffffffull;
+    uint64_t q = r / v1, rh = r - q * v1;
+    while ((q >> 32) || q * v0 > (rh << 32)) {
+        q--;
+        rh += v1;
+        if (rh >> 32) break;
+    }
+    return q;
+}
+__host__ __device__ __forceinline__ void q64_div(uint64_t N, uint64_t D, unsigned long long& wi,
+                                                 unsigned long long& wf) {
+    const uint64_t i = N / D;
+    uint64_t r = N - i * D;
+    wi = i;
+    if ((D >> 32) == 0) {
+        r <<= 32;
+        const uint64_t q1 = r / D;
+        r = (r - q1 * D) << 32;
+        wf = (q1 << 32) | (r / D);
+        return;
+    }
+#ifdef __CUDA_ARCH__
+    const int s = __clzll((long long)D);
+#else
+    const int s = __builtin_clzll(D);
+#endif
+    D <<= s;
+    r <<= s;
+    const uint64_t q1 = q64_digit(r, D);
+    r = (r << 32) - q1 * D;   // mod 2^64: the true remainder is below D
+    wf = (q1 << 32) | q64_digit(r, D);
+}
+
+// c delta / (c delta - dur) in Q64 (64 fraction bits, rounded down), bit by bit: for the matcher's
+// instances without a table, where q64_div's registers would spill the hot loop (the replay of
+// 18 queries on 1e5 edges ran 1.5 % slower with it)
 __device__ __forceinline__ void q64_weight(int64_t cd, int64_t dur, unsigned long long& wi,
                                         unsigned long long& wf) {
     unsigned long long D = (unsigned long long)(cd - dur);
@@ -501,7 +544,7 @@ __device__ __forceinline__ void ride_weight(const QPlan& R, int64_t dur, unsigne
         wi = e.x;
         wf = e.y;
     } else {
-        q64_weight(R.cd, dur, wi, wf);
+        q64_div((uint64_t)R.cd, (uint64_t)(R.cd - dur), wi, wf);
     }
     lo = wf * n;
     hi = wi * n + __umul64hi(wf, n);
@@ -608,24 +651,24 @@ size_t match_smem_bytes(int nq, int threads, bool ride_tab = false) {
 }
 
 // ----------------------------------------------------------------- kernels
-__global__ void k_wtab(uint64_t* __restrict__ tab, int64_t delta, int64_t cd) {
-    for (int64_t d = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; d <= delta;
-         d += (int64_t)gridDim.x * blockDim.x) {
-        unsigned long long D = (unsigned long long)(cd - d);
-        if (D == 0) {  // duration c*delta (c = 1) never fits inside a window of c*delta ticks
-            tab[2 * d] = 0;
-            tab[2 * d + 1] = 0;
-            continue;
+// Every weight table of the batch in one launch, table y by row y of the grid (plan own[y]'s;
+// plans with the same delta and c delta share a table).  A weight costs three divisions, so
+// that a long table is bound by the 16 bytes it writes per duration.  A bench batch on 1e6 edges
+// ran 592 -> 555 us with one launch instead of nine; six tables of a graph in milliseconds, the
+// longest 3.6e6 durations, took 393 us with 64 shift-and-subtract steps per weight (the call
+// 3,034 -> 2,666 us).
+__global__ void k_wtab(const QPlan* __restrict__ plans, const int32_t* __restrict__ own, int n_tab) {
+    for (int y = blockIdx.y; y < n_tab; y += gridDim.y) {
+        const QPlan& Q = plans[own[y]];
+        ulonglong2* tab = reinterpret_cast<ulonglong2*>(const_cast<uint64_t*>(Q.wtab));
+        const int64_t cd = Q.cd, delta = Q.delta;
+        for (int64_t d = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; d <= delta;
+             d += (int64_t)gridDim.x * blockDim.x) {
+            ulonglong2 e = make_ulonglong2(0, 0);
+            // (duration c delta (c = 1) never fits inside a window of c delta ticks)
+            if (cd > d) q64_div((uint64_t)cd, (uint64_t)(cd - d), e.x, e.y);
+            tab[d] = e;
         }
-        unsigned long long N = (unsigned long long)cd;
-        unsigned long long wi = N / D, r = N - wi * D, wf = 0;
-        for (int i = 0; i < 64; i++) {
-            r <<= 1;
-            wf <<= 1;
-            if (r >= D) { r -= D; wf |= 1; }
-        }
-        tab[2 * d] = wi;
-        tab[2 * d + 1] = wf;
     }
 }
 
@@ -1919,6 +1962,50 @@ size_t per_first_scratch_bytes(int64_t F, bool hoist, size_t rec_bytes) {
 constexpr size_t kBoundScratchBytes = (size_t)2 << 30;
 
 
+// Weight tables of a batch's estimates: their places from base on, and the bytes they need.
+// Estimates with the same delta and c delta read one table: 192 seeds of one query need as many
+// tables as there are values of c.  Only spans up to kWtabMax get one; the others divide per
+// instance.  own: the plan that each table is made for.
+size_t place_wtabs(std::vector<QPlan>& hp, char* base, std::vector<int32_t>& own) {
+    size_t off = 0;
+    own.clear();
+    std::map<std::pair<int64_t, int64_t>, const uint64_t*> have;
+    for (size_t i = 0; i < hp.size(); i++) {
+        QPlan& P = hp[i];
+        P.wtab = nullptr;
+        if (P.l <= 0 || P.mode != TM_MODE_ESTIMATE || P.delta + 1 > kWtabMax) continue;
+        auto ins = have.emplace(std::make_pair(P.delta, P.cd), (const uint64_t*)(base + off));
+        P.wtab = ins.first->second;
+        if (!ins.second) continue;
+        off += a256(16 * (size_t)(P.delta + 1));
+        own.push_back((int32_t)i);
+    }
+    return off;
+}
+
+// The plans and, behind them, the owners of the weight tables: one copy to the device, from h,
+// which the caller keeps until the stream has passed it
+size_t plans_bytes(size_t nq) { return (sizeof(QPlan) + sizeof(int32_t)) * nq; }
+cudaError_t copy_plans(const std::vector<QPlan>& hp, const std::vector<int32_t>& own, std::vector<char>& h,
+                       QPlan* dplans, cudaStream_t st) {
+    const size_t np = sizeof(QPlan) * hp.size(), no = sizeof(int32_t) * own.size();
+    h.resize(np + no);
+    std::memcpy(h.data(), hp.data(), np);
+    if (no) std::memcpy(h.data() + np, own.data(), no);
+    return cudaMemcpyAsync(dplans, h.data(), np + no, cudaMemcpyHostToDevice, st);
+}
+
+// fills the tables (dplans as copy_plans left it)
+void launch_wtabs(const std::vector<QPlan>& hp, const std::vector<int32_t>& own, const QPlan* dplans, cudaStream_t st) {
+    if (own.empty()) return;
+    int64_t dmax = 0;
+    for (int32_t i : own) dmax = std::max(dmax, hp[(size_t)i].delta);
+    const unsigned gx = (unsigned)std::min<int64_t>(dmax / 256 + 1, 2048);
+    k_wtab<<<dim3(gx, (unsigned)std::min<size_t>(own.size(), 65535)), 256, 0, st>>>(
+        dplans, reinterpret_cast<const int32_t*>(dplans + hp.size()), (int)own.size());
+    count_launch();
+}
+
 template <typename TT>
 int run_batch_t(const tm_graph* g, const tm_query* qs, int nq, tm_result* res, cudaStream_t st,
                 BatchOut* dbg) {
@@ -1931,7 +2018,7 @@ int run_batch_t(const tm_graph* g, const tm_query* qs, int nq, tm_result* res, c
     int64_t NW = 0, n_sums = 0, F_ub = 0;
     int lmax = 1, kmax = 2;
     bool any_hoist = false, any_full = false;
-    size_t wtab_bytes = 0, full_bytes = 0;
+    size_t full_bytes = 0;
     for (int i = 0; i < nq; i++) {
         std::string why;
         int s = validate_query(g, qs[i], why);
@@ -1988,8 +2075,6 @@ int run_batch_t(const tm_graph* g, const tm_query* qs, int nq, tm_result* res, c
         lmax = std::max(lmax, hp[(size_t)i].l);
         kmax = std::max(kmax, hp[(size_t)i].k);
         any_hoist |= hp[(size_t)i].hoist != 0 || hp[(size_t)i].ex23 != 0;
-        if (hp[(size_t)i].mode == TM_MODE_ESTIMATE && hp[(size_t)i].delta + 1 <= kWtabMax)
-            wtab_bytes += a256(16 * (size_t)(hp[(size_t)i].delta + 1));
         if (hp[(size_t)i].full) {
             any_full = true;
             full_bytes += a256(4 * (size_t)hp[(size_t)i].b * (size_t)g->m) +
@@ -2014,9 +2099,11 @@ int run_batch_t(const tm_graph* g, const tm_query* qs, int nq, tm_result* res, c
     const int64_t n_parts = fold_parts(hp, smax);
     int bmax = 1;
     for (const QPlan& P : hp) bmax = std::max(bmax, P.b);
+    std::vector<int32_t> wown;
+    const size_t wtab_bytes = place_wtabs(hp, nullptr, wown);
     size_t NWs = (size_t)std::max<int64_t>(NW, 1);
     size_t Ms = (size_t)std::max<int64_t>(g->m, 1);
-    size_t sz = a256(sizeof(QPlan) * (size_t)nq) + a256(sizeof(tm_result) * (size_t)nq) + wtab_bytes +
+    size_t sz = a256(plans_bytes((size_t)nq)) + a256(sizeof(tm_result) * (size_t)nq) + wtab_bytes +
                 9 * a256(8 * NWs) + 3 * a256(4 * NWs) + a256(8 * NWs) + a256(8 * A_N * NWs) + 4 * 256 +
                 full_bytes + (any_full ? 3 * a256(4 * Ms) : 0) +
                 a256(sizeof(ShiftSums) * (size_t)std::max<int64_t>(n_sums, 1)) +
@@ -2026,13 +2113,11 @@ int run_batch_t(const tm_graph* g, const tm_query* qs, int nq, tm_result* res, c
     TM_CUDA(cudaMallocAsync((void**)&sb, sz, st));
     char* p = sb;
     auto take = [&](size_t bytes) { char* r = p; p += a256(bytes); return (void*)r; };
-    QPlan* dplans = (QPlan*)take(sizeof(QPlan) * (size_t)nq);
+    QPlan* dplans = (QPlan*)take(plans_bytes((size_t)nq));
     tm_result* dres = (tm_result*)take(sizeof(tm_result) * (size_t)nq);
+    place_wtabs(hp, (char*)take(wtab_bytes), wown);
     for (int i = 0; i < nq; i++) {
         QPlan& P = hp[(size_t)i];
-        if (P.l > 0 && P.mode == TM_MODE_ESTIMATE && P.delta + 1 <= kWtabMax) {
-            P.wtab = (const uint64_t*)take(16 * (size_t)(P.delta + 1));
-        }
         if (P.full) {
             P.perm = (const int32_t*)take(4 * (size_t)P.b * (size_t)g->m);
             P.woff = (const int64_t*)take(8 * (size_t)P.b * (size_t)(P.J + 1));
@@ -2081,20 +2166,16 @@ int run_batch_t(const tm_graph* g, const tm_query* qs, int nq, tm_result* res, c
     int ev_w0 = pe.mark(st), ev_w1 = -1, ev_l0 = -1, ev_l1 = -1, ev_l2 = -1, ev_m1 = -1, ev_r1 = -1, ev_f1 = -1;
     int64_t hW2 = 0;
     unsigned long long h_rcount = 0;
-    fail(cudaMemcpyAsync(dplans, hp.data(), sizeof(QPlan) * (size_t)nq, cudaMemcpyHostToDevice, st), "plans");
+    std::vector<char> h_plans;
+    fail(copy_plans(hp, wown, h_plans, dplans, st), "plans");
     if (!h_shifts.empty())
         fail(cudaMemcpyAsync(dshifts, h_shifts.data(), 8 * h_shifts.size(), cudaMemcpyHostToDevice, st), "shifts");
     fail(cudaMemsetAsync(W.acc, 0, 8 * A_N * NWs, st), "acc");
     fail(cudaMemsetAsync(dctr, 0, 8, st), "counter");
     fail(cudaMemsetAsync(drcount, 0, 8, st), "record counter");
-    for (int i = 0; i < nq && rc == TM_OK; i++) {
-        const QPlan& P = hp[(size_t)i];
-        if (P.wtab) {
-            int64_t n = P.delta + 1;
-            unsigned gr = (unsigned)std::min<int64_t>((n + 255) / 256, 4096);
-            k_wtab<<<gr, 256, 0, st>>>((uint64_t*)P.wtab, P.delta, P.cd); count_launch();
-            fail(cudaGetLastError(), "k_wtab");
-        }
+    if (rc == TM_OK) {
+        launch_wtabs(hp, wown, dplans, st);
+        fail(cudaGetLastError(), "k_wtab");
     }
     GraphDevT<TT> G = typed<TT>(g->dev);
     if (rc == TM_OK) rc = ex_tables_for(g, hp, st, G);
@@ -2768,7 +2849,6 @@ int batch_create_t(const tm_graph* g, const tm_query* qs, int nq, tm_batch** out
     int64_t NW = 0, Fmax = 0, n_sums = 0;
     int lmax = 1, kmax = 2, bmax = 1;
     bool any_hoist = false;
-    size_t wtab_bytes = 0;
     for (int i = 0; i < nq; i++) {
         std::string why;
         int s = validate_query(g, qs[i], why);
@@ -2797,14 +2877,15 @@ int batch_create_t(const tm_graph* g, const tm_query* qs, int nq, tm_batch** out
         lmax = std::max(lmax, P.l);
         kmax = std::max(kmax, P.k);
         any_hoist |= P.hoist != 0 || P.ex23 != 0;
-        if (P.mode == TM_MODE_ESTIMATE && P.delta + 1 <= kWtabMax) wtab_bytes += a256(16 * (size_t)(P.delta + 1));
     }
     int smax = 1;
     const int64_t n_parts = fold_parts(hp, smax);
+    std::vector<int32_t> wown;
+    const size_t wtab_bytes = place_wtabs(hp, nullptr, wown);
     size_t NWs = (size_t)std::max<int64_t>(NW, 1), Fs = (size_t)std::max<int64_t>(Fmax, 1);
     int64_t ws1 = 2 * ((NW + 2047) / 2048) + 2;
     int64_t ws2 = scan_dn_ws_elems(Fmax) + 2;
-    size_t sz = a256(sizeof(QPlan) * (size_t)nq) + a256(sizeof(tm_result) * (size_t)nq) + wtab_bytes +
+    size_t sz = a256(plans_bytes((size_t)nq)) + a256(sizeof(tm_result) * (size_t)nq) + wtab_bytes +
                 9 * a256(8 * NWs) + 3 * a256(4 * NWs) + a256(8 * NWs) + a256(8 * A_N * NWs) + 3 * 256 +
                 a256(sizeof(FRec<TT>) * Fs) + (any_hoist ? 3 : 1) * a256(8 * Fs) + a256(8 * (size_t)ws1) +
                 a256(8 * (size_t)ws2) +
@@ -2820,13 +2901,9 @@ int batch_create_t(const tm_graph* g, const tm_query* qs, int nq, tm_batch** out
     }
     char* p = (char*)b->scratch;
     auto take = [&](size_t bytes) { char* r = p; p += a256(bytes); return (void*)r; };
-    QPlan* dplans = (QPlan*)take(sizeof(QPlan) * (size_t)nq);
+    QPlan* dplans = (QPlan*)take(plans_bytes((size_t)nq));
     tm_result* dres = (tm_result*)take(sizeof(tm_result) * (size_t)nq);
-    for (int i = 0; i < nq; i++) {
-        QPlan& P = hp[(size_t)i];
-        if (P.l > 0 && P.mode == TM_MODE_ESTIMATE && P.delta + 1 <= kWtabMax)
-            P.wtab = (const uint64_t*)take(16 * (size_t)(P.delta + 1));
-    }
+    place_wtabs(hp, (char*)take(wtab_bytes), wown);
     WinDev W;
     W.lo = (int64_t*)take(8 * NWs);
     W.hi = (int64_t*)take(8 * NWs);
@@ -2863,15 +2940,11 @@ int batch_create_t(const tm_graph* g, const tm_query* qs, int nq, tm_batch** out
         if (rc == TM_OK && ee != cudaSuccess) rc = cuda_status(ee, what, __FILE__, __LINE__);
     };
     // once: plans and weight tables
-    fail(cudaMemcpyAsync(dplans, hp.data(), sizeof(QPlan) * (size_t)nq, cudaMemcpyHostToDevice, st), "plans");
-    for (int i = 0; i < nq && rc == TM_OK; i++) {
-        const QPlan& P = hp[(size_t)i];
-        if (P.wtab) {
-            int64_t n = P.delta + 1;
-            k_wtab<<<(unsigned)std::min<int64_t>((n + 255) / 256, 4096), 256, 0, st>>>((uint64_t*)P.wtab, P.delta, P.cd);
-            count_launch();
-            fail(cudaGetLastError(), "k_wtab");
-        }
+    std::vector<char> h_plans;
+    fail(copy_plans(hp, wown, h_plans, dplans, st), "plans");
+    if (rc == TM_OK) {
+        launch_wtabs(hp, wown, dplans, st);
+        fail(cudaGetLastError(), "k_wtab");
     }
     fail(cudaStreamSynchronize(st), "batch setup");
     if (rc != TM_OK) { batch_release(b); return rc; }
