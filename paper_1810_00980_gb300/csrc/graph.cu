@@ -6,6 +6,7 @@
 #include <algorithm>
 #include <cstring>
 #include <mutex>
+#include <new>
 
 #include "tm_internal.cuh"
 
@@ -44,28 +45,69 @@ __global__ void k_validate(const int32_t* __restrict__ src, const int32_t* __res
     if ((threadIdx.x & 31) == 0) atomicMax(&flags[2], mx);
 }
 
+// Copies the edges into the graph (times minus tmin, in the graph's time type), counts the digits
+// of both endpoints for the sorts and checks the input on the way: flags[0] unsorted, flags[1] id
+// outside [0, n) (taken as node 0 until the build is given up), flags[3] some edge is a loop.
+// One read of the input in place of three (check, copy, digit counts); bound by its 16 bytes in
+// and 12 (16 with 64-bit times) out per edge.
+constexpr int kIngestThreads = 512;
 template <typename TT>
-__global__ void k_ingest(const int32_t* __restrict__ src, const int32_t* __restrict__ dst,
-                         const int64_t* __restrict__ t, int64_t m, int64_t tmin,
+__global__ void __launch_bounds__(kIngestThreads) k_ingest(const int32_t* __restrict__ src, const int32_t* __restrict__ dst,
+                         const int64_t* __restrict__ t, int64_t m, int64_t tmin, int32_t n,
                          int32_t* __restrict__ gs, int32_t* __restrict__ gd, TT* __restrict__ gt,
-                         uint32_t* __restrict__ key_src, uint32_t* __restrict__ key_dst,
-                         uint32_t* __restrict__ iota_a, uint32_t* __restrict__ iota_b) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < m;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        int32_t s = src[i], d = dst[i];
-        gs[i] = s;
-        gd[i] = d;
-        gt[i] = (TT)(t[i] - tmin);
-        key_src[i] = (uint32_t)s;
-        key_dst[i] = (uint32_t)d;
-        iota_a[i] = (uint32_t)i;
-        iota_b[i] = (uint32_t)i;
+                         uint32_t* __restrict__ flags, SortDigits D, uint32_t* __restrict__ counts) {
+    extern __shared__ uint32_t sm_counts[];   // [source, destination][pass][digit]
+    const int words = D.passes << D.db;
+    for (int i = threadIdx.x; i < 2 * words; i += blockDim.x) sm_counts[i] = 0;
+    __syncthreads();
+    bool unsorted = false, bad = false, loop = false;
+    constexpr int U = 4;   // independent loads in flight per thread
+    const int64_t span = (int64_t)blockDim.x * U;
+    for (int64_t base = blockIdx.x * span; base < m; base += gridDim.x * span) {
+        int32_t s[U], d[U];
+        int64_t tt[U], tp[U];
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+            const int64_t i = base + (int64_t)u * blockDim.x + threadIdx.x;
+            const bool in = i < m;
+            s[u] = in ? src[i] : 0;
+            d[u] = in ? dst[i] : 0;
+            tt[u] = in ? t[i] : 0;
+            tp[u] = in && i > 0 ? t[i - 1] : tt[u];
+        }
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+            const int64_t i = base + (int64_t)u * blockDim.x + threadIdx.x;
+            if (i >= m) continue;
+            unsorted |= tt[u] < tp[u];
+            if ((uint32_t)s[u] >= (uint32_t)n || (uint32_t)d[u] >= (uint32_t)n) {
+                bad = true;
+                s[u] = d[u] = 0;
+            }
+            loop |= s[u] == d[u];
+            gs[i] = s[u];
+            gd[i] = d[u];
+            gt[i] = (TT)(tt[u] - tmin);
+            count_digits(sm_counts, D, (uint32_t)s[u]);
+            count_digits(sm_counts + words, D, (uint32_t)d[u]);
+        }
     }
+    const bool any_unsorted = __syncthreads_or(unsorted), any_bad = __syncthreads_or(bad), any_loop = __syncthreads_or(loop);
+    if (threadIdx.x == 0) {
+        if (any_unsorted) atomicOr(flags, 1u);
+        if (any_bad) atomicOr(flags + 1, 1u);
+        if (any_loop) atomicOr(flags + 3, 1u);
+    }
+    for (int i = threadIdx.x; i < 2 * words; i += blockDim.x)
+        if (sm_counts[i]) atomicAdd(counts + i, sm_counts[i]);
 }
 
-// off[v] = first position whose sorted key is >= v, for v in [0, n]
-__global__ void k_offsets(const uint32_t* __restrict__ keys, int64_t m, int32_t n,
-                          int64_t* __restrict__ off) {
+// off[v] = first position whose sorted key is >= v, for v in [0, n]; row 0 of the grid the out
+// view's, row 1 the in view's
+__global__ void k_offsets(const uint32_t* __restrict__ out_keys, const uint32_t* __restrict__ in_keys, int64_t m,
+                          int32_t n, int64_t* __restrict__ out_off, int64_t* __restrict__ in_off) {
+    const uint32_t* keys = blockIdx.y ? in_keys : out_keys;
+    int64_t* off = blockIdx.y ? in_off : out_off;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i <= m;
          i += (int64_t)gridDim.x * blockDim.x) {
         int64_t prev = i == 0 ? -1 : (int64_t)keys[i - 1];
@@ -74,118 +116,76 @@ __global__ void k_offsets(const uint32_t* __restrict__ keys, int64_t m, int32_t 
     }
 }
 
-// out_nbr/out_t (or in_*) gathered through the sort permutation
-template <typename TT>
-__global__ void k_gather_view(const uint32_t* __restrict__ perm, const int32_t* __restrict__ other,
-                              const TT* __restrict__ t, int64_t m, int32_t* __restrict__ nbr,
-                              TT* __restrict__ tv) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < m;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        uint32_t e = perm[i];
-        nbr[i] = other[e];
-        tv[i] = t[e];
+// Pair index of every pair-view position and the start of every pair, in one pass: a pair starts
+// where (source, destination) changes; ballots number the starts inside a warp's 512 positions, a
+// block scan and the look-back over earlier tiles number them across the graph.  8 bytes read
+// and 4 (8 more per pair) written per edge; it replaces a flag array of 8 bytes per edge, its
+// three-kernel scan and two passes over both.
+constexpr int kPairItems = 16;
+constexpr int kPairTile = kThreads * kPairItems;
+__global__ void __launch_bounds__(kThreads) k_pairs(const uint32_t* __restrict__ src, const uint32_t* __restrict__ dst, int64_t m,
+                        int32_t* __restrict__ pair_pid, int64_t* __restrict__ pair_off, uint32_t* ticket,
+                        uint32_t* words, uint32_t* err, int64_t* __restrict__ P) {
+    __shared__ uint32_t s_tile, s_warp[kThreads / 32];
+    if (threadIdx.x == 0) s_tile = atomicAdd(ticket, 1u);
+    __syncthreads();
+    const int64_t tile = s_tile, tbase = tile * kPairTile;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int64_t base = tbase + (int64_t)w * (kPairItems * 32) + lane;
+    uint32_t s[kPairItems], d[kPairItems], heads[kPairItems];
+#pragma unroll
+    for (int r = 0; r < kPairItems; r++) {
+        const int64_t i = base + r * 32;
+        s[r] = i < m ? src[i] : 0;
+        d[r] = i < m ? dst[i] : 0;
     }
-}
-
-// pair view: positions sorted by (src, dst, time); head flag where the pair changes
-template <typename TT>
-__global__ void k_pair_heads(const uint32_t* __restrict__ perm, const int32_t* __restrict__ src,
-                             const int32_t* __restrict__ dst, const TT* __restrict__ t,
-                             int64_t m, int64_t* __restrict__ head, TT* __restrict__ pair_t) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < m;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        uint32_t e = perm[i];
-        pair_t[i] = t[e];
-        int64_t h = 1;
-        if (i > 0) {
-            uint32_t f = perm[i - 1];
-            h = (src[e] != src[f] || dst[e] != dst[f]) ? 1 : 0;
+    // the position before the warp's first; every other one is a neighbouring lane's or round's
+    uint32_t ls = 0, ld = 0;
+    if (lane == 0 && base > 0 && base < m) {
+        ls = src[base - 1];
+        ld = dst[base - 1];
+    }
+    uint32_t mine = 0;
+#pragma unroll
+    for (int r = 0; r < kPairItems; r++) {
+        const int64_t i = base + r * 32;
+        uint32_t ps = __shfl_up_sync(kFull, s[r], 1), pd = __shfl_up_sync(kFull, d[r], 1);
+        if (lane == 0) {
+            ps = ls;
+            pd = ld;
         }
-        head[i] = h;
+        heads[r] = __ballot_sync(kFull, i < m && (i == 0 || s[r] != ps || d[r] != pd));
+        mine += __popc(heads[r]);
+        ls = __shfl_sync(kFull, s[r], 31);
+        ld = __shfl_sync(kFull, d[r], 31);
     }
-}
-
-// ---- views for 32-bit times: each sort carries its payload (the other endpoint and the
-// time packed in 64 bits) instead of an edge index, so no view is gathered through a
-// permutation (random reads of the edge arrays) after the sort
-__global__ void k_ingest_kv(const int32_t* __restrict__ src, const int32_t* __restrict__ dst,
-                            const int64_t* __restrict__ t, int64_t m, int64_t tmin,
-                            int32_t* __restrict__ gs, int32_t* __restrict__ gd, int32_t* __restrict__ gt,
-                            uint32_t* __restrict__ key_src, uint32_t* __restrict__ key_dst,
-                            uint64_t* __restrict__ pay_out, uint64_t* __restrict__ pay_in) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < m;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        int32_t s = src[i], d = dst[i];
-        uint32_t tt = (uint32_t)(t[i] - tmin);
-        gs[i] = s;
-        gd[i] = d;
-        gt[i] = (int32_t)tt;
-        key_src[i] = (uint32_t)s;
-        key_dst[i] = (uint32_t)d;
-        pay_out[i] = (uint64_t)(uint32_t)d | ((uint64_t)tt << 32);
-        pay_in[i] = (uint64_t)(uint32_t)s | ((uint64_t)tt << 32);
+    if (lane == 0) s_warp[w] = mine;
+    __syncthreads();
+    uint32_t total = 0, below = 0;
+#pragma unroll
+    for (int i = 0; i < kThreads / 32; i++) {
+        below += i < w ? s_warp[i] : 0;
+        total += s_warp[i];
     }
-}
-
-// a sorted view's neighbour and time arrays from its payload
-__global__ void k_split_view(const uint64_t* __restrict__ pay, int64_t m, int32_t* __restrict__ nbr,
-                             int32_t* __restrict__ tv) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < m;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        uint64_t v = pay[i];
-        nbr[i] = (int32_t)(uint32_t)v;
-        tv[i] = (int32_t)(uint32_t)(v >> 32);
-    }
-}
-
-// the in view as sort input for the pair view: key = source, payload = destination | time
-__global__ void k_pair_keys(const int32_t* __restrict__ in_nbr, const uint32_t* __restrict__ in_dst,
-                            const int32_t* __restrict__ in_t, int64_t m, uint32_t* __restrict__ key,
-                            uint64_t* __restrict__ pay) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < m;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        key[i] = (uint32_t)in_nbr[i];
-        pay[i] = (uint64_t)in_dst[i] | ((uint64_t)(uint32_t)in_t[i] << 32);
-    }
-}
-
-// pair view from (source, destination | time) sorted by source: times, head flags
-__global__ void k_pair_heads_kv(const uint32_t* __restrict__ key, const uint64_t* __restrict__ pay,
-                                int64_t m, int64_t* __restrict__ head, int32_t* __restrict__ pair_t) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < m;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        uint64_t v = pay[i];
-        pair_t[i] = (int32_t)(uint32_t)(v >> 32);
-        head[i] = (i == 0 || key[i] != key[i - 1] || (uint32_t)v != (uint32_t)pay[i - 1]) ? 1 : 0;
-    }
-}
-
-__global__ void k_pair_index_kv(const uint32_t* __restrict__ key, const uint64_t* __restrict__ pay,
-                                const int64_t* __restrict__ head, const int64_t* __restrict__ pid_excl,
-                                int64_t m, int32_t* __restrict__ pair_dst, int64_t* __restrict__ pair_off,
-                                int32_t* __restrict__ pair_src) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < m;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        if (head[i]) {
-            int64_t p = pid_excl[i];
-            pair_dst[p] = (int32_t)(uint32_t)pay[i];
-            pair_off[p] = i;
-            pair_src[p] = (int32_t)key[i];
+    if (threadIdx.x == 0) st_tile(words + tile, tile == 0 ? (kTilePrefix | total) : total + 1);
+    const uint32_t before = look_back_block(words, tile, err);
+    if (threadIdx.x == 0) {
+        if (tile > 0) st_tile(words + tile, kTilePrefix | (before + total));
+        if (tbase + kPairTile >= m) {   // the last tile knows how many pairs there are
+            *P = (int64_t)before + total;
+            pair_off[(int64_t)before + total] = m;
         }
     }
-}
-
-// pid_excl[i] = number of heads before i; a head at i starts pair pid_excl[i]
-__global__ void k_pair_index(const uint32_t* __restrict__ perm, const int32_t* __restrict__ dst,
-                             const int64_t* __restrict__ head, const int64_t* __restrict__ pid_excl,
-                             int64_t m, int32_t* __restrict__ pair_dst, int64_t* __restrict__ pair_off) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < m;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        if (head[i]) {
-            int64_t p = pid_excl[i];
-            pair_dst[p] = dst[perm[i]];
-            pair_off[p] = i;
+    uint32_t run = before + below;   // starts before this round's 32 positions
+#pragma unroll
+    for (int r = 0; r < kPairItems; r++) {
+        const int64_t i = base + r * 32;
+        const uint32_t pid = run + __popc(heads[r] & (0xffffffffu >> (31 - lane))) - 1;
+        if (i < m) {
+            pair_pid[i] = (int32_t)pid;
+            if ((heads[r] >> lane) & 1u) pair_off[TM_CHK_IDX(pid, m, kChkSort)] = i;
         }
+        run += __popc(heads[r]);
     }
 }
 
@@ -193,15 +193,15 @@ __global__ void k_pair_index(const uint32_t* __restrict__ perm, const int32_t* _
 // time-sorted segment of pair_t, stored in the slot as (begin, length) so that a
 // lookup is one 16-byte load.  Capacity is a power of two >= 2 P, so every probe
 // chain ends at an empty slot.
-__global__ void k_hash_insert(const int32_t* __restrict__ pair_src, const int32_t* __restrict__ pair_dst,
+__global__ void k_hash_insert(const int32_t* __restrict__ out_src, const int32_t* __restrict__ pair_dst,
                               const int64_t* __restrict__ pair_off, int64_t P,
                               unsigned long long* __restrict__ slots, unsigned long long mask,
                               uint32_t* __restrict__ filt, unsigned long long fmask) {
     for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < P;
          p += (int64_t)gridDim.x * blockDim.x) {
-        unsigned long long key = ((unsigned long long)(uint32_t)pair_src[p] << 32) | (uint32_t)pair_dst[p];
-        unsigned long long seg = ((unsigned long long)(uint32_t)(pair_off[p + 1] - pair_off[p]) << 32) |
-                                 (uint32_t)pair_off[p];
+        const int64_t at = pair_off[p];   // (the out view and the pair view hold a source at the same positions)
+        unsigned long long key = ((unsigned long long)(uint32_t)out_src[at] << 32) | (uint32_t)pair_dst[at];
+        unsigned long long seg = ((unsigned long long)(uint32_t)(pair_off[p + 1] - at) << 32) | (uint32_t)at;
         unsigned long long h0 = sm64_mix(key);
         atomicOr(filt + ((h0 >> 32) & fmask), (1u << (h0 & 31)) | (1u << ((h0 >> 5) & 31)));
         unsigned long long h = h0 & mask;
@@ -216,37 +216,6 @@ __global__ void k_hash_insert(const int32_t* __restrict__ pair_src, const int32_
     }
 }
 
-__global__ void k_pair_src(const uint32_t* __restrict__ perm, const int32_t* __restrict__ src,
-                           const int64_t* __restrict__ head, const int64_t* __restrict__ pid_excl,
-                           int64_t m, int32_t* __restrict__ pair_src) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < m;
-         i += (int64_t)gridDim.x * blockDim.x)
-        if (head[i]) pair_src[pid_excl[i]] = src[perm[i]];
-}
-
-// pair index of every pair-view position: heads up to and including it, minus one
-__global__ void k_pair_pid(const int64_t* __restrict__ head, const int64_t* __restrict__ pid_excl, int64_t m,
-                           int32_t* __restrict__ pair_pid) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < m;
-         i += (int64_t)gridDim.x * blockDim.x)
-        pair_pid[i] = (int32_t)(pid_excl[i] + head[i] - 1);
-}
-
-__global__ void k_pair_tail(int64_t* __restrict__ pair_off, const int64_t* __restrict__ P, int64_t m) {
-    pair_off[*P] = m;
-}
-
-// pk_off[u] = pair index of the first pair whose source is >= u
-__global__ void k_pk_off(const int64_t* __restrict__ out_off, const int64_t* __restrict__ head,
-                         const int64_t* __restrict__ pid_excl, const int64_t* __restrict__ P,
-                         int64_t m, int32_t n, int64_t* __restrict__ pk_off) {
-    for (int64_t u = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; u <= n;
-         u += (int64_t)gridDim.x * blockDim.x) {
-        int64_t pos = out_off[u];
-        pk_off[u] = pos >= m ? *P : pid_excl[pos];
-    }
-}
-
 int bits_for(int32_t n) {
     int b = 0;
     while (b < 31 && ((int64_t)1 << b) < (int64_t)n) b++;
@@ -255,30 +224,32 @@ int bits_for(int32_t n) {
 
 size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
-// A second stream of the calling thread on device dev, with two events, for the in-view sort
-// that runs beside the out-view sort (null when it cannot be created: the sorts then share st)
-struct SideStream {
-    cudaStream_t s = nullptr;
-    cudaEvent_t fork = nullptr, join = nullptr;
-};
-SideStream* side_stream(int dev) {
-    constexpr int kDevs = 64;
-    thread_local SideStream ss[kDevs];
-    if (dev < 0 || dev >= kDevs) return nullptr;
-    SideStream& x = ss[dev];
-    if (!x.s) {
-        if (cudaStreamCreateWithFlags(&x.s, cudaStreamNonBlocking) != cudaSuccess ||
-            cudaEventCreateWithFlags(&x.fork, cudaEventDisableTiming) != cudaSuccess ||
-            cudaEventCreateWithFlags(&x.join, cudaEventDisableTiming) != cudaSuccess) {
-            cudaGetLastError();
-            x.s = nullptr;
-            return nullptr;
-        }
+// the input checks on their own, for callers that give no n_nodes or whose times span too much:
+// max id through *n_ids
+int check_edges(const int32_t* d_src, const int32_t* d_dst, const int64_t* d_t, int64_t m, int32_t n_nodes,
+                cudaStream_t st, int32_t* n_ids) {
+    int32_t* flags = nullptr;
+    TM_CUDA(cudaMallocAsync((void**)&flags, 4 * sizeof(int32_t), st));
+    int32_t hf[4] = {0, 0, -1, 0};
+    cudaError_t e = cudaMemcpyAsync(flags, hf, sizeof(hf), cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess) {
+        k_validate<<<grid_for(m), kThreads, 0, st>>>(d_src, d_dst, d_t, m, n_nodes, flags); count_launch();
+        e = cudaGetLastError();
     }
-    return &x;
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);   // hf has been read
+    if (e == cudaSuccess) e = cudaMemcpyAsync(hf, flags, sizeof(hf), cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    cudaFreeAsync(flags, st);
+    TM_CUDA(e);
+    if (hf[0]) { set_error("timestamps are not sorted non-decreasingly"); return TM_EUNSORTED; }
+    if (hf[1]) { set_error("node id outside [0, n_nodes)"); return TM_ERANGE; }
+    *n_ids = hf[2] + 1;
+    return TM_OK;
 }
 
-int build_graph(const int32_t* d_src, const int32_t* d_dst, const int64_t* d_t, int64_t m,
+}  // namespace
+
+int build_graph(const int32_t* d_src, const int32_t* d_dst, const int64_t* d_t, const int64_t* h_t, int64_t m,
                 int32_t n_nodes, cudaStream_t st, tm_graph** out) {
     if (!out) { set_error("out is NULL"); return TM_EINVAL; }
     *out = nullptr;
@@ -293,42 +264,39 @@ int build_graph(const int32_t* d_src, const int32_t* d_dst, const int64_t* d_t, 
     nv.next("tm_graph_build");
     int ev0 = pe.mark(st);
     int64_t tmin = 0, tmax = 0;
-    int32_t loops = 0;
     int32_t n = n_nodes < 0 ? 0 : n_nodes;
     if (m > 0) {
-        int32_t* flags = nullptr;
-        TM_CUDA(cudaMallocAsync((void**)&flags, 4 * sizeof(int32_t), st));
-        int32_t init[4] = {0, 0, -1, 0};
-        TM_CUDA(cudaMemcpyAsync(flags, init, sizeof(init), cudaMemcpyHostToDevice, st));
-        k_validate<<<grid_for(m), kThreads, 0, st>>>(d_src, d_dst, d_t, m, n_nodes, flags); count_launch();
-        TM_CUDA(cudaGetLastError());
-        int32_t hf[4];
         int64_t tt[2];
-        TM_CUDA(cudaMemcpyAsync(hf, flags, sizeof(hf), cudaMemcpyDeviceToHost, st));
-        TM_CUDA(cudaMemcpyAsync(&tt[0], d_t, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
-        TM_CUDA(cudaMemcpyAsync(&tt[1], d_t + (m - 1), sizeof(int64_t), cudaMemcpyDeviceToHost, st));
-        TM_CUDA(cudaStreamSynchronize(st));
-        cudaFreeAsync(flags, st);
-        if (hf[0]) { set_error("timestamps are not sorted non-decreasingly"); return TM_EUNSORTED; }
-        if (hf[1]) { set_error("node id outside [0, n_nodes)"); return TM_ERANGE; }
+        if (h_t) {
+            tt[0] = h_t[0];
+            tt[1] = h_t[m - 1];
+        } else {
+            TM_CUDA(cudaMemcpyAsync(&tt[0], d_t, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
+            TM_CUDA(cudaMemcpyAsync(&tt[1], d_t + (m - 1), sizeof(int64_t), cudaMemcpyDeviceToHost, st));
+            TM_CUDA(cudaStreamSynchronize(st));
+        }
+        if (tt[1] < tt[0]) { set_error("timestamps are not sorted non-decreasingly"); return TM_EUNSORTED; }
         tmin = tt[0];
-        tmax = tt[1] - tt[0];
-        if (tt[1] < tt[0] || tmax >= ((int64_t)1 << 61)) { set_error("time span >= 2^61"); return TM_EINVAL; }
-        if (n_nodes < 0) n = hf[2] + 1;
-        loops = hf[3];
+        const uint64_t span = (uint64_t)tt[1] - (uint64_t)tt[0];
+        if (n <= 0 || span >= (uint64_t)1 << 61) {   // ids counted, or a wrong input told apart, first
+            int32_t ids = 0;
+            TM_TRY(check_edges(d_src, d_dst, d_t, m, n_nodes, st, &ids));
+            if (span >= (uint64_t)1 << 61) { set_error("time span >= 2^61"); return TM_EINVAL; }
+            if (n_nodes < 0) n = ids;
+        }
+        tmax = (int64_t)span;
     }
 
     // ---- one allocation for the resident graph
     size_t nN = (size_t)n + 1, M = (size_t)m;
     // time arrays hold int32 when every normalised time fits, else int64
     const int tb = tmax <= (int64_t)INT32_MAX ? 4 : 8;
-    size_t sz_i32m = align256(4 * M), sz_i64m = align256(8 * M), sz_off = align256(8 * nN);
+    size_t sz_i32m = align256(4 * M), sz_off = align256(8 * nN);
     size_t sz_tm = align256((size_t)tb * M);
-    size_t total = 2 * sz_i32m + sz_tm          // src, dst, t
-                 + sz_off + sz_i32m + sz_tm     // out view
-                 + sz_off + sz_i32m + sz_tm     // in view
-                 + sz_off + sz_i32m + align256(8 * (M + 1)) + sz_tm   // pair view (P <= m)
-                 + 3 * sz_i32m;                                          // view keys, pair index
+    size_t total = 2 * sz_i32m + sz_tm              // src, dst, t
+                 + sz_off + 2 * sz_i32m + sz_tm     // out view
+                 + sz_off + 2 * sz_i32m + sz_tm     // in view
+                 + 2 * sz_i32m + align256(8 * (M + 1)) + sz_tm;   // pair view (P <= m)
     tm_graph* g = new (std::nothrow) tm_graph();
     if (!g) { set_error("host allocation failed"); return TM_ENOMEM; }
     g->device = dev;
@@ -349,25 +317,24 @@ int build_graph(const int32_t* d_src, const int32_t* d_dst, const int64_t* d_t, 
     int32_t* gd = (int32_t*)take(sz_i32m);
     void* gt = take(sz_tm);
     int64_t* out_off = (int64_t*)take(sz_off);
+    int32_t* out_src = (int32_t*)take(sz_i32m);
     int32_t* out_nbr = (int32_t*)take(sz_i32m);
     void* out_t = take(sz_tm);
     int64_t* in_off = (int64_t*)take(sz_off);
+    int32_t* in_dst = (int32_t*)take(sz_i32m);
     int32_t* in_nbr = (int32_t*)take(sz_i32m);
     void* in_t = take(sz_tm);
-    int64_t* pk_off = (int64_t*)take(sz_off);
     int32_t* pair_dst = (int32_t*)take(sz_i32m);
+    int32_t* pair_pid = (int32_t*)take(sz_i32m);
     int64_t* pair_off = (int64_t*)take(align256(8 * (M + 1)));
     void* pair_t = take(sz_tm);
-    int32_t* out_src = (int32_t*)take(sz_i32m);
-    int32_t* in_dst = (int32_t*)take(sz_i32m);
-    int32_t* pair_pid = (int32_t*)take(sz_i32m);
 
     GraphDev& G = g->dev;
-    G.m = m; G.n = n; G.tbytes = tb; G.loops = loops;
+    G.m = m; G.n = n; G.tbytes = tb; G.loops = 0;
     G.src = gs; G.dst = gd; G.t = gt;
     G.out_off = out_off; G.out_nbr = out_nbr; G.out_t = out_t;
     G.in_off = in_off; G.in_nbr = in_nbr; G.in_t = in_t;
-    G.pk_off = pk_off; G.pair_dst = pair_dst; G.pair_off = pair_off; G.pair_t = pair_t;
+    G.pair_dst = pair_dst; G.pair_off = pair_off; G.pair_t = pair_t;
     G.out_src = out_src; G.in_dst = in_dst; G.pair_pid = pair_pid;
     G.hslots = nullptr; G.hmask = 0;
     G.pfilt = nullptr; G.pfmask = 0;
@@ -379,7 +346,6 @@ int build_graph(const int32_t* d_src, const int32_t* d_dst, const int64_t* d_t, 
     if (m == 0) {
         TM_CUDA(cudaMemsetAsync(out_off, 0, 8 * nN, st));
         TM_CUDA(cudaMemsetAsync(in_off, 0, 8 * nN, st));
-        TM_CUDA(cudaMemsetAsync(pk_off, 0, 8 * nN, st));
         TM_CUDA(cudaMemsetAsync(pair_off, 0, 8, st));
         TM_CUDA(cudaStreamSynchronize(st));
         g->P = 0;
@@ -388,17 +354,13 @@ int build_graph(const int32_t* d_src, const int32_t* d_dst, const int64_t* d_t, 
         return TM_OK;
     }
 
-    // ---- scratch: keys/values for three sorts (double-buffered) + pair scan
-    uint32_t *ks, *kd, *va, *vb, *kt, *vt;
-    int64_t *head, *pid, *dP;
-    // index path: 6 u32 + 2 i64 per edge; payload path (32-bit times): 3 u32 + 3 u64
-    // (the payload path takes a fourth key and value array when the in-view sort runs on a side
-    // stream beside the out-view sort)
-    SideStream* side = tb == 4 ? side_stream(dev) : nullptr;
-    const int kv = side ? 4 : 3;
-    size_t scratch = std::max(6 * align256(4 * M) + 2 * sz_i64m, kv * align256(4 * M) + kv * sz_i64m) + 256;
+    // ---- scratch: the lists between the passes of two sorts, the sorts' counts and tile words,
+    // and the pair index's tile words.  The sorts' spare words hold the flags and the pair count.
+    const SortDigits D = sort_digits(bits_for(n));
+    const size_t set = 2 * sz_i32m + sz_tm, ws_bytes = align256(sort_ws_bytes(m, D, 3, 2));
+    const size_t pair_tiles = (size_t)((m + kPairTile - 1) / kPairTile), pair_ws = align256(4 * (pair_tiles + 64));
     ScratchLease lease;
-    int lrc = scratch_acquire(scratch, st, lease);
+    int lrc = scratch_acquire(2 * set + ws_bytes + pair_ws, st, lease);
     if (lrc != TM_OK) {
         cudaStreamSynchronize(st);
         pool_free(g->block, dev);
@@ -406,159 +368,80 @@ int build_graph(const int32_t* d_src, const int32_t* d_dst, const int64_t* d_t, 
         return lrc;
     }
     char* q = (char*)lease.p;
-    auto takes = [&](size_t bytes) { char* r = q; q += align256(bytes); return (void*)r; };
-    ks = (uint32_t*)takes(4 * M);
-    kd = (uint32_t*)takes(4 * M);
-    va = (uint32_t*)takes(4 * M);
-    vb = (uint32_t*)takes(4 * M);
-    kt = (uint32_t*)takes(4 * M);
-    vt = (uint32_t*)takes(4 * M);
-    head = (int64_t*)takes(8 * M);
-    pid = (int64_t*)takes(8 * M);
-    dP = (int64_t*)((char*)lease.p + scratch - 256);
+    const SortWs W = sort_ws(q, m, D, 3, 2);
+    uint32_t* flags = W.err + 8;
+    int64_t* dP = (int64_t*)(W.err + 16);
+    uint32_t* pw = (uint32_t*)(q + ws_bytes);
+    q += ws_bytes + pair_ws;
+    SortIo io[2];   // out view: (source; destination, time) by source; in view the other way round
+    for (int k = 0; k < 2; k++) {
+        io[k].key_in = (const uint32_t*)(k ? gd : gs);
+        io[k].a_in = (const uint32_t*)(k ? gs : gd);
+        io[k].t_in = gt;
+        io[k].key_out = (uint32_t*)(k ? in_dst : out_src);
+        io[k].a_out = (uint32_t*)(k ? in_nbr : out_nbr);
+        io[k].t_out = k ? in_t : out_t;
+        io[k].key_tmp = (uint32_t*)q;
+        io[k].a_tmp = (uint32_t*)(q + sz_i32m);
+        io[k].t_tmp = q + 2 * sz_i32m;
+        io[k].counts = k;
+        io[k].keep_key = true;
+        q += set;
+    }
+    // pair view: the in view stably re-sorted by source = (source, destination, time); its
+    // sources are the out view's, so the last pass need not write them
+    SortIo pr = io[0];
+    pr.key_in = (const uint32_t*)in_nbr;
+    pr.a_in = (const uint32_t*)in_dst;
+    pr.t_in = in_t;
+    pr.key_out = io[1].key_tmp;   // (three or more passes go through it)
+    pr.a_out = (uint32_t*)pair_dst;
+    pr.t_out = pair_t;
+    pr.keep_key = false;
 
-    int bits = bits_for(n);
-    unsigned gr = grid_for(m);
-    // the launches below that move timestamps, for the chosen element type
-    auto typed_launch = [&](auto tag, int which, const uint32_t* perm, const int32_t* other, int32_t* nbr,
-                            void* tv) {
-        using TT = decltype(tag);
-        if (which == 0)
-            k_ingest<TT><<<gr, kThreads, 0, st>>>(d_src, d_dst, d_t, m, tmin, gs, gd, (TT*)gt, ks, kd, va, vb);
-        else if (which == 1)
-            k_gather_view<TT><<<gr, kThreads, 0, st>>>(perm, other, (const TT*)gt, m, nbr, (TT*)tv);
-        else
-            k_pair_heads<TT><<<gr, kThreads, 0, st>>>(perm, gs, gd, (const TT*)gt, m, head, (TT*)tv);
+    auto launched = [&]() {
         count_launch();
-    };
-    auto tlaunch = [&](int which, const uint32_t* perm, const int32_t* other, int32_t* nbr, void* tv) {
-        if (tb == 4) typed_launch(int32_t{}, which, perm, other, nbr, tv);
-        else typed_launch(int64_t{}, which, perm, other, nbr, tv);
-    };
-    uint32_t* psrc = nullptr;   // pair sources (the hash keys), in pair order
-    if (tb == 4) {
-        // payload path: scratch laid out as three u32 and three u64 arrays
-        char* q2 = (char*)lease.p;
-        auto take2 = [&](size_t bytes) { char* r = q2; q2 += align256(bytes); return (void*)r; };
-        uint32_t* k0 = (uint32_t*)take2(4 * M);
-        uint32_t* k1 = (uint32_t*)take2(4 * M);
-        uint32_t* k2 = (uint32_t*)take2(4 * M);
-        uint32_t* k3 = side ? (uint32_t*)take2(4 * M) : k0;
-        uint64_t* p0 = (uint64_t*)take2(8 * M);
-        uint64_t* p1 = (uint64_t*)take2(8 * M);
-        uint64_t* p2 = (uint64_t*)take2(8 * M);
-        uint64_t* p3 = side ? (uint64_t*)take2(8 * M) : p0;
-        uint32_t* kr = nullptr;
-        uint64_t* pr = nullptr;
-        k_ingest_kv<<<gr, kThreads, 0, st>>>(d_src, d_dst, d_t, m, tmin, gs, gd, (int32_t*)gt, k0, k1, p0, p1);
-        count_launch();
-        if (cudaGetLastError() != cudaSuccess) rc = TM_ECUDA;
-        // in view: (destination; source | time) stably sorted by destination -- on the side
-        // stream when there is one, beside the out view's sort
-        cudaStream_t sin = side ? side->s : st;
-        if (rc == TM_OK && side && (cudaEventRecord(side->fork, st) != cudaSuccess ||
-                                    cudaStreamWaitEvent(sin, side->fork, 0) != cudaSuccess))
+        if (rc == TM_OK && cudaGetLastError() != cudaSuccess) {
+            set_error("graph build launch failed");
             rc = TM_ECUDA;
-        uint32_t* kr_in = nullptr;
-        uint64_t* pr_in = nullptr;
-        auto in_view = [&]() {
-            if (rc == TM_OK) rc = radix_sort_kv64(k1, p1, k3, p3, m, bits, sin, &kr_in, &pr_in);
-            if (rc == TM_OK) {
-                k_offsets<<<grid_for(m + 1), kThreads, 0, sin>>>(kr_in, m, n, in_off); count_launch();
-                k_split_view<<<gr, kThreads, 0, sin>>>(pr_in, m, in_nbr, (int32_t*)in_t); count_launch();
-                if (cudaGetLastError() != cudaSuccess) rc = TM_ECUDA;
-                if (rc == TM_OK && cudaMemcpyAsync(in_dst, kr_in, 4 * M, cudaMemcpyDeviceToDevice, sin) != cudaSuccess)
-                    rc = TM_ECUDA;
-            }
-            if (side && cudaEventRecord(side->join, sin) != cudaSuccess && rc == TM_OK) rc = TM_ECUDA;
-        };
-        if (side) in_view();
-        // out view: (source; destination | time) stably sorted by source
-        if (rc == TM_OK) rc = radix_sort_kv64(k0, p0, k2, p2, m, bits, st, &kr, &pr);
-        if (rc == TM_OK) {
-            k_offsets<<<grid_for(m + 1), kThreads, 0, st>>>(kr, m, n, out_off); count_launch();
-            k_split_view<<<gr, kThreads, 0, st>>>(pr, m, out_nbr, (int32_t*)out_t); count_launch();
-            if (cudaGetLastError() != cudaSuccess) rc = TM_ECUDA;
-            if (rc == TM_OK && cudaMemcpyAsync(out_src, kr, 4 * M, cudaMemcpyDeviceToDevice, st) != cudaSuccess)
-                rc = TM_ECUDA;
         }
-        if (side) {
-            // the pair view needs the in view, and reuses the in-view sort's arrays
-            if (cudaStreamWaitEvent(st, side->join, 0) != cudaSuccess && rc == TM_OK) rc = TM_ECUDA;
-        } else {
-            in_view();   // after the out view, in its arrays (k0 / p0 are free again)
-        }
-        // pair view: the in view stably re-sorted by source = (source, destination, time)
-        if (rc == TM_OK) {
-            k_pair_keys<<<gr, kThreads, 0, st>>>(in_nbr, (const uint32_t*)in_dst, (const int32_t*)in_t, m, k2, p2);
-            count_launch();
-            if (cudaGetLastError() != cudaSuccess) rc = TM_ECUDA;
-        }
-        if (rc == TM_OK) rc = radix_sort_kv64(k2, p2, k0, p0, m, bits, st, &kr, &pr);
-        // heads and pair indices in the u64 arrays the sort left free; sources in a free u32 one
-        int64_t* hd = (int64_t*)p1;
-        int64_t* pd = (int64_t*)(pr == p2 ? p0 : p2);
-        psrc = kr == k2 ? k0 : k2;
-        if (rc == TM_OK) {
-            k_pair_heads_kv<<<gr, kThreads, 0, st>>>(kr, pr, m, hd, (int32_t*)pair_t); count_launch();
-            if (cudaGetLastError() != cudaSuccess) rc = TM_ECUDA;
-        }
-        if (rc == TM_OK) rc = scan_exclusive_i64(hd, pd, m, dP, st);
-        if (rc == TM_OK) {
-            k_pair_index_kv<<<gr, kThreads, 0, st>>>(kr, pr, hd, pd, m, pair_dst, pair_off, (int32_t*)psrc);
-            count_launch();
-            k_pair_tail<<<1, 1, 0, st>>>(pair_off, dP, m); count_launch();
-            k_pk_off<<<grid_for((int64_t)n + 1), kThreads, 0, st>>>(out_off, hd, pd, dP, m, n, pk_off); count_launch();
-            k_pair_pid<<<gr, kThreads, 0, st>>>(hd, pd, m, pair_pid); count_launch();
-            if (cudaGetLastError() != cudaSuccess) rc = TM_ECUDA;
-        }
-    } else {
-        tlaunch(0, nullptr, nullptr, nullptr, nullptr);
-        if (cudaGetLastError() != cudaSuccess) rc = TM_ECUDA;
-        // out view: edges stably sorted by source (time order kept inside a source)
-        if (rc == TM_OK) rc = radix_sort_pairs(ks, va, kt, vt, m, bits, st);
-        if (rc == TM_OK) {
-            k_offsets<<<grid_for(m + 1), kThreads, 0, st>>>(ks, m, n, out_off); count_launch();
-            tlaunch(1, va, gd, out_nbr, out_t);
-            if (cudaGetLastError() != cudaSuccess) rc = TM_ECUDA;
-            if (rc == TM_OK && cudaMemcpyAsync(out_src, ks, 4 * M, cudaMemcpyDeviceToDevice, st) != cudaSuccess)
-                rc = TM_ECUDA;
-        }
-        // in view: stably sorted by destination
-        if (rc == TM_OK) rc = radix_sort_pairs(kd, vb, kt, vt, m, bits, st);
-        if (rc == TM_OK) {
-            k_offsets<<<grid_for(m + 1), kThreads, 0, st>>>(kd, m, n, in_off); count_launch();
-            tlaunch(1, vb, gs, in_nbr, in_t);
-            if (cudaGetLastError() != cudaSuccess) rc = TM_ECUDA;
-            if (rc == TM_OK && cudaMemcpyAsync(in_dst, kd, 4 * M, cudaMemcpyDeviceToDevice, st) != cudaSuccess)
-                rc = TM_ECUDA;
-        }
-        // pair view: the in-view order stably re-sorted by source = (src, dst, time)
-        if (rc == TM_OK) {
-            tlaunch(1, vb, gs, (int32_t*)ks, head);   // sources in in-view order; times go to scratch
-            if (cudaGetLastError() != cudaSuccess) rc = TM_ECUDA;
-        }
-        if (rc == TM_OK) rc = radix_sort_pairs(ks, vb, kt, vt, m, bits, st);
-        if (rc == TM_OK) {
-            tlaunch(2, vb, nullptr, nullptr, pair_t);
-            if (cudaGetLastError() != cudaSuccess) rc = TM_ECUDA;
-        }
-        if (rc == TM_OK) rc = scan_exclusive_i64(head, pid, m, dP, st);
-        if (rc == TM_OK) {
-            k_pair_index<<<gr, kThreads, 0, st>>>(vb, gd, head, pid, m, pair_dst, pair_off); count_launch();
-            k_pair_tail<<<1, 1, 0, st>>>(pair_off, dP, m); count_launch();
-            k_pk_off<<<grid_for((int64_t)n + 1), kThreads, 0, st>>>(out_off, head, pid, dP, m, n, pk_off); count_launch();
-            k_pair_src<<<gr, kThreads, 0, st>>>(vb, gs, head, pid, m, (int32_t*)kt); count_launch();
-            psrc = kt;
-            k_pair_pid<<<gr, kThreads, 0, st>>>(head, pid, m, pair_pid); count_launch();
-            if (cudaGetLastError() != cudaSuccess) rc = TM_ECUDA;
-        }
+    };
+    rc = sort_clear(W, st);
+    if (rc == TM_OK && cudaMemsetAsync(pw, 0, pair_ws, st) != cudaSuccess) rc = TM_ECUDA;
+    if (rc == TM_OK) {
+        const size_t sm = (size_t)8 * D.passes << D.db;
+        const unsigned gi = (unsigned)std::min<int64_t>((m + 4 * kIngestThreads - 1) / (4 * kIngestThreads), (int64_t)sm_count() * 4);
+        if (tb == 4)
+            k_ingest<int32_t><<<gi, kIngestThreads, sm, st>>>(d_src, d_dst, d_t, m, tmin, n, gs, gd, (int32_t*)gt, flags, D, W.counts);
+        else
+            k_ingest<int64_t><<<gi, kIngestThreads, sm, st>>>(d_src, d_dst, d_t, m, tmin, n, gs, gd, (int64_t*)gt, flags, D, W.counts);
+        launched();
+    }
+    if (rc == TM_OK) rc = sort_bases(W, st);
+    if (rc == TM_OK) rc = sort_run(W, io, 2, 0, tb, st);
+    if (rc == TM_OK) rc = sort_run(W, &pr, 1, 2, tb, st);
+    if (rc == TM_OK) {
+        k_offsets<<<dim3(grid_for(m + 1), 2), kThreads, 0, st>>>((const uint32_t*)out_src, (const uint32_t*)in_dst, m, n, out_off, in_off);
+        launched();
+    }
+    if (rc == TM_OK) {
+        k_pairs<<<(unsigned)pair_tiles, kThreads, 0, st>>>((const uint32_t*)out_src, (const uint32_t*)pair_dst, m, pair_pid,
+                                                           pair_off, pw, pw + 64, W.err, dP);
+        launched();
     }
     int64_t P = 0;
     if (rc == TM_OK) {
-        e = cudaMemcpyAsync(&P, dP, 8, cudaMemcpyDeviceToHost, st);
+        uint32_t h[24];   // error word, flags, pair count
+        e = cudaMemcpyAsync(h, W.err, sizeof(h), cudaMemcpyDeviceToHost, st);
         if (e == cudaSuccess) e = cudaStreamSynchronize(st);
         if (e != cudaSuccess) rc = cuda_status(e, "graph build", __FILE__, __LINE__);
+        else if (h[8]) { set_error("timestamps are not sorted non-decreasingly"); rc = TM_EUNSORTED; }
+        else if (h[9]) { set_error("node id outside [0, n_nodes)"); rc = TM_ERANGE; }
+        else if (h[0]) { set_error("graph build: a wait for an earlier tile expired"); rc = TM_ECUDA; }
+        else {
+            G.loops = h[11] ? 1 : 0;
+            std::memcpy(&P, h + 16, 8);
+        }
     }
     // pair hash: capacity the next power of two >= 2 P; then the pair filter: 8 bits per pair
     // (a power of two of 32-bit words), at most 32 MB so that it stays in L2
@@ -579,7 +462,7 @@ int build_graph(const int32_t* d_src, const int32_t* d_dst, const int64_t* d_t, 
             e = cudaMemsetAsync(g->hash_block, 0xff, 16 * cap, st);
             if (e == cudaSuccess) e = cudaMemsetAsync(filt, 0, 4 * fw, st);
             if (e == cudaSuccess) {
-                k_hash_insert<<<grid_for(P), kThreads, 0, st>>>((const int32_t*)psrc, pair_dst, pair_off, P,
+                k_hash_insert<<<grid_for(P), kThreads, 0, st>>>(out_src, pair_dst, pair_off, P,
                                                                (unsigned long long*)g->hash_block, cap - 1,
                                                                filt, fw - 1);
                 count_launch();
@@ -605,6 +488,8 @@ int build_graph(const int32_t* d_src, const int32_t* d_dst, const int64_t* d_t, 
     return TM_OK;
 }
 
+namespace {
+
 // Two-node tables.  For pair-view position e of pair (u, v) at time t_e:
 //   own[e] = number of (u, v) edges with time < t_e, rev[e] = number of (v, u) edges with
 //   time < t_e;
@@ -622,7 +507,7 @@ __global__ void k_ex_rank(GraphDevT<TT> G, int reverse, int64_t* __restrict__ ou
             if (e > pa && (int64_t)G.pair_t[e - 1] == te) r = lower_bound_i64(G.pair_t, pa, e, te) - pa;
             out[e] = r;
         } else {
-            int32_t u = G.out_src[e], v = G.pair_dst[pid];
+            int32_t u = G.out_src[e], v = G.pair_dst[e];
             int64_t ra, rb;
             out[e] = pair_segment(G, v, u, ra, rb) ? lower_bound_i64(G.pair_t, ra, rb, te) - ra : 0;
         }
@@ -682,7 +567,7 @@ extern "C" {
 
 int tm_graph_load_device(const int32_t* d_src, const int32_t* d_dst, const int64_t* d_t, int64_t m,
                          int32_t n_nodes, void* stream, tm_graph** out) {
-    return tmo::build_graph(d_src, d_dst, d_t, m, n_nodes, (cudaStream_t)stream, out);
+    return tmo::build_graph(d_src, d_dst, d_t, nullptr, m, n_nodes, (cudaStream_t)stream, out);
 }
 
 int tm_graph_load(const int32_t* src, const int32_t* dst, const int64_t* t, int64_t m,
@@ -708,7 +593,7 @@ int tm_graph_load(const int32_t* src, const int32_t* dst, const int64_t* t, int6
     if (e == cudaSuccess && m > 0) e = cudaMemcpyAsync(dd, dst, 4 * (size_t)m, cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess && m > 0) e = cudaMemcpyAsync(dt, t, 8 * (size_t)m, cudaMemcpyHostToDevice, st);
     if (e != cudaSuccess) rc = tmo::cuda_status(e, "tm_graph_load copy", __FILE__, __LINE__);
-    if (rc == TM_OK) rc = tmo::build_graph(ds, dd, dt, m, n_nodes, st, out);
+    if (rc == TM_OK) rc = tmo::build_graph(ds, dd, dt, t, m, n_nodes, st, out);
     tmo::scratch_release(lease, st);
     cudaStreamSynchronize(st);
     cudaStreamDestroy(st);

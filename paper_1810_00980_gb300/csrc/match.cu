@@ -240,7 +240,7 @@ __device__ __forceinline__ void first_edge(const GraphDevT<TT>& G, int order, in
         s = __ldg(G.in_nbr + e); d = __ldg(G.in_dst + e); t = __ldg(G.in_t + e);
     } else if (order == kOrdPair) {
         // the pair view is grouped by source at the same positions as the out view
-        s = __ldg(G.out_src + e); d = __ldg(G.pair_dst + __ldg(G.pair_pid + e)); t = __ldg(G.pair_t + e);
+        s = __ldg(G.out_src + e); d = __ldg(G.pair_dst + e); t = __ldg(G.pair_t + e);
     } else {
         s = __ldg(G.src + e); d = __ldg(G.dst + e); t = __ldg(G.t + e);
     }
@@ -2104,7 +2104,7 @@ int run_batch_t(const tm_graph* g, const tm_query* qs, int nq, tm_result* res, c
     size_t NWs = (size_t)std::max<int64_t>(NW, 1);
     size_t Ms = (size_t)std::max<int64_t>(g->m, 1);
     size_t sz = a256(plans_bytes((size_t)nq)) + a256(sizeof(tm_result) * (size_t)nq) + wtab_bytes +
-                9 * a256(8 * NWs) + 3 * a256(4 * NWs) + a256(8 * NWs) + a256(8 * A_N * NWs) + 4 * 256 +
+                9 * a256(8 * NWs) + 3 * a256(4 * NWs) + a256(8 * NWs) + a256(8 * A_N * NWs) + 5 * 256 +
                 full_bytes + (any_full ? 3 * a256(4 * Ms) : 0) +
                 a256(sizeof(ShiftSums) * (size_t)std::max<int64_t>(n_sums, 1)) +
                 a256(sizeof(ShiftSums) * (size_t)n_parts) +
@@ -2145,6 +2145,7 @@ int run_batch_t(const tm_graph* g, const tm_query* qs, int nq, tm_result* res, c
     int64_t* dW2 = (int64_t*)take(8);
     unsigned long long* dctr = (unsigned long long*)take(8);
     unsigned long long* drcount = (unsigned long long*)take(8);
+    uint32_t* dserr = (uint32_t*)take(8);   // the window sorts' error word
     ShiftSums* dsums = (ShiftSums*)take(sizeof(ShiftSums) * (size_t)std::max<int64_t>(n_sums, 1));
     ShiftSums* dpart = (ShiftSums*)take(sizeof(ShiftSums) * (size_t)n_parts);
     unsigned long long* dsubc = (unsigned long long*)take(8 * kMaxSub * (size_t)nq);
@@ -2166,6 +2167,7 @@ int run_batch_t(const tm_graph* g, const tm_query* qs, int nq, tm_result* res, c
     int ev_w0 = pe.mark(st), ev_w1 = -1, ev_l0 = -1, ev_l1 = -1, ev_l2 = -1, ev_m1 = -1, ev_r1 = -1, ev_f1 = -1;
     int64_t hW2 = 0;
     unsigned long long h_rcount = 0;
+    uint32_t h_serr = 0;
     std::vector<char> h_plans;
     fail(copy_plans(hp, wown, h_plans, dplans, st), "plans");
     if (!h_shifts.empty())
@@ -2173,6 +2175,7 @@ int run_batch_t(const tm_graph* g, const tm_query* qs, int nq, tm_result* res, c
     fail(cudaMemsetAsync(W.acc, 0, 8 * A_N * NWs, st), "acc");
     fail(cudaMemsetAsync(dctr, 0, 8, st), "counter");
     fail(cudaMemsetAsync(drcount, 0, 8, st), "record counter");
+    if (any_full) fail(cudaMemsetAsync(dserr, 0, 8, st), "sort error word");
     if (rc == TM_OK) {
         launch_wtabs(hp, wown, dplans, st);
         fail(cudaGetLastError(), "k_wtab");
@@ -2193,7 +2196,7 @@ int run_batch_t(const tm_graph* g, const tm_query* qs, int nq, tm_result* res, c
             unsigned gr = (unsigned)std::min<int64_t>((g->m + 255) / 256, (int64_t)nsm * 8);
             k_winkey<TT><<<gr, 256, 0, st>>>(tv, g->m, sft, P.cd, pk_key, vals); count_launch();
             fail(cudaGetLastError(), "k_winkey");
-            if (rc == TM_OK) rc = radix_sort_pairs(pk_key, vals, pk_ktmp, pk_vtmp, g->m, bits, st);
+            if (rc == TM_OK) rc = radix_sort_pairs(pk_key, vals, pk_ktmp, pk_vtmp, g->m, bits, dserr, st);
             if (rc == TM_OK) {
                 k_woff<<<(unsigned)std::min<int64_t>((g->m + 256) / 256, (int64_t)nsm * 8), 256, 0, st>>>(
                     pk_key, g->m, P.J, (int64_t*)(P.woff + (size_t)k * (size_t)(P.J + 1)));
@@ -2294,6 +2297,7 @@ int run_batch_t(const tm_graph* g, const tm_query* qs, int nq, tm_result* res, c
         if (ev_m1 < 0) ev_m1 = ev_f0;
         if (ev_r1 < 0) ev_r1 = ev_m1;
     }
+    if (rc == TM_OK && any_full) fail(cudaMemcpyAsync(&h_serr, dserr, 4, cudaMemcpyDeviceToHost, st), "sort error word");
     if (rc == TM_OK && any_share) fail(cudaMemcpyAsync(&h_rcount, drcount, 8, cudaMemcpyDeviceToHost, st), "records");
     if (rc == TM_OK) fail(cudaMemcpyAsync(res, dres, sizeof(tm_result) * (size_t)nq, cudaMemcpyDeviceToHost, st), "results");
     if (rc == TM_OK && dbg && dbg->sub_count)
@@ -2331,6 +2335,10 @@ int run_batch_t(const tm_graph* g, const tm_query* qs, int nq, tm_result* res, c
     }
     cudaError_t se = cudaStreamSynchronize(st);
     fail(se, "batch sync");
+    if (rc == TM_OK && h_serr) {
+        set_error("window partition: a wait for an earlier tile expired");
+        rc = TM_ECUDA;
+    }
     if (pe.on && rc == TM_OK) {
         double wall = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - wall0).count();
         store_profile_batch(pe.ms(ev_w0, ev_w1), pe.ms(ev_l0, ev_l2), ev_l1 >= 0 ? pe.ms(ev_l1, ev_m1) : 0.0,

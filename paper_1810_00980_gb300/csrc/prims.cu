@@ -1,7 +1,7 @@
-// Device primitives: exclusive scan of int64 and a stable LSD radix sort of
-// (uint32 key, uint32 value) pairs.  Neither waits on other blocks: the scan
-// is reduce-then-scan over tiles, the sort is histogram / scan / scatter per
-// digit, so no launch can spin.
+// Device primitives: exclusive scan of int64 (reduce-then-scan over tiles: no block waits on
+// another) and a stable LSD radix sort of 32-bit keys with up to 12 bytes of payload (a tile
+// waits, with a limit, for the counts of earlier tiles).
+#include <algorithm>
 #include <mutex>
 #include <vector>
 
@@ -236,192 +236,252 @@ __global__ void k_scan_small_dn(const int64_t* in, int64_t* out, const int64_t* 
 }
 
 // ------------------------------------------------------------------ radix sort
+// Stable LSD radix sort of (key, a[, t]) triples by digits of up to 10 bits, one kernel per
+// digit.  The digit counts of the whole input, for every digit, come from one earlier read
+// (digit_count_block, inside the kernel that produces the keys, or k_digit_count); a pass then
+// finds each tile's place in every digit's run from the tiles before it (decoupled look-back:
+// Merrill and Garland, "Single-pass parallel prefix scan with decoupled look-back", 2016; used
+// for radix sorting by Adinets and Merrill, "Onesweep", 2022), so it reads and writes each
+// triple once and nothing else of size n.  The passes it replaces read every key a second time
+// for a histogram per tile and scanned 2^bits x tiles counters with three more kernels.
+//
+// What bounds a pass: HBM, at 2 x 12 bytes per key with 32-bit times.  A tile is 4096 keys, all
+// of its loads in flight at once, so that three tiles per SM cover the memory's latency; each
+// digit's run of the tile leaves shared memory as neighbouring addresses.
 constexpr int kSortThreads = 256;
 constexpr int kSortWarps = kSortThreads / 32;
-constexpr int kSortItems = 16;                       // per lane
+constexpr int kSortItems = 16;                       // per thread
 constexpr int kSortTile = kSortThreads * kSortItems; // 4096
-constexpr int kMaxDigitBits = 10;
 
-__global__ void k_radix_hist(const uint32_t* __restrict__ keys, int64_t n, int shift, int db,
-                             int32_t* __restrict__ hist, int64_t ntiles) {
-    __shared__ int32_t h[1 << kMaxDigitBits];
-    int nd = 1 << db;
-    for (int i = threadIdx.x; i < nd; i += blockDim.x) h[i] = 0;
-    __syncthreads();
-    int64_t base = (int64_t)blockIdx.x * kSortTile;
-    uint32_t mask = (uint32_t)nd - 1;
-    for (int i = threadIdx.x; i < kSortTile; i += blockDim.x) {
-        int64_t idx = base + i;
-        if (idx < n) atomicAdd(&h[(keys[idx] >> shift) & mask], 1);
+// lanes of `act` holding the same DB-bit digit: one ballot per bit (independent of one another,
+// unlike the compare-and-vote loop behind __match_any_sync)
+template <int DB>
+__device__ __forceinline__ unsigned same_digit(uint32_t d, unsigned act) {
+    unsigned m = act;
+#pragma unroll
+    for (int b = 0; b < DB; b++) {
+        const bool bit = (d >> b) & 1u;
+        const unsigned v = __ballot_sync(kFull, bit);
+        m &= bit ? v : ~v;
     }
-    __syncthreads();
-    for (int i = threadIdx.x; i < nd; i += blockDim.x) hist[(int64_t)i * ntiles + blockIdx.x] = h[i];
+    return m;
 }
 
-// Stable scatter of one tile: warp w owns items [w*512, w*512+512) of the
-// tile, taken 32 at a time in index order; ranks among equal digits come from
-// __match_any_sync and per-warp running counters, then warps are offset by
-// the counts of lower warps.  The tile is first reordered by digit in shared
-// memory, so that neighbouring threads write neighbouring addresses of one
-// digit's output run (coalesced) instead of scattering single words.
-// Dynamic shared memory: kSortTile keys and values, per-warp digit counters,
-// and per-digit tile starts and output bases (sort_smem_bytes(db)).
-template <typename V>
-__global__ void __launch_bounds__(kSortThreads)
-k_radix_scatter(const uint32_t* __restrict__ kin, const V* __restrict__ vin,
-                uint32_t* __restrict__ kout, V* __restrict__ vout, int64_t n, int shift,
-                int db, const int64_t* __restrict__ offs, int64_t ntiles) {
+// exclusive scan over the block of one value per thread (sm: one word per warp)
+__device__ __forceinline__ uint32_t block_excl_scan_u32(uint32_t v, uint32_t* sm) {
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    uint32_t inc = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(kFull, inc, o);
+        if (lane >= o) inc += y;
+    }
+    if (lane == 31) sm[w] = inc;
+    __syncthreads();
+    uint32_t before = 0;
+#pragma unroll
+    for (int i = 0; i < kSortWarps; i++) before += i < w ? sm[i] : 0;
+    return before + inc - v;
+}
+
+template <int TB> struct SortTime { using type = uint64_t; };
+template <> struct SortTime<4> { using type = uint32_t; };
+
+template <int TB, int DB>
+constexpr size_t sort_smem_bytes() {
+    constexpr size_t cnt = (size_t)2 * kSortWarps << DB, keys = (size_t)4 * kSortTile;
+    return (size_t)kSortTile * (TB + 4 + 2) + (cnt > keys ? cnt : keys) + ((size_t)8 << DB);
+}
+
+// `bytes` bytes from src to the tile's place in shared memory without going through registers:
+// 16 at a time where src allows it, else word by word
+__device__ __forceinline__ void stage_tile(void* dst, const void* src, uint32_t bytes) {
+    const uint32_t to = (uint32_t)__cvta_generic_to_shared(dst);
+    const char* from = (const char*)src;
+    if (((uintptr_t)from & 15) == 0) {
+        for (uint32_t o = threadIdx.x * 16; o < bytes; o += kSortThreads * 16) {
+            const uint32_t left = bytes - o < 16 ? bytes - o : 16;
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(to + o), "l"(from + o), "r"(left) : "memory");
+        }
+    } else {
+        for (uint32_t o = threadIdx.x * 4; o < bytes; o += kSortThreads * 4)
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(to + o), "l"(from + o) : "memory");
+    }
+}
+
+// One pass of one or two independent sorts (block b works on sort b mod J.jobs): warp w of a tile
+// owns its items [512 w, 512 w + 512), 32 at a time in index order; ranks among equal digits are
+// the lane order inside a ballot and the warp's running counters, then warps are offset by the
+// counts of lower warps.  The payload waits in shared memory in input order while the keys are
+// ranked (held in registers it spilled); the tile is put in digit order as (key, input slot).
+template <int TB, int DB>
+__global__ void __launch_bounds__(kSortThreads, TB == 8 ? 2 : 3) k_sort_pass(SortJobs J, int64_t n, int shift) {
+    using T = typename SortTime<TB>::type;
+    constexpr int ND = 1 << DB;
+    constexpr int PER = ND > kSortThreads ? ND / kSortThreads : 1;   // digits per thread
+    static_assert(ND <= kSortThreads || ND % kSortThreads == 0, "a thread's digits must not pass the last");
     extern __shared__ __align__(16) unsigned char sm_sort[];
-    int nd = 1 << db;
-    uint32_t* skey = (uint32_t*)sm_sort;                        // [kSortTile]
-    V* sval = (V*)(skey + kSortTile);                           // [kSortTile]
-    int64_t* gbase = (int64_t*)(sval + kSortTile);              // [nd] output index of tile slot 0 of digit d
-    int32_t* cnt = (int32_t*)(gbase + nd);                      // [kSortWarps][nd]
-    int32_t* tds = cnt + kSortWarps * nd;                       // [nd] tile start of digit d
-    uint32_t mask = (uint32_t)nd - 1;
-    int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    for (int i = lane; i < nd; i += 32) cnt[w * nd + i] = 0;
-    __syncwarp();
-    int64_t tbase = (int64_t)blockIdx.x * kSortTile;
-    int64_t base = tbase + (int64_t)w * (kSortItems * 32);
-    uint32_t key[kSortItems];
-    int32_t rank[kSortItems];
-    unsigned lt = (1u << lane) - 1u;
+    T* st = (T*)sm_sort;                                            // [TB ? tile : 0] input order
+    uint32_t* sa = (uint32_t*)(sm_sort + (size_t)TB * kSortTile);   // [tile] input order
+    uint32_t* gbase = sa + kSortTile;                        // [ND] output index of tile slot 0 of the digit
+    uint32_t* tds = gbase + ND;                              // [ND] tile start of the digit
+    uint16_t* slot = (uint16_t*)(tds + ND);                  // [tile] digit order -> input order
+    uint32_t* sk = (uint32_t*)(slot + kSortTile);            // [tile] keys in digit order, once the
+    uint16_t* cnt = (uint16_t*)sk;                           // [warps][ND] counters are done with
+    __shared__ uint32_t s_tile, red[kSortWarps];
+    const SortJob job = (J.jobs == 2 && (blockIdx.x & 1)) ? J.job[1] : J.job[0];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    if (threadIdx.x == 0) s_tile = atomicAdd(job.ticket, 1u);
+    for (int i = threadIdx.x; i < kSortWarps * ND / 2; i += kSortThreads) ((uint32_t*)cnt)[i] = 0;
+    __syncthreads();
+    const int64_t tile = s_tile;
+    const int64_t tbase = tile * kSortTile;
+    const int tn = (int)min((int64_t)kSortTile, n - tbase);
+    if (tn <= 0) return;
+    const int wbase = w * (kSortItems * 32) + lane;
+    uint32_t key[kSortItems], rank[kSortItems];
+#pragma unroll
+    for (int r = 0; r < kSortItems; r++) key[r] = wbase + r * 32 < tn ? __ldg(job.key_in + tbase + wbase + r * 32) : 0u;
+    stage_tile(sa, job.a_in + tbase, 4u * (uint32_t)tn);
+    if constexpr (TB != 0) stage_tile(st, (const T*)job.t_in + tbase, (uint32_t)TB * (uint32_t)tn);
+    uint16_t* wc = cnt + w * ND;
 #pragma unroll
     for (int r = 0; r < kSortItems; r++) {
-        int64_t idx = base + r * 32 + lane;
-        bool ok = idx < n;
-        key[r] = ok ? kin[idx] : 0u;
-        uint32_t d = ok ? ((key[r] >> shift) & mask) : 0xffffffffu;
-        unsigned peers = __match_any_sync(kFull, d);
-        int before = __popc(peers & lt);
-        int32_t c0 = ok ? cnt[w * nd + d] : 0;
-        rank[r] = c0 + before;
+        const bool ok = wbase + r * 32 < tn;
+        const uint32_t d = (key[r] >> shift) & (ND - 1);
+        const unsigned peers = same_digit<DB>(d, __ballot_sync(kFull, ok));
+        const uint32_t c0 = wc[d];
+        rank[r] = c0 + __popc(peers & ((1u << lane) - 1u));
         __syncwarp();
-        int leader = 31 - __clz(peers);
-        if (ok && lane == leader) cnt[w * nd + d] = c0 + __popc(peers);
+        if (ok && (peers >> lane) == 1u) wc[d] = (uint16_t)(c0 + __popc(peers));   // the highest peer
         __syncwarp();
     }
     __syncthreads();
-    // per digit: warp offsets inside the digit, the digit's total in tds (scanned below)
-    for (int d = threadIdx.x; d < nd; d += blockDim.x) {
-        int32_t run = 0;
+    // per digit: the warps' offsets inside it and the tile's count, told to the tiles behind
+    uint32_t tot[PER], sum = 0;
+    uint32_t* words = job.words + tile * ND;
+    const int d0 = threadIdx.x * PER;
+    if (d0 < ND) {
 #pragma unroll
-        for (int ww = 0; ww < kSortWarps; ww++) {
-            int32_t c = cnt[ww * nd + d];
-            cnt[ww * nd + d] = run;
-            run += c;
-        }
-        tds[d] = run;
-    }
-    __syncthreads();
-    if (w == 0) {   // exclusive scan of the digit totals (nd <= 1024: 32 per lane at most)
-        int per = (nd + 31) / 32;
-        int32_t sum = 0;
-        for (int i = 0; i < per; i++) {
-            int d = lane * per + i;
-            if (d < nd) sum += tds[d];
-        }
-        int32_t inc = sum;
+        for (int x = 0; x < PER; x++) {
+            uint32_t run = 0;
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            int32_t y = __shfl_up_sync(kFull, inc, o);
-            if (lane >= o) inc += y;
-        }
-        int32_t run = inc - sum;
-        for (int i = 0; i < per; i++) {
-            int d = lane * per + i;
-            if (d < nd) {
-                int32_t c = tds[d];
-                tds[d] = run;
+            for (int i = 0; i < kSortWarps; i++) {
+                const uint32_t c = cnt[i * ND + d0 + x];
+                cnt[i * ND + d0 + x] = (uint16_t)run;
                 run += c;
             }
+            tot[x] = run;
+            sum += run;
+            st_tile(words + d0 + x, tile == 0 ? (kTilePrefix | run) : run + 1);
+        }
+    }
+    uint32_t at = block_excl_scan_u32(sum, red);
+    if (d0 < ND) {
+#pragma unroll
+        for (int x = 0; x < PER; x++) {
+            tds[d0 + x] = at;
+            at += tot[x];
         }
     }
     __syncthreads();
-    for (int d = threadIdx.x; d < nd; d += blockDim.x)
-        gbase[d] = offs[(int64_t)d * ntiles + blockIdx.x] - tds[d];
 #pragma unroll
     for (int r = 0; r < kSortItems; r++) {
-        int64_t idx = base + r * 32 + lane;
-        if (idx < n) {
-            uint32_t d = (key[r] >> shift) & mask;
-            int32_t lp = tds[d] + cnt[w * nd + d] + rank[r];
-            skey[lp] = key[r];
-            sval[lp] = vin[idx];   // values are read here, not held through the ranking
+        const uint32_t d = (key[r] >> shift) & (ND - 1);
+        rank[r] += tds[d] + wc[d];
+    }
+    __syncthreads();   // the counters give way to the keys
+#pragma unroll
+    for (int r = 0; r < kSortItems; r++) {
+        if (wbase + r * 32 < tn) {
+            sk[rank[r]] = key[r];
+            slot[rank[r]] = (uint16_t)(wbase + r * 32);
         }
     }
+    // each digit's place in the output
+    if (d0 < ND) {
+#pragma unroll
+        for (int x = 0; x < PER; x++) {
+            uint32_t before = 0;
+            if (tile > 0) {
+                before = look_back(job.words + d0 + x, tile, ND, J.err);
+                st_tile(words + d0 + x, kTilePrefix | (before + tot[x]));
+            }
+            gbase[d0 + x] = job.base[d0 + x] + before - tds[d0 + x];
+        }
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();
-    int64_t tn = min((int64_t)kSortTile, n - tbase);
-    for (int i = threadIdx.x; i < tn; i += blockDim.x) {
-        uint32_t k = skey[i];
-        int64_t pos = TM_CHK_IDX(gbase[(k >> shift) & mask] + i, n, kChkSort);
-        kout[pos] = k;
-        vout[pos] = sval[i];
+    for (int i = threadIdx.x; i < tn; i += kSortThreads) {
+        const uint32_t k = sk[i], o = slot[i];
+        const int64_t pos = TM_CHK_IDX((int64_t)(uint32_t)(gbase[(k >> shift) & (ND - 1)] + (uint32_t)i), n, kChkSort);
+        if (job.key_out) job.key_out[pos] = k;
+        job.a_out[pos] = sa[o];
+        if constexpr (TB != 0) ((T*)job.t_out)[pos] = st[o];
     }
 }
 
-template <typename V>
-size_t sort_smem_bytes(int db) {
-    size_t nd = (size_t)1 << db;
-    return (4 + sizeof(V)) * (size_t)kSortTile + 8 * nd + 4 * nd * (kSortWarps + 1);
+// counts of every digit of every pass of `keys` (counts[pass][digit], zeroed before)
+__global__ void k_digit_count(const uint32_t* __restrict__ keys, int64_t n, SortDigits D, uint32_t* __restrict__ counts) {
+    extern __shared__ uint32_t sm_digits[];
+    const int words = D.passes << D.db;
+    for (int i = threadIdx.x; i < words; i += blockDim.x) sm_digits[i] = 0;
+    __syncthreads();
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+        count_digits(sm_digits, D, keys[i]);
+    __syncthreads();
+    for (int i = threadIdx.x; i < words; i += blockDim.x)
+        if (sm_digits[i]) atomicAdd(counts + i, sm_digits[i]);
 }
 
-// LSD radix sort of (u32 key, V value) by the low `bits` bits of the key, stable; the
-// sorted arrays end in whichever of (keys, vals) / (keys_tmp, vals_tmp) the last pass
-// wrote, returned through kres / vres
-template <typename V>
-int radix_sort_t(uint32_t* keys, V* vals, uint32_t* keys_tmp, V* vals_tmp, int64_t n, int bits,
-                 cudaStream_t st, uint32_t** kres, V** vres) {
-    *kres = keys;
-    *vres = vals;
-    if (n <= 1 || bits <= 0) return TM_OK;
-    int passes = (bits + kMaxDigitBits - 1) / kMaxDigitBits;
-    int db = (bits + passes - 1) / passes;
+// counts of each (sort, pass) -> the start of each digit's run, in place (one block each)
+__global__ void __launch_bounds__(kSortThreads) k_digit_base(uint32_t* __restrict__ counts, int db) {
+    __shared__ uint32_t red[kSortWarps];
+    uint32_t* c = counts + ((size_t)blockIdx.x << db);
+    const int per = max(1, (1 << db) / kSortThreads), d0 = threadIdx.x * per;
+    uint32_t sum = 0;
+    for (int x = 0; x < per; x++) sum += d0 + x < (1 << db) ? c[d0 + x] : 0;
+    uint32_t at = block_excl_scan_u32(sum, red);
+    for (int x = 0; x < per; x++)
+        if (d0 + x < (1 << db)) {
+            const uint32_t v = c[d0 + x];
+            c[d0 + x] = at;
+            at += v;
+        }
+}
+
+template <int TB, int DB>
+int sort_pass(const SortJobs& J, int64_t n, int shift, cudaStream_t st) {
     {
-        // the scatter's dynamic shared memory can exceed the 48 KB default: allow the
-        // largest digit width once per device and value type
+        // the tile's shared memory exceeds the 48 KB default: allowed once per device
         static std::mutex mu;
         static bool done[64] = {};
         int dev = 0;
         TM_CUDA(cudaGetDevice(&dev));
         std::lock_guard<std::mutex> lk(mu);
-        if (dev >= 0 && dev < 64 && !done[dev]) {
-            TM_CUDA(cudaFuncSetAttribute(k_radix_scatter<V>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)sort_smem_bytes<V>(kMaxDigitBits)));
-            done[dev] = true;
+        if (dev < 0 || dev >= 64 || !done[dev]) {
+            TM_CUDA(cudaFuncSetAttribute(k_sort_pass<TB, DB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)sort_smem_bytes<TB, DB>()));
+            if (dev >= 0 && dev < 64) done[dev] = true;
         }
     }
-    int64_t ntiles = (n + kSortTile - 1) / kSortTile;
-    int64_t nh = ((int64_t)1 << db) * ntiles;
-    int32_t* hist = nullptr;
-    int64_t* offs = nullptr;
-    TM_CUDA(cudaMallocAsync((void**)&hist, sizeof(int32_t) * (size_t)nh, st));
-    TM_CUDA(cudaMallocAsync((void**)&offs, sizeof(int64_t) * (size_t)nh * 2, st));
-    int64_t* hist64 = offs + nh;
-    uint32_t *ka = keys, *kb = keys_tmp;
-    V *va = vals, *vb = vals_tmp;
-    int rc = TM_OK;
-    for (int p = 0; p < passes && rc == TM_OK; p++) {
-        int shift = p * db;
-        int width = (shift + db > bits) ? bits - shift : db;
-        k_radix_hist<<<(unsigned)ntiles, kSortThreads, 0, st>>>(ka, n, shift, width, hist, ntiles); count_launch();
-        int64_t nhp = ((int64_t)1 << width) * ntiles;
-        rc = scan_lengths(hist, offs, nhp, nullptr, nullptr, nh >= 8 ? hist64 : nullptr, nh, st);
-        if (rc != TM_OK) break;
-        k_radix_scatter<V><<<(unsigned)ntiles, kSortThreads, sort_smem_bytes<V>(width), st>>>(
-            ka, va, kb, vb, n, shift, width, offs, ntiles);
-        count_launch();
-        if (cudaGetLastError() != cudaSuccess) { rc = TM_ECUDA; break; }
-        std::swap(ka, kb);
-        std::swap(va, vb);
+    const int64_t blocks = J.jobs * ((n + kSortTile - 1) / kSortTile);
+    k_sort_pass<TB, DB><<<(unsigned)blocks, kSortThreads, sort_smem_bytes<TB, DB>(), st>>>(J, n, shift);
+    count_launch();
+    TM_CUDA(cudaGetLastError());
+    return TM_OK;
+}
+
+template <int TB>
+int sort_pass_db(const SortJobs& J, int64_t n, int shift, int db, cudaStream_t st) {
+    switch (db) {
+        case 5: return sort_pass<TB, 5>(J, n, shift, st);
+        case 6: return sort_pass<TB, 6>(J, n, shift, st);
+        case 7: return sort_pass<TB, 7>(J, n, shift, st);
+        case 8: return sort_pass<TB, 8>(J, n, shift, st);
+        case 9: return sort_pass<TB, 9>(J, n, shift, st);
+        default: return sort_pass<TB, 10>(J, n, shift, st);
     }
-    cudaFreeAsync(hist, st);
-    cudaFreeAsync(offs, st);
-    if (rc != TM_OK) set_error("radix sort launch failed");
-    *kres = ka;
-    *vres = va;
-    return rc;
 }
 
 }  // namespace
@@ -552,22 +612,115 @@ int scan_exclusive_i64_dn(const int64_t* in, int64_t* out, int64_t n_max, const 
     return TM_OK;
 }
 
-int radix_sort_pairs(uint32_t* keys, uint32_t* vals, uint32_t* keys_tmp, uint32_t* vals_tmp,
-                     int64_t n, int bits, cudaStream_t st) {
-    // Sorts (keys, vals) stably by the low `bits` bits of keys; the result ends
-    // in keys/vals.  bits <= 32.
-    uint32_t *kr, *vr;
-    int rc = radix_sort_t<uint32_t>(keys, vals, keys_tmp, vals_tmp, n, bits, st, &kr, &vr);
-    if (rc == TM_OK && kr != keys) {
-        TM_CUDA(cudaMemcpyAsync(keys, kr, sizeof(uint32_t) * (size_t)n, cudaMemcpyDeviceToDevice, st));
-        TM_CUDA(cudaMemcpyAsync(vals, vr, sizeof(uint32_t) * (size_t)n, cudaMemcpyDeviceToDevice, st));
-    }
-    return rc;
+SortDigits sort_digits(int bits) {
+    SortDigits D;
+    D.bits = std::max(bits, 1);
+    D.passes = (D.bits + 9) / 10;
+    D.db = std::max(5, (D.bits + D.passes - 1) / D.passes);
+    return D;
 }
 
-int radix_sort_kv64(uint32_t* keys, uint64_t* vals, uint32_t* keys_tmp, uint64_t* vals_tmp, int64_t n,
-                    int bits, cudaStream_t st, uint32_t** kres, uint64_t** vres) {
-    return radix_sort_t<uint64_t>(keys, vals, keys_tmp, vals_tmp, n, bits, st, kres, vres);
+// words of one sort's scratch: tickets and tile words of every pass (zeroed by sort_clear)
+static size_t sort_pass_words(int64_t n, const SortDigits& D) {
+    const size_t ntiles = (size_t)((n + kSortTile - 1) / kSortTile);
+    return ((ntiles << D.db) + 63) / 64 * 64 + 64;
+}
+size_t sort_ws_bytes(int64_t n, const SortDigits& D, int sorts, int counted) {
+    return 4 * ((size_t)sorts * D.passes * sort_pass_words(n, D) + ((size_t)counted * D.passes << D.db) + 64);
+}
+
+SortWs sort_ws(void* mem, int64_t n, const SortDigits& D, int sorts, int counted) {
+    SortWs W;
+    W.D = D;
+    W.n = n;
+    W.err = (uint32_t*)mem;
+    W.counts = W.err + 64;
+    W.words = W.counts + ((size_t)counted * D.passes << D.db);
+    W.counted = counted;
+    W.bytes = sort_ws_bytes(n, D, sorts, counted);
+    return W;
+}
+
+int sort_clear(const SortWs& W, cudaStream_t st) {
+    TM_CUDA(cudaMemsetAsync(W.err, 0, W.bytes, st));
+    return TM_OK;
+}
+
+int sort_bases(const SortWs& W, cudaStream_t st) {
+    k_digit_base<<<(unsigned)(W.counted * W.D.passes), kSortThreads, 0, st>>>(W.counts, W.D.db);
+    count_launch();
+    TM_CUDA(cudaGetLastError());
+    return TM_OK;
+}
+
+int sort_run(const SortWs& W, const SortIo* io, int sorts, int first, int tbytes, cudaStream_t st) {
+    const size_t pw = sort_pass_words(W.n, W.D);
+    for (int p = 0; p < W.D.passes; p++) {
+        SortJobs J;
+        J.jobs = sorts;
+        J.err = W.err;
+        for (int s = 0; s < sorts; s++) {
+            const SortIo& x = io[s];
+            // an odd number of passes still to come writes the final arrays, an even one the others
+            const bool from_final = (W.D.passes - p) % 2 == 0, last = p + 1 == W.D.passes;
+            SortJob& j = J.job[s];
+            j.key_in = p == 0 ? x.key_in : from_final ? x.key_out : x.key_tmp;
+            j.a_in = p == 0 ? x.a_in : from_final ? x.a_out : x.a_tmp;
+            j.t_in = p == 0 ? x.t_in : from_final ? x.t_out : x.t_tmp;
+            j.key_out = last && !x.keep_key ? nullptr : from_final ? x.key_tmp : x.key_out;
+            j.a_out = from_final ? x.a_tmp : x.a_out;
+            j.t_out = from_final ? x.t_tmp : x.t_out;
+            uint32_t* w = W.words + pw * ((size_t)(first + s) * W.D.passes + p);
+            j.ticket = w;
+            j.words = w + 64;
+            j.base = W.counts + (((size_t)x.counts * W.D.passes + p) << W.D.db);
+        }
+        const int shift = p * W.D.db;
+        int rc;
+        if (tbytes == 8) rc = sort_pass_db<8>(J, W.n, shift, W.D.db, st);
+        else if (tbytes == 4) rc = sort_pass_db<4>(J, W.n, shift, W.D.db, st);
+        else rc = sort_pass_db<0>(J, W.n, shift, W.D.db, st);
+        if (rc != TM_OK) return rc;
+    }
+    return TM_OK;
+}
+
+int radix_sort_pairs(uint32_t* keys, uint32_t* vals, uint32_t* keys_tmp, uint32_t* vals_tmp,
+                     int64_t n, int bits, uint32_t* d_err, cudaStream_t st) {
+    // Sorts (keys, vals) stably by the low `bits` bits of keys; the result ends
+    // in keys/vals.  bits <= 32.
+    if (n <= 1 || bits <= 0) return TM_OK;
+    const SortDigits D = sort_digits(bits);
+    void* mem = nullptr;
+    TM_CUDA(cudaMallocAsync(&mem, sort_ws_bytes(n, D, 1, 1), st));
+    SortWs W = sort_ws(mem, n, D, 1, 1);
+    int rc = sort_clear(W, st);
+    W.err = d_err;
+    if (rc == TM_OK) {
+        k_digit_count<<<(unsigned)std::min<int64_t>((n + 255) / 256, (int64_t)sm_count() * 8), 256,
+                        (size_t)4 * D.passes << D.db, st>>>(keys, n, D, W.counts);
+        count_launch();
+        if (cudaGetLastError() != cudaSuccess) rc = TM_ECUDA;
+    }
+    if (rc == TM_OK) rc = sort_bases(W, st);
+    SortIo io;
+    io.key_in = keys; io.a_in = vals; io.t_in = nullptr;
+    // an even number of passes ends where it began, an odd one in the other arrays
+    const bool even = D.passes % 2 == 0;
+    io.key_out = even ? keys : keys_tmp; io.a_out = even ? vals : vals_tmp; io.t_out = nullptr;
+    io.key_tmp = even ? keys_tmp : keys; io.a_tmp = even ? vals_tmp : vals; io.t_tmp = nullptr;
+    io.counts = 0;
+    io.keep_key = true;
+    if (rc == TM_OK) rc = sort_run(W, &io, 1, 0, 0, st);
+    if (rc == TM_OK && !even) {
+        cudaError_t e = cudaMemcpyAsync(keys, keys_tmp, sizeof(uint32_t) * (size_t)n, cudaMemcpyDeviceToDevice, st);
+        if (e == cudaSuccess)
+            e = cudaMemcpyAsync(vals, vals_tmp, sizeof(uint32_t) * (size_t)n, cudaMemcpyDeviceToDevice, st);
+        if (e != cudaSuccess) rc = TM_ECUDA;
+    }
+    cudaFreeAsync(mem, st);
+    if (rc != TM_OK) set_error("radix sort launch failed");
+    return rc;
 }
 
 namespace {

@@ -303,7 +303,7 @@ extern "C" int tm_stream_run(const int32_t* src, const int32_t* dst, const int64
         // this segment: graph, then one batch of the queries with work in it
         tm_graph* g = nullptr;
         int64_t n = cur.eb - cur.ea;
-        rc = tm_graph_load_device(dev[slot].src, dev[slot].dst, dev[slot].t, n, n_nodes, st, &g);
+        rc = build_graph(dev[slot].src, dev[slot].dst, dev[slot].t, t + cur.ea, n, n_nodes, st, &g);
         if (rc == TM_OK) {
             size_t k = cur.qidx.size();
             sq.resize(k);

@@ -103,8 +103,7 @@ struct GraphDev {
     const int64_t* in_off;  // [n+1]
     const int32_t* in_nbr;  // [m] source
     const void* in_t;       // [m]
-    const int64_t* pk_off;  // [n+1] pair index range of each source
-    const int32_t* pair_dst;// [P]
+    const int32_t* pair_dst;// [m] destination of each pair-view entry
     const int64_t* pair_off;// [P+1]
     const void* pair_t;     // [m]
     const int32_t* out_src; // [m] source of each out-view entry (the sort key)
@@ -134,7 +133,6 @@ struct GraphDevT {
     const int64_t* in_off;
     const int32_t* in_nbr;
     const TT* in_t;
-    const int64_t* pk_off;
     const int32_t* pair_dst;
     const int64_t* pair_off;
     const TT* pair_t;
@@ -160,7 +158,7 @@ inline GraphDevT<TT> typed(const GraphDev& g) {
     r.src = g.src; r.dst = g.dst; r.t = (const TT*)g.t;
     r.out_off = g.out_off; r.out_nbr = g.out_nbr; r.out_t = (const TT*)g.out_t;
     r.in_off = g.in_off; r.in_nbr = g.in_nbr; r.in_t = (const TT*)g.in_t;
-    r.pk_off = g.pk_off; r.pair_dst = g.pair_dst; r.pair_off = g.pair_off; r.pair_t = (const TT*)g.pair_t;
+    r.pair_dst = g.pair_dst; r.pair_off = g.pair_off; r.pair_t = (const TT*)g.pair_t;
     r.out_src = g.out_src; r.in_dst = g.in_dst; r.pair_pid = g.pair_pid;
     r.hslots = g.hslots; r.hmask = g.hmask; r.loops = g.loops;
     r.pfilt = g.pfilt; r.pfmask = g.pfmask;
@@ -333,11 +331,63 @@ int check_query(int64_t t_max, const tm_query& q, std::string& why);
 int scan_exclusive_i64(const int64_t* in, int64_t* out, int64_t n, int64_t* d_total,
                        cudaStream_t st);
 int radix_sort_pairs(uint32_t* keys, uint32_t* vals, uint32_t* keys_tmp, uint32_t* vals_tmp,
-                     int64_t n, int bits, cudaStream_t st);
-// the same with 64-bit values; the sorted arrays end in (keys, vals) or (keys_tmp, vals_tmp),
-// returned through kres / vres (no copy back)
-int radix_sort_kv64(uint32_t* keys, uint64_t* vals, uint32_t* keys_tmp, uint64_t* vals_tmp, int64_t n,
-                    int bits, cudaStream_t st, uint32_t** kres, uint64_t** vres);
+                     int64_t n, int bits, uint32_t* d_err, cudaStream_t st);   // *d_err as SortWs::err
+
+// The radix sort in parts, for callers that produce the keys themselves and sort several lists
+// of n triples (key, a, t) by the same number of bits:
+//   sort_digits    how the bits are cut into passes
+//   sort_ws        places the scratch of `sorts` sorts, `counted` of them with counts of their
+//                  own, in sort_ws_bytes(...) bytes; sort_clear zeroes it
+//   count_digits   (device) adds a key to the block's counts [pass][digit] in shared memory, which
+//                  the caller adds to W.counts + (c * passes << db) for counted list c
+//   sort_bases     counts -> starts of the digits' runs
+//   sort_run       the passes of sorts [first, first + sorts) side by side in one launch per pass
+//                  (SortIo::counts names the counted list with the same keys)
+// Asynchronous; *W.err is non-zero afterwards if a wait between tiles expired.
+struct SortDigits { int bits, passes, db; };
+struct SortWs {
+    SortDigits D;
+    int64_t n;
+    int counted;
+    uint32_t* err;
+    uint32_t* counts;
+    uint32_t* words;
+    size_t bytes;
+};
+struct SortIo {
+    const uint32_t *key_in, *a_in;
+    const void* t_in;
+    uint32_t *key_out, *a_out;    // the sorted lists
+    void* t_out;
+    uint32_t *key_tmp, *a_tmp;    // between passes (unused by a single pass)
+    void* t_tmp;
+    int counts;
+    bool keep_key;                // false: the last pass leaves key_out unwritten
+};
+struct SortJob {
+    const uint32_t *key_in, *a_in;
+    const void* t_in;
+    uint32_t *key_out, *a_out;
+    void* t_out;
+    uint32_t *ticket, *words;
+    const uint32_t* base;
+};
+constexpr int kMaxSortJobs = 2;
+struct SortJobs {
+    SortJob job[kMaxSortJobs];
+    int jobs;
+    uint32_t* err;
+};
+SortDigits sort_digits(int bits);
+size_t sort_ws_bytes(int64_t n, const SortDigits& D, int sorts, int counted);
+SortWs sort_ws(void* mem, int64_t n, const SortDigits& D, int sorts, int counted);
+int sort_clear(const SortWs& W, cudaStream_t st);
+int sort_bases(const SortWs& W, cudaStream_t st);
+int sort_run(const SortWs& W, const SortIo* io, int sorts, int first, int tbytes, cudaStream_t st);
+__device__ __forceinline__ void count_digits(uint32_t* sm, const SortDigits& D, uint32_t key) {
+    for (int p = 0; p < D.passes; p++)
+        atomicAdd(sm + (p << D.db) + ((key >> (p * D.db)) & ((1u << D.db) - 1u)), 1u);
+}
 // exclusive scan with the tile sums in caller workspace (2 * ceil(n/2048) int64, n <= 2048^2)
 int scan_exclusive_i64_ws(const int64_t* in, int64_t* out, int64_t n, int64_t* d_total,
                           int64_t* ws, int64_t ws_elems, cudaStream_t st);
@@ -353,6 +403,10 @@ int scan_exclusive_i64_dn(const int64_t* in, int64_t* out, int64_t n_max, const 
                           int64_t* d_total, int64_t* ws, int64_t ws_elems, cudaStream_t st);
 
 int sm_count();
+// a graph from device arrays (tm_graph_load_device); h_t: the same times on the host when the
+// caller has them there (their first and last are then read without waiting for the device)
+int build_graph(const int32_t* d_src, const int32_t* d_dst, const int64_t* d_t, const int64_t* h_t, int64_t m,
+                int32_t n_nodes, cudaStream_t st, tm_graph** out);
 // the graph's two-node tables (own, rev: [m+1] each) that are asked for, each built on
 // the first call that needs it (thread-safe; synchronises the stream when it builds);
 // null for an empty graph or when not asked for
@@ -454,6 +508,94 @@ __device__ __forceinline__ int64_t lower_bound_i32(const int32_t* __restrict__ a
         if (__ldg(a + mid) < v) lo = mid + 1; else hi = mid;
     }
     return lo;
+}
+
+// Decoupled look-back.  A tile's word (for one digit of a sort, or for a scan): 0 not yet known; count + 1 (below 2^31) once the tile
+// has counted; kTilePrefix | sum over the tiles up to and including it once that is known (below
+// 2^31, as n is).
+constexpr uint32_t kTilePrefix = 0x80000000u;
+constexpr int kSpinLimit = 1 << 22;   // polls of one word, about a second: then the error word is set
+
+__device__ __forceinline__ uint32_t ld_tile(const uint32_t* p) {
+    uint32_t v;
+    asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ void st_tile(uint32_t* p, uint32_t v) {
+    asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+
+// Sum of the words of tiles tile-1, tile-2, ... at `stride` apart, back to the first that holds a
+// prefix, kLookBack of them read at a time (the reads are a serial chain otherwise: prefixes
+// travel forward at most that many tiles per memory latency).  Tiles are numbered in the order
+// blocks start, so every word waited for belongs to a block that already runs; if one still
+// never comes the error word is set and the sum so far returned (positions stay in range: it is
+// too small, never too large).
+constexpr int kLookBack = 4;
+__device__ __forceinline__ uint32_t look_back(const uint32_t* words, int64_t tile, int64_t stride, uint32_t* err) {
+    uint32_t sum = 0;
+    int64_t at = tile - 1;
+    int spins = 0;
+    while (at >= 0) {
+        uint32_t v[kLookBack];
+#pragma unroll
+        for (int i = 0; i < kLookBack; i++) v[i] = at - i >= 0 ? ld_tile(words + (at - i) * stride) : kTilePrefix;
+        bool open = true;   // no prefix and no missing word among those taken so far
+#pragma unroll
+        for (int i = 0; i < kLookBack; i++) {
+            if (open) {
+                if (v[i] & kTilePrefix) return sum + (v[i] & ~kTilePrefix);
+                open = v[i] != 0;
+                if (open) {
+                    sum += v[i] - 1;
+                    at--;
+                }
+            }
+        }
+        if (v[0] == 0 && ++spins > kSpinLimit) {
+            atomicOr(err, 1u);
+            return sum;
+        }
+    }
+    return sum;
+}
+
+// The same by a whole block, blockDim.x words at a time (a multiple of 32, at most 1024; every
+// thread returns the sum).  For scans with one word per tile, where a narrower look-back is the
+// chain that bounds the kernel: the tiles in flight then find their prefixes one hop after
+// another instead of reading all of each other's counts at once.
+__device__ __forceinline__ uint32_t look_back_block(const uint32_t* words, int64_t tile, uint32_t* err) {
+    __shared__ uint32_t s_sum[32];
+    __shared__ int s_gap, s_pre;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nt = blockDim.x;
+    uint32_t sum = 0;
+    int64_t at = tile - 1;
+    int spins = 0;
+    while (at >= 0) {
+        if (threadIdx.x == 0) s_gap = s_pre = nt;
+        __syncthreads();
+        const int64_t mine = at - (int64_t)threadIdx.x;
+        const uint32_t v = mine >= 0 ? ld_tile(words + mine) : kTilePrefix;
+        if (v == 0) atomicMin(&s_gap, (int)threadIdx.x);
+        if (v & kTilePrefix) atomicMin(&s_pre, (int)threadIdx.x);
+        __syncthreads();
+        // the words before the first missing one, up to and including the first prefix
+        const int gap = s_gap, pre = s_pre;
+        uint32_t x = (int)threadIdx.x < gap && (int)threadIdx.x <= pre ? ((v & kTilePrefix) ? (v & ~kTilePrefix) : v - 1) : 0;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(kFull, x, o);
+        if (lane == 0) s_sum[w] = x;
+        __syncthreads();
+        for (int i = 0; i < (nt >> 5); i++) sum += s_sum[i];
+        if (pre < gap) break;
+        at -= gap;
+        if (gap == 0 && ++spins > kSpinLimit) {
+            if (threadIdx.x == 0) atomicOr(err, 1u);
+            break;
+        }
+        __syncthreads();   // s_sum and the two marks are written again
+    }
+    return sum;
 }
 
 // SplitMix64 (Steele, Lea & Flood 2014): output n (n >= 1) of the generator
