@@ -879,9 +879,8 @@ __global__ void __launch_bounds__(256, 8) k_level2(MatchArgs<TT> A, FRec<TT>* __
                 bool have_own = false, have_rev = false;
                 auto own_side = [&]() {
                     if (Q.order == kOrdPair) {
-                        int32_t pid = __ldg(G.pair_pid + e1);
-                        pa = __ldg(G.pair_off + pid);
-                        pb = __ldg(G.pair_off + pid + 1);
+                        pa = __ldg(G.pair_beg + e1);
+                        pb = __ldg(G.pair_end + e1);
                         own_ub = gallop_ub(G.pair_t, e1 + 1, pb, t1);
                     } else {
                         pair_segment(G, s1, d1, pa, pb, false);   // e1 is one of the pair's edges
@@ -942,7 +941,7 @@ __global__ void __launch_bounds__(256, 8) k_level2(MatchArgs<TT> A, FRec<TT>* __
                     // first edges with no closing edge skip every other search
                     if (Q.order == kOrdPair) {
                         // the first edge's own pair: its entries after e1 up to thi
-                        int64_t pend = __ldg(G.pair_off + __ldg(G.pair_pid + e1) + 1);
+                        int64_t pend = __ldg(G.pair_end + e1);
                         ha = gallop_ub(G.pair_t, e1 + 1, pend, t1);
                         hh = thi > t1 ? gallop_ub(G.pair_t, ha, pend, thi) : ha;
                     } else {

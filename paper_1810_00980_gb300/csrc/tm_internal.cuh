@@ -104,13 +104,15 @@ struct GraphDev {
     const int32_t* in_nbr;  // [m] source
     const void* in_t;       // [m]
     const int32_t* pair_dst;// [m] destination of each pair-view entry
-    const int64_t* pair_off;// [P+1]
+    const int32_t* pair_beg;// [m] start and end of the segment of the entry's pair
+    const int32_t* pair_end;// [m]
     const void* pair_t;     // [m]
     const int32_t* out_src; // [m] source of each out-view entry (the sort key)
     const int32_t* in_dst;  // [m] destination of each in-view entry
-    const int32_t* pair_pid;// [m] pair index of each pair-view entry
-    const unsigned long long* hslots;  // [2*(hmask+1)]: key, then (length << 32 | begin) of the pair's segment
-    unsigned long long hmask;          // hash capacity - 1 (power of two)
+    // pair table: hparts parts of hmask + 1 slots, open addressing inside a part; a slot is the key
+    // (src << 32 | dst), then (length << 32 | begin) of the pair's segment
+    const unsigned long long* hslots;
+    uint32_t hparts, hmask;
     // pair filter: two bits per pair in one 32-bit word; a lookup whose two bits are not both
     // set has no pair (most lookups of absent pairs end in this L2-resident array)
     const uint32_t* pfilt;             // [pfmask+1] or null
@@ -134,13 +136,13 @@ struct GraphDevT {
     const int32_t* in_nbr;
     const TT* in_t;
     const int32_t* pair_dst;
-    const int64_t* pair_off;
+    const int32_t* pair_beg;
+    const int32_t* pair_end;
     const TT* pair_t;
     const int32_t* out_src;
     const int32_t* in_dst;
-    const int32_t* pair_pid;
     const unsigned long long* hslots;
-    unsigned long long hmask;
+    uint32_t hparts, hmask;
     const uint32_t* pfilt;
     unsigned long long pfmask;
     int32_t loops;
@@ -158,9 +160,9 @@ inline GraphDevT<TT> typed(const GraphDev& g) {
     r.src = g.src; r.dst = g.dst; r.t = (const TT*)g.t;
     r.out_off = g.out_off; r.out_nbr = g.out_nbr; r.out_t = (const TT*)g.out_t;
     r.in_off = g.in_off; r.in_nbr = g.in_nbr; r.in_t = (const TT*)g.in_t;
-    r.pair_dst = g.pair_dst; r.pair_off = g.pair_off; r.pair_t = (const TT*)g.pair_t;
-    r.out_src = g.out_src; r.in_dst = g.in_dst; r.pair_pid = g.pair_pid;
-    r.hslots = g.hslots; r.hmask = g.hmask; r.loops = g.loops;
+    r.pair_dst = g.pair_dst; r.pair_beg = g.pair_beg; r.pair_end = g.pair_end; r.pair_t = (const TT*)g.pair_t;
+    r.out_src = g.out_src; r.in_dst = g.in_dst;
+    r.hslots = g.hslots; r.hparts = g.hparts; r.hmask = g.hmask; r.loops = g.loops;
     r.pfilt = g.pfilt; r.pfmask = g.pfmask;
     r.ex_own = nullptr; r.ex_rev = nullptr;
     return r;
@@ -179,7 +181,8 @@ struct tm_graph {
     int64_t t_max;          // normalised
     int64_t bytes;
     void* block;            // one device allocation holding every array
-    void* hash_block;       // the (src, dst) -> pair index hash table
+    void* hash_block;       // the pair filter, after a small graph's pair table
+    void* table_block;      // a large graph's pair table (or null)
     void* ex_own_block;     // the two-node tables ([m+1] each), built on first use (or null)
     void* ex_rev_block;
     tmo::GraphDev dev;
@@ -510,7 +513,7 @@ __device__ __forceinline__ int64_t lower_bound_i32(const int32_t* __restrict__ a
     return lo;
 }
 
-// Decoupled look-back.  A tile's word (for one digit of a sort, or for a scan): 0 not yet known; count + 1 (below 2^31) once the tile
+// Decoupled look-back.  A tile's word for one digit: 0 not yet known; count + 1 (below 2^31) once the tile
 // has counted; kTilePrefix | sum over the tiles up to and including it once that is known (below
 // 2^31, as n is).
 constexpr uint32_t kTilePrefix = 0x80000000u;
@@ -560,44 +563,6 @@ __device__ __forceinline__ uint32_t look_back(const uint32_t* words, int64_t til
     return sum;
 }
 
-// The same by a whole block, blockDim.x words at a time (a multiple of 32, at most 1024; every
-// thread returns the sum).  For scans with one word per tile, where a narrower look-back is the
-// chain that bounds the kernel: the tiles in flight then find their prefixes one hop after
-// another instead of reading all of each other's counts at once.
-__device__ __forceinline__ uint32_t look_back_block(const uint32_t* words, int64_t tile, uint32_t* err) {
-    __shared__ uint32_t s_sum[32];
-    __shared__ int s_gap, s_pre;
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nt = blockDim.x;
-    uint32_t sum = 0;
-    int64_t at = tile - 1;
-    int spins = 0;
-    while (at >= 0) {
-        if (threadIdx.x == 0) s_gap = s_pre = nt;
-        __syncthreads();
-        const int64_t mine = at - (int64_t)threadIdx.x;
-        const uint32_t v = mine >= 0 ? ld_tile(words + mine) : kTilePrefix;
-        if (v == 0) atomicMin(&s_gap, (int)threadIdx.x);
-        if (v & kTilePrefix) atomicMin(&s_pre, (int)threadIdx.x);
-        __syncthreads();
-        // the words before the first missing one, up to and including the first prefix
-        const int gap = s_gap, pre = s_pre;
-        uint32_t x = (int)threadIdx.x < gap && (int)threadIdx.x <= pre ? ((v & kTilePrefix) ? (v & ~kTilePrefix) : v - 1) : 0;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(kFull, x, o);
-        if (lane == 0) s_sum[w] = x;
-        __syncthreads();
-        for (int i = 0; i < (nt >> 5); i++) sum += s_sum[i];
-        if (pre < gap) break;
-        at -= gap;
-        if (gap == 0 && ++spins > kSpinLimit) {
-            if (threadIdx.x == 0) atomicOr(err, 1u);
-            break;
-        }
-        __syncthreads();   // s_sum and the two marks are written again
-    }
-    return sum;
-}
-
 // SplitMix64 (Steele, Lea & Flood 2014): output n (n >= 1) of the generator
 // seeded with s is mix(s + n * 0x9E3779B97F4A7C15).
 __host__ __device__ __forceinline__ uint64_t sm64_mix(uint64_t z) {
@@ -613,23 +578,33 @@ __host__ __device__ __forceinline__ uint64_t draw(uint64_t seed, uint64_t k, uin
     return sm64_output(sm64_output(seed, k + 1), n + 1);
 }
 
+// a pair's key, its bits in the filter (word (h >> 10) & pfmask), its part of the table (by the
+// hash's upper half, in order) and its first slot there
+__device__ __forceinline__ unsigned long long pair_key(int32_t u, int32_t v) {
+    return ((unsigned long long)(uint32_t)u << 32) | (uint32_t)v;
+}
+__device__ __forceinline__ uint32_t pair_bits(unsigned long long h) { return (1u << (h & 31)) | (1u << ((h >> 5) & 31)); }
+__device__ __forceinline__ uint32_t pair_part(unsigned long long h, uint32_t parts) { return __umulhi((uint32_t)(h >> 32), parts); }
+
 // the time-sorted segment [a, b) of pair (u, v) in the pair view, by one hash lookup
-// (after the pair filter, which answers most lookups of absent pairs from L2)
+// (after the pair filter, which answers most lookups of absent pairs from L2).  (Slots grouped by
+// source, 8 bytes with the segment's end beside the entries, made the matcher 7 % slower: two
+// more dependent loads; a table two thirds full 2 %: longer probe chains.)
 template <typename TT>
 __device__ __forceinline__ bool pair_segment(const GraphDevT<TT>& G, int32_t u, int32_t v, int64_t& a,
                                              int64_t& b, bool filter = true) {
-    unsigned long long key = ((unsigned long long)(uint32_t)u << 32) | (uint32_t)v;
-    unsigned long long h0 = sm64_mix(key);
+    const unsigned long long key = pair_key(u, v);
+    const unsigned long long h = sm64_mix(key);
+    a = b = 0;
     if (filter && G.pfilt) {   // callers that know the pair exists skip the filter
-        uint32_t w = __ldg(G.pfilt + ((h0 >> 32) & G.pfmask));
-        if (!((w >> (h0 & 31)) & (w >> ((h0 >> 5) & 31)) & 1u)) {
-            a = b = 0;
-            return false;
-        }
+        const uint32_t w = __ldg(G.pfilt + ((h >> 10) & G.pfmask));
+        if (!((w >> (h & 31)) & (w >> ((h >> 5) & 31)) & 1u)) return false;
     }
-    unsigned long long h = h0 & G.hmask;
-    for (unsigned long long it = 0; it <= G.hmask; it++) {
-        ulonglong2 sl = __ldg(reinterpret_cast<const ulonglong2*>(G.hslots) + h);
+    const ulonglong2* slots = reinterpret_cast<const ulonglong2*>(G.hslots) +
+                              (size_t)pair_part(h, G.hparts) * ((size_t)G.hmask + 1);
+    uint32_t x = (uint32_t)h & G.hmask;
+    for (uint32_t it = 0; it <= G.hmask; it++) {
+        const ulonglong2 sl = __ldg(slots + x);
         if (sl.x == key) {
             a = (int64_t)(uint32_t)sl.y;
             b = a + (int64_t)(sl.y >> 32);
@@ -639,11 +614,9 @@ __device__ __forceinline__ bool pair_segment(const GraphDevT<TT>& G, int32_t u, 
 #endif
             return true;
         }
-        unsigned long long k = sl.x;
-        if (k == kHashEmpty) break;
-        h = (h + 1) & G.hmask;
+        if (sl.x == kHashEmpty) break;
+        x = (x + 1) & G.hmask;
     }
-    a = b = 0;
     return false;
 }
 

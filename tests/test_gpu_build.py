@@ -84,3 +84,43 @@ def test_wrong_inputs_keep_their_order_of_blame():
     assert status(bad_id, ids, far, 7) == tm.TM_ERANGE
     with tm.Graph(*(torch.from_numpy(x).cuda() for x in (ids, ids, base)), -1) as g:
         assert g.info().n_nodes == 7
+
+
+@pytest.mark.parametrize("crowded", [False, True])
+def test_pair_table_filled_by_parts(crowded):
+    """A graph large enough for the pair table to be filled part by part, and one whose pairs all
+    hash into a single part (more than its list holds): every reply pair is found."""
+    import torch
+    import __graft_entry__
+    __graft_entry__.build()
+    torch.cuda.set_device(0)
+    from paper_1810_00980_gb300 import tm
+    rng = np.random.default_rng(8)
+    n, m = 20_000, (3 << 20) + 1
+    u, v = rng.integers(0, n, 6_000_000), rng.integers(0, n, 6_000_000)
+    if crowded:
+        x = (u.astype(np.uint64) << np.uint64(32)) | v.astype(np.uint64)
+        x = (x ^ (x >> np.uint64(30))) * np.uint64(0xBF58476D1CE4E5B9)
+        x = (x ^ (x >> np.uint64(27))) * np.uint64(0x94D049BB133111EB)
+        x ^= x >> np.uint64(31)
+        keep = np.flatnonzero((x >> np.uint64(58)) == 5)
+        assert len(keep) > 80_000
+        u, v = u[keep], v[keep]
+        pick = rng.integers(0, len(u), m)
+        src, dst = u[pick].astype(np.int32), v[pick].astype(np.int32)
+    else:
+        half = m // 2   # replies are common
+        src = np.concatenate([u[:half], v[:m - half]]).astype(np.int32)
+        dst = np.concatenate([v[:half], u[:m - half]]).astype(np.int32)
+        order = rng.permutation(m)
+        src, dst = src[order], dst[order]
+    t = np.sort(rng.integers(0, 50_000, m)).astype(np.int64)
+    delta, span = 20_000, 100_000
+    pair = src.astype(np.int64) * n + dst
+    keys = np.sort(pair * span + t)
+    rev = (dst.astype(np.int64) * n + src) * span + t
+    ok = src != dst
+    want = int((np.searchsorted(keys, rev + delta, "right") - np.searchsorted(keys, rev, "right"))[ok].sum())
+    with tm.Graph(*(torch.from_numpy(x).cuda() for x in (src, dst, t)), n) as g:
+        assert g.info().n_pairs == len(np.unique(pair))
+        assert tm.count_exact(g, tm.Motif([0, 1], [1, 0]), delta) == want
