@@ -473,11 +473,11 @@ __device__ __forceinline__ int64_t div_nonneg(int64_t x, int64_t d) {
     return x / d;
 }
 
-__device__ __forceinline__ void ride_window(const QPlan& R, int k, int64_t t1, int64_t& w, int64_t& thi) {
-    int64_t s = __ldg(R.shifts + k);
-    int64_t j = div_nonneg(t1 - s, R.cd);   // 0-based window of t1
-    w = R.win_base + (int64_t)k * R.J + j;
-    thi = min(t1 + R.delta, s + (j + 1) * R.cd - 1);
+__device__ __forceinline__ void ride_window(const RideEnt& E, int64_t t1, int64_t& w, int64_t& thi) {
+    const int64_t x = t1 - E.shift;
+    const int64_t j = E.sh ? (int64_t)(((uint64_t)(uint32_t)x * E.mul) >> E.sh) : div_nonneg(x, E.cd);   // 0-based window of t1
+    w = E.wbase + j;
+    thi = min(t1 + E.delta, E.shift + (j + 1) * E.cd - 1);
 }
 
 // Rider sums go through a per-block table in shared memory keyed by window (when c delta is
@@ -536,7 +536,7 @@ __device__ __forceinline__ void ride_add(unsigned long long* acc, int64_t w, uns
     atomic_add_u128(p + A_WLO, lo, hi);
 }
 
-__device__ __forceinline__ void ride_weight(const QPlan& R, int64_t dur, unsigned long long n,
+__device__ __forceinline__ void ride_weight(const RideEnt& R, int64_t dur, unsigned long long n,
                                             unsigned long long& lo, unsigned long long& hi) {
     unsigned long long wi, wf;
     if (R.wtab) {
@@ -551,53 +551,43 @@ __device__ __forceinline__ void ride_weight(const QPlan& R, int64_t dur, unsigne
 }
 
 // cnt instances closed by the edge at t3
-__device__ __forceinline__ void ride_at(const QPlan* __restrict__ PL, const QPlan& Q, const int32_t* __restrict__ kept,
-                                     unsigned long long* acc, int64_t t1, int64_t t3, unsigned long long cnt) {
+__device__ __forceinline__ void ride_at(const QPlan& Q, const int32_t* __restrict__ kept, unsigned long long* acc,
+                                        int64_t t1, int64_t t3, unsigned long long cnt) {
     for (int r = 0; r < Q.nride; r++) {
-        const QPlan& R = PL[Q.ride_q[r]];
-        if (t3 - t1 > R.delta) continue;
-        const bool all_kept = R.q_mode == TM_Q_UNIFORM && R.p >= 1.0;   // no keep flag to read
-        for (int k = 0; k < R.b; k++) {
-            int64_t w, thi;
-            ride_window(R, k, t1, w, thi);
-            if (t3 > thi || !(all_kept || kept[w])) continue;
-            unsigned long long lo, hi;
-            ride_weight(R, t3 - t1, cnt, lo, hi);
-            ride_add(acc, w, cnt, lo, hi);
-        }
+        const RideEnt& R = Q.rides[r];
+        int64_t w, thi;
+        ride_window(R, t1, w, thi);
+        if (t3 > thi || !(R.all_kept || kept[w])) continue;
+        unsigned long long lo, hi;
+        ride_weight(R, t3 - t1, cnt, lo, hi);
+        ride_add(acc, w, cnt, lo, hi);
     }
 }
 
 // one instance per closing entry of the time-sorted range [lo, hi) (entries after tc); the most
 // entries read for one rider shift count as the exact query's last-edge entries read one by one
 template <typename TT>
-__device__ __forceinline__ void ride_range(const QPlan* __restrict__ PL, const QPlan& Q,
-                                        const int32_t* __restrict__ kept, unsigned long long* acc,
-                                        const TT* __restrict__ ta, int64_t clo, int64_t chi, int64_t t1,
-                                        int64_t tc) {
+__device__ __forceinline__ void ride_range(const QPlan& Q, const int32_t* __restrict__ kept, unsigned long long* acc,
+                                           const TT* __restrict__ ta, int64_t clo, int64_t chi, int64_t t1, int64_t tc) {
     unsigned long long nread = 0;
     for (int r = 0; r < Q.nride; r++) {
-        const QPlan& R = PL[Q.ride_q[r]];
-        if (t1 + R.delta <= tc) continue;   // no closing edge after tc fits the span
-        const bool all_kept = R.q_mode == TM_Q_UNIFORM && R.p >= 1.0;   // no keep flag to read
-        for (int k = 0; k < R.b; k++) {
-            int64_t w, thi;
-            ride_window(R, k, t1, w, thi);
-            if (thi <= tc || !(all_kept || kept[w])) continue;
-            unsigned long long cnt = 0, wl = 0, wh = 0;
-            for (int64_t x = clo; x < chi; x++) {
-                int64_t t3 = (int64_t)ta[x];
-                if (t3 > thi) break;   // times increase
-                unsigned long long l, h;
-                ride_weight(R, t3 - t1, 1, l, h);
-                unsigned long long y = wl + l;
-                wh += h + (y < wl ? 1ull : 0ull);
-                wl = y;
-                cnt++;
-            }
-            ride_add(acc, w, cnt, wl, wh);
-            nread = max(nread, cnt);
+        const RideEnt& R = Q.rides[r];
+        int64_t w, thi;
+        ride_window(R, t1, w, thi);
+        if (thi <= tc || !(R.all_kept || kept[w])) continue;   // no closing edge after tc fits
+        unsigned long long cnt = 0, wl = 0, wh = 0;
+        for (int64_t x = clo; x < chi; x++) {
+            int64_t t3 = (int64_t)ta[x];
+            if (t3 > thi) break;   // times increase
+            unsigned long long l, h;
+            ride_weight(R, t3 - t1, 1, l, h);
+            unsigned long long y = wl + l;
+            wh += h + (y < wl ? 1ull : 0ull);
+            wl = y;
+            cnt++;
         }
+        ride_add(acc, w, cnt, wl, wh);
+        nread = max(nread, cnt);
     }
     if (nread) ride_add(acc, (int64_t)(kInstKey | (unsigned long long)Q.win_base), nread, 0, 0);
 }
@@ -913,13 +903,10 @@ __global__ void __launch_bounds__(256, 8) k_level2(MatchArgs<TT> A, FRec<TT>* __
                             // latest end of a kept rider window holding t1
                             int64_t thr = t1;
                             for (int r = 0; r < Q.nride; r++) {
-                                const QPlan& R = PL[Q.ride_q[r]];
-                                const bool all_kept = R.q_mode == TM_Q_UNIFORM && R.p >= 1.0;
-                                for (int k = 0; k < R.b; k++) {
-                                    int64_t w, th;
-                                    ride_window(R, k, t1, w, th);
-                                    if (all_kept || A.W.kept[w]) thr = max(thr, th);
-                                }
+                                const RideEnt& R = Q.rides[r];
+                                int64_t w, th;
+                                ride_window(R, t1, w, th);
+                                if (th > thr && (R.all_kept || A.W.kept[w])) thr = th;
                             }
                             if (thr > t1) {
                                 len = gallop_ub(G.pair_t, ha, hh, thr) - ha;   // items for the riders only
@@ -1033,10 +1020,31 @@ __global__ void __launch_bounds__(256, 8) k_level2(MatchArgs<TT> A, FRec<TT>* __
     acc_flush_warp(acc, A.W.acc);
 }
 
+// The warp's deferred rider / smaller-span records (lanes with rn != 0), appended with one atomic
+template <typename TT>
+__device__ __forceinline__ void ride_emit(const MatchArgs<TT>& A, int64_t rx, int32_t rn, int64_t t1, int64_t tc, int32_t q) {
+    const int lane = threadIdx.x & 31;
+    const unsigned rm = __ballot_sync(kFull, rn != 0);
+    if (!rm) return;
+    unsigned long long rb = 0;
+    if (lane == 0) rb = atomicAdd(A.rcount, (unsigned long long)__popc(rm));
+    rb = __shfl_sync(kFull, rb, 0) + __popc(rm & ((1u << lane) - 1u));
+    if (rn && (int64_t)rb < A.rcap) {
+        RideRec<TT> rr;
+        rr.x = rx;
+        rr.t1 = (TT)t1;
+        rr.tc = (TT)tc;
+        rr.q = q;
+        rr.n = rn;
+        A.rrec[rb] = rr;
+    }
+}
+
 // Warp-cooperative expansion of motif edge D (0-based) for the 32 partial
 // instances held by the lanes (valid ones have edges 0..D-1 matched).
 // (ha, hh): the closing pair range when the query fixed it at the first edge.
-template <typename TT, int D, int LMAX, int KMAX>
+// RIDE: exact queries may carry riders (their instances then also go to k_ride as records).
+template <typename TT, int D, int LMAX, int KMAX, bool RIDE>
 __device__ void expand(const MatchArgs<TT>& A, const QPlan* __restrict__ PL, bool valid, int32_t q, int64_t win,
                        int32_t (&phi)[KMAX], int64_t t1, int64_t tprev, int64_t thi, int64_t ha,
                        int64_t hh, Acc& acc) {
@@ -1044,6 +1052,7 @@ __device__ void expand(const MatchArgs<TT>& A, const QPlan* __restrict__ PL, boo
     int lane = threadIdx.x & 31;
     int64_t lo = 0, len = 0;
     int dir = 0;   // 1: this lane's candidates are the last edge's (two-sided closing)
+    int32_t closed = 0;   // RIDE: instances closed by the range at lo
     if (valid) {
         const QPlan& Q = PL[q];
         const LevelPlan P = Q.lv[D];
@@ -1081,6 +1090,7 @@ __device__ void expand(const MatchArgs<TT>& A, const QPlan* __restrict__ PL, boo
             if (Q.mode == TM_MODE_EXACT) {
                 if (P.view == kPair) {
                     acc.f[A_COUNT] += len;
+                    if (RIDE && Q.nride) closed = (int32_t)len;
                     len = 0;
                 } else if (len > A.enum_threshold && P.view != kAll) {
                     acc.f[A_COUNT] += last_count_subtract(G, P, phi, len, tprev, thi);
@@ -1089,6 +1099,7 @@ __device__ void expand(const MatchArgs<TT>& A, const QPlan* __restrict__ PL, boo
             }
         }
     }
+    if constexpr (RIDE) ride_emit(A, lo, closed, t1, tprev, q);
     int64_t incl = warp_incl_scan64(len);
     int64_t total = __shfl_sync(kFull, incl, 31);
     int64_t mystart = incl - len;
@@ -1121,6 +1132,8 @@ __device__ void expand(const MatchArgs<TT>& A, const QPlan* __restrict__ PL, boo
         for (int i = 0; i < KMAX; i++) ophi[i] = __shfl_sync(kFull, phi[i], o);
         bool ok = false, deeper = false;
         int64_t tc = 0;
+        int64_t rx = 0;
+        int32_t rn = 0;
         if (has) {
             const QPlan& Q = PL[oq];
             const LevelPlan P = Q.lv[D];
@@ -1142,6 +1155,7 @@ __device__ void expand(const MatchArgs<TT>& A, const QPlan* __restrict__ PL, boo
                     if (cnt) {
                         acc.f[A_COUNT] += cnt;
                         if (Q.mode == TM_MODE_ESTIMATE) add_weight_n(acc, Q, tl - ot1, (unsigned long long)cnt);
+                        if (RIDE && Q.nride) { rx = tl; rn = -(int32_t)cnt; }
                     }
                 }
             } else {
@@ -1161,17 +1175,21 @@ __device__ void expand(const MatchArgs<TT>& A, const QPlan* __restrict__ PL, boo
                         const LevelPlan L = Q.lv[Q.l - 1];
                         if (ok && D == Q.l - 2 && Q.mode == TM_MODE_EXACT && L.view == kPair && !Q.hoist) {
                             // close here: the last edge counted by range length
-                            acc.f[A_COUNT] += pair_count(G, phi_get(ophi, L.su), phi_get(ophi, L.sv), tc, othi);
+                            int64_t clo, chi;
+                            pair_range(G, phi_get(ophi, L.su), phi_get(ophi, L.sv), tc, othi, clo, chi);
+                            acc.f[A_COUNT] += chi - clo;
                             acc.s(A_LAST) += 1;
+                            if (RIDE && Q.nride) { rx = clo; rn = (int32_t)(chi - clo); }
                             deeper = false;
                         }
                     }
                 }
             }
         }
+        if constexpr (RIDE) ride_emit(A, rx, rn, ot1, tc, oq);
         if constexpr (D + 1 < LMAX) {
             if (__any_sync(kFull, deeper))
-                expand<TT, D + 1, LMAX, KMAX>(A, PL, deeper, oq, ow, ophi, ot1, tc, othi, oha, ohh, acc);
+                expand<TT, D + 1, LMAX, KMAX, RIDE>(A, PL, deeper, oq, ow, ophi, ot1, tc, othi, oha, ohh, acc);
         }
     }
 }
@@ -1184,7 +1202,7 @@ __device__ void expand(const MatchArgs<TT>& A, const QPlan* __restrict__ PL, boo
 // bound nodes, two-node, riding along, or of at most two edges): the code the hot loop does
 // not run still takes registers, and without it the 3-cycle enumeration of the benchmark
 // batch runs 1.50 -> 1.32 ms
-template <typename TT, int LMAX, int KMAX, int OCC = (LMAX <= 3 ? 4 : 1), bool EXPAND = true>
+template <typename TT, int LMAX, int KMAX, int OCC = (LMAX <= 3 ? 4 : 1), bool EXPAND = true, bool RIDE = false>
 __global__ void __launch_bounds__(256, OCC) k_match(MatchArgs<TT> A) {
     const GraphDevT<TT>& G = A.G;
     extern __shared__ __align__(16) unsigned char smem_plans[];
@@ -1379,25 +1397,10 @@ __global__ void __launch_bounds__(256, OCC) k_match(MatchArgs<TT> A) {
                 }
                 }
             }
-            // the round's deferred records, appended with one atomic per warp
-            const unsigned rm = __ballot_sync(kFull, rn != 0);
-            if (rm) {
-                unsigned long long rb = 0;
-                if (lane == 0) rb = atomicAdd(A.rcount, (unsigned long long)__popc(rm));
-                rb = __shfl_sync(kFull, rb, 0) + __popc(rm & ((1u << lane) - 1u));
-                if (rn && (int64_t)rb < A.rcap) {
-                    RideRec<TT> rr;
-                    rr.x = rx;
-                    rr.t1 = (TT)t1;
-                    rr.tc = (TT)tc;
-                    rr.q = q;
-                    rr.n = rn;
-                    A.rrec[rb] = rr;
-                }
-            }
+            ride_emit(A, rx, rn, t1, tc, q);
             if constexpr (EXPAND) {
                 if (__any_sync(kFull, deeper))
-                    expand<TT, 2, LMAX, KMAX>(A, PL, deeper, q, win, phi, t1, tc, thi, ha, hh, acc);
+                    expand<TT, 2, LMAX, KMAX, RIDE>(A, PL, deeper, q, win, phi, t1, tc, thi, ha, hh, acc);
             } else {
                 TM_CHK(!deeper, kChkQueue);   // the host's choice of EXPAND = false must hold
             }
@@ -1412,60 +1415,56 @@ __global__ void __launch_bounds__(256, OCC) k_match(MatchArgs<TT> A) {
 // usual case: neighbouring records come from the same first edges) their sums are added once,
 // by one lane, instead of 32 times to the same shared-memory slot.
 template <typename TT>
-__device__ __forceinline__ void ride_warp(const QPlan* __restrict__ PL, const QPlan& Q,
-                                          const int32_t* __restrict__ kept, unsigned long long* acc,
+__device__ __forceinline__ void ride_warp(const QPlan& Q, const int32_t* __restrict__ kept, unsigned long long* acc,
                                           const TT* __restrict__ ta, bool valid, const RideRec<TT>& r) {
     const int lane = threadIdx.x & 31;
     const int64_t t1 = (int64_t)r.t1, tc = (int64_t)r.tc;
     const bool at = r.n < 0;
     unsigned long long nread = 0;
     for (int rr = 0; rr < Q.nride; rr++) {
-        const QPlan& R = PL[Q.ride_q[rr]];
-        const bool all_kept = R.q_mode == TM_Q_UNIFORM && R.p >= 1.0;   // no keep flag to read
-        for (int k = 0; k < R.b; k++) {
-            unsigned long long cnt = 0, wl = 0, wh = 0;
-            int64_t w = -1;
-            if (valid) {
-                int64_t thi;
-                ride_window(R, k, t1, w, thi);
-                if (at) {
-                    const int64_t t3 = r.x;   // -n instances closed at t3
-                    if (t3 - t1 <= R.delta && t3 <= thi && (all_kept || kept[w])) {
-                        cnt = (unsigned long long)(-(int64_t)r.n);
-                        ride_weight(R, t3 - t1, cnt, wl, wh);
-                    }
-                } else if (t1 + R.delta > tc && thi > tc && (all_kept || kept[w])) {
-                    for (int64_t x = r.x; x < r.x + r.n; x++) {
-                        const int64_t t3 = (int64_t)ta[x];
-                        if (t3 > thi) break;   // times increase
-                        unsigned long long l, h;
-                        ride_weight(R, t3 - t1, 1, l, h);
-                        const unsigned long long y = wl + l;
-                        wh += h + (y < wl ? 1ull : 0ull);
-                        wl = y;
-                        cnt++;
-                    }
-                    nread = max(nread, cnt);
+        const RideEnt R = Q.rides[rr];
+        unsigned long long cnt = 0, wl = 0, wh = 0;
+        int64_t w = -1;
+        if (valid) {
+            int64_t thi;
+            ride_window(R, t1, w, thi);
+            if (at) {
+                const int64_t t3 = r.x;   // -n instances closed at t3
+                if (t3 <= thi && (R.all_kept || kept[w])) {
+                    cnt = (unsigned long long)(-(int64_t)r.n);
+                    ride_weight(R, t3 - t1, cnt, wl, wh);
                 }
-            }
-            const unsigned hm = __ballot_sync(kFull, cnt != 0);
-            if (!hm) continue;
-            const int first = __ffs(hm) - 1;
-            const int64_t w0 = __shfl_sync(kFull, w, first);
-            if (__all_sync(kFull, cnt == 0 || w == w0)) {
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) {
-                    cnt += __shfl_xor_sync(kFull, cnt, o);
-                    const unsigned long long l2 = __shfl_xor_sync(kFull, wl, o);
-                    const unsigned long long h2 = __shfl_xor_sync(kFull, wh, o);
-                    const unsigned long long y = wl + l2;
-                    wh = wh + h2 + (y < wl ? 1ull : 0ull);
+            } else if (thi > tc && (R.all_kept || kept[w])) {
+                for (int64_t x = r.x; x < r.x + r.n; x++) {
+                    const int64_t t3 = (int64_t)ta[x];
+                    if (t3 > thi) break;   // times increase
+                    unsigned long long l, h;
+                    ride_weight(R, t3 - t1, 1, l, h);
+                    const unsigned long long y = wl + l;
+                    wh += h + (y < wl ? 1ull : 0ull);
                     wl = y;
+                    cnt++;
                 }
-                if (lane == first) ride_add(acc, w0, cnt, wl, wh);
-            } else if (cnt) {
-                ride_add(acc, w, cnt, wl, wh);
+                nread = max(nread, cnt);
             }
+        }
+        const unsigned hm = __ballot_sync(kFull, cnt != 0);
+        if (!hm) continue;
+        const int first = __ffs(hm) - 1;
+        const int64_t w0 = __shfl_sync(kFull, w, first);
+        if (__all_sync(kFull, cnt == 0 || w == w0)) {
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                cnt += __shfl_xor_sync(kFull, cnt, o);
+                const unsigned long long l2 = __shfl_xor_sync(kFull, wl, o);
+                const unsigned long long h2 = __shfl_xor_sync(kFull, wh, o);
+                const unsigned long long y = wl + l2;
+                wh = wh + h2 + (y < wl ? 1ull : 0ull);
+                wl = y;
+            }
+            if (lane == first) ride_add(acc, w0, cnt, wl, wh);
+        } else if (cnt) {
+            ride_add(acc, w, cnt, wl, wh);
         }
     }
     // entries read one by one: per record the most any rider shift read, summed over the warp
@@ -1532,11 +1531,11 @@ __global__ void __launch_bounds__(256) k_ride(MatchArgs<TT> A) {
         const int32_t q0 = __shfl_sync(kFull, q, 0);
         const bool uniform = __all_sync(kFull, !valid || q == q0);
         if (uniform && q0 >= 0) {
-            if (PL[q0].nride) ride_warp(PL, PL[q0], A.W.kept, A.W.acc, G.pair_t, valid, r);
+            if (PL[q0].nride) ride_warp(PL[q0], A.W.kept, A.W.acc, G.pair_t, valid, r);
         } else if (!uniform && valid && PL[q].nride) {
             const QPlan& Q = PL[q];
-            if (r.n < 0) ride_at(PL, Q, A.W.kept, A.W.acc, (int64_t)r.t1, r.x, (unsigned long long)(-(int64_t)r.n));
-            else ride_range(PL, Q, A.W.kept, A.W.acc, G.pair_t, r.x, r.x + r.n, (int64_t)r.t1, (int64_t)r.tc);
+            if (r.n < 0) ride_at(Q, A.W.kept, A.W.acc, (int64_t)r.t1, r.x, (unsigned long long)(-(int64_t)r.n));
+            else ride_range(Q, A.W.kept, A.W.acc, G.pair_t, r.x, r.x + r.n, (int64_t)r.t1, (int64_t)r.tc);
         }
     }
     acc_flush_warp(acc, A.W.acc);
@@ -1734,6 +1733,7 @@ void launch_match(const MatchArgs<TT>& A, int lmax, int kmax, const Tuning& tu, 
         else k_match<TT, 3, 4, 4, false><<<gm, bt, sm, st>>>(A);
     } else if (lmax <= 3 && kmax <= 4 && bps >= 6) k_match<TT, 3, 4, 6><<<gm, bt, sm, st>>>(A);
     else if (lmax <= 3 && kmax <= 4) k_match<TT, 3, 4><<<gm, bt, sm, st>>>(A);
+    else if (lmax <= 4 && kmax <= 4 && A.rrec) k_match<TT, 4, 4, 4, true, true><<<gm, bt, sm, st>>>(A);
     else if (lmax <= 4 && kmax <= 4 && bps >= 4) k_match<TT, 4, 4, 4><<<gm, bt, sm, st>>>(A);
     else if (lmax <= 4 && kmax <= 4) k_match<TT, 4, 4><<<gm, bt, sm, st>>>(A);
     else if (lmax <= 4) k_match<TT, 4, TM_K_MAX><<<gm, bt, sm, st>>>(A);
@@ -2005,6 +2005,25 @@ void launch_wtabs(const std::vector<QPlan>& hp, const std::vector<int32_t>& own,
     count_launch();
 }
 
+// shift k of rider R (a plan with its windows placed)
+RideEnt ride_entry(const QPlan& R, int k, int64_t t_max) {
+    RideEnt E;
+    std::memset(&E, 0, sizeof(E));
+    E.shift = -(int64_t)(draw(R.seed, (uint64_t)k, 0) % (uint64_t)R.cd) - R.t_off;
+    E.wbase = R.win_base + (int64_t)k * R.J;
+    E.cd = R.cd;
+    E.delta = R.delta;
+    E.all_kept = R.q_mode == TM_Q_UNIFORM && R.p >= 1.0;
+    // every t1 - shift below 2^31: the reciprocal is exact (its error times 2^31 stays below 2^sh)
+    if (t_max - E.shift < (int64_t)1 << 31 && R.cd > 1 && R.cd < (int64_t)1 << 31) {
+        int l = 1;
+        while (((int64_t)1 << l) < R.cd) l++;
+        E.sh = (uint32_t)(31 + l);
+        E.mul = (uint32_t)((((unsigned __int128)1 << E.sh) + (unsigned __int128)R.cd - 1) / (unsigned __int128)R.cd);
+    }
+    return E;
+}
+
 template <typename TT>
 int run_batch_t(const tm_graph* g, const tm_query* qs, int nq, tm_result* res, cudaStream_t st,
                 BatchOut* dbg) {
@@ -2018,6 +2037,12 @@ int run_batch_t(const tm_graph* g, const tm_query* qs, int nq, tm_result* res, c
     int lmax = 1, kmax = 2;
     bool any_hoist = false, any_full = false;
     size_t full_bytes = 0;
+    std::vector<char> is_rider;
+    if (dbg && dbg->riders) {
+        is_rider.assign((size_t)nq, 0);
+        for (const std::vector<int>& v : *dbg->riders)
+            for (int r : v) is_rider[(size_t)r] = 1;
+    }
     for (int i = 0; i < nq; i++) {
         std::string why;
         int s = validate_query(g, qs[i], why);
@@ -2053,12 +2078,7 @@ int run_batch_t(const tm_graph* g, const tm_query* qs, int nq, tm_result* res, c
             P.nsub = std::min(dbg->nsub[i], (int32_t)kMaxSub);
             for (int x = 0; x < P.nsub; x++) P.dsub[x] = dbg->sub_delta[(size_t)i * kMaxSub + x];
         }
-        if (dbg && dbg->ride_q && hp[(size_t)i].mode == TM_MODE_EXACT) {
-            QPlan& P = hp[(size_t)i];
-            for (int x = 0; x < kMaxRide; x++)
-                if (dbg->ride_q[(size_t)i * kMaxRide + x] >= 0) P.ride_q[P.nride++] = dbg->ride_q[(size_t)i * kMaxRide + x];
-        }
-        if (dbg && dbg->riding && dbg->riding[i] && hp[(size_t)i].mode == TM_MODE_ESTIMATE) {
+        if (!is_rider.empty() && is_rider[(size_t)i]) {
             QPlan& P = hp[(size_t)i];
             undo_wclamp(P);   // its instances arrive per window
             P.riding = 1;
@@ -2083,16 +2103,23 @@ int run_batch_t(const tm_graph* g, const tm_query* qs, int nq, tm_result* res, c
     // exact queries with riders or smaller spans leave that work to k_ride in records; the
     // record buffer holds as many as the largest batch so far needed (a batch that needs more
     // runs again with room for all of them)
+    // the riders' shifts, one entry each, in their exact query's order
+    std::vector<RideEnt> h_rides;
+    std::vector<size_t> ride_at0((size_t)nq, 0);
+    if (dbg && dbg->riders)
+        for (int i = 0; i < nq; i++) {
+            QPlan& P = hp[(size_t)i];
+            ride_at0[(size_t)i] = h_rides.size();
+            for (int r : (*dbg->riders)[(size_t)i]) {
+                const QPlan& R = hp[(size_t)r];
+                for (int k = 0; k < R.b; k++) h_rides.push_back(ride_entry(R, k, g->t_max));
+            }
+            P.nride = (int32_t)(h_rides.size() - ride_at0[(size_t)i]);
+        }
     bool any_share = false;
     for (const QPlan& P : hp) any_share |= P.nsub > 0 || P.nride > 0;
     const int64_t rcap = any_share ? ride_capacity().load() : 0;
     const size_t rrec_bytes = any_share ? a256(sizeof(RideRec<TT>) * (size_t)rcap) : 0;
-    // window origins of the riding estimates' shifts, read per instance on the device
-    std::vector<int64_t> h_shifts;
-    for (const QPlan& P : hp)
-        if (P.riding)
-            for (int k = 0; k < P.b; k++)
-                h_shifts.push_back(-(int64_t)(draw(P.seed, (uint64_t)k, 0) % (uint64_t)P.cd) - P.t_off);
     // ---- scratch layout
     int smax = 1;
     const int64_t n_parts = fold_parts(hp, smax);
@@ -2107,7 +2134,7 @@ int run_batch_t(const tm_graph* g, const tm_query* qs, int nq, tm_result* res, c
                 full_bytes + (any_full ? 3 * a256(4 * Ms) : 0) +
                 a256(sizeof(ShiftSums) * (size_t)std::max<int64_t>(n_sums, 1)) +
                 a256(sizeof(ShiftSums) * (size_t)n_parts) +
-                a256(8 * kMaxSub * (size_t)nq) + a256(8 * std::max<size_t>(h_shifts.size(), 1));
+                a256(8 * kMaxSub * (size_t)nq) + a256(sizeof(RideEnt) * std::max<size_t>(h_rides.size(), 1));
     char* sb = nullptr;
     TM_CUDA(cudaMallocAsync((void**)&sb, sz, st));
     char* p = sb;
@@ -2148,11 +2175,13 @@ int run_batch_t(const tm_graph* g, const tm_query* qs, int nq, tm_result* res, c
     ShiftSums* dsums = (ShiftSums*)take(sizeof(ShiftSums) * (size_t)std::max<int64_t>(n_sums, 1));
     ShiftSums* dpart = (ShiftSums*)take(sizeof(ShiftSums) * (size_t)n_parts);
     unsigned long long* dsubc = (unsigned long long*)take(8 * kMaxSub * (size_t)nq);
-    int64_t* dshifts = (int64_t*)take(8 * std::max<size_t>(h_shifts.size(), 1));
-    for (size_t i = 0, o = 0; i < (size_t)nq; i++)
-        if (hp[i].riding) {
-            hp[i].shifts = dshifts + o;
-            o += (size_t)hp[i].b;
+    RideEnt* drides = (RideEnt*)take(sizeof(RideEnt) * std::max<size_t>(h_rides.size(), 1));
+    for (int i = 0; i < nq; i++) hp[(size_t)i].rides = drides + ride_at0[(size_t)i];
+    if (!h_rides.empty())   // their weight tables have places now
+        for (int i = 0; i < nq; i++) {
+            size_t o = ride_at0[(size_t)i];
+            for (int r : (*dbg->riders)[(size_t)i])
+                for (int k = 0; k < hp[(size_t)r].b; k++) h_rides[o++].wtab = hp[(size_t)r].wtab;
         }
 
     int rc = TM_OK;
@@ -2169,8 +2198,8 @@ int run_batch_t(const tm_graph* g, const tm_query* qs, int nq, tm_result* res, c
     uint32_t h_serr = 0;
     std::vector<char> h_plans;
     fail(copy_plans(hp, wown, h_plans, dplans, st), "plans");
-    if (!h_shifts.empty())
-        fail(cudaMemcpyAsync(dshifts, h_shifts.data(), 8 * h_shifts.size(), cudaMemcpyHostToDevice, st), "shifts");
+    if (!h_rides.empty())
+        fail(cudaMemcpyAsync(drides, h_rides.data(), sizeof(RideEnt) * h_rides.size(), cudaMemcpyHostToDevice, st), "riders");
     fail(cudaMemsetAsync(W.acc, 0, 8 * A_N * NWs, st), "acc");
     fail(cudaMemsetAsync(dctr, 0, 8, st), "counter");
     fail(cudaMemsetAsync(drcount, 0, 8, st), "record counter");
@@ -2383,7 +2412,7 @@ int run_batch_t(const tm_graph* g, const tm_query* qs, int nq, tm_result* res, c
         if (qstat[(size_t)i] != TM_OK) {
             std::memset(&res[i], 0, sizeof(tm_result));
             res[i].status = qstat[(size_t)i];
-        } else if (res[i].status != TM_OK && first_err == TM_OK) {
+        } else if (res[i].status != TM_OK && first_err == TM_OK && i < nq - (dbg ? dbg->hidden : 0)) {
             first_err = res[i].status;
             set_error("query " + std::to_string(i) + ": count or weight sum overflowed 2^63");
         }
@@ -2407,6 +2436,12 @@ bool same_motif(const tm_motif* a, const tm_motif* b) {
     if (a->l != b->l || a->k != b->k) return false;
     return std::memcmp(a->lv, b->lv, sizeof(LevelPlan) * (size_t)a->l) == 0;
 }
+
+// When estimates share an enumeration of their own (run_batch_once).  Both sides, us a call on 1e7
+// edges: the nine calibrated estimates (sums 1.5 to 2.6 first edges per motif, candidates 1.02 to
+// 1.04) 6,362 apart and 3,352 sharing; 192 seeds of the 4-cycle (10.6 of each) 49,200 apart and
+// 6,580 sharing, build included.  The margin over 1 pays for the records and their weighing.
+constexpr double kHideFirst = 1.4, kHideCand = 0.9;
 
 int run_batch_once(const tm_graph* g, const tm_query* qs, int nq, tm_result* res, cudaStream_t st,
                    BatchOut* dbg) {
@@ -2444,14 +2479,22 @@ int run_batch_once(const tm_graph* g, const tm_query* qs, int nq, tm_result* res
     // along with it: each instance that query enumerates also adds its weight to the window of
     // an estimate when it lies inside one of its kept windows and within its span, so the
     // estimate needs no enumeration of its own (its windows and fold stay its own)
-    std::vector<int> host((size_t)nq, -1);    // estimate -> its exact head
+    std::vector<int> host((size_t)nq, -1);    // estimate -> its exact head (nq + h: hidden head h)
     std::vector<int> nrid((size_t)nq, 0);
+    std::vector<int> alone;                   // estimates that could ride and have no head
+    int lmax = 1, kmax = 2;
+    for (int i = 0; i < nq; i++)
+        if (qs[i].motif) {
+            lmax = std::max(lmax, qs[i].motif->l);
+            kmax = std::max(kmax, qs[i].motif->k);
+        }
     for (int i = 0; i < nq; i++) {
         const tm_query& q = qs[i];
         std::string why;
         if (q.mode != TM_MODE_ESTIMATE || (q.q_mode != TM_Q_UNIFORM && q.q_mode != TM_Q_EDGES)) continue;
-        if (!q.motif || q.motif->l != 3 || q.motif->lv[2].view != kPair) continue;
-        if (validate_query(g, q, why) != TM_OK) continue;
+        // (four edges: the matcher's four-edge instantiation emits the records)
+        if (!q.motif || (q.motif->l != 3 && !(q.motif->l == 4 && lmax <= 4 && kmax <= 4))) continue;
+        if (q.motif->lv[q.motif->l - 1].view != kPair || validate_query(g, q, why) != TM_OK) continue;
         for (int L : heads)
             if (nrid[(size_t)L] < kMaxRide && qs[L].delta >= q.delta && same_motif(qs[L].motif, q.motif)) {
                 host[(size_t)i] = L;
@@ -2459,21 +2502,53 @@ int run_batch_once(const tm_graph* g, const tm_query* qs, int nq, tm_result* res
                 any = true;
                 break;
             }
+        if (host[(size_t)i] < 0) alone.push_back(i);
+    }
+    // Estimates of one motif without such an exact query: when together they keep enough windows,
+    // one enumeration of the whole graph for all of them costs less than their own, so they ride
+    // along with an exact query that nobody asked for.  Theirs cost, in first edges, sum b p, and in
+    // candidates (which grow with the span) sum b p delta; the shared one 1 and its span.  It is
+    // taken for the longest span for which the first sum is at least kHideFirst and the second at
+    // least kHideCand of it (measured: see kHideFirst).
+    std::vector<tm_query> hidden;
+    std::vector<int> top;                     // per hidden head, the estimate whose span it has
+    for (size_t x = 0; x < alone.size(); x++) {
+        if (host[(size_t)alone[x]] >= 0) continue;
+        std::vector<int> gr;
+        for (size_t y = x; y < alone.size(); y++)
+            if (host[(size_t)alone[y]] < 0 && same_motif(qs[alone[x]].motif, qs[alone[y]].motif)) gr.push_back(alone[y]);
+        std::stable_sort(gr.begin(), gr.end(), [&](int a, int b) { return qs[a].delta > qs[b].delta; });
+        for (size_t y = 0; y < gr.size(); y++) {
+            double first = 0.0, cand = 0.0;
+            const size_t n = std::min(gr.size() - y, (size_t)kMaxRide);
+            for (size_t z = y; z < y + n; z++) {
+                const tm_query& q = qs[gr[z]];
+                const double J = 1.0 + (double)g->t_max / ((double)q.c * (double)q.delta);
+                const double p = q.q_mode == TM_Q_UNIFORM ? q.p : std::min(1.0, q.p / J);
+                first += p * q.b;
+                cand += p * q.b * ((double)q.delta / (double)qs[gr[y]].delta);
+            }
+            if (first < kHideFirst || cand < kHideCand) continue;
+            tm_query e = qs[gr[y]];
+            e.mode = TM_MODE_EXACT;
+            for (size_t z = y; z < y + n; z++) host[(size_t)gr[z]] = nq + (int)hidden.size();
+            hidden.push_back(e);
+            top.push_back(gr[y]);
+            any = true;
+            break;
+        }
     }
     if (!any) return run_batch_typed(g, qs, nq, res, st, nullptr);
     // the batch without the span members, each head carrying its members' spans and riders
     std::vector<tm_query> qc;
-    std::vector<int> pos((size_t)nq, -1);
+    std::vector<int> pos((size_t)nq + hidden.size(), -1);
     for (int i = 0; i < nq; i++)
         if (lead[(size_t)i] < 0) { pos[(size_t)i] = (int)qc.size(); qc.push_back(qs[i]); }
+    for (size_t h = 0; h < hidden.size(); h++) { pos[(size_t)nq + h] = (int)qc.size(); qc.push_back(hidden[h]); }
     int nc = (int)qc.size();
-    std::vector<int32_t> riding((size_t)nc, 0), ride_q((size_t)nc * kMaxRide, -1), fill((size_t)nc, 0);
-    for (int i = 0; i < nq; i++) {
-        if (host[(size_t)i] < 0) continue;
-        int c = pos[(size_t)i], h = pos[(size_t)host[(size_t)i]];
-        riding[(size_t)c] = 1;
-        ride_q[(size_t)h * kMaxRide + fill[(size_t)h]++] = c;
-    }
+    std::vector<std::vector<int>> riders((size_t)nc);
+    for (int i = 0; i < nq; i++)
+        if (host[(size_t)i] >= 0) riders[(size_t)pos[(size_t)host[(size_t)i]]].push_back(pos[(size_t)i]);
     std::vector<int32_t> nsub((size_t)nc, 0);
     std::vector<int64_t> sd((size_t)nc * kMaxSub, 0);
     for (int i = 0; i < nq; i++) {
@@ -2488,8 +2563,8 @@ int run_batch_once(const tm_graph* g, const tm_query* qs, int nq, tm_result* res
     bo.nsub = nsub.data();
     bo.sub_delta = sd.data();
     bo.sub_count = sc.data();
-    bo.riding = riding.data();
-    bo.ride_q = ride_q.data();
+    bo.riders = &riders;
+    bo.hidden = (int)hidden.size();
     int rc = run_batch_typed(g, qc.data(), nc, rc_res.data(), st, &bo);
     for (int i = 0; i < nq; i++) {
         if (lead[(size_t)i] < 0) {
@@ -2502,6 +2577,14 @@ int run_batch_once(const tm_graph* g, const tm_query* qs, int nq, tm_result* res
         r.estimate = (double)r.count;
         r.first_edges = r.cand_edges = r.last_ranges = r.inst_read = 0;   // the work is the leader's
         res[i] = r;
+    }
+    for (size_t h = 0; h < hidden.size(); h++) {   // its work is reported by the estimate with its span
+        const tm_result& w = rc_res[(size_t)pos[(size_t)nq + h]];
+        tm_result& r = res[top[h]];
+        r.first_edges += w.first_edges;
+        r.cand_edges += w.cand_edges;
+        r.last_ranges += w.last_ranges;
+        r.inst_read += w.inst_read;
     }
     return rc;
 }

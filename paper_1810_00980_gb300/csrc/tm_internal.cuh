@@ -7,6 +7,7 @@
 
 #include <atomic>
 #include <string>
+#include <vector>
 
 #include "../../include/tm.h"
 
@@ -223,6 +224,19 @@ enum FirstOrder : int32_t { kOrdTime = 0, kOrdOut = 1, kOrdIn = 2, kOrdPair = 3 
 // the last edge each either repeat (u,v) or reverse it (v,u)
 enum Ex23Bits : int32_t { kEx23On = 1, kEx23MidRev = 2, kEx23LastRev = 4 };
 
+// one shift of an estimate riding along with an exact query
+struct alignas(16) RideEnt {
+    int64_t shift;        // window origin -(shift draw mod cd) - t_off
+    int64_t wbase;        // the shift's first window slot
+    int64_t cd, delta;
+    const uint64_t* wtab; // as QPlan::wtab
+    // (t1 - shift) / cd as (t1 - shift) * mul >> sh for every time of the graph, by the rounded-up
+    // reciprocal of Granlund and Montgomery (1994); sh = 0: divide
+    uint32_t mul, sh;
+    int32_t all_kept;     // uniform p = 1: no keep flag to read
+    int32_t pad0[3];
+};
+
 struct QPlan {
     int32_t l, k;
     int32_t mode;        // TM_MODE_*
@@ -267,14 +281,17 @@ struct QPlan {
     // estimates of the same motif riding along with this exact query: every instance this
     // query enumerates is also added, with the rider's weight, to the rider's window when it
     // lies inside a kept window of the rider and within the rider's span
-    int32_t nride;
+    int32_t nride;       // entries of `rides`: one per shift of every rider
     int32_t riding;      // 1: this estimate rides along with an exact query (no first edges)
-    int32_t ride_q[6];   // plan indices of the riders
-    const int64_t* shifts;   // riding estimates: [b] window origins -(shift draw mod cd) - t_off
+    const RideEnt* rides;
+    // (a stride of 320 bytes: plans staged in shared memory at 328 made the replay of a batch 1.5 %
+    // slower)
+    int64_t pad0[3];
     LevelPlan lv[TM_L_MAX];
 };
 constexpr int kMaxSub = 3;
-constexpr int kMaxRide = 6;
+constexpr int kMaxRide = 4096;   // riders of one exact query
+static_assert(sizeof(QPlan) == 320, "plan stride");
 
 struct Tuning {
     int block_threads = 256;
@@ -317,8 +334,8 @@ struct BatchOut {                 // optional per-window readback for one query
     int64_t shift = 0;
     const SegSpec* seg = nullptr; // per query, or null (whole graph)
     ShiftSums* sums = nullptr;    // host: per query, per shift (exact: one), or null
-    const int32_t* riding = nullptr;          // per query: 1 if it rides along (no first edges)
-    const int32_t* ride_q = nullptr;          // per query: [kMaxRide] plan indices of its riders, -1 unused
+    const std::vector<std::vector<int>>* riders = nullptr;   // per query: plan indices of its riders
+    int hidden = 0;                           // trailing queries whose results nobody asked for
     const int32_t* nsub = nullptr;            // per query: spans counted alongside (exact)
     const int64_t* sub_delta = nullptr;       // [nq][kMaxSub]
     unsigned long long* sub_count = nullptr;  // host out: [nq][kMaxSub]
