@@ -15,8 +15,7 @@
 //              expanded warp-cooperatively (range lengths scanned across the
 //              warp, each lane takes one candidate, owner found by shuffles);
 //              in exact mode the last motif edge is counted by range length.
-//   k_fold_shift, k_fold_final
-//              per query, shift and slice of windows the partial sums, then per
+//   k_fold     per query, shift and slice of windows the partial sums, then per
 //              query: Z_k = sum_j W_j / q_j per shift and the mean over shifts
 //              (Algorithm 1's return value).
 #include <algorithm>
@@ -119,7 +118,7 @@ struct MatchArgs {
     int64_t chunk;
     int enum_threshold;
     const int32_t* blockwin = nullptr;  // [ceil(F/32)] window of first edge 32 b (null: searched)
-    const int64_t* chunkf = nullptr;    // [nchunkf] first edge of work item i * chunk (null: searched)
+    const int64_t* chunkf = nullptr;    // [nchunkf] first edge of work item i * kItemGrain (null: searched)
     int64_t nchunkf = 0;
     RideRec<TT>* rrec = nullptr;        // [rcap] deferred rider / smaller-span work (see RideRec)
     unsigned long long* rcount = nullptr;   // records appended (counts past rcap: the batch reruns)
@@ -641,6 +640,8 @@ size_t match_smem_bytes(int nq, int threads, bool ride_tab = false) {
 }
 
 // ----------------------------------------------------------------- kernels
+constexpr int kWindowThreads = 256;
+
 // Every weight table of the batch in one launch, table y by row y of the grid (plan own[y]'s;
 // plans with the same delta and c delta share a table).  A weight costs three divisions, so
 // that a long table is bound by the 16 bytes it writes per duration.  A bench batch on 1e6 edges
@@ -662,8 +663,11 @@ __global__ void k_wtab(const QPlan* __restrict__ plans, const int32_t* __restric
     }
 }
 
+// (dF given, by a caller with no more windows than the one block's threads: their first edges'
+// offsets and number too, instead of by a scan of their own)
 template <typename TT>
-__global__ void k_windows(GraphDevT<TT> G, const QPlan* __restrict__ plans, int nq, WinDev W, int64_t NW) {
+__global__ void k_windows(GraphDevT<TT> G, const QPlan* __restrict__ plans, int nq, WinDev W, int64_t NW,
+                          int64_t* __restrict__ dF) {
     for (int64_t w = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; w < NW;
          w += (int64_t)gridDim.x * blockDim.x) {
         int lo_q = 0, hi_q = nq;
@@ -719,6 +723,26 @@ __global__ void k_windows(GraphDevT<TT> G, const QPlan* __restrict__ plans, int 
         W.q[w] = lo_q; W.k[w] = k; W.kept[w] = kept; W.qj[w] = qj;
         W.nfirst[w] = (kept && !Q.riding) ? hi - lo : 0;   // riders take no first edges
     }
+    if (!dF) return;
+    __shared__ int64_t s_warp[kWindowThreads / 32];
+    const int64_t mine = threadIdx.x < NW ? W.nfirst[threadIdx.x] : 0, inc = warp_incl_scan64(mine);
+    if ((threadIdx.x & 31) == 31) s_warp[threadIdx.x >> 5] = inc;
+    __syncthreads();
+    int64_t before = 0;
+    for (int i = 0; i < (int)(threadIdx.x >> 5); i++) before += s_warp[i];
+    if (threadIdx.x < NW) W.fbase[threadIdx.x] = before + inc - mine;
+    if (threadIdx.x == NW - 1) *dF = before + inc;
+}
+
+// windows of a batch, and the scan of their first edges' numbers (words: scan_once_words(NW))
+template <typename TT>
+int launch_windows(const GraphDevT<TT>& G, const QPlan* dplans, int nq, const WinDev& W, int64_t NW, int64_t* dF,
+                   unsigned long long* words, uint32_t* err, int nsm, cudaStream_t st) {
+    const bool one = NW <= kWindowThreads;
+    const unsigned gr = (unsigned)std::min<int64_t>((NW + kWindowThreads - 1) / kWindowThreads, (int64_t)nsm * 16);
+    k_windows<TT><<<gr, kWindowThreads, 0, st>>>(G, dplans, nq, W, NW, one ? dF : nullptr); count_launch();
+    TM_CUDA(cudaGetLastError());
+    return one ? TM_OK : scan_once_i64(W.nfirst, W.fbase, NW, dF, words, err, st);
 }
 
 // window index (0-based) of every position of a node-grouped view for shift s
@@ -767,18 +791,6 @@ __global__ void k_blockwin(const int64_t* __restrict__ fbase, int64_t NW, int64_
         }
         bw[b] = (int32_t)lo;
     }
-}
-
-// first edge of work item i * chunk (the start of k_match's i-th chunk), for the first
-// cap chunks and the one after the last
-__global__ void k_chunkf(const int64_t* __restrict__ excl, int64_t Fh, const int64_t* __restrict__ d_F,
-                         const int64_t* __restrict__ d_W2, int64_t chunk, int64_t cap,
-                         int64_t* __restrict__ cf) {
-    const int64_t F = d_F ? *d_F : Fh;
-    int64_t n = min(cap, (*d_W2 + chunk - 1) / chunk + 1);
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x)
-        cf[i] = upper_bound_i64(excl, 0, F, i * chunk) - 1;
 }
 
 // one warp-uniform grid-stride loop over first edges f
@@ -1213,19 +1225,23 @@ __global__ void __launch_bounds__(256, OCC) k_match(MatchArgs<TT> A) {
     Acc acc;
     acc_init(acc, smem_plans, A.nq);
     acc_zero(acc);
+    // few items: smaller chunks, so that every warp gets some (17,000 items in chunks of 256 kept 67
+    // warps busy for eight rounds each: 43 us of a 20,000-edge count)
+    const int64_t share = (W2 / (((int64_t)gridDim.x * blockDim.x) >> 5) + kItemGrain) / kItemGrain * kItemGrain;
+    const int64_t chunk = min(A.chunk, share);
     for (;;) {
         unsigned long long c0u = 0;
-        if (lane == 0) c0u = atomicAdd(A.counter, (unsigned long long)A.chunk);
+        if (lane == 0) c0u = atomicAdd(A.counter, (unsigned long long)chunk);
         int64_t c0 = (int64_t)__shfl_sync(kFull, c0u, 0);
         if (c0 >= W2) break;
-        int64_t c1 = min(c0 + A.chunk, W2);
+        int64_t c1 = min(c0 + chunk, W2);
         int64_t fb = 0, fe = 0;
-        int64_t ci = c0 / A.chunk;
-        if (A.chunkf && ci + 1 < A.nchunkf) {
+        const int64_t ci = c0 / kItemGrain, ce = (c1 + kItemGrain - 1) / kItemGrain;
+        if (A.chunkf && ce < A.nchunkf) {
             // first edges of this chunk's first item and of the next chunk's (a bound on
             // the last item's: first edges in between have no items below c1)
             fb = __ldg(A.chunkf + ci);
-            fe = __ldg(A.chunkf + ci + 1);
+            fe = __ldg(A.chunkf + ce);
         } else {
             if (lane < 2) {
                 int64_t key = lane == 0 ? c0 : c1 - 1;
@@ -1553,70 +1569,77 @@ __global__ void __launch_bounds__(256) k_ride(MatchArgs<TT> A) {
     }
 }
 
-// Windows of one shift that a block of k_fold_shift sums: a query's shifts are cut into
+// Windows of one shift that a block of k_fold sums: a query's shifts are cut into
 // fold_slices(J) slices of whole windows, a function of the query alone, so that its
 // result does not depend on the batch it runs in.
 constexpr int kFoldThreads = 256;
-constexpr int kFoldMaxSlices = 32;
+constexpr int kFoldMaxSlices = 32;   // one per lane when they are added
 __host__ __device__ inline int fold_slices(int64_t nwin) {
-    int64_t s = (nwin + 8 * kFoldThreads - 1) / (8 * kFoldThreads);
+    int64_t s = (nwin + 2 * kFoldThreads - 1) / (2 * kFoldThreads);
     return (int)(s < 1 ? 1 : (s > kFoldMaxSlices ? kFoldMaxSlices : s));
 }
 
-// Fold, first half: block (query, shift k, slice) sums the kept windows of its slice —
-// counts and work counters as integers, the Q64 weight sum W_j as a 128-bit integer, and
-// the doubles sum_j W_j / q_j (the shift's Z_k when q_j varies, Algorithm 1) and
-// sum_j W_j^2 (1 - q_j) / q_j^2 (Lemma 4.4) — into part[part_base + k * slices + slice].
+// the 32 lanes' sums in every lane (the doubles in a fixed order)
+__device__ __forceinline__ void warp_add_sums(ShiftSums& a) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        ShiftSums b;
+        b.count = __shfl_xor_sync(kFull, a.count, o);
+        b.wlo = __shfl_xor_sync(kFull, a.wlo, o);
+        b.whi = __shfl_xor_sync(kFull, a.whi, o);
+        b.first = __shfl_xor_sync(kFull, a.first, o);
+        b.cand = __shfl_xor_sync(kFull, a.cand, o);
+        b.last = __shfl_xor_sync(kFull, a.last, o);
+        b.inst = __shfl_xor_sync(kFull, a.inst, o);
+        b.kept = __shfl_xor_sync(kFull, a.kept, o);
+        b.zq = __shfl_xor_sync(kFull, a.zq, o);
+        b.vq = __shfl_xor_sync(kFull, a.vq, o);
+        add_shift_sums(a, b);
+    }
+}
+
+// The fold.  Block (query, shift k, slice) sums the kept windows of its slice — counts and work
+// counters as integers, the Q64 weight sum W_j as a 128-bit integer, and the doubles
+// sum_j W_j / q_j (the shift's Z_k when q_j varies, Algorithm 1) and
+// sum_j W_j^2 (1 - q_j) / q_j^2 (Lemma 4.4) — into part[part_base + k * slices + slice]; the last of
+// the query's blocks to get there adds the slices of each shift, a warp per shift, and then
+// the shifts in order: Z_k, their mean (the estimate of Algorithm 1), the mean variance
+// estimate and the spread of the Z_k (Welford).
 // The grid's y extent is capped at the hardware limit; a block then also takes the shifts
 // k + gridDim.y, k + 2 gridDim.y, ... (a loop that is uniform across the block).
-__global__ void __launch_bounds__(kFoldThreads) k_fold_shift(const QPlan* __restrict__ plans, WinDev W,
-                                                             ShiftSums* __restrict__ part) {
-    const QPlan& Q = plans[blockIdx.x];
+// A chain of dependent loads bounds it, not bytes: two windows per thread and one launch (eight
+// windows and a second launch with a thread per query took 24 + 18 us for the 18 queries of a
+// batch on 1e6 edges).
+__global__ void __launch_bounds__(kFoldThreads) k_fold(const QPlan* __restrict__ plans, WinDev W, ShiftSums* part,
+                                                       uint32_t* __restrict__ folded, tm_result* __restrict__ res,
+                                                       ShiftSums* __restrict__ sums, unsigned long long* __restrict__ subc) {
+    const int qi = blockIdx.x;
+    const QPlan& Q = plans[qi];
     const int sl = blockIdx.z;
     const int nsh = Q.l <= 0 ? 0 : (Q.mode == TM_MODE_EXACT ? 1 : Q.b);
     const int64_t nwin = Q.mode == TM_MODE_EXACT ? 1 : Q.J;
     const int ns = fold_slices(nwin);
-    if (sl >= ns) return;
+    if (sl >= ns || (int)blockIdx.y >= max(nsh, 1)) return;
     __shared__ ShiftSums sh[kFoldThreads / 32];
-    int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    __shared__ int s_last;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     for (int k = blockIdx.y; k < nsh; k += gridDim.y) {
-        unsigned long long c[6] = {0, 0, 0, 0, 0, 0};   // count, first, cand, last, inst, kept
-        unsigned long long wlo = 0, whi = 0;
-        double zq = 0.0, vq = 0.0;
+        ShiftSums a = {};
         for (int64_t r = (int64_t)sl * kFoldThreads + threadIdx.x; r < nwin; r += (int64_t)ns * kFoldThreads) {
-            int64_t w = Q.win_base + (int64_t)k * nwin + r;
+            const int64_t w = Q.win_base + (int64_t)k * nwin + r;
             if (!W.kept[w]) continue;
-            const unsigned long long* a = W.acc + w * A_N;
-            c[0] += a[A_COUNT];
-            c[1] += a[A_FIRST];
-            c[2] += a[A_CAND];
-            c[3] += a[A_LAST];
-            c[4] += a[A_INST];
-            c[5] += 1;
-            unsigned long long x = wlo + a[A_WLO];
-            whi += a[A_WHI] + (x < wlo ? 1ull : 0ull);
-            wlo = x;
-            double y = (double)a[A_WHI] + (double)a[A_WLO] * 0x1.0p-64;
-            double qj = W.qj[w];
-            if (Q.q_mode == TM_Q_EDGES) zq += y / qj;
-            vq += y * y * (1.0 - qj) / (qj * qj);
+            const unsigned long long* x = W.acc + w * A_N;
+            const double qj = W.qj[w];
+            ShiftSums b;
+            b.count = x[A_COUNT]; b.wlo = x[A_WLO]; b.whi = x[A_WHI]; b.first = x[A_FIRST];
+            b.cand = x[A_CAND]; b.last = x[A_LAST]; b.inst = x[A_INST]; b.kept = 1;
+            const double y = (double)b.whi + (double)b.wlo * 0x1.0p-64;
+            b.zq = Q.q_mode == TM_Q_EDGES ? y / qj : 0.0;
+            b.vq = y * y * (1.0 - qj) / (qj * qj);
+            add_shift_sums(a, b);
         }
-        for (int o = 16; o > 0; o >>= 1) {
-#pragma unroll
-            for (int i = 0; i < 6; i++) c[i] += __shfl_xor_sync(kFull, c[i], o);
-            unsigned long long l2 = __shfl_xor_sync(kFull, wlo, o);
-            unsigned long long h2 = __shfl_xor_sync(kFull, whi, o);
-            unsigned long long x = wlo + l2;
-            whi = whi + h2 + (x < wlo ? 1ull : 0ull);
-            wlo = x;
-            zq += __shfl_xor_sync(kFull, zq, o);
-            vq += __shfl_xor_sync(kFull, vq, o);
-        }
-        if (lane == 0) {
-            ShiftSums& o = sh[wid];
-            o.count = c[0]; o.first = c[1]; o.cand = c[2]; o.last = c[3]; o.inst = c[4]; o.kept = c[5];
-            o.wlo = wlo; o.whi = whi; o.zq = zq; o.vq = vq;
-        }
+        warp_add_sums(a);
+        if (lane == 0) sh[wid] = a;
         __syncthreads();
         if (threadIdx.x == 0) {
             ShiftSums t = sh[0];
@@ -1625,37 +1648,53 @@ __global__ void __launch_bounds__(kFoldThreads) k_fold_shift(const QPlan* __rest
         }
         __syncthreads();   // sh is written again by the next shift
     }
-}
-
-// Fold, second half: one thread per query adds its slices in order, then its shifts in
-// order: Z_k, their mean (the estimate of Algorithm 1), the mean variance estimate and
-// the spread of the Z_k (Welford).
-__global__ void k_fold_final(const QPlan* __restrict__ plans, int nq, WinDev W, const ShiftSums* __restrict__ part,
-                             tm_result* __restrict__ res, ShiftSums* __restrict__ sums,
-                             unsigned long long* __restrict__ subc) {
-    int qi = blockIdx.x * blockDim.x + threadIdx.x;
-    if (qi >= nq) return;
-    const QPlan& Q = plans[qi];
-    const int nsh = Q.l <= 0 ? 0 : (Q.mode == TM_MODE_EXACT ? 1 : Q.b);
-    const int ns = fold_slices(Q.mode == TM_MODE_EXACT ? 1 : Q.J);
-    double zsum = 0.0, vsum = 0.0, wmean = 0.0, wm2 = 0.0;
+    // the query's last block goes on
+    if (threadIdx.x == 0) {
+        const uint32_t blocks = (uint32_t)(min(max(nsh, 1), (int)gridDim.y) * ns);
+        __threadfence();
+        s_last = atomicAdd(folded + qi, 1u) + 1 == blocks;
+        __threadfence();
+    }
+    __syncthreads();
+    if (!s_last) return;
+    double zsum = 0.0, vsum = 0.0, wmean = 0.0, wm2 = 0.0;   // thread 0's
     ShiftSums tot = {};
     int overflow = 0;
-    for (int k = 0; k < nsh; k++) {
-        const ShiftSums* pk = part + Q.part_base + (int64_t)k * ns;
-        ShiftSums u = pk[0];
-        for (int x = 1; x < ns; x++) add_shift_sums(u, pk[x]);
-        if (sums) sums[Q.sum_base + k] = u;
-        if (u.whi >= (1ull << 63) || u.count >= (1ull << 63)) overflow = 1;
-        add_shift_sums(tot, u);
-        double Wd = (double)u.whi + (double)u.wlo * 0x1.0p-64;
-        double zk = Q.q_mode == TM_Q_EDGES ? u.zq : Wd / Q.p;
-        zsum += zk;
-        vsum += u.vq;
-        double dz = zk - wmean;
-        wmean += dz / (k + 1);
-        wm2 += dz * (zk - wmean);
+    constexpr int kWarps = kFoldThreads / 32;
+    for (int k0 = 0; k0 < nsh; k0 += kWarps) {
+        if (k0 + wid < nsh) {
+            const ShiftSums* pk = part + Q.part_base + (int64_t)(k0 + wid) * ns;
+            ShiftSums u = {};
+            if (lane < ns) {
+                const unsigned long long* x = reinterpret_cast<const unsigned long long*>(pk + lane);
+                unsigned long long* y = reinterpret_cast<unsigned long long*>(&u);
+#pragma unroll
+                for (int i = 0; i < (int)(sizeof(ShiftSums) / 8); i++) y[i] = __ldcg(x + i);   // other blocks wrote them
+            }
+            warp_add_sums(u);
+            if (lane == 0) {
+                sh[wid] = u;
+                if (sums) sums[Q.sum_base + k0 + wid] = u;
+            }
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            for (int k = k0; k < min(k0 + kWarps, nsh); k++) {
+                const ShiftSums& u = sh[k - k0];
+                if (u.whi >= (1ull << 63) || u.count >= (1ull << 63)) overflow = 1;
+                add_shift_sums(tot, u);
+                const double Wd = (double)u.whi + (double)u.wlo * 0x1.0p-64;
+                const double zk = Q.q_mode == TM_Q_EDGES ? u.zq : Wd / Q.p;
+                zsum += zk;
+                vsum += u.vq;
+                const double dz = zk - wmean;
+                wmean += dz / (k + 1);
+                wm2 += dz * (zk - wmean);
+            }
+        }
+        __syncthreads();
     }
+    if (threadIdx.x != 0) return;
     if (subc) {
         // counts of the exact queries at smaller spans (one window: the whole graph)
         const unsigned long long* a = W.acc + Q.win_base * A_N;
@@ -1703,13 +1742,12 @@ int64_t fold_parts(std::vector<QPlan>& hp, int& smax) {
 
 constexpr int kMaxGridY = 65535;
 
-// both halves of the fold on st
-void launch_fold(const QPlan* dplans, int nq, int bmax, int smax, const WinDev& W, ShiftSums* part,
+// the fold on st (folded: one zeroed counter per query)
+void launch_fold(const QPlan* dplans, int nq, int bmax, int smax, const WinDev& W, ShiftSums* part, uint32_t* folded,
                  tm_result* dres, ShiftSums* sums, unsigned long long* subc, cudaStream_t st) {
     unsigned gy = (unsigned)std::min(std::max(bmax, 1), kMaxGridY);
-    k_fold_shift<<<dim3((unsigned)nq, gy, (unsigned)smax), kFoldThreads, 0, st>>>(dplans, W, part);
-    k_fold_final<<<(unsigned)((nq + 63) / 64), 64, 0, st>>>(dplans, nq, W, part, dres, sums, subc);
-    count_launch(2);
+    k_fold<<<dim3((unsigned)nq, gy, (unsigned)smax), kFoldThreads, 0, st>>>(dplans, W, part, folded, dres, sums, subc);
+    count_launch();
 }
 
 // the persistent matcher for a batch whose deepest motif has lmax edges on kmax nodes: the
@@ -2129,9 +2167,12 @@ int run_batch_t(const tm_graph* g, const tm_query* qs, int nq, tm_result* res, c
     const size_t wtab_bytes = place_wtabs(hp, nullptr, wown);
     size_t NWs = (size_t)std::max<int64_t>(NW, 1);
     size_t Ms = (size_t)std::max<int64_t>(g->m, 1);
+    // (a bound too large for one launch: the first edges counted later may not be)
+    const size_t n_words_w = scan_once_words(NW);
+    const size_t n_words_f = scan_once_words(F_ub) ? scan_once_words(F_ub) : 8 + (size_t)kOnePassTiles;
     size_t sz = a256(plans_bytes((size_t)nq)) + a256(sizeof(tm_result) * (size_t)nq) + wtab_bytes +
-                9 * a256(8 * NWs) + 3 * a256(4 * NWs) + a256(8 * NWs) + a256(8 * A_N * NWs) + 5 * 256 +
-                full_bytes + (any_full ? 3 * a256(4 * Ms) : 0) +
+                9 * a256(8 * NWs) + 3 * a256(4 * NWs) + a256(8 * NWs) + a256(8 * A_N * NWs) + 4 * 256 +
+                a256(4 * (size_t)nq) + a256(8 * n_words_w) + a256(8 * n_words_f) + full_bytes + (any_full ? 3 * a256(4 * Ms) : 0) +
                 a256(sizeof(ShiftSums) * (size_t)std::max<int64_t>(n_sums, 1)) +
                 a256(sizeof(ShiftSums) * (size_t)n_parts) +
                 a256(8 * kMaxSub * (size_t)nq) + a256(sizeof(RideEnt) * std::max<size_t>(h_rides.size(), 1));
@@ -2140,7 +2181,6 @@ int run_batch_t(const tm_graph* g, const tm_query* qs, int nq, tm_result* res, c
     char* p = sb;
     auto take = [&](size_t bytes) { char* r = p; p += a256(bytes); return (void*)r; };
     QPlan* dplans = (QPlan*)take(plans_bytes((size_t)nq));
-    tm_result* dres = (tm_result*)take(sizeof(tm_result) * (size_t)nq);
     place_wtabs(hp, (char*)take(wtab_bytes), wown);
     for (int i = 0; i < nq; i++) {
         QPlan& P = hp[(size_t)i];
@@ -2166,12 +2206,21 @@ int run_batch_t(const tm_graph* g, const tm_query* qs, int nq, tm_result* res, c
     W.k = (int32_t*)take(4 * NWs);
     W.kept = (int32_t*)take(4 * NWs);
     W.qj = (double*)take(8 * NWs);
+    // the results and, right behind them (one copy brings all back), the record count and the
+    // error word of the kernels that wait between blocks; from there on everything starts at zero
+    const size_t res_bytes = sizeof(tm_result) * (size_t)nq;
+    static_assert(sizeof(tm_result) % 8 == 0, "the counters follow the results");
+    tm_result* dres = (tm_result*)take(res_bytes + 16);
+    unsigned long long* drcount = (unsigned long long*)((char*)dres + res_bytes);
+    uint32_t* dserr = (uint32_t*)(drcount + 1);
     W.acc = (unsigned long long*)take(8 * A_N * NWs);
     int64_t* dF = (int64_t*)take(8);
     int64_t* dW2 = (int64_t*)take(8);
     unsigned long long* dctr = (unsigned long long*)take(8);
-    unsigned long long* drcount = (unsigned long long*)take(8);
-    uint32_t* dserr = (uint32_t*)take(8);   // the window sorts' error word
+    uint32_t* dfolded = (uint32_t*)take(4 * (size_t)nq);
+    unsigned long long* words_w = (unsigned long long*)take(8 * n_words_w);
+    unsigned long long* words_f = (unsigned long long*)take(8 * n_words_f);
+    char* const zero_end = p;
     ShiftSums* dsums = (ShiftSums*)take(sizeof(ShiftSums) * (size_t)std::max<int64_t>(n_sums, 1));
     ShiftSums* dpart = (ShiftSums*)take(sizeof(ShiftSums) * (size_t)n_parts);
     unsigned long long* dsubc = (unsigned long long*)take(8 * kMaxSub * (size_t)nq);
@@ -2200,10 +2249,7 @@ int run_batch_t(const tm_graph* g, const tm_query* qs, int nq, tm_result* res, c
     fail(copy_plans(hp, wown, h_plans, dplans, st), "plans");
     if (!h_rides.empty())
         fail(cudaMemcpyAsync(drides, h_rides.data(), sizeof(RideEnt) * h_rides.size(), cudaMemcpyHostToDevice, st), "riders");
-    fail(cudaMemsetAsync(W.acc, 0, 8 * A_N * NWs, st), "acc");
-    fail(cudaMemsetAsync(dctr, 0, 8, st), "counter");
-    fail(cudaMemsetAsync(drcount, 0, 8, st), "record counter");
-    if (any_full) fail(cudaMemsetAsync(dserr, 0, 8, st), "sort error word");
+    fail(cudaMemsetAsync(drcount, 0, (size_t)(zero_end - (char*)drcount), st), "accumulators");
     if (rc == TM_OK) {
         launch_wtabs(hp, wown, dplans, st);
         fail(cudaGetLastError(), "k_wtab");
@@ -2233,12 +2279,7 @@ int run_batch_t(const tm_graph* g, const tm_query* qs, int nq, tm_result* res, c
             }
         }
     }
-    if (rc == TM_OK && NW > 0) {
-        unsigned gr = (unsigned)std::min<int64_t>((NW + 255) / 256, (int64_t)nsm * 16);
-        k_windows<TT><<<gr, 256, 0, st>>>(G, dplans, nq, W, NW); count_launch();
-        fail(cudaGetLastError(), "k_windows");
-    }
-    if (rc == TM_OK) rc = scan_exclusive_i64(W.nfirst, W.fbase, NW, dF, st);
+    if (rc == TM_OK && NW > 0) rc = launch_windows<TT>(G, dplans, nq, W, NW, dF, words_w, dserr, nsm, st);
     // The per-first-edge scratch is sized for the bound on F when that fits in
     // kBoundScratchBytes, and the kernels read F on the device: no host round trip
     // between the window partition and the matcher.  Otherwise F is read back first.
@@ -2279,22 +2320,20 @@ int run_batch_t(const tm_graph* g, const tm_query* qs, int nq, tm_result* res, c
             A.rcount = drcount;
             A.rcap = rcap;
             int64_t gl2 = std::min<int64_t>((Fa + 255) / 256, (int64_t)nsm * 8);
-            k_blockwin<<<(unsigned)std::min<int64_t>(((int64_t)nbw + 255) / 256, (int64_t)nsm * 8), 256, 0, st>>>(
-                W.fbase, NW, Fa, d_Fk, bwin);
-            count_launch();
+            if (NW > 1) {   // (one window: nothing to search)
+                k_blockwin<<<(unsigned)std::min<int64_t>(((int64_t)nbw + 255) / 256, (int64_t)nsm * 8), 256, 0, st>>>(
+                    W.fbase, NW, Fa, d_Fk, bwin);
+                count_launch();
+            } else {
+                A.blockwin = nullptr;
+            }
             ev_l0 = pe.mark(st);
             nv.next("tm_level2");
             k_level2<TT><<<(unsigned)std::max<int64_t>(gl2, 1), 256, match_smem_bytes(A.nq, 256), st>>>(A, rec, len32, hs_a, hs_hi); count_launch();
             fail(cudaGetLastError(), "k_level2");
             ev_l2 = pe.mark(st);
             nv.next("tm_scan");
-            if (rc == TM_OK) rc = scan_lengths(len32, excl, Fa, d_Fk, dW2, nullptr, 0, st);
-            if (rc == TM_OK) {
-                k_chunkf<<<(unsigned)std::min<int64_t>(((int64_t)ncf + 255) / 256, (int64_t)nsm * 8), 256, 0, st>>>(
-                    excl, Fa, d_Fk, dW2, A.chunk, (int64_t)ncf, cf);
-                count_launch();
-                fail(cudaGetLastError(), "k_chunkf");
-            }
+            if (rc == TM_OK) rc = scan_lengths(len32, excl, Fa, d_Fk, dW2, cf, (int64_t)ncf, words_f, dserr, nullptr, 0, st);
             ev_l1 = pe.mark(st);
             nv.next("tm_match");
             if (rc == TM_OK) {
@@ -2317,7 +2356,7 @@ int run_batch_t(const tm_graph* g, const tm_query* qs, int nq, tm_result* res, c
     if (rc == TM_OK) {
         int ev_f0 = pe.mark(st);
         nv.next("tm_fold");
-        launch_fold(dplans, nq, bmax, smax, W, dpart, dres, dbg && dbg->sums ? dsums : nullptr,
+        launch_fold(dplans, nq, bmax, smax, W, dpart, dfolded, dres, dbg && dbg->sums ? dsums : nullptr,
                     dbg && dbg->sub_count ? dsubc : nullptr, st);
         fail(cudaGetLastError(), "fold");
         ev_f1 = pe.mark(st);
@@ -2325,9 +2364,8 @@ int run_batch_t(const tm_graph* g, const tm_query* qs, int nq, tm_result* res, c
         if (ev_m1 < 0) ev_m1 = ev_f0;
         if (ev_r1 < 0) ev_r1 = ev_m1;
     }
-    if (rc == TM_OK && any_full) fail(cudaMemcpyAsync(&h_serr, dserr, 4, cudaMemcpyDeviceToHost, st), "sort error word");
-    if (rc == TM_OK && any_share) fail(cudaMemcpyAsync(&h_rcount, drcount, 8, cudaMemcpyDeviceToHost, st), "records");
-    if (rc == TM_OK) fail(cudaMemcpyAsync(res, dres, sizeof(tm_result) * (size_t)nq, cudaMemcpyDeviceToHost, st), "results");
+    std::vector<char> h_res(res_bytes + 16);
+    if (rc == TM_OK) fail(cudaMemcpyAsync(h_res.data(), dres, res_bytes + 16, cudaMemcpyDeviceToHost, st), "results");
     if (rc == TM_OK && dbg && dbg->sub_count)
         fail(cudaMemcpyAsync(dbg->sub_count, dsubc, 8 * kMaxSub * (size_t)nq, cudaMemcpyDeviceToHost, st),
              "span counts");
@@ -2363,9 +2401,14 @@ int run_batch_t(const tm_graph* g, const tm_query* qs, int nq, tm_result* res, c
     }
     cudaError_t se = cudaStreamSynchronize(st);
     fail(se, "batch sync");
-    if (rc == TM_OK && h_serr) {
-        set_error("window partition: a wait for an earlier tile expired");
-        rc = TM_ECUDA;
+    if (rc == TM_OK) {
+        std::memcpy(res, h_res.data(), res_bytes);
+        std::memcpy(&h_rcount, h_res.data() + res_bytes, 8);
+        std::memcpy(&h_serr, h_res.data() + res_bytes + 8, 4);
+        if (h_serr) {
+            set_error("batch: a wait for an earlier tile expired");
+            rc = TM_ECUDA;
+        }
     }
     if (pe.on && rc == TM_OK) {
         double wall = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - wall0).count();
@@ -2830,17 +2873,18 @@ int count_exact_noalloc_t(const tm_graph* g, const tm_motif* m, int64_t delta, c
     P.win_base = 0;
     P.hoist = 0;   // no per-first-edge closing ranges: keeps the scratch at its stated size
     P.ex23 = 0;    // nor the two-node tables (an allocation)
-    // every call starts from zeroed accumulators and queue counter
+    // every call starts from zeroed accumulators, queue counter (with the fold's counter and the
+    // error word behind it) and scan words, which fill the last part of the scan workspace
+    uint32_t* dfolded = (uint32_t*)(dctr + 1);
+    uint32_t* derr = (uint32_t*)(dctr + 2);
+    unsigned long long* words = (unsigned long long*)(ws + kNaWsElems / 2);
     cudaError_t e = cudaMemcpyAsync(dplan, &P, sizeof(P), cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(W.acc, 0, 8 * A_N, st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(dctr, 0, 8, st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(W.acc, 0, (size_t)((unsigned char*)dctr + 256 - (unsigned char*)W.acc), st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(words, 0, 8 * (size_t)kNaWsElems / 2, st);
     if (e != cudaSuccess) return na_status(e);
     GraphDevT<TT> G = typed<TT>(g->dev);
-    k_windows<TT><<<1, 32, 0, st>>>(G, dplan, 1, W, 1); count_launch();
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return na_status(e);
-    rc = scan_exclusive_i64_ws(W.nfirst, W.fbase, 1, dF, ws, kNaWsElems, st);
-    if (rc != TM_OK) return rc;
+    rc = launch_windows<TT>(G, dplan, 1, W, 1, dF, nullptr, nullptr, sm_count(), st);
+    if (rc != TM_OK) return TM_ECUDA;
     int64_t F = g->m;   // one window holding every edge
     if (F > 0) {
         const Tuning tu = tuning();
@@ -2856,21 +2900,28 @@ int count_exact_noalloc_t(const tm_graph* g, const tm_motif* m, int64_t delta, c
         count_launch();
         e = cudaGetLastError();
         if (e != cudaSuccess) return na_status(e);
-        // the 32-bit lengths fill the first half of their 8-byte-per-edge region; the scan's
-        // workspace takes the second half
-        rc = scan_lengths((const int32_t*)len2, excl, F, nullptr, dW2, len2 + kNaMaxEdges / 2, kNaMaxEdges / 2, st);
+        // the 32-bit lengths fill the first half of their 8-byte-per-edge region, the item starts
+        // the second
+        A.chunkf = len2 + kNaMaxEdges / 2;
+        A.nchunkf = kNaMaxEdges / 2;
+        if ((int64_t)scan_once_words(F) > kNaWsElems / 2 || !scan_once_words(F)) return TM_EINVAL;
+        rc = scan_lengths((const int32_t*)len2, excl, F, nullptr, dW2, len2 + kNaMaxEdges / 2, A.nchunkf, words, derr,
+                          nullptr, 0, st);
         if (rc != TM_OK) return rc;
         launch_match<TT>(A, P.l, std::max(P.k, 2), tu, nsm, st, plan_expands(P));
         e = cudaGetLastError();
         if (e != cudaSuccess) return na_status(e);
     }
     // the scan workspace is free again: it holds the fold's one partial record
-    launch_fold(dplan, 1, 1, 1, W, (ShiftSums*)ws, dres, nullptr, nullptr, st);
+    launch_fold(dplan, 1, 1, 1, W, (ShiftSums*)ws, dfolded, dres, nullptr, nullptr, st);
     e = cudaGetLastError();
     tm_result hres;
+    uint32_t herr = 0;
     if (e == cudaSuccess) e = cudaMemcpyAsync(&hres, dres, sizeof(hres), cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&herr, derr, sizeof(herr), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) return na_status(e);
+    if (herr) return TM_ECUDA;
     if (hres.status != TM_OK) return hres.status;
     *count = hres.count;
     return TM_OK;
@@ -2902,7 +2953,8 @@ struct tm_batch {
     std::vector<int> qstat;
     int first_err = TM_OK;
     void* scratch = nullptr;
-    tm_result* h_res = nullptr;       // pinned: the graph's last node copies results here
+    tm_result* h_res = nullptr;       // pinned: the graph's last nodes copy results here,
+    uint32_t* h_err = nullptr;        // and the error word of kernels that wait between blocks
     cudaStream_t cap = nullptr;
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
@@ -2973,16 +3025,21 @@ int batch_create_t(const tm_graph* g, const tm_query* qs, int nq, tm_batch** out
     std::vector<int32_t> wown;
     const size_t wtab_bytes = place_wtabs(hp, nullptr, wown);
     size_t NWs = (size_t)std::max<int64_t>(NW, 1), Fs = (size_t)std::max<int64_t>(Fmax, 1);
+    const size_t n_words_w = scan_once_words(NW), n_words_f = scan_once_words(Fmax);
     int64_t ws1 = 2 * ((NW + 2047) / 2048) + 2;
     int64_t ws2 = scan_dn_ws_elems(Fmax) + 2;
     size_t sz = a256(plans_bytes((size_t)nq)) + a256(sizeof(tm_result) * (size_t)nq) + wtab_bytes +
-                9 * a256(8 * NWs) + 3 * a256(4 * NWs) + a256(8 * NWs) + a256(8 * A_N * NWs) + 3 * 256 +
-                a256(sizeof(FRec<TT>) * Fs) + (any_hoist ? 3 : 1) * a256(8 * Fs) + a256(8 * (size_t)ws1) +
+                9 * a256(8 * NWs) + 3 * a256(4 * NWs) + a256(8 * NWs) + a256(8 * A_N * NWs) + 4 * 256 +
+                a256(4 * (size_t)nq) + a256(8 * n_words_w) + a256(8 * n_words_f) + a256(sizeof(FRec<TT>) * Fs) + (any_hoist ? 3 : 1) * a256(8 * Fs) + a256(8 * (size_t)ws1) +
                 a256(8 * (size_t)ws2) +
                 a256(4 * (Fs / 32 + 1)) + a256(8 * (Fs / 4 + 2)) + a256(4 * Fs) +
                 a256(sizeof(ShiftSums) * (size_t)n_parts);
     cudaError_t e = cudaMalloc(&b->scratch, sz);
-    if (e == cudaSuccess) e = cudaMallocHost((void**)&b->h_res, sizeof(tm_result) * (size_t)nq);
+    if (e == cudaSuccess) e = cudaMallocHost((void**)&b->h_res, sizeof(tm_result) * (size_t)nq + 8);
+    if (e == cudaSuccess) {
+        b->h_err = (uint32_t*)(b->h_res + nq);
+        *b->h_err = 0;
+    }
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&b->cap, cudaStreamNonBlocking);
     if (e != cudaSuccess) {
         int rc = cuda_status(e, "tm_batch_create", __FILE__, __LINE__);
@@ -3012,6 +3069,11 @@ int batch_create_t(const tm_graph* g, const tm_query* qs, int nq, tm_batch** out
     int64_t* dF = (int64_t*)take(8);
     int64_t* dW2 = (int64_t*)take(8);
     unsigned long long* dctr = (unsigned long long*)take(8);
+    uint32_t* derr = (uint32_t*)take(8);
+    uint32_t* dfolded = (uint32_t*)take(4 * (size_t)nq);
+    unsigned long long* words_w = (unsigned long long*)take(8 * n_words_w);
+    unsigned long long* words_f = (unsigned long long*)take(8 * n_words_f);
+    char* const zero_end = p;
     FRec<TT>* rec = (FRec<TT>*)take(sizeof(FRec<TT>) * Fs);
     int64_t* excl = (int64_t*)take(8 * Fs);
     int32_t* len32 = (int32_t*)take(4 * Fs);
@@ -3048,14 +3110,15 @@ int batch_create_t(const tm_graph* g, const tm_query* qs, int nq, tm_batch** out
     tm_profile pr0;
     tm_profile_last(&pr0);
     fail(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal), "begin capture");
-    fail(cudaMemsetAsync(W.acc, 0, 8 * A_N * NWs, st), "acc");
-    fail(cudaMemsetAsync(dctr, 0, 8, st), "counter");
-    if (rc == TM_OK && NW > 0) {
+    fail(cudaMemsetAsync(W.acc, 0, (size_t)(zero_end - (char*)W.acc), st), "accumulators");
+    if (rc == TM_OK && NW > 0 && (n_words_w || NW <= kWindowThreads)) {
+        rc = launch_windows<TT>(G, dplans, nq, W, NW, dF, words_w, derr, nsm, st);
+    } else if (rc == TM_OK && NW > 0) {   // (a scan too long for one launch, in the batch's own workspace)
         unsigned gr = (unsigned)std::min<int64_t>((NW + 255) / 256, (int64_t)nsm * 16);
-        k_windows<TT><<<gr, 256, 0, st>>>(G, dplans, nq, W, NW); count_launch();
+        k_windows<TT><<<gr, kWindowThreads, 0, st>>>(G, dplans, nq, W, NW, nullptr); count_launch();
         fail(cudaGetLastError(), "k_windows");
+        if (rc == TM_OK) rc = scan_exclusive_i64_ws(W.nfirst, W.fbase, NW, dF, wsp1, ws1, st);
     }
-    if (rc == TM_OK) rc = scan_exclusive_i64_ws(W.nfirst, W.fbase, NW, dF, wsp1, ws1, st);
     if (rc == TM_OK && Fmax > 0) {
         MatchArgs<TT> A;
         A.G = G; A.plans = dplans; A.nq = nq; A.W = W; A.NW = NW; A.F = Fmax; A.d_F = dF;
@@ -3070,13 +3133,7 @@ int batch_create_t(const tm_graph* g, const tm_query* qs, int nq, tm_batch** out
         count_launch();
         k_level2<TT><<<(unsigned)std::max<int64_t>(gl2, 1), 256, match_smem_bytes(A.nq, 256), st>>>(A, rec, len32, hs_a, hs_hi); count_launch();
         fail(cudaGetLastError(), "k_level2");
-        if (rc == TM_OK) rc = scan_lengths(len32, excl, Fmax, dF, dW2, wsp2, ws2, st);
-        if (rc == TM_OK) {
-            k_chunkf<<<(unsigned)std::min<int64_t>(((int64_t)ncf + 255) / 256, (int64_t)nsm * 8), 256, 0, st>>>(
-                excl, Fmax, dF, dW2, A.chunk, (int64_t)ncf, cf);
-            count_launch();
-            fail(cudaGetLastError(), "k_chunkf");
-        }
+        if (rc == TM_OK) rc = scan_lengths(len32, excl, Fmax, dF, dW2, cf, (int64_t)ncf, words_f, derr, wsp2, ws2, st);
         if (rc == TM_OK) {
             launch_match<TT>(A, lmax, kmax, tu, nsm, st,
                              std::any_of(hp.begin(), hp.end(), [](const QPlan& P) { return plan_expands(P); }));
@@ -3084,10 +3141,11 @@ int batch_create_t(const tm_graph* g, const tm_query* qs, int nq, tm_batch** out
         }
     }
     if (rc == TM_OK) {
-        launch_fold(dplans, nq, bmax, smax, W, dpart, dres, nullptr, nullptr, st);
+        launch_fold(dplans, nq, bmax, smax, W, dpart, dfolded, dres, nullptr, nullptr, st);
         fail(cudaGetLastError(), "fold");
     }
     fail(cudaMemcpyAsync(b->h_res, dres, sizeof(tm_result) * (size_t)nq, cudaMemcpyDeviceToHost, st), "results");
+    fail(cudaMemcpyAsync(b->h_err, derr, 4, cudaMemcpyDeviceToHost, st), "error word");
     cudaGraph_t graph = nullptr;
     cudaError_t ee = cudaStreamEndCapture(st, &graph);
     fail(ee, "end capture");
@@ -3130,6 +3188,7 @@ int tm_batch_launch(tm_batch* b, void* stream) {
 int tm_batch_results(tm_batch* b, void* stream, tm_result* results) {
     if (!b || !results) { tmo::set_error("bad argument"); return TM_EINVAL; }
     TM_CUDA(cudaStreamSynchronize((cudaStream_t)stream));
+    if (*b->h_err) { tmo::set_error("batch: a wait for an earlier tile expired"); return TM_ECUDA; }
     int first = b->first_err;
     for (int i = 0; i < b->nq; i++) {
         results[i] = b->h_res[i];

@@ -99,12 +99,40 @@ __global__ void k_len_reduce(const int32_t* __restrict__ in, int64_t n_max, cons
     if (threadIdx.x == 0) sums[blockIdx.x] = total;
 }
 
+// Item starts: cf[i] = the element whose range holds item i * kItemGrain.  Each thread notes its own
+// elements' (those of a range past kBigRange are left to the whole block: noted by one thread, the
+// range of a hub's burst would be a long serial run of stores).
+constexpr int64_t kBigRange = 64 * kItemGrain;
+struct BigRanges {
+    int n;
+    int64_t e[32], from[32], len[32];
+};
+__device__ __forceinline__ void note_items(BigRanges& B, int64_t* cf, int64_t ncf, int64_t e, int64_t from, int64_t len) {
+    if (len > kBigRange) {
+        const int k = atomicAdd(&B.n, 1);
+        if (k < 32) {
+            B.e[k] = e; B.from[k] = from; B.len[k] = len;
+            return;
+        }
+    }
+    for (int64_t i = (from + kItemGrain - 1) / kItemGrain; i * kItemGrain < from + len && i < ncf; i++) cf[i] = e;
+}
+__device__ __forceinline__ void note_big(const BigRanges& B, int64_t* cf, int64_t ncf) {
+    for (int k = 0; k < min(B.n, 32); k++)
+        for (int64_t i = (B.from[k] + kItemGrain - 1) / kItemGrain + threadIdx.x;
+             i * kItemGrain < B.from[k] + B.len[k] && i < ncf; i += blockDim.x)
+            cf[i] = B.e[k];
+}
+
 // ... then each tile's exclusive scan plus the tile's offset; the tile passes through shared
-// memory so that both the 32-bit loads and the 64-bit stores are coalesced
+// memory so that both the 32-bit loads and the 64-bit stores are coalesced.  cf: as k_scan_once
 __global__ void k_len_scan(const int32_t* __restrict__ in, int64_t* __restrict__ out, int64_t n_max,
-                           const int64_t* __restrict__ d_n, const int64_t* __restrict__ offs) {
+                           const int64_t* __restrict__ d_n, const int64_t* __restrict__ offs,
+                           int64_t* __restrict__ cf, int64_t ncf) {
     __shared__ int64_t smem[33];
     __shared__ int64_t tile[kScanTile + kScanTile / 16];   // one pad word per 16: no bank conflicts
+    __shared__ BigRanges big;
+    if (threadIdx.x == 0) big.n = 0;
     int64_t n = d_n ? min(*d_n, n_max) : n_max;
     int64_t t0 = (int64_t)blockIdx.x * kScanTile;
     if (t0 >= n) return;
@@ -123,12 +151,18 @@ __global__ void k_len_scan(const int32_t* __restrict__ in, int64_t* __restrict__
     }
     int64_t total;
     int64_t run = block_excl_scan(loc, smem, &total) + offs[blockIdx.x];
+    if (threadIdx.x == 0 && t0 + kScanTile >= n) {
+        const int64_t end = (run + total + kItemGrain - 1) / kItemGrain;
+        if (end < ncf) cf[end] = n - 1;
+    }
 #pragma unroll
     for (int i = 0; i < kScanItems; i++) {
+        note_items(big, cf, ncf, t0 + b + i, run, v[i]);
         tile[b + i + ((b + i) >> 4)] = run;
         run += v[i];
     }
     __syncthreads();
+    note_big(big, cf, ncf);
     for (int i = threadIdx.x; i < kScanTile; i += blockDim.x) {
         int64_t idx = t0 + i;
         if (idx < n) out[idx] = tile[i + (i >> 4)];
@@ -169,70 +203,106 @@ __global__ void k_scan_small(const int64_t* in, int64_t* out, int64_t n, int64_t
 
 __global__ void k_set_i64(int64_t* p, int64_t v) { *p = v; }
 
-// the same scans for an element count held in device memory (*d_n <= n_max);
-// tiles past *d_n contribute nothing and write nothing
-__global__ void k_scan_tiles_dn(const int64_t* in, int64_t* out, const int64_t* __restrict__ d_n,
-                                int64_t* __restrict__ sums) {
+// Exclusive scan of lengths (TI = int32_t or int64_t) into 64-bit offsets in one launch: a tile's
+// sum, then its prefix, go through one word (top two bits: 1 sum known, 2 prefix known; sums below
+// 2^62), and a warp looks back over 32 tiles at a time.  Prefixes travel 32 tiles per memory
+// latency, so beyond kOnePassTiles tiles the two-pass form is as quick; below, one launch takes
+// the place of three to five (a 20,000-edge count spent 22 of its 118 us on them).
+// CF also notes the first edge of every kItemGrain-th item (cf[i]: the element whose range holds
+// item i * kItemGrain; past the last, n - 1), as far as cf's ncf entries go.
+constexpr int kOneThreads = 256;
+constexpr int kOneItems = 16;
+constexpr int kOneTile = kOneThreads * kOneItems;
+
+__device__ __forceinline__ unsigned long long ld_tile64(const unsigned long long* p) {
+    unsigned long long v;
+    asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ void st_tile64(unsigned long long* p, unsigned long long v) {
+    asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+}
+
+template <typename TI, bool CF>
+__global__ void __launch_bounds__(kOneThreads) k_scan_once(const TI* __restrict__ in, int64_t* __restrict__ out, int64_t n_max,
+                            const int64_t* __restrict__ d_n, int64_t* __restrict__ d_total, unsigned long long* words,
+                            uint32_t* err, int64_t* __restrict__ cf, int64_t ncf) {
     __shared__ int64_t smem[33];
-    int64_t n = *d_n;
-    if ((int64_t)blockIdx.x * kScanTile >= n) {
-        if (threadIdx.x == 0) sums[blockIdx.x] = 0;
+    __shared__ int64_t tile[kOneTile + kOneTile / 16];   // one pad word per 16: no bank conflicts
+    __shared__ int64_t s_before;
+    __shared__ uint32_t s_tile;
+    __shared__ BigRanges big;
+    if (CF && threadIdx.x == 0) big.n = 0;
+    const int64_t n = d_n ? min(*d_n, n_max) : n_max;
+    if (threadIdx.x == 0) s_tile = (uint32_t)atomicAdd(words, 1ull);
+    __syncthreads();
+    const int64_t t = s_tile, t0 = t * kOneTile;
+    words += 8;
+    if (t0 >= n) {
+        if (n == 0 && t == 0 && threadIdx.x == 0) *d_total = 0;
         return;
     }
-    int64_t base = (int64_t)blockIdx.x * kScanTile + (int64_t)threadIdx.x * kScanItems;
-    int64_t v[kScanItems];
+    for (int i = threadIdx.x; i < kOneTile; i += kOneThreads) {
+        const int64_t idx = t0 + i;
+        tile[i + (i >> 4)] = idx < n ? (int64_t)in[idx] : 0;
+    }
+    __syncthreads();
+    const int b = threadIdx.x * kOneItems;
     int64_t loc = 0;
 #pragma unroll
-    for (int i = 0; i < kScanItems; i++) {
-        int64_t idx = base + i;
-        v[i] = idx < n ? in[idx] : 0;
-        loc += v[i];
-    }
+    for (int i = 0; i < kOneItems; i++) loc += tile[b + i + ((b + i) >> 4)];
     int64_t total;
-    int64_t run = block_excl_scan(loc, smem, &total);
+    const int64_t off = block_excl_scan(loc, smem, &total);
+    if (threadIdx.x < 32) {
+        const int lane = threadIdx.x;
+        int64_t before = 0;
+        if (t > 0) {
+            if (lane == 0) st_tile64(words + t, (1ull << 62) | (unsigned long long)total);
+            int64_t at = t - 1;
+            int spins = 0;
+            while (at >= 0) {
+                const unsigned long long v = at - lane >= 0 ? ld_tile64(words + (at - lane)) : 2ull << 62;
+                const unsigned pre = __ballot_sync(kFull, (v >> 62) == 2), gap = __ballot_sync(kFull, v == 0);
+                const int first_gap = gap ? __ffs(gap) - 1 : 32, first_pre = pre ? __ffs(pre) - 1 : 32;
+                int64_t x = lane < first_gap && lane <= first_pre ? (int64_t)(v & ((1ull << 62) - 1)) : 0;
 #pragma unroll
-    for (int i = 0; i < kScanItems; i++) {
-        int64_t idx = base + i;
-        if (idx < n) out[idx] = run;
-        run += v[i];
+                for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(kFull, x, o);
+                before += x;
+                if (first_pre < first_gap) break;
+                at -= first_gap;
+                if (first_gap == 0 && ++spins > kSpinLimit) {
+                    if (lane == 0) atomicOr(err, 1u);
+                    break;
+                }
+            }
+        }
+        if (lane == 0) {
+            st_tile64(words + t, (2ull << 62) | (unsigned long long)(before + total));
+            s_before = before;
+            if (t0 + kOneTile >= n) {
+                *d_total = before + total;
+                if (CF) {
+                    const int64_t end = (before + total + kItemGrain - 1) / kItemGrain;
+                    if (end < ncf) cf[end] = n - 1;
+                }
+            }
+        }
     }
-    if (threadIdx.x == 0) sums[blockIdx.x] = total;
-}
-
-__global__ void k_scan_add_dn(int64_t* __restrict__ out, const int64_t* __restrict__ d_n,
-                              const int64_t* __restrict__ offs) {
-    int64_t n = *d_n;
-    int64_t base = (int64_t)blockIdx.x * kScanTile;
-    if (base >= n) return;
-    int64_t add = offs[blockIdx.x];
-    for (int i = threadIdx.x; i < kScanTile; i += blockDim.x) {
-        int64_t idx = base + i;
-        if (idx < n) out[idx] += add;
-    }
-}
-
-__global__ void k_scan_small_dn(const int64_t* in, int64_t* out, const int64_t* __restrict__ d_n,
-                                int64_t* __restrict__ d_total) {
-    __shared__ int64_t smem[33];
-    int64_t n = *d_n;
-    int64_t base = (int64_t)threadIdx.x * kScanItems;
-    int64_t v[kScanItems];
-    int64_t loc = 0;
+    __syncthreads();
+    int64_t run = s_before + off;
 #pragma unroll
-    for (int i = 0; i < kScanItems; i++) {
-        int64_t idx = base + i;
-        v[i] = idx < n ? in[idx] : 0;
-        loc += v[i];
+    for (int i = 0; i < kOneItems; i++) {
+        const int64_t v = tile[b + i + ((b + i) >> 4)];
+        if (CF) note_items(big, cf, ncf, t0 + b + i, run, v);
+        tile[b + i + ((b + i) >> 4)] = run;
+        run += v;
     }
-    int64_t total;
-    int64_t run = block_excl_scan(loc, smem, &total);
-#pragma unroll
-    for (int i = 0; i < kScanItems; i++) {
-        int64_t idx = base + i;
-        if (idx < n) out[idx] = run;
-        run += v[i];
+    __syncthreads();
+    if (CF) note_big(big, cf, ncf);
+    for (int i = threadIdx.x; i < kOneTile; i += kOneThreads) {
+        const int64_t idx = t0 + i;
+        if (idx < n) out[idx] = tile[i + (i >> 4)];
     }
-    if (threadIdx.x == 0 && d_total) *d_total = total;
 }
 
 // ------------------------------------------------------------------ radix sort
@@ -544,12 +614,18 @@ int scan_exclusive_i64_ws(const int64_t* in, int64_t* out, int64_t n, int64_t* d
 }
 
 int scan_lengths(const int32_t* in, int64_t* out, int64_t n_max, const int64_t* d_n, int64_t* d_total,
-                 int64_t* ws, int64_t ws_elems, cudaStream_t st) {
+                 int64_t* cf, int64_t ncf, unsigned long long* words, uint32_t* err, int64_t* ws, int64_t ws_elems,
+                 cudaStream_t st) {
     if (n_max <= 0) {
-        if (d_total) {
-            k_set_i64<<<1, 1, 0, st>>>(d_total, 0); count_launch();
-            TM_CUDA(cudaGetLastError());
-        }
+        k_set_i64<<<1, 1, 0, st>>>(d_total, 0); count_launch();
+        TM_CUDA(cudaGetLastError());
+        return TM_OK;
+    }
+    if (scan_once_words(n_max)) {
+        k_scan_once<int32_t, true><<<(unsigned)((n_max + kOneTile - 1) / kOneTile), kOneThreads, 0, st>>>(
+            in, out, n_max, d_n, d_total, words, err, cf, ncf);
+        count_launch();
+        TM_CUDA(cudaGetLastError());
         return TM_OK;
     }
     int64_t ntiles = (n_max + kScanTile - 1) / kScanTile;
@@ -569,7 +645,7 @@ int scan_lengths(const int32_t* in, int64_t* out, int64_t n_max, const int64_t* 
         if (cudaGetLastError() != cudaSuccess) rc = TM_ECUDA;
         if (rc == TM_OK) rc = scan_exclusive_i64_ws(sums, soffs, ntiles, d_total, ws + 2 * ntiles, need - 2 * ntiles, st);
         if (rc == TM_OK) {
-            k_len_scan<<<(unsigned)ntiles, kScanThreads, 0, st>>>(in, out, n_max, d_n, soffs); count_launch();
+            k_len_scan<<<(unsigned)ntiles, kScanThreads, 0, st>>>(in, out, n_max, d_n, soffs, cf, ncf); count_launch();
             if (cudaGetLastError() != cudaSuccess) rc = TM_ECUDA;
         }
     }
@@ -584,30 +660,17 @@ int64_t scan_dn_ws_elems(int64_t n_max) {
     return 2 * ntiles + 2 * ((ntiles + kScanTile - 1) / kScanTile) + 2;
 }
 
-int scan_exclusive_i64_dn(const int64_t* in, int64_t* out, int64_t n_max, const int64_t* d_n,
-                          int64_t* d_total, int64_t* ws, int64_t ws_elems, cudaStream_t st) {
-    if (n_max <= 0) {
-        if (d_total) {
-            k_set_i64<<<1, 1, 0, st>>>(d_total, 0); count_launch();
-            TM_CUDA(cudaGetLastError());
-        }
-        return TM_OK;
-    }
-    if (n_max <= kScanTile) {
-        k_scan_small_dn<<<1, kScanThreads, 0, st>>>(in, out, d_n, d_total); count_launch();
-        TM_CUDA(cudaGetLastError());
-        return TM_OK;
-    }
-    int64_t ntiles = (n_max + kScanTile - 1) / kScanTile;
-    if (ws_elems < scan_dn_ws_elems(n_max)) return TM_EINVAL;
-    int64_t* sums = ws;
-    int64_t* soffs = ws + ntiles;
-    int64_t* inner = ws + 2 * ntiles;
-    k_scan_tiles_dn<<<(unsigned)ntiles, kScanThreads, 0, st>>>(in, out, d_n, sums); count_launch();
-    TM_CUDA(cudaGetLastError());
-    int rc = scan_exclusive_i64_ws(sums, soffs, ntiles, d_total, inner, ws_elems - 2 * ntiles, st);
-    if (rc != TM_OK) return rc;
-    k_scan_add_dn<<<(unsigned)ntiles, kScanThreads, 0, st>>>(out, d_n, soffs); count_launch();
+size_t scan_once_words(int64_t n_max) {
+    const int64_t tiles = (n_max + kOneTile - 1) / kOneTile;
+    return n_max > 0 && tiles <= kOnePassTiles ? 8 + (size_t)tiles : 0;
+}
+
+int scan_once_i64(const int64_t* in, int64_t* out, int64_t n, int64_t* d_total, unsigned long long* words, uint32_t* err,
+                  cudaStream_t st) {
+    if (!scan_once_words(n)) return scan_exclusive_i64(in, out, n, d_total, st);
+    k_scan_once<int64_t, false><<<(unsigned)((n + kOneTile - 1) / kOneTile), kOneThreads, 0, st>>>(
+        in, out, n, nullptr, d_total, words, err, nullptr, 0);
+    count_launch();
     TM_CUDA(cudaGetLastError());
     return TM_OK;
 }

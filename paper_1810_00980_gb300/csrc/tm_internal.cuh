@@ -412,15 +412,20 @@ __device__ __forceinline__ void count_digits(uint32_t* sm, const SortDigits& D, 
 int scan_exclusive_i64_ws(const int64_t* in, int64_t* out, int64_t n, int64_t* d_total,
                           int64_t* ws, int64_t ws_elems, cudaStream_t st);
 
-// exclusive scan of the first *d_n (<= n_max) elements, the count read on the
-// device; workspace of scan_dn_ws_elems(n_max) int64 (no allocation, capturable)
 int64_t scan_dn_ws_elems(int64_t n_max);
-// exclusive scan of 32-bit lengths into 64-bit offsets (the first *d_n, or n_max when d_n is
-// null); workspace scan_dn_ws_elems(n_max), or null to allocate it on the stream
+// Exclusive scan of 32-bit range lengths into 64-bit offsets (the first *d_n, or n_max when d_n is
+// null) with, in cf, the element that holds every kItemGrain-th item (as far as ncf goes).  words:
+// scan_once_words(n_max) zeroed words; when that is 0 (too many tiles for one launch) ws of
+// scan_dn_ws_elems(n_max), or null to allocate it on the stream.  *err: as SortWs::err
+constexpr int kItemGrain = 32;
+constexpr int64_t kOnePassTiles = 1024;
+size_t scan_once_words(int64_t n_max);
 int scan_lengths(const int32_t* in, int64_t* out, int64_t n_max, const int64_t* d_n, int64_t* d_total,
-                 int64_t* ws, int64_t ws_elems, cudaStream_t st);
-int scan_exclusive_i64_dn(const int64_t* in, int64_t* out, int64_t n_max, const int64_t* d_n,
-                          int64_t* d_total, int64_t* ws, int64_t ws_elems, cudaStream_t st);
+                 int64_t* cf, int64_t ncf, unsigned long long* words, uint32_t* err, int64_t* ws, int64_t ws_elems,
+                 cudaStream_t st);
+// scan_exclusive_i64 in one launch when scan_once_words(n) > 0 (that many zeroed words)
+int scan_once_i64(const int64_t* in, int64_t* out, int64_t n, int64_t* d_total, unsigned long long* words, uint32_t* err,
+                  cudaStream_t st);
 
 int sm_count();
 // a graph from device arrays (tm_graph_load_device); h_t: the same times on the host when the
