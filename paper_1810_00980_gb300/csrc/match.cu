@@ -1206,15 +1206,13 @@ __device__ void expand(const MatchArgs<TT>& A, const QPlan* __restrict__ PL, boo
     }
 }
 
-// OCC: resident 256-thread blocks per SM the register allocation must allow
-// (three-edge motifs: 4 without spills, 6 with spilled registers; four-edge motifs: 1 leaves
-// the compiler 118 registers, 4 caps them at 64 with spills -- the autotuner picks)
+// OCC: resident 256-thread blocks per SM the register allocation must allow (launch_match picks)
 // EXPAND = false leaves out the warp-cooperative expansion of deeper motif edges, for batches
 // whose items all end at their second edge (every query exact with the last edge between two
 // bound nodes, two-node, riding along, or of at most two edges): the code the hot loop does
 // not run still takes registers, and without it the 3-cycle enumeration of the benchmark
 // batch runs 1.50 -> 1.32 ms
-template <typename TT, int LMAX, int KMAX, int OCC = (LMAX <= 3 ? 4 : 1), bool EXPAND = true, bool RIDE = false>
+template <typename TT, int LMAX, int KMAX, int OCC = 4, bool EXPAND = true, bool RIDE = false>
 __global__ void __launch_bounds__(256, OCC) k_match(MatchArgs<TT> A) {
     const GraphDevT<TT>& G = A.G;
     extern __shared__ __align__(16) unsigned char smem_plans[];
@@ -1763,7 +1761,12 @@ bool plan_expands(const QPlan& P) {
 template <typename TT>
 void launch_match(const MatchArgs<TT>& A, int lmax, int kmax, const Tuning& tu, int nsm, cudaStream_t st,
                   bool expand) {
-    const int bps = tu.blocks_per_sm, bt = tu.block_threads;
+    // Every instantiation waits on chains of dependent loads, so six blocks per SM at 40 registers
+    // beat fewer with more registers and less spilling (k_match, ms, at 6 / 4 / 2 / 1 blocks: the
+    // benchmark batch on 1e7 edges 1.35 / 1.56; 192 seeds of the 4-cycle there 3.54 / 4.29 / 5.11 /
+    // 9.00; four- and five-edge counts on 1.25e6 edges 1.00 / 1.02 / 1.21 / 2.12, by the deepest
+    // instantiation at 4 / 3 / 2 / 1 blocks 1.17 / 1.27 / 1.53 / 2.17; eight blocks are no better).  A tuning that was set or found picks the one for its blocks per SM.
+    const int bps = tu.blocks_set ? tu.blocks_per_sm : 6, bt = tu.block_threads;
     const unsigned gm = (unsigned)(nsm * bps);
     const size_t sm = match_smem_bytes(A.nq, bt);
     if (lmax <= 3 && kmax <= 4 && !expand) {
@@ -1771,11 +1774,11 @@ void launch_match(const MatchArgs<TT>& A, int lmax, int kmax, const Tuning& tu, 
         else k_match<TT, 3, 4, 4, false><<<gm, bt, sm, st>>>(A);
     } else if (lmax <= 3 && kmax <= 4 && bps >= 6) k_match<TT, 3, 4, 6><<<gm, bt, sm, st>>>(A);
     else if (lmax <= 3 && kmax <= 4) k_match<TT, 3, 4><<<gm, bt, sm, st>>>(A);
-    else if (lmax <= 4 && kmax <= 4 && A.rrec) k_match<TT, 4, 4, 4, true, true><<<gm, bt, sm, st>>>(A);
-    else if (lmax <= 4 && kmax <= 4 && bps >= 4) k_match<TT, 4, 4, 4><<<gm, bt, sm, st>>>(A);
-    else if (lmax <= 4 && kmax <= 4) k_match<TT, 4, 4><<<gm, bt, sm, st>>>(A);
-    else if (lmax <= 4) k_match<TT, 4, TM_K_MAX><<<gm, bt, sm, st>>>(A);
-    else k_match<TT, TM_L_MAX, TM_K_MAX><<<gm, bt, sm, st>>>(A);
+    else if (lmax <= 4 && kmax <= 4 && A.rrec) k_match<TT, 4, 4, 6, true, true><<<gm, bt, sm, st>>>(A);
+    else if (lmax <= 4 && kmax <= 4 && bps >= 6) k_match<TT, 4, 4, 6><<<gm, bt, sm, st>>>(A);
+    else if (lmax <= 4 && kmax <= 4) k_match<TT, 4, 4, 4><<<gm, bt, sm, st>>>(A);
+    else if (lmax <= 5 && kmax <= 5) k_match<TT, 5, 5, 6><<<gm, bt, sm, st>>>(A);
+    else k_match<TT, TM_L_MAX, TM_K_MAX, 4><<<gm, bt, sm, st>>>(A);
     count_launch();
 }
 
