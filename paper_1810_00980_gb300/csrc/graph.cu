@@ -548,6 +548,7 @@ int build_graph(const int32_t* d_src, const int32_t* d_dst, const int64_t* d_t, 
 
     GraphDev& G = g->dev;
     G.m = m; G.n = n; G.tbytes = tb; G.loops = 0;
+    G.per_tick = 1.0f / ((float)tmax + 1.0f);
     G.src = gs; G.dst = gd; G.t = gt;
     G.out_off = out_off; G.out_nbr = out_nbr; G.out_t = out_t;
     G.in_off = in_off; G.in_nbr = in_nbr; G.in_t = in_t;

@@ -209,7 +209,7 @@ __device__ __forceinline__ void level_range(const GraphDevT<TT>& G, const LevelP
     } else {
         ta = G.t; a = 0; b = G.m;
     }
-    lo = upper_bound_i64(ta, a, b, tprev);
+    lo = P.view == kPair ? upper_bound_i64(ta, a, b, tprev) : time_ub(ta, a, b, tprev, G.per_tick);
     len = gallop_ub(ta, lo, b, thi) - lo;
 }
 
@@ -976,7 +976,7 @@ __global__ void __launch_bounds__(256, 8) k_level2(MatchArgs<TT> A, FRec<TT>* __
                     const TT* ta = x_src ? G.in_t : G.out_t;
                     const int64_t* off = x_src ? G.in_off : G.out_off;
                     int64_t a = __ldg(off + bn), b = __ldg(off + bn + 1);
-                    int64_t rlo = upper_bound_i64(ta, a, b, t1);
+                    int64_t rlo = time_ub(ta, a, b, t1, G.per_tick);
                     int64_t rlen = gallop_ub(ta, rlo, b, thi) - rlo;
                     if (rlen == 0) {
                         len = 0;                 // nothing can close an instance
@@ -1085,7 +1085,7 @@ __device__ void expand(const MatchArgs<TT>& A, const QPlan* __restrict__ PL, boo
                 const TT* ta = x_src ? G.in_t : G.out_t;
                 const int64_t* off = x_src ? G.in_off : G.out_off;
                 int64_t a = __ldg(off + bn), b = __ldg(off + bn + 1);
-                int64_t rlo = upper_bound_i64(ta, a, b, tprev);
+                int64_t rlo = time_ub(ta, a, b, tprev, G.per_tick);
                 int64_t rlen = gallop_ub(ta, rlo, b, thi) - rlo;
                 if (rlen == 0) {
                     len = 0;
