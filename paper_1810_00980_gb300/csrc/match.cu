@@ -780,6 +780,7 @@ __device__ __forceinline__ int64_t first_thi(const QPlan& Q, const WinDev& W, in
 // run at full occupancy instead of on the critical path of k_level2's warps
 __global__ void k_blockwin(const int64_t* __restrict__ fbase, int64_t NW, int64_t Fh,
                            const int64_t* __restrict__ d_F, int32_t* __restrict__ bw) {
+    grid_wait();
     const int64_t F = d_F ? *d_F : Fh;
     int64_t nb = (F + 31) >> 5;
     for (int64_t b = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; b < nb;
@@ -807,6 +808,7 @@ __global__ void __launch_bounds__(256, 8) k_level2(MatchArgs<TT> A, FRec<TT>* __
     Acc acc;
     acc_init(acc, smem_plans, A.nq);
     acc_zero(acc);
+    grid_wait();
     const int64_t F = A.d_F ? *A.d_F : A.F;
     for (int64_t base = warp * 32; base < F; base += nwarps * 32) {
         int64_t f = base + lane;
@@ -1218,20 +1220,20 @@ __global__ void __launch_bounds__(256, OCC) k_match(MatchArgs<TT> A) {
     extern __shared__ __align__(16) unsigned char smem_plans[];
     const QPlan* PL = stage_plans(A.plans, A.nq, smem_plans);
     int lane = threadIdx.x & 31;
-    int64_t W2 = *A.d_W2;
-    const int64_t F = A.d_F ? *A.d_F : A.F;
     Acc acc;
     acc_init(acc, smem_plans, A.nq);
     acc_zero(acc);
+    grid_wait();
+    int64_t W2 = *A.d_W2;
+    const int64_t F = A.d_F ? *A.d_F : A.F;
     // few items: smaller chunks, so that every warp gets some (17,000 items in chunks of 256 kept 67
     // warps busy for eight rounds each: 43 us of a 20,000-edge count)
-    const int64_t share = (W2 / (((int64_t)gridDim.x * blockDim.x) >> 5) + kItemGrain) / kItemGrain * kItemGrain;
+    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    const int64_t share = (W2 / nwarps + kItemGrain) / kItemGrain * kItemGrain;
     const int64_t chunk = min(A.chunk, share);
-    for (;;) {
-        unsigned long long c0u = 0;
-        if (lane == 0) c0u = atomicAdd(A.counter, (unsigned long long)chunk);
-        int64_t c0 = (int64_t)__shfl_sync(kFull, c0u, 0);
-        if (c0 >= W2) break;
+    // a warp's first chunk is its own, the others come from the counter (with few items no warp
+    // asks it: 7,000 atomics on one word take longer than such a batch's items)
+    for (int64_t c0 = ((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5) * chunk; c0 < W2;) {
         int64_t c1 = min(c0 + chunk, W2);
         int64_t fb = 0, fe = 0;
         const int64_t ci = c0 / kItemGrain, ce = (c1 + kItemGrain - 1) / kItemGrain;
@@ -1420,6 +1422,10 @@ __global__ void __launch_bounds__(256, OCC) k_match(MatchArgs<TT> A) {
             }
         }
         acc_flush_warp(acc, A.W.acc);
+        if (nwarps * chunk >= W2) break;
+        unsigned long long c0u = 0;
+        if (lane == 0) c0u = atomicAdd(A.counter, (unsigned long long)chunk);
+        c0 = nwarps * chunk + (int64_t)__shfl_sync(kFull, c0u, 0);
     }
     acc_flush_warp(acc, A.W.acc);
 }
@@ -1505,6 +1511,7 @@ __global__ void __launch_bounds__(256) k_ride(MatchArgs<TT> A) {
         tab->cnt[i] = tab->lo[i] = tab->hi[i] = 0;
     }
     __syncthreads();
+    grid_wait();
     const int64_t nrec = min((int64_t)*A.rcount, A.rcap);
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     // whole warps step together, so that the accumulator flushes see every lane
@@ -1596,35 +1603,40 @@ __device__ __forceinline__ void warp_add_sums(ShiftSums& a) {
     }
 }
 
-// The fold.  Block (query, shift k, slice) sums the kept windows of its slice — counts and work
+// The fold.  A block per (query, shift k, slice), found from the plans' part_base, sums the kept
+// windows of its slice — counts and work
 // counters as integers, the Q64 weight sum W_j as a 128-bit integer, and the doubles
 // sum_j W_j / q_j (the shift's Z_k when q_j varies, Algorithm 1) and
 // sum_j W_j^2 (1 - q_j) / q_j^2 (Lemma 4.4) — into part[part_base + k * slices + slice]; the last of
 // the query's blocks to get there adds the slices of each shift, a warp per shift, and then
 // the shifts in order: Z_k, their mean (the estimate of Algorithm 1), the mean variance
 // estimate and the spread of the Z_k (Welford).
-// The grid's y extent is capped at the hardware limit; a block then also takes the shifts
-// k + gridDim.y, k + 2 gridDim.y, ... (a loop that is uniform across the block).
-// A chain of dependent loads bounds it, not bytes: two windows per thread and one launch (eight
-// windows and a second launch with a thread per query took 24 + 18 us for the 18 queries of a
-// batch on 1e6 edges).
-__global__ void __launch_bounds__(kFoldThreads) k_fold(const QPlan* __restrict__ plans, WinDev W, ShiftSums* part,
+// A chain of dependent loads bounds it, not bytes: two windows per thread and one launch of just
+// the blocks there is work for (eight windows and a second launch with a thread per query took
+// 24 + 18 us for the 18 queries of a batch on 1e6 edges).
+__global__ void __launch_bounds__(kFoldThreads) k_fold(const QPlan* __restrict__ plans, int nq, WinDev W, ShiftSums* part,
                                                        uint32_t* __restrict__ folded, tm_result* __restrict__ res,
                                                        ShiftSums* __restrict__ sums, unsigned long long* __restrict__ subc) {
-    const int qi = blockIdx.x;
+    int qi = 0, q_hi = nq;   // the query whose parts this block's is one of
+    while (q_hi - qi > 1) {
+        const int mid = (qi + q_hi) >> 1;
+        if (plans[mid].part_base <= (int64_t)blockIdx.x) qi = mid; else q_hi = mid;
+    }
     const QPlan& Q = plans[qi];
-    const int sl = blockIdx.z;
     const int nsh = Q.l <= 0 ? 0 : (Q.mode == TM_MODE_EXACT ? 1 : Q.b);
     const int64_t nwin = Q.mode == TM_MODE_EXACT ? 1 : Q.J;
     const int ns = fold_slices(nwin);
-    if (sl >= ns || (int)blockIdx.y >= max(nsh, 1)) return;
+    const int64_t mine = (int64_t)blockIdx.x - Q.part_base;
+    const int sl = (int)(mine % ns);
     __shared__ ShiftSums sh[kFoldThreads / 32];
     __shared__ int s_last;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    for (int k = blockIdx.y; k < nsh; k += gridDim.y) {
+    grid_wait();
+    if (nsh > 0) {
+        const int64_t k = mine / ns;
         ShiftSums a = {};
         for (int64_t r = (int64_t)sl * kFoldThreads + threadIdx.x; r < nwin; r += (int64_t)ns * kFoldThreads) {
-            const int64_t w = Q.win_base + (int64_t)k * nwin + r;
+            const int64_t w = Q.win_base + k * nwin + r;
             if (!W.kept[w]) continue;
             const unsigned long long* x = W.acc + w * A_N;
             const double qj = W.qj[w];
@@ -1636,19 +1648,19 @@ __global__ void __launch_bounds__(kFoldThreads) k_fold(const QPlan* __restrict__
             b.vq = y * y * (1.0 - qj) / (qj * qj);
             add_shift_sums(a, b);
         }
-        warp_add_sums(a);
+        if (__any_sync(kFull, a.kept != 0)) warp_add_sums(a);
         if (lane == 0) sh[wid] = a;
         __syncthreads();
         if (threadIdx.x == 0) {
             ShiftSums t = sh[0];
-            for (int ww = 1; ww < kFoldThreads / 32; ww++) add_shift_sums(t, sh[ww]);
-            part[Q.part_base + (int64_t)k * ns + sl] = t;
+            for (int ww = 1; ww < kFoldThreads / 32; ww++)
+                if (sh[ww].kept) add_shift_sums(t, sh[ww]);
+            part[blockIdx.x] = t;
         }
-        __syncthreads();   // sh is written again by the next shift
     }
     // the query's last block goes on
     if (threadIdx.x == 0) {
-        const uint32_t blocks = (uint32_t)(min(max(nsh, 1), (int)gridDim.y) * ns);
+        const uint32_t blocks = (uint32_t)max(nsh, 1) * (uint32_t)ns;
         __threadfence();
         s_last = atomicAdd(folded + qi, 1u) + 1 == blocks;
         __threadfence();
@@ -1669,7 +1681,7 @@ __global__ void __launch_bounds__(kFoldThreads) k_fold(const QPlan* __restrict__
 #pragma unroll
                 for (int i = 0; i < (int)(sizeof(ShiftSums) / 8); i++) y[i] = __ldcg(x + i);   // other blocks wrote them
             }
-            warp_add_sums(u);
+            if (ns > 1) warp_add_sums(u);
             if (lane == 0) {
                 sh[wid] = u;
                 if (sums) sums[Q.sum_base + k0 + wid] = u;
@@ -1723,28 +1735,23 @@ __global__ void __launch_bounds__(kFoldThreads) k_fold(const QPlan* __restrict__
     res[qi] = r;
 }
 
-// the fold's partial records: part_base of every plan (a query's shifts times its slices,
-// one after another); returns the total and, through smax, the most slices of a query
-int64_t fold_parts(std::vector<QPlan>& hp, int& smax) {
+// the fold's parts: part_base of every plan (a query's shifts times its slices, one after
+// another; a rejected query has one for its status); returns how many there are
+int64_t fold_parts(std::vector<QPlan>& hp) {
     int64_t n = 0;
-    smax = 1;
     for (QPlan& P : hp) {
         P.part_base = n;
-        if (P.l <= 0) continue;
-        int ns = fold_slices(P.mode == TM_MODE_EXACT ? 1 : P.J);
-        smax = std::max(smax, ns);
-        n += (int64_t)(P.mode == TM_MODE_EXACT ? 1 : P.b) * ns;
+        if (P.l <= 0) n++;
+        else if (P.mode == TM_MODE_EXACT) n += fold_slices(1);
+        else n += (int64_t)P.b * fold_slices(P.J);
     }
-    return std::max<int64_t>(n, 1);
+    return n;
 }
 
-constexpr int kMaxGridY = 65535;
-
 // the fold on st (folded: one zeroed counter per query)
-void launch_fold(const QPlan* dplans, int nq, int bmax, int smax, const WinDev& W, ShiftSums* part, uint32_t* folded,
+void launch_fold(const QPlan* dplans, int nq, int64_t n_parts, const WinDev& W, ShiftSums* part, uint32_t* folded,
                  tm_result* dres, ShiftSums* sums, unsigned long long* subc, cudaStream_t st) {
-    unsigned gy = (unsigned)std::min(std::max(bmax, 1), kMaxGridY);
-    k_fold<<<dim3((unsigned)nq, gy, (unsigned)smax), kFoldThreads, 0, st>>>(dplans, W, part, folded, dres, sums, subc);
+    launch_after(k_fold, dim3((unsigned)n_parts), kFoldThreads, 0, st, dplans, nq, W, part, folded, dres, sums, subc);
     count_launch();
 }
 
@@ -1770,15 +1777,15 @@ void launch_match(const MatchArgs<TT>& A, int lmax, int kmax, const Tuning& tu, 
     const unsigned gm = (unsigned)(nsm * bps);
     const size_t sm = match_smem_bytes(A.nq, bt);
     if (lmax <= 3 && kmax <= 4 && !expand) {
-        if (bps >= 6) k_match<TT, 3, 4, 6, false><<<gm, bt, sm, st>>>(A);
-        else k_match<TT, 3, 4, 4, false><<<gm, bt, sm, st>>>(A);
-    } else if (lmax <= 3 && kmax <= 4 && bps >= 6) k_match<TT, 3, 4, 6><<<gm, bt, sm, st>>>(A);
-    else if (lmax <= 3 && kmax <= 4) k_match<TT, 3, 4><<<gm, bt, sm, st>>>(A);
-    else if (lmax <= 4 && kmax <= 4 && A.rrec) k_match<TT, 4, 4, 6, true, true><<<gm, bt, sm, st>>>(A);
-    else if (lmax <= 4 && kmax <= 4 && bps >= 6) k_match<TT, 4, 4, 6><<<gm, bt, sm, st>>>(A);
-    else if (lmax <= 4 && kmax <= 4) k_match<TT, 4, 4, 4><<<gm, bt, sm, st>>>(A);
-    else if (lmax <= 5 && kmax <= 5) k_match<TT, 5, 5, 6><<<gm, bt, sm, st>>>(A);
-    else k_match<TT, TM_L_MAX, TM_K_MAX, 4><<<gm, bt, sm, st>>>(A);
+        if (bps >= 6) launch_after(k_match<TT, 3, 4, 6, false>, dim3(gm), bt, sm, st, A);
+        else launch_after(k_match<TT, 3, 4, 4, false>, dim3(gm), bt, sm, st, A);
+    } else if (lmax <= 3 && kmax <= 4 && bps >= 6) launch_after(k_match<TT, 3, 4, 6>, dim3(gm), bt, sm, st, A);
+    else if (lmax <= 3 && kmax <= 4) launch_after(k_match<TT, 3, 4>, dim3(gm), bt, sm, st, A);
+    else if (lmax <= 4 && kmax <= 4 && A.rrec) launch_after(k_match<TT, 4, 4, 6, true, true>, dim3(gm), bt, sm, st, A);
+    else if (lmax <= 4 && kmax <= 4 && bps >= 6) launch_after(k_match<TT, 4, 4, 6>, dim3(gm), bt, sm, st, A);
+    else if (lmax <= 4 && kmax <= 4) launch_after(k_match<TT, 4, 4, 4>, dim3(gm), bt, sm, st, A);
+    else if (lmax <= 5 && kmax <= 5) launch_after(k_match<TT, 5, 5, 6>, dim3(gm), bt, sm, st, A);
+    else launch_after(k_match<TT, TM_L_MAX, TM_K_MAX, 4>, dim3(gm), bt, sm, st, A);
     count_launch();
 }
 
@@ -2162,10 +2169,7 @@ int run_batch_t(const tm_graph* g, const tm_query* qs, int nq, tm_result* res, c
     const int64_t rcap = any_share ? ride_capacity().load() : 0;
     const size_t rrec_bytes = any_share ? a256(sizeof(RideRec<TT>) * (size_t)rcap) : 0;
     // ---- scratch layout
-    int smax = 1;
-    const int64_t n_parts = fold_parts(hp, smax);
-    int bmax = 1;
-    for (const QPlan& P : hp) bmax = std::max(bmax, P.b);
+    const int64_t n_parts = fold_parts(hp);
     std::vector<int32_t> wown;
     const size_t wtab_bytes = place_wtabs(hp, nullptr, wown);
     size_t NWs = (size_t)std::max<int64_t>(NW, 1);
@@ -2324,15 +2328,15 @@ int run_batch_t(const tm_graph* g, const tm_query* qs, int nq, tm_result* res, c
             A.rcap = rcap;
             int64_t gl2 = std::min<int64_t>((Fa + 255) / 256, (int64_t)nsm * 8);
             if (NW > 1) {   // (one window: nothing to search)
-                k_blockwin<<<(unsigned)std::min<int64_t>(((int64_t)nbw + 255) / 256, (int64_t)nsm * 8), 256, 0, st>>>(
-                    W.fbase, NW, Fa, d_Fk, bwin);
+                launch_after(k_blockwin, dim3((unsigned)std::min<int64_t>(((int64_t)nbw + 255) / 256, (int64_t)nsm * 8)), 256, 0, st,
+                             W.fbase, NW, Fa, d_Fk, bwin);
                 count_launch();
             } else {
                 A.blockwin = nullptr;
             }
             ev_l0 = pe.mark(st);
             nv.next("tm_level2");
-            k_level2<TT><<<(unsigned)std::max<int64_t>(gl2, 1), 256, match_smem_bytes(A.nq, 256), st>>>(A, rec, len32, hs_a, hs_hi); count_launch();
+            launch_after(k_level2<TT>, dim3((unsigned)std::max<int64_t>(gl2, 1)), 256, match_smem_bytes(A.nq, 256), st, A, rec, len32, hs_a, hs_hi); count_launch();
             fail(cudaGetLastError(), "k_level2");
             ev_l2 = pe.mark(st);
             nv.next("tm_scan");
@@ -2346,7 +2350,7 @@ int run_batch_t(const tm_graph* g, const tm_query* qs, int nq, tm_result* res, c
                 ev_m1 = pe.mark(st);
                 if (any_share && rc == TM_OK) {
                     nv.next("tm_ride");
-                    k_ride<TT><<<(unsigned)(nsm * 8), 256, match_smem_bytes(A.nq, 256, true), st>>>(A);
+                    launch_after(k_ride<TT>, dim3((unsigned)(nsm * 8)), 256, match_smem_bytes(A.nq, 256, true), st, A);
                     count_launch();
                     fail(cudaGetLastError(), "k_ride");
                     ev_r1 = pe.mark(st);
@@ -2359,7 +2363,7 @@ int run_batch_t(const tm_graph* g, const tm_query* qs, int nq, tm_result* res, c
     if (rc == TM_OK) {
         int ev_f0 = pe.mark(st);
         nv.next("tm_fold");
-        launch_fold(dplans, nq, bmax, smax, W, dpart, dfolded, dres, dbg && dbg->sums ? dsums : nullptr,
+        launch_fold(dplans, nq, n_parts, W, dpart, dfolded, dres, dbg && dbg->sums ? dsums : nullptr,
                     dbg && dbg->sub_count ? dsubc : nullptr, st);
         fail(cudaGetLastError(), "fold");
         ev_f1 = pe.mark(st);
@@ -2899,7 +2903,7 @@ int count_exact_noalloc_t(const tm_graph* g, const tm_motif* m, int64_t delta, c
         A.chunk = tu.chunk_items;
         int nsm = sm_count();
         int64_t gl2 = std::min<int64_t>((F + 255) / 256, (int64_t)nsm * 8);
-        k_level2<TT><<<(unsigned)std::max<int64_t>(gl2, 1), 256, match_smem_bytes(A.nq, 256), st>>>(A, rec, (int32_t*)len2, nullptr, nullptr);
+        launch_after(k_level2<TT>, dim3((unsigned)std::max<int64_t>(gl2, 1)), 256, match_smem_bytes(A.nq, 256), st, A, rec, (int32_t*)len2, nullptr, nullptr);
         count_launch();
         e = cudaGetLastError();
         if (e != cudaSuccess) return na_status(e);
@@ -2916,7 +2920,7 @@ int count_exact_noalloc_t(const tm_graph* g, const tm_motif* m, int64_t delta, c
         if (e != cudaSuccess) return na_status(e);
     }
     // the scan workspace is free again: it holds the fold's one partial record
-    launch_fold(dplan, 1, 1, 1, W, (ShiftSums*)ws, dfolded, dres, nullptr, nullptr, st);
+    launch_fold(dplan, 1, 1, W, (ShiftSums*)ws, dfolded, dres, nullptr, nullptr, st);
     e = cudaGetLastError();
     tm_result hres;
     uint32_t herr = 0;
@@ -2992,7 +2996,7 @@ int batch_create_t(const tm_graph* g, const tm_query* qs, int nq, tm_batch** out
     b->qstat.assign((size_t)nq, TM_OK);
     std::vector<QPlan> hp((size_t)nq);
     int64_t NW = 0, Fmax = 0, n_sums = 0;
-    int lmax = 1, kmax = 2, bmax = 1;
+    int lmax = 1, kmax = 2;
     bool any_hoist = false;
     for (int i = 0; i < nq; i++) {
         std::string why;
@@ -3016,15 +3020,13 @@ int batch_create_t(const tm_graph* g, const tm_query* qs, int nq, tm_batch** out
         P.win_base = NW;
         P.sum_base = n_sums;
         n_sums += P.mode == TM_MODE_EXACT ? 1 : P.b;
-        bmax = std::max(bmax, P.b);
         NW += P.mode == TM_MODE_EXACT ? 1 : P.J * P.b;
         Fmax += P.mode == TM_MODE_EXACT ? g->m : (int64_t)P.b * g->m;
         lmax = std::max(lmax, P.l);
         kmax = std::max(kmax, P.k);
         any_hoist |= P.hoist != 0 || P.ex23 != 0;
     }
-    int smax = 1;
-    const int64_t n_parts = fold_parts(hp, smax);
+    const int64_t n_parts = fold_parts(hp);
     std::vector<int32_t> wown;
     const size_t wtab_bytes = place_wtabs(hp, nullptr, wown);
     size_t NWs = (size_t)std::max<int64_t>(NW, 1), Fs = (size_t)std::max<int64_t>(Fmax, 1);
@@ -3052,7 +3054,6 @@ int batch_create_t(const tm_graph* g, const tm_query* qs, int nq, tm_batch** out
     char* p = (char*)b->scratch;
     auto take = [&](size_t bytes) { char* r = p; p += a256(bytes); return (void*)r; };
     QPlan* dplans = (QPlan*)take(plans_bytes((size_t)nq));
-    tm_result* dres = (tm_result*)take(sizeof(tm_result) * (size_t)nq);
     place_wtabs(hp, (char*)take(wtab_bytes), wown);
     WinDev W;
     W.lo = (int64_t*)take(8 * NWs);
@@ -3068,11 +3069,12 @@ int batch_create_t(const tm_graph* g, const tm_query* qs, int nq, tm_batch** out
     W.k = (int32_t*)take(4 * NWs);
     W.kept = (int32_t*)take(4 * NWs);
     W.qj = (double*)take(8 * NWs);
+    tm_result* dres = (tm_result*)take(sizeof(tm_result) * (size_t)nq + 8);   // the error word behind them
+    uint32_t* derr = (uint32_t*)(dres + nq);   // from there on everything starts at zero
     W.acc = (unsigned long long*)take(8 * A_N * NWs);
     int64_t* dF = (int64_t*)take(8);
     int64_t* dW2 = (int64_t*)take(8);
     unsigned long long* dctr = (unsigned long long*)take(8);
-    uint32_t* derr = (uint32_t*)take(8);
     uint32_t* dfolded = (uint32_t*)take(4 * (size_t)nq);
     unsigned long long* words_w = (unsigned long long*)take(8 * n_words_w);
     unsigned long long* words_f = (unsigned long long*)take(8 * n_words_f);
@@ -3113,7 +3115,7 @@ int batch_create_t(const tm_graph* g, const tm_query* qs, int nq, tm_batch** out
     tm_profile pr0;
     tm_profile_last(&pr0);
     fail(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal), "begin capture");
-    fail(cudaMemsetAsync(W.acc, 0, (size_t)(zero_end - (char*)W.acc), st), "accumulators");
+    fail(cudaMemsetAsync(derr, 0, (size_t)(zero_end - (char*)derr), st), "accumulators");
     if (rc == TM_OK && NW > 0 && (n_words_w || NW <= kWindowThreads)) {
         rc = launch_windows<TT>(G, dplans, nq, W, NW, dF, words_w, derr, nsm, st);
     } else if (rc == TM_OK && NW > 0) {   // (a scan too long for one launch, in the batch's own workspace)
@@ -3131,10 +3133,10 @@ int batch_create_t(const tm_graph* g, const tm_query* qs, int nq, tm_batch** out
         A.chunk = tu.chunk_items;
         A.blockwin = bwin; A.chunkf = cf; A.nchunkf = (int64_t)ncf;
         int64_t gl2 = std::min<int64_t>((Fmax + 255) / 256, (int64_t)nsm * 8);
-        k_blockwin<<<(unsigned)std::min<int64_t>(((int64_t)nbw + 255) / 256, (int64_t)nsm * 8), 256, 0, st>>>(
-            W.fbase, NW, Fmax, dF, bwin);
+        launch_after(k_blockwin, dim3((unsigned)std::min<int64_t>(((int64_t)nbw + 255) / 256, (int64_t)nsm * 8)), 256, 0, st,
+                     W.fbase, NW, Fmax, dF, bwin);
         count_launch();
-        k_level2<TT><<<(unsigned)std::max<int64_t>(gl2, 1), 256, match_smem_bytes(A.nq, 256), st>>>(A, rec, len32, hs_a, hs_hi); count_launch();
+        launch_after(k_level2<TT>, dim3((unsigned)std::max<int64_t>(gl2, 1)), 256, match_smem_bytes(A.nq, 256), st, A, rec, len32, hs_a, hs_hi); count_launch();
         fail(cudaGetLastError(), "k_level2");
         if (rc == TM_OK) rc = scan_lengths(len32, excl, Fmax, dF, dW2, cf, (int64_t)ncf, words_f, derr, wsp2, ws2, st);
         if (rc == TM_OK) {
@@ -3144,11 +3146,10 @@ int batch_create_t(const tm_graph* g, const tm_query* qs, int nq, tm_batch** out
         }
     }
     if (rc == TM_OK) {
-        launch_fold(dplans, nq, bmax, smax, W, dpart, dfolded, dres, nullptr, nullptr, st);
+        launch_fold(dplans, nq, n_parts, W, dpart, dfolded, dres, nullptr, nullptr, st);
         fail(cudaGetLastError(), "fold");
     }
-    fail(cudaMemcpyAsync(b->h_res, dres, sizeof(tm_result) * (size_t)nq, cudaMemcpyDeviceToHost, st), "results");
-    fail(cudaMemcpyAsync(b->h_err, derr, 4, cudaMemcpyDeviceToHost, st), "error word");
+    fail(cudaMemcpyAsync(b->h_res, dres, sizeof(tm_result) * (size_t)nq + 8, cudaMemcpyDeviceToHost, st), "results");
     cudaGraph_t graph = nullptr;
     cudaError_t ee = cudaStreamEndCapture(st, &graph);
     fail(ee, "end capture");

@@ -233,8 +233,9 @@ __global__ void __launch_bounds__(kOneThreads) k_scan_once(const TI* __restrict_
     __shared__ uint32_t s_tile;
     __shared__ BigRanges big;
     if (CF && threadIdx.x == 0) big.n = 0;
+    grid_wait();
     const int64_t n = d_n ? min(*d_n, n_max) : n_max;
-    if (threadIdx.x == 0) s_tile = (uint32_t)atomicAdd(words, 1ull);
+    if (threadIdx.x == 0) s_tile = gridDim.x == 1 ? 0u : (uint32_t)atomicAdd(words, 1ull);
     __syncthreads();
     const int64_t t = s_tile, t0 = t * kOneTile;
     words += 8;
@@ -277,7 +278,7 @@ __global__ void __launch_bounds__(kOneThreads) k_scan_once(const TI* __restrict_
             }
         }
         if (lane == 0) {
-            st_tile64(words + t, (2ull << 62) | (unsigned long long)(before + total));
+            if (gridDim.x > 1) st_tile64(words + t, (2ull << 62) | (unsigned long long)(before + total));
             s_before = before;
             if (t0 + kOneTile >= n) {
                 *d_total = before + total;
@@ -622,10 +623,9 @@ int scan_lengths(const int32_t* in, int64_t* out, int64_t n_max, const int64_t* 
         return TM_OK;
     }
     if (scan_once_words(n_max)) {
-        k_scan_once<int32_t, true><<<(unsigned)((n_max + kOneTile - 1) / kOneTile), kOneThreads, 0, st>>>(
-            in, out, n_max, d_n, d_total, words, err, cf, ncf);
         count_launch();
-        TM_CUDA(cudaGetLastError());
+        TM_CUDA(launch_after(k_scan_once<int32_t, true>, dim3((unsigned)((n_max + kOneTile - 1) / kOneTile)), kOneThreads, 0, st,
+                             in, out, n_max, d_n, d_total, words, err, cf, ncf));
         return TM_OK;
     }
     int64_t ntiles = (n_max + kScanTile - 1) / kScanTile;
@@ -668,10 +668,9 @@ size_t scan_once_words(int64_t n_max) {
 int scan_once_i64(const int64_t* in, int64_t* out, int64_t n, int64_t* d_total, unsigned long long* words, uint32_t* err,
                   cudaStream_t st) {
     if (!scan_once_words(n)) return scan_exclusive_i64(in, out, n, d_total, st);
-    k_scan_once<int64_t, false><<<(unsigned)((n + kOneTile - 1) / kOneTile), kOneThreads, 0, st>>>(
-        in, out, n, nullptr, d_total, words, err, nullptr, 0);
     count_launch();
-    TM_CUDA(cudaGetLastError());
+    TM_CUDA(launch_after(k_scan_once<int64_t, false>, dim3((unsigned)((n + kOneTile - 1) / kOneTile)), kOneThreads, 0, st,
+                         in, out, n, nullptr, d_total, words, err, nullptr, 0));
     return TM_OK;
 }
 

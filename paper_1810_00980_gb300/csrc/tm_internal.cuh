@@ -506,6 +506,26 @@ struct PhaseEvents {
     }
 };
 
+// A launch that may begin before the stream's previous kernel has ended (programmatic dependent
+// launch): its blocks set up what no kernel of the stream writes and then call grid_wait(), which
+// returns once every earlier kernel has completed.  Every kernel launched this way calls it in
+// every block, so that its own completion implies theirs.
+template <typename... P, typename... A>
+cudaError_t launch_after(void (*kernel)(P...), dim3 grid, unsigned threads, size_t smem, cudaStream_t st, A... args) {
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t c = {};
+    c.gridDim = grid;
+    c.blockDim = dim3(threads);
+    c.dynamicSmemBytes = smem;
+    c.stream = st;
+    c.attrs = &at;
+    c.numAttrs = 1;
+    return cudaLaunchKernelEx(&c, kernel, static_cast<P>(args)...);
+}
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // ----------------------------------------------------------------------------
 // device helpers
 // ----------------------------------------------------------------------------
