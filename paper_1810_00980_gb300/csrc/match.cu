@@ -1655,24 +1655,29 @@ __global__ void __launch_bounds__(kFoldThreads) k_fold(const QPlan* __restrict__
             ShiftSums t = sh[0];
             for (int ww = 1; ww < kFoldThreads / 32; ww++)
                 if (sh[ww].kept) add_shift_sums(t, sh[ww]);
-            part[blockIdx.x] = t;
+            if (nsh * (int64_t)ns > 1) part[blockIdx.x] = t;
+            else sh[0] = t;
         }
     }
-    // the query's last block goes on
-    if (threadIdx.x == 0) {
-        const uint32_t blocks = (uint32_t)max(nsh, 1) * (uint32_t)ns;
-        __threadfence();
-        s_last = atomicAdd(folded + qi, 1u) + 1 == blocks;
-        __threadfence();
+    // the query's last block goes on (one with a single part is all there is)
+    const bool single = nsh * (int64_t)ns <= 1;
+    if (!single) {
+        if (threadIdx.x == 0) {
+            __threadfence();
+            s_last = atomicAdd(folded + qi, 1u) + 1 == (uint32_t)nsh * (uint32_t)ns;
+            __threadfence();
+        }
+        __syncthreads();
+        if (!s_last) return;
     }
-    __syncthreads();
-    if (!s_last) return;
     double zsum = 0.0, vsum = 0.0, wmean = 0.0, wm2 = 0.0;   // thread 0's
     ShiftSums tot = {};
     int overflow = 0;
     constexpr int kWarps = kFoldThreads / 32;
     for (int k0 = 0; k0 < nsh; k0 += kWarps) {
-        if (k0 + wid < nsh) {
+        if (single) {
+            if (threadIdx.x == 0 && sums) sums[Q.sum_base] = sh[0];
+        } else if (k0 + wid < nsh) {
             const ShiftSums* pk = part + Q.part_base + (int64_t)(k0 + wid) * ns;
             ShiftSums u = {};
             if (lane < ns) {
@@ -2844,7 +2849,7 @@ int count_exact_noalloc_t(const tm_graph* g, const tm_motif* m, int64_t delta, c
     unsigned char* p = base;
     auto take = [&](size_t bytes) { unsigned char* r = p; p += na_a256(bytes); return (void*)r; };
     QPlan* dplan = (QPlan*)take(sizeof(QPlan));
-    tm_result* dres = (tm_result*)take(sizeof(tm_result));
+    take(sizeof(tm_result));
     WinDev W;
     W.lo = (int64_t*)take(8);
     W.hi = (int64_t*)take(8);
@@ -2884,6 +2889,8 @@ int count_exact_noalloc_t(const tm_graph* g, const tm_motif* m, int64_t delta, c
     // error word behind it) and scan words, which fill the last part of the scan workspace
     uint32_t* dfolded = (uint32_t*)(dctr + 1);
     uint32_t* derr = (uint32_t*)(dctr + 2);
+    static_assert(3 * 8 + sizeof(tm_result) <= 256, "the result follows the error word (one copy brings both back)");
+    tm_result* dres = (tm_result*)(dctr + 3);
     unsigned long long* words = (unsigned long long*)(ws + kNaWsElems / 2);
     cudaError_t e = cudaMemcpyAsync(dplan, &P, sizeof(P), cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess) e = cudaMemsetAsync(W.acc, 0, (size_t)((unsigned char*)dctr + 256 - (unsigned char*)W.acc), st);
@@ -2922,13 +2929,15 @@ int count_exact_noalloc_t(const tm_graph* g, const tm_motif* m, int64_t delta, c
     // the scan workspace is free again: it holds the fold's one partial record
     launch_fold(dplan, 1, 1, W, (ShiftSums*)ws, dfolded, dres, nullptr, nullptr, st);
     e = cudaGetLastError();
-    tm_result hres;
-    uint32_t herr = 0;
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&hres, dres, sizeof(hres), cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&herr, derr, sizeof(herr), cudaMemcpyDeviceToHost, st);
+    struct {
+        unsigned long long err;
+        tm_result res;
+    } h;
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&h, derr, sizeof(h), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) return na_status(e);
-    if (herr) return TM_ECUDA;
+    if (h.err) return TM_ECUDA;
+    const tm_result& hres = h.res;
     if (hres.status != TM_OK) return hres.status;
     *count = hres.count;
     return TM_OK;
