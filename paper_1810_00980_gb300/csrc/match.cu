@@ -2567,30 +2567,36 @@ int run_batch_once(const tm_graph* g, const tm_query* qs, int nq, tm_result* res
     // least kHideCand of it (measured: see kHideFirst).
     std::vector<tm_query> hidden;
     std::vector<int> top;                     // per hidden head, the estimate whose span it has
-    for (size_t x = 0; x < alone.size(); x++) {
-        if (host[(size_t)alone[x]] >= 0) continue;
-        std::vector<int> gr;
-        for (size_t y = x; y < alone.size(); y++)
-            if (host[(size_t)alone[y]] < 0 && same_motif(qs[alone[x]].motif, qs[alone[y]].motif)) gr.push_back(alone[y]);
+    std::vector<std::vector<int>> kinds;      // the estimates of each motif
+    for (int i : alone) {
+        size_t k = 0;
+        while (k < kinds.size() && !same_motif(qs[kinds[k][0]].motif, qs[i].motif)) k++;
+        if (k == kinds.size()) kinds.emplace_back();
+        kinds[k].push_back(i);
+    }
+    for (std::vector<int>& gr : kinds) {
         std::stable_sort(gr.begin(), gr.end(), [&](int a, int b) { return qs[a].delta > qs[b].delta; });
-        for (size_t y = 0; y < gr.size(); y++) {
-            double first = 0.0, cand = 0.0;
-            const size_t n = std::min(gr.size() - y, (size_t)kMaxRide);
-            for (size_t z = y; z < y + n; z++) {
-                const tm_query& q = qs[gr[z]];
-                const double J = 1.0 + (double)g->t_max / ((double)q.c * (double)q.delta);
-                const double p = q.q_mode == TM_Q_UNIFORM ? q.p : std::min(1.0, q.p / J);
-                first += p * q.b;
-                cand += p * q.b * ((double)q.delta / (double)qs[gr[y]].delta);
+        std::vector<double> first(1, 0.0), cand(1, 0.0);   // sums of b p and of b p delta, longest spans first
+        for (int i : gr) {
+            const tm_query& q = qs[i];
+            const double J = 1.0 + (double)g->t_max / ((double)q.c * (double)q.delta);
+            const double bp = q.b * (q.q_mode == TM_Q_UNIFORM ? q.p : std::min(1.0, q.p / J));
+            first.push_back(first.back() + bp);
+            cand.push_back(cand.back() + bp * (double)q.delta);
+        }
+        for (size_t y = 0; y < gr.size();) {
+            const size_t e = std::min(gr.size(), y + (size_t)kMaxRide);
+            if (first[e] - first[y] < kHideFirst || cand[e] - cand[y] < kHideCand * (double)qs[gr[y]].delta) {
+                y++;   // the next shorter span
+                continue;
             }
-            if (first < kHideFirst || cand < kHideCand) continue;
-            tm_query e = qs[gr[y]];
-            e.mode = TM_MODE_EXACT;
-            for (size_t z = y; z < y + n; z++) host[(size_t)gr[z]] = nq + (int)hidden.size();
-            hidden.push_back(e);
+            tm_query h = qs[gr[y]];
+            h.mode = TM_MODE_EXACT;
+            for (size_t z = y; z < e; z++) host[(size_t)gr[z]] = nq + (int)hidden.size();
+            hidden.push_back(h);
             top.push_back(gr[y]);
             any = true;
-            break;
+            y = e;
         }
     }
     if (!any) return run_batch_typed(g, qs, nq, res, st, nullptr);
