@@ -674,10 +674,14 @@ int scan_once_i64(const int64_t* in, int64_t* out, int64_t n, int64_t* d_total, 
     return TM_OK;
 }
 
+// Digits of at most nine bits (ten when one pass then does): a tile's run of a digit is four keys
+// at ten bits, 16 bytes in each array, 32 at seven, and the stores bound the pass.  Build of 1e8
+// edges between 1e6 nodes (20 bits): two passes of ten 11.0 ms, three of seven 9.0, four of five
+// 9.8; of 1e7 between 1e5 (17 bits): two of nine 0.90 ms, three of six 0.91.
 SortDigits sort_digits(int bits) {
     SortDigits D;
     D.bits = std::max(bits, 1);
-    D.passes = (D.bits + 9) / 10;
+    D.passes = D.bits <= 10 ? 1 : (D.bits + 8) / 9;
     D.db = std::max(5, (D.bits + D.passes - 1) / D.passes);
     return D;
 }
