@@ -119,6 +119,8 @@ typedef struct {
     int64_t cand_edges;   /* adjacency entries read at intermediate levels (N_cand) */
     int64_t last_ranges;  /* partial instances closed at the last motif edge (N_last) */
     int64_t inst_read;    /* last-edge entries read one by one (estimate mode) */
+    /* (queries that share an enumeration report its work on one of them: the exact query of the
+     * largest span, or among estimates alone the one of the largest span; the others report 0) */
     double var_hat;       /* estimate: unbiased estimate of Var[Z | s] averaged over shifts
                              (Lemma 4.4: sum_j Q_j Y_j^2 (1-q_j)/q_j^2); exact: 0 */
     double shift_var;     /* estimate with b >= 2: sample variance of the b per-shift Z_k (an
@@ -281,7 +283,8 @@ void tm_batch_free(tm_batch* b);
  * (tm_autotune) writes these after timing candidates on a graph. */
 typedef struct {
     int32_t block_threads;     /* threads per block of the matcher (multiple of 32) */
-    int32_t blocks_per_sm;     /* persistent blocks per SM */
+    int32_t blocks_per_sm;     /* persistent blocks per SM (until it is set or found by the
+                                  autotuner, the matcher takes the number that suits its kernel) */
     int32_t chunk_items;       /* level-2 items a warp takes per queue grab (multiple of 32) */
     int32_t enum_threshold;    /* last-level ranges longer than this are counted by
                                   subtraction instead of being read entry by entry */

@@ -1,8 +1,9 @@
 // Graph ingest and adjacency build (temporal graph T and its static graph G,
-// Section 2).  Everything after the input copy runs on the device: validation,
-// normalisation t' = t - t_min (Algorithm 1 assumes times start at 0), three
-// stable radix sorts that leave every adjacency segment in time order, and
-// segment offsets found from the sorted keys.
+// Section 2).  Everything after the input copy runs on the device: one read that
+// validates, normalises t' = t - t_min (Algorithm 1 assumes times start at 0) and
+// counts the sorts' digits, three stable radix sorts that leave every adjacency
+// segment in time order, segment offsets and pair bounds found from the sorted
+// keys, and the table of the static edges.
 #include <algorithm>
 #include <cstring>
 #include <mutex>

@@ -2077,6 +2077,9 @@ RideEnt ride_entry(const QPlan& R, int k, int64_t t_max) {
     return E;
 }
 
+// most deferred records made room for on behalf of estimates that could do without (12.9 GB)
+constexpr int64_t kHiddenRecords = (int64_t)1 << 29;
+
 template <typename TT>
 int run_batch_t(const tm_graph* g, const tm_query* qs, int nq, tm_result* res, cudaStream_t st,
                 BatchOut* dbg) {
@@ -2171,7 +2174,7 @@ int run_batch_t(const tm_graph* g, const tm_query* qs, int nq, tm_result* res, c
         }
     bool any_share = false;
     for (const QPlan& P : hp) any_share |= P.nsub > 0 || P.nride > 0;
-    const int64_t rcap = any_share ? ride_capacity().load() : 0;
+    const int64_t rcap = any_share ? std::max(ride_capacity().load(), dbg->need_records) : 0;   // (shares come with dbg)
     const size_t rrec_bytes = any_share ? a256(sizeof(RideRec<TT>) * (size_t)rcap) : 0;
     // ---- scratch layout
     const int64_t n_parts = fold_parts(hp);
@@ -2436,9 +2439,13 @@ int run_batch_t(const tm_graph* g, const tm_query* qs, int nq, tm_result* res, c
     if ((int64_t)h_rcount > rcap) {
         // more deferred records than the buffer held: run again with room for all of them
         int64_t want = (int64_t)h_rcount + (int64_t)(h_rcount >> 3) + 1024;
+        if (dbg->hidden && want > kHiddenRecords) return TM_ENOMEM;   // run_batch_once runs the estimates apart
+        dbg->need_records = want;
+        rc = run_batch_t<TT>(g, qs, nq, res, st, dbg);
+        if (rc == TM_ENOMEM) return rc;   // (the next batches keep the capacity that fits)
         int64_t cur = ride_capacity().load();
         while (cur < want && !ride_capacity().compare_exchange_weak(cur, want)) {}
-        return run_batch_t<TT>(g, qs, nq, res, st, dbg);
+        return rc;
     }
     if (dbg && dq_n > 0) {
         const QPlan& P = hp[(size_t)dbg->query];
@@ -2499,7 +2506,7 @@ bool same_motif(const tm_motif* a, const tm_motif* b) {
 constexpr double kHideFirst = 1.4, kHideCand = 0.9;
 
 int run_batch_once(const tm_graph* g, const tm_query* qs, int nq, tm_result* res, cudaStream_t st,
-                   BatchOut* dbg) {
+                   BatchOut* dbg, bool hide = true) {
     if (dbg || !g || !qs || !res || nq < 2) return run_batch_typed(g, qs, nq, res, st, dbg);
     std::vector<int> lead((size_t)nq, -1), slot((size_t)nq, -1);   // span members: their leader
     std::vector<std::vector<int>> groups;
@@ -2574,6 +2581,7 @@ int run_batch_once(const tm_graph* g, const tm_query* qs, int nq, tm_result* res
         if (k == kinds.size()) kinds.emplace_back();
         kinds[k].push_back(i);
     }
+    if (!hide) kinds.clear();
     for (std::vector<int>& gr : kinds) {
         std::stable_sort(gr.begin(), gr.end(), [&](int a, int b) { return qs[a].delta > qs[b].delta; });
         std::vector<double> first(1, 0.0), cand(1, 0.0);   // sums of b p and of b p delta, longest spans first
@@ -2627,6 +2635,9 @@ int run_batch_once(const tm_graph* g, const tm_query* qs, int nq, tm_result* res
     bo.riders = &riders;
     bo.hidden = (int)hidden.size();
     int rc = run_batch_typed(g, qc.data(), nc, rc_res.data(), st, &bo);
+    // the shared enumeration's records (one per group of instances) may not fit where the
+    // estimates' own enumerations, which keep none, do
+    if (rc == TM_ENOMEM && !hidden.empty()) return run_batch_once(g, qs, nq, res, st, dbg, false);
     for (int i = 0; i < nq; i++) {
         if (lead[(size_t)i] < 0) {
             res[i] = rc_res[(size_t)pos[(size_t)i]];

@@ -307,8 +307,7 @@ __global__ void __launch_bounds__(kOneThreads) k_scan_once(const TI* __restrict_
 }
 
 // ------------------------------------------------------------------ radix sort
-// Stable LSD radix sort of (key, a[, t]) triples by digits of up to 10 bits, one kernel per
-// digit.  The digit counts of the whole input, for every digit, come from one earlier read
+// Stable LSD radix sort of (key, a[, t]) triples, one kernel per digit.  The digit counts of the whole input, for every digit, come from one earlier read
 // (digit_count_block, inside the kernel that produces the keys, or k_digit_count); a pass then
 // finds each tile's place in every digit's run from the tiles before it (decoupled look-back:
 // Merrill and Garland, "Single-pass parallel prefix scan with decoupled look-back", 2016; used
@@ -316,9 +315,12 @@ __global__ void __launch_bounds__(kOneThreads) k_scan_once(const TI* __restrict_
 // triple once and nothing else of size n.  The passes it replaces read every key a second time
 // for a histogram per tile and scanned 2^bits x tiles counters with three more kernels.
 //
-// What bounds a pass: HBM, at 2 x 12 bytes per key with 32-bit times.  A tile is 4096 keys, all
-// of its loads in flight at once, so that three tiles per SM cover the memory's latency; each
-// digit's run of the tile leaves shared memory as neighbouring addresses.
+// A tile is 4096 keys, all of its loads in flight at once, so that three tiles per SM cover the
+// memory's latency; each digit's run of the tile leaves shared memory as neighbouring
+// addresses.  A pass moves 2.3 to 3.0 TB/s of its 2 x 12 bytes per key (1e7 keys, nine-bit
+// digits: 93 to 106 us, 159 to 176 for both views at once; histogram, scan and scatter took 140
+// to 180 per sort): 58 % of the LSU's wavefronts, for stores that reach four to eight runs each,
+// and 55 % of the ALU, for a ballot per digit bit, are what bounds it.
 constexpr int kSortThreads = 256;
 constexpr int kSortWarps = kSortThreads / 32;
 constexpr int kSortItems = 16;                       // per thread

@@ -339,6 +339,7 @@ struct BatchOut {                 // optional per-window readback for one query
     ShiftSums* sums = nullptr;    // host: per query, per shift (exact: one), or null
     const std::vector<std::vector<int>>* riders = nullptr;   // per query: plan indices of its riders
     int hidden = 0;                           // trailing queries whose results nobody asked for
+    int64_t need_records = 0;                 // deferred records to make room for, past the usual capacity
     const int32_t* nsub = nullptr;            // per query: spans counted alongside (exact)
     const int64_t* sub_delta = nullptr;       // [nq][kMaxSub]
     unsigned long long* sub_count = nullptr;  // host out: [nq][kMaxSub]

@@ -64,3 +64,27 @@ def test_few_windows_stay_alone():
     with tm.Graph(*(torch.from_numpy(x).cuda() for x in (src, dst, t)), 700) as g:
         res = tm.run_batch(g, [tm.estimate_query(mo, 3600, 10, 0.2, s) for s in range(4)])
         assert all(r["first_edges"] > 0 for r in res)
+
+
+def test_no_room_for_the_records_runs_the_estimates_apart():
+    """The shared enumeration needs a record buffer that the estimates alone do not: when it
+    cannot be had, the batch still runs and equals itself."""
+    import torch
+    import __graft_entry__
+    __graft_entry__.build()
+    torch.cuda.set_device(0)
+    from paper_1810_00980_gb300 import tm
+    src, dst, t = synth.chung_lu_hawkes(700, 40_000, 2.1, seed=13, horizon=2_000_000)
+    mo = tm.Motif(*MOTIFS["cycle3"])
+    with tm.Graph(*(torch.from_numpy(x).cuda() for x in (src, dst, t)), 700) as g:
+        qs = [tm.estimate_query(mo, 3600, 10, 0.8, s) for s in range(3)]
+        ref = tm.run_batch(g, qs)
+        assert sum(r["first_edges"] > 0 for r in ref) == 1
+        try:
+            tm.set_ride_capacity(1 << 36)   # 1.6 TB of records
+            res = tm.run_batch(g, qs)
+        finally:
+            tm.set_ride_capacity(1 << 23)
+        assert all(r["first_edges"] > 0 for r in res)
+        assert [{k: r[k] for k in KEYS} for r in res] == [{k: r[k] for k in KEYS} for r in ref]
+        assert tm.run_batch(g, qs)[0]["estimate"] == ref[0]["estimate"]
