@@ -437,12 +437,13 @@ def cpu_baselines(src, dst, t, meta):
 
 
 def sampled_leg(tm, torch, g, qs, meta, exact, stream, steps=5, warmup=2):
-    """The estimator's own sampled-window path on the resident graph: the nine
-    estimates of the benchmark batch in a batch of their own (no exact query of
-    their motif beside them, so none rides along and each enumerates its own
-    kept windows), with each estimate's relative error; beside them the nine
-    exact queries in one batch, each query alone in its own batched launch, and
-    (measured separately) plain one-query-per-launch exact counting.  Times are
+    """The estimator's own path on the resident graph: the nine estimates of the
+    benchmark batch in a batch of their own (no exact query of their motif
+    beside them; those of a motif share one enumeration when together they
+    keep enough windows), with each estimate's relative error; beside them the
+    nine exact queries in one batch, each query alone in its own batched launch
+    (an estimate then enumerates its own kept windows), and (measured
+    separately) plain one-query-per-launch exact counting.  Times are
     CUDA events around `steps` synchronous tm_run_batch calls."""
     sh = stream.cuda_stream
 
@@ -479,7 +480,7 @@ def sampled_leg(tm, torch, g, qs, meta, exact, stream, steps=5, warmup=2):
             "exact_one_per_launch_qps": len(exq) / (ex_alone_ms / 1e3),
             "estimates_rel_err_max": max(v["rel_err"] for v in per.values()),
             "per_estimate": per,
-            "note": "estimates alone (no riders); graph resident, not rebuilt; one tm_run_batch per step"}
+            "note": "estimates without exact queries; graph resident, not rebuilt; one tm_run_batch per step"}
 
 
 # ------------------------------------------------------------------ main ---
