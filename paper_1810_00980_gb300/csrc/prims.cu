@@ -307,13 +307,14 @@ __global__ void __launch_bounds__(kOneThreads) k_scan_once(const TI* __restrict_
 }
 
 // ------------------------------------------------------------------ radix sort
-// Stable LSD radix sort of (key, a[, t]) triples, one kernel per digit.  The digit counts of the whole input, for every digit, come from one earlier read
-// (digit_count_block, inside the kernel that produces the keys, or k_digit_count); a pass then
-// finds each tile's place in every digit's run from the tiles before it (decoupled look-back:
-// Merrill and Garland, "Single-pass parallel prefix scan with decoupled look-back", 2016; used
-// for radix sorting by Adinets and Merrill, "Onesweep", 2022), so it reads and writes each
-// triple once and nothing else of size n.  The passes it replaces read every key a second time
-// for a histogram per tile and scanned 2^bits x tiles counters with three more kernels.
+// Stable LSD radix sort of (key, a[, t]) triples, one kernel per digit.  The counts of the whole
+// input, for every digit, come from one earlier read (count_digits, inside the kernel that
+// produces the keys, or k_digit_count); a pass then finds each tile's place in every digit's run
+// from the tiles before it (decoupled look-back: Merrill and Garland, "Single-pass parallel
+// prefix scan with decoupled look-back", 2016; used for radix sorting by Adinets and Merrill,
+// "Onesweep", 2022), so it reads and writes each triple once and nothing else of size n.  The
+// passes it replaces read every key a second time for a histogram per tile and scanned
+// 2^bits x tiles counters with three more kernels.
 //
 // A tile is 4096 keys, all of its loads in flight at once, so that three tiles per SM cover the
 // memory's latency; each digit's run of the tile leaves shared memory as neighbouring
