@@ -118,8 +118,9 @@ struct MatchArgs {
     int64_t chunk;
     int enum_threshold;
     const int32_t* blockwin = nullptr;  // [ceil(F/32)] window of first edge 32 b (null: searched)
-    const int64_t* chunkf = nullptr;    // [nchunkf] first edge of work item i * kItemGrain (null: searched)
+    const int64_t* chunkf = nullptr;    // [nchunkf] first edge of work item i << grain_log
     int64_t nchunkf = 0;
+    int grain_log = 5;                  // log2 of item_grain of the first edges' bound
     RideRec<TT>* rrec = nullptr;        // [rcap] deferred rider / smaller-span work (see RideRec)
     unsigned long long* rcount = nullptr;   // records appended (counts past rcap: the batch reruns)
     int64_t rcap = 0;
@@ -1229,15 +1230,16 @@ __global__ void __launch_bounds__(256, OCC) k_match(MatchArgs<TT> A) {
     // few items: smaller chunks, so that every warp gets some (17,000 items in chunks of 256 kept 67
     // warps busy for eight rounds each: 43 us of a 20,000-edge count)
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    const int64_t share = (W2 / nwarps + kItemGrain) / kItemGrain * kItemGrain;
-    const int64_t chunk = min(A.chunk, share);
+    const int gl = A.grain_log;
+    const int64_t share = ((W2 / nwarps >> gl) + 1) << gl;
+    const int64_t chunk = min((((A.chunk - 1) >> gl) + 1) << gl, share);
     // a warp's first chunk is its own, the others come from the counter (with few items no warp
     // asks it: 7,000 atomics on one word take longer than such a batch's items)
     for (int64_t c0 = ((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5) * chunk; c0 < W2;) {
         int64_t c1 = min(c0 + chunk, W2);
         int64_t fb = 0, fe = 0;
-        const int64_t ci = c0 / kItemGrain, ce = (c1 + kItemGrain - 1) / kItemGrain;
-        if (A.chunkf && ce < A.nchunkf) {
+        const int64_t ci = c0 >> gl, ce = ((c1 - 1) >> gl) + 1;
+        if (ce < A.nchunkf) {
             // first edges of this chunk's first item and of the next chunk's (a bound on
             // the last item's: first edges in between have no items below c1)
             fb = __ldg(A.chunkf + ci);
@@ -2008,7 +2010,7 @@ int ex_tables_for(const tm_graph* g, const std::vector<QPlan>& hp, cudaStream_t 
 // chunk-start tables
 size_t per_first_scratch_bytes(int64_t F, bool hoist, size_t rec_bytes) {
     size_t Fs = (size_t)std::max<int64_t>(F, 1);
-    size_t nbw = Fs / 32 + 1, ncf = Fs / 4 + 2;
+    size_t nbw = Fs / 32 + 1, ncf = item_starts(Fs);
     return a256(rec_bytes * Fs) + a256(4 * Fs) + (hoist ? 3 : 1) * a256(8 * Fs) + a256(4 * nbw) + a256(8 * ncf);
 }
 constexpr size_t kBoundScratchBytes = (size_t)2 << 30;
@@ -2310,7 +2312,7 @@ int run_batch_t(const tm_graph* g, const tm_query* qs, int nq, tm_result* res, c
     ScratchLease fb;
     if (rc == TM_OK && Fa > 0) {
         size_t Fs = (size_t)Fa;
-        size_t nbw = Fs / 32 + 1, ncf = Fs / 4 + 2;
+        size_t nbw = Fs / 32 + 1, ncf = item_starts(Fs);
         rc = scratch_acquire(per_first_scratch_bytes(Fa, any_hoist, sizeof(FRec<TT>)) + rrec_bytes, st, fb);
         if (rc == TM_OK) {
             char* q2 = (char*)fb.p;
@@ -2330,7 +2332,7 @@ int run_batch_t(const tm_graph* g, const tm_query* qs, int nq, tm_result* res, c
             A.d_W2 = dW2; A.counter = dctr;
             A.enum_threshold = tu.enum_threshold;
             A.chunk = tu.chunk_items;
-            A.blockwin = bwin; A.chunkf = cf; A.nchunkf = (int64_t)ncf;
+            A.blockwin = bwin; A.chunkf = cf; A.nchunkf = (int64_t)ncf; A.grain_log = item_grain_log(Fa);
             A.rrec = rrec;
             A.rcount = drcount;
             A.rcap = rcap;
@@ -2935,6 +2937,7 @@ int count_exact_noalloc_t(const tm_graph* g, const tm_motif* m, int64_t delta, c
         // the second
         A.chunkf = len2 + kNaMaxEdges / 2;
         A.nchunkf = kNaMaxEdges / 2;
+        A.grain_log = item_grain_log(F);
         if ((int64_t)scan_once_words(F) > kNaWsElems / 2 || !scan_once_words(F)) return TM_EINVAL;
         rc = scan_lengths((const int32_t*)len2, excl, F, nullptr, dW2, len2 + kNaMaxEdges / 2, A.nchunkf, words, derr,
                           nullptr, 0, st);
@@ -3063,7 +3066,7 @@ int batch_create_t(const tm_graph* g, const tm_query* qs, int nq, tm_batch** out
                 9 * a256(8 * NWs) + 3 * a256(4 * NWs) + a256(8 * NWs) + a256(8 * A_N * NWs) + 4 * 256 +
                 a256(4 * (size_t)nq) + a256(8 * n_words_w) + a256(8 * n_words_f) + a256(sizeof(FRec<TT>) * Fs) + (any_hoist ? 3 : 1) * a256(8 * Fs) + a256(8 * (size_t)ws1) +
                 a256(8 * (size_t)ws2) +
-                a256(4 * (Fs / 32 + 1)) + a256(8 * (Fs / 4 + 2)) + a256(4 * Fs) +
+                a256(4 * (Fs / 32 + 1)) + a256(8 * item_starts(Fs)) + a256(4 * Fs) +
                 a256(sizeof(ShiftSums) * (size_t)n_parts);
     cudaError_t e = cudaMalloc(&b->scratch, sz);
     if (e == cudaSuccess) e = cudaMallocHost((void**)&b->h_res, sizeof(tm_result) * (size_t)nq + 8);
@@ -3112,7 +3115,7 @@ int batch_create_t(const tm_graph* g, const tm_query* qs, int nq, tm_batch** out
     int64_t* hs_hi = any_hoist ? (int64_t*)take(8 * Fs) : nullptr;
     int64_t* wsp1 = (int64_t*)take(8 * (size_t)ws1);
     int64_t* wsp2 = (int64_t*)take(8 * (size_t)ws2);
-    size_t nbw = Fs / 32 + 1, ncf = Fs / 4 + 2;
+    size_t nbw = Fs / 32 + 1, ncf = item_starts(Fs);
     int32_t* bwin = (int32_t*)take(4 * nbw);
     int64_t* cf = (int64_t*)take(8 * ncf);
     ShiftSums* dpart = (ShiftSums*)take(sizeof(ShiftSums) * (size_t)n_parts);
@@ -3157,7 +3160,7 @@ int batch_create_t(const tm_graph* g, const tm_query* qs, int nq, tm_batch** out
         A.d_W2 = dW2; A.counter = dctr;
         A.enum_threshold = tu.enum_threshold;
         A.chunk = tu.chunk_items;
-        A.blockwin = bwin; A.chunkf = cf; A.nchunkf = (int64_t)ncf;
+        A.blockwin = bwin; A.chunkf = cf; A.nchunkf = (int64_t)ncf; A.grain_log = item_grain_log(Fmax);
         int64_t gl2 = std::min<int64_t>((Fmax + 255) / 256, (int64_t)nsm * 8);
         launch_after(k_blockwin, dim3((unsigned)std::min<int64_t>(((int64_t)nbw + 255) / 256, (int64_t)nsm * 8)), 256, 0, st,
                      W.fbase, NW, Fmax, dF, bwin);

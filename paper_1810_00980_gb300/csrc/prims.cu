@@ -99,15 +99,16 @@ __global__ void k_len_reduce(const int32_t* __restrict__ in, int64_t n_max, cons
     if (threadIdx.x == 0) sums[blockIdx.x] = total;
 }
 
-// Item starts: cf[i] = the element whose range holds item i * kItemGrain.  Each thread notes its own
+// Item starts: cf[i] = the element whose range holds item i * grain.  Each thread notes its own
 // elements' (those of a range past kBigRange are left to the whole block: noted by one thread, the
 // range of a hub's burst would be a long serial run of stores).
-constexpr int64_t kBigRange = 64 * kItemGrain;
+constexpr int64_t kBigRange = 2048;
 struct BigRanges {
     int n;
     int64_t e[32], from[32], len[32];
 };
-__device__ __forceinline__ void note_items(BigRanges& B, int64_t* cf, int64_t ncf, int64_t e, int64_t from, int64_t len) {
+__device__ __forceinline__ void note_items(BigRanges& B, int64_t* cf, int64_t ncf, int grain, int64_t e, int64_t from,
+                                           int64_t len) {
     if (len > kBigRange) {
         const int k = atomicAdd(&B.n, 1);
         if (k < 32) {
@@ -115,12 +116,12 @@ __device__ __forceinline__ void note_items(BigRanges& B, int64_t* cf, int64_t nc
             return;
         }
     }
-    for (int64_t i = (from + kItemGrain - 1) / kItemGrain; i * kItemGrain < from + len && i < ncf; i++) cf[i] = e;
+    for (int64_t i = (from + grain - 1) / grain; i * grain < from + len && i < ncf; i++) cf[i] = e;
 }
-__device__ __forceinline__ void note_big(const BigRanges& B, int64_t* cf, int64_t ncf) {
+__device__ __forceinline__ void note_big(const BigRanges& B, int64_t* cf, int64_t ncf, int grain) {
     for (int k = 0; k < min(B.n, 32); k++)
-        for (int64_t i = (B.from[k] + kItemGrain - 1) / kItemGrain + threadIdx.x;
-             i * kItemGrain < B.from[k] + B.len[k] && i < ncf; i += blockDim.x)
+        for (int64_t i = (B.from[k] + grain - 1) / grain + threadIdx.x;
+             i * grain < B.from[k] + B.len[k] && i < ncf; i += blockDim.x)
             cf[i] = B.e[k];
 }
 
@@ -132,6 +133,7 @@ __global__ void k_len_scan(const int32_t* __restrict__ in, int64_t* __restrict__
     __shared__ int64_t smem[33];
     __shared__ int64_t tile[kScanTile + kScanTile / 16];   // one pad word per 16: no bank conflicts
     __shared__ BigRanges big;
+    const int grain = item_grain(n_max);
     if (threadIdx.x == 0) big.n = 0;
     int64_t n = d_n ? min(*d_n, n_max) : n_max;
     int64_t t0 = (int64_t)blockIdx.x * kScanTile;
@@ -152,17 +154,17 @@ __global__ void k_len_scan(const int32_t* __restrict__ in, int64_t* __restrict__
     int64_t total;
     int64_t run = block_excl_scan(loc, smem, &total) + offs[blockIdx.x];
     if (threadIdx.x == 0 && t0 + kScanTile >= n) {
-        const int64_t end = (run + total + kItemGrain - 1) / kItemGrain;
+        const int64_t end = (run + total + grain - 1) / grain;
         if (end < ncf) cf[end] = n - 1;
     }
 #pragma unroll
     for (int i = 0; i < kScanItems; i++) {
-        note_items(big, cf, ncf, t0 + b + i, run, v[i]);
+        note_items(big, cf, ncf, grain, t0 + b + i, run, v[i]);
         tile[b + i + ((b + i) >> 4)] = run;
         run += v[i];
     }
     __syncthreads();
-    note_big(big, cf, ncf);
+    note_big(big, cf, ncf, grain);
     for (int i = threadIdx.x; i < kScanTile; i += blockDim.x) {
         int64_t idx = t0 + i;
         if (idx < n) out[idx] = tile[i + (i >> 4)];
@@ -208,8 +210,8 @@ __global__ void k_set_i64(int64_t* p, int64_t v) { *p = v; }
 // 2^62), and a warp looks back over 32 tiles at a time.  Prefixes travel 32 tiles per memory
 // latency, so beyond kOnePassTiles tiles the two-pass form is as quick; below, one launch takes
 // the place of three to five (a 20,000-edge count spent 22 of its 118 us on them).
-// CF also notes the first edge of every kItemGrain-th item (cf[i]: the element whose range holds
-// item i * kItemGrain; past the last, n - 1), as far as cf's ncf entries go.
+// CF also notes the first edge of every grain-th item (cf[i]: the element whose range holds item
+// i * grain, grain = item_grain(n_max); past the last, n - 1), as far as cf's ncf entries go.
 constexpr int kOneThreads = 256;
 constexpr int kOneItems = 16;
 constexpr int kOneTile = kOneThreads * kOneItems;
@@ -232,6 +234,7 @@ __global__ void __launch_bounds__(kOneThreads) k_scan_once(const TI* __restrict_
     __shared__ int64_t s_before;
     __shared__ uint32_t s_tile;
     __shared__ BigRanges big;
+    const int grain = item_grain(n_max);
     if (CF && threadIdx.x == 0) big.n = 0;
     grid_wait();
     const int64_t n = d_n ? min(*d_n, n_max) : n_max;
@@ -283,7 +286,7 @@ __global__ void __launch_bounds__(kOneThreads) k_scan_once(const TI* __restrict_
             if (t0 + kOneTile >= n) {
                 *d_total = before + total;
                 if (CF) {
-                    const int64_t end = (before + total + kItemGrain - 1) / kItemGrain;
+                    const int64_t end = (before + total + grain - 1) / grain;
                     if (end < ncf) cf[end] = n - 1;
                 }
             }
@@ -294,12 +297,12 @@ __global__ void __launch_bounds__(kOneThreads) k_scan_once(const TI* __restrict_
 #pragma unroll
     for (int i = 0; i < kOneItems; i++) {
         const int64_t v = tile[b + i + ((b + i) >> 4)];
-        if (CF) note_items(big, cf, ncf, t0 + b + i, run, v);
+        if (CF) note_items(big, cf, ncf, grain, t0 + b + i, run, v);
         tile[b + i + ((b + i) >> 4)] = run;
         run += v;
     }
     __syncthreads();
-    if (CF) note_big(big, cf, ncf);
+    if (CF) note_big(big, cf, ncf, grain);
     for (int i = threadIdx.x; i < kOneTile; i += kOneThreads) {
         const int64_t idx = t0 + i;
         if (idx < n) out[idx] = tile[i + (i >> 4)];

@@ -418,10 +418,17 @@ int scan_exclusive_i64_ws(const int64_t* in, int64_t* out, int64_t n, int64_t* d
 
 int64_t scan_dn_ws_elems(int64_t n_max);
 // Exclusive scan of 32-bit range lengths into 64-bit offsets (the first *d_n, or n_max when d_n is
-// null) with, in cf, the element that holds every kItemGrain-th item (as far as ncf goes).  words:
+// null) with, in cf, the element that holds every grain-th item (as far as ncf goes).  words:
 // scan_once_words(n_max) zeroed words; when that is 0 (too many tiles for one launch) ws of
 // scan_dn_ws_elems(n_max), or null to allocate it on the stream.  *err: as SortWs::err
-constexpr int kItemGrain = 32;
+// The matcher's chunks are whole grains.  Few first edges: 32 items, so that small batches cut
+// small chunks, with entries for 64 items per first edge; many: 256, where every chunk is at
+// least that long anyway, for as many items in an eighth of the memory.  (The bound counts: a
+// captured batch of 18 queries on 1e5 edges has one of 2.1e6, and at 256 took 275 instead of
+// 234 us.)
+__host__ __device__ inline int item_grain_log(int64_t n_max) { return n_max <= (int64_t)1 << 22 ? 5 : 8; }
+__host__ __device__ inline int item_grain(int64_t n_max) { return 1 << item_grain_log(n_max); }
+inline size_t item_starts(size_t n_max) { return n_max <= (size_t)1 << 22 ? 2 * n_max + 2 : n_max / 4 + 2; }
 constexpr int64_t kOnePassTiles = 1024;
 size_t scan_once_words(int64_t n_max);
 int scan_lengths(const int32_t* in, int64_t* out, int64_t n_max, const int64_t* d_n, int64_t* d_total,
