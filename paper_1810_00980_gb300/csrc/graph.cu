@@ -157,6 +157,7 @@ __device__ __forceinline__ void pair_insert(unsigned long long* slots, uint32_t 
         }
         x = (x + 1) & mask;
     }
+    TM_CHK(false, kChkRange);   // no empty slot
 }
 
 // every pair into a table of one part (emptied before)
@@ -204,7 +205,7 @@ __global__ void __launch_bounds__(kThreads) k_pair_split(PairBuckets B, uint32_t
 #pragma unroll
     for (int u = 0; u < kSplitItems; u++) {
         if (u * kThreads + threadIdx.x < tn) {
-            part[u] = pair_part(sm64_mix(rec[u].x), parts) - b * sub;
+            part[u] = (uint32_t)TM_CHK_IDX(pair_part(sm64_mix(rec[u].x), parts) - b * sub, sub, kChkRange);
             rank[u] = atomicAdd(&s_cnt[part[u]], 1u);
         }
     }
@@ -238,7 +239,7 @@ __global__ void __launch_bounds__(kThreads) k_pair_split(PairBuckets B, uint32_t
     __syncthreads();
     for (uint32_t y = threadIdx.x; y < tn; y += kThreads) {
         const ulonglong2 e = s_rec[y];
-        const uint32_t q = pair_part(sm64_mix(e.x), parts) - b * sub, at = s_at[q] + y;
+        const uint32_t q = (uint32_t)TM_CHK_IDX(pair_part(sm64_mix(e.x), parts) - b * sub, sub, kChkRange), at = s_at[q] + y;
         if (at < (uint32_t)kPartSlots) slots[(size_t)(b * sub + q) * kPartSlots + at] = e;
         else *B.full = 1;
     }
@@ -285,7 +286,7 @@ constexpr int kPairTile = kThreads * kPairItems;
 constexpr int kPairWords = kPairTile / 32;
 template <bool BUCKETS>
 __global__ void __launch_bounds__(kThreads) k_pairs(const uint32_t* __restrict__ src, const int32_t* __restrict__ dst,
-                        const int64_t* __restrict__ out_off, int64_t m, int32_t* __restrict__ pair_beg,
+                        const int64_t* __restrict__ out_off, int64_t m, int32_t n, int32_t* __restrict__ pair_beg,
                         int32_t* __restrict__ pair_end, PairBuckets B, uint32_t* __restrict__ filt, unsigned long long fmask, unsigned long long* __restrict__ P) {
     __shared__ uint32_t s_head[kPairWords];
     __shared__ int s_prev[kPairWords], s_next[kPairWords];   // last start before the word, first after it
@@ -311,11 +312,11 @@ __global__ void __launch_bounds__(kThreads) k_pairs(const uint32_t* __restrict__
         ls = src[base - 1];
         ld = dst[base - 1];
     }
-    if (threadIdx.x == 0) s_beg = (int32_t)lower_bound_i32(dst, out_off[s[0]], tbase, d[0]);
+    if (threadIdx.x == 0) s_beg = (int32_t)lower_bound_i32(dst, out_off[TM_CHK_IDX(s[0], n, kChkNode)], tbase, d[0]);
     if (threadIdx.x == 32) {
         const int64_t last = min(m, tbase + kPairTile) - 1;
         const int32_t dl = dst[last];
-        int64_t lo = last + 1, hi = out_off[src[last] + 1];
+        int64_t lo = last + 1, hi = out_off[TM_CHK_IDX(src[last], n, kChkNode) + 1];
         while (lo < hi) {
             const int64_t mid = lo + ((hi - lo) >> 1);
             if (dst[mid] <= dl) lo = mid + 1; else hi = mid;
@@ -383,7 +384,9 @@ __global__ void __launch_bounds__(kThreads) k_pairs(const uint32_t* __restrict__
         const int pb = le ? 32 * k + 31 - __clz(le) : s_prev[k];
         const int pe = gt ? 32 * k + __ffs(gt) - 1 : s_next[k];
         const int32_t end = pe < kPairTile ? (int32_t)(tbase + pe) : s_end;
-        pair_beg[i] = pb >= 0 ? (int32_t)(tbase + pb) : s_beg;
+        const int32_t beg = pb >= 0 ? (int32_t)(tbase + pb) : s_beg;
+        TM_CHK(beg >= 0 && beg <= i && i < end && end <= m, kChkRange);
+        pair_beg[i] = beg;
         pair_end[i] = end;
         if ((h >> lane) & 1u) {
             const unsigned long long key = pair_key((int32_t)s[r], d[r]), hash = sm64_mix(key);
@@ -679,9 +682,9 @@ int build_graph(const int32_t* d_src, const int32_t* d_dst, const int64_t* d_t, 
     if (rc == TM_OK) {
         const unsigned gp = (unsigned)((m + kPairTile - 1) / kPairTile);
         if (parted)
-            k_pairs<true><<<gp, kThreads, 0, st>>>((const uint32_t*)out_src, pair_dst, out_off, m, pair_beg, pair_end, B, filt, fw - 1, dP);
+            k_pairs<true><<<gp, kThreads, 0, st>>>((const uint32_t*)out_src, pair_dst, out_off, m, n, pair_beg, pair_end, B, filt, fw - 1, dP);
         else
-            k_pairs<false><<<gp, kThreads, 0, st>>>((const uint32_t*)out_src, pair_dst, out_off, m, pair_beg, pair_end, B, filt, fw - 1, dP);
+            k_pairs<false><<<gp, kThreads, 0, st>>>((const uint32_t*)out_src, pair_dst, out_off, m, n, pair_beg, pair_end, B, filt, fw - 1, dP);
         launched();
     }
     uint32_t h[24];   // error word, flags, pair count, list-full mark

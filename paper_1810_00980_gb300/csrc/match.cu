@@ -1242,8 +1242,9 @@ __global__ void __launch_bounds__(256, OCC) k_match(MatchArgs<TT> A) {
         if (ce < A.nchunkf) {
             // first edges of this chunk's first item and of the next chunk's (a bound on
             // the last item's: first edges in between have no items below c1)
-            fb = __ldg(A.chunkf + ci);
-            fe = __ldg(A.chunkf + ce);
+            fb = TM_CHK_IDX(__ldg(A.chunkf + ci), F, kChkQueue);
+            fe = TM_CHK_IDX(__ldg(A.chunkf + ce), F, kChkQueue);
+            TM_CHK(fb <= fe && A.excl[fb] <= c0, kChkQueue);
         } else {
             if (lane < 2) {
                 int64_t key = lane == 0 ? c0 : c1 - 1;

@@ -116,13 +116,13 @@ __device__ __forceinline__ void note_items(BigRanges& B, int64_t* cf, int64_t nc
             return;
         }
     }
-    for (int64_t i = (from + grain - 1) / grain; i * grain < from + len && i < ncf; i++) cf[i] = e;
+    for (int64_t i = (from + grain - 1) / grain; i * grain < from + len && i < ncf; i++) cf[TM_CHK_IDX(i, ncf, kChkSort)] = e;
 }
 __device__ __forceinline__ void note_big(const BigRanges& B, int64_t* cf, int64_t ncf, int grain) {
     for (int k = 0; k < min(B.n, 32); k++)
         for (int64_t i = (B.from[k] + grain - 1) / grain + threadIdx.x;
              i * grain < B.from[k] + B.len[k] && i < ncf; i += blockDim.x)
-            cf[i] = B.e[k];
+            cf[TM_CHK_IDX(i, ncf, kChkSort)] = B.e[k];
 }
 
 // ... then each tile's exclusive scan plus the tile's offset; the tile passes through shared
@@ -155,7 +155,7 @@ __global__ void k_len_scan(const int32_t* __restrict__ in, int64_t* __restrict__
     int64_t run = block_excl_scan(loc, smem, &total) + offs[blockIdx.x];
     if (threadIdx.x == 0 && t0 + kScanTile >= n) {
         const int64_t end = (run + total + grain - 1) / grain;
-        if (end < ncf) cf[end] = n - 1;
+        if (end < ncf) cf[TM_CHK_IDX(end, ncf, kChkSort)] = n - 1;
     }
 #pragma unroll
     for (int i = 0; i < kScanItems; i++) {
@@ -287,7 +287,7 @@ __global__ void __launch_bounds__(kOneThreads) k_scan_once(const TI* __restrict_
                 *d_total = before + total;
                 if (CF) {
                     const int64_t end = (before + total + grain - 1) / grain;
-                    if (end < ncf) cf[end] = n - 1;
+                    if (end < ncf) cf[TM_CHK_IDX(end, ncf, kChkSort)] = n - 1;
                 }
             }
         }
