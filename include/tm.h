@@ -351,9 +351,14 @@ int tm_profile_last(tm_profile* out);
  *   tm_check_selftest runs one deliberately out-of-range index (one past a one-element
  *                     device array) through the check, which reads element 0 and sets
  *                     bit 64, so that a test can see the mechanism work.
- * In the ordinary build both return TM_EINVAL (*word = 0). */
+ *   tm_check_expire   the nth launch from now (0: none) of a kernel whose tiles wait for earlier
+ *                     ones runs without its first tile and with a short limit, so that the wait
+ *                     expires and the call ends with TM_ECUDA; *left = launches that were still
+ *                     to come of the last one asked for (0: it has happened).
+ * In the ordinary build all return TM_EINVAL (*word = *left = 0). */
 int tm_check_status(uint32_t* word, int32_t clear);
 int tm_check_selftest(void);
+int tm_check_expire(int32_t nth, int32_t* left);
 
 /* ---- serving -----------------------------------------------------------------
  * A server keeps graphs resident, accepts queries from any thread, and runs

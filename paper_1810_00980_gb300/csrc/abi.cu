@@ -337,6 +337,18 @@ int tm_check_status(uint32_t* word, int32_t clear) {
 
 int tm_check_selftest(void) { return check_selftest(); }
 
+int tm_check_expire(int32_t nth, int32_t* left) {
+    if (!left || nth < 0) { set_error("bad argument"); return TM_EINVAL; }
+    *left = 0;
+#ifndef TM_CHECKED
+    set_error("bounds checks are not compiled into this build");
+    return TM_EINVAL;
+#else
+    *left = check_expire(nth);
+    return TM_OK;
+#endif
+}
+
 int tm_profile_enable(int32_t on) {
     g_prof_on.store(on != 0);
     return TM_OK;

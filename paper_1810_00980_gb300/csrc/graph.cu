@@ -107,11 +107,11 @@ __global__ void __launch_bounds__(kIngestThreads) k_ingest(const int32_t* __rest
 // view's, row 1 the in view's.  Four keys per thread and load (one at a time, a thread waited out
 // a memory latency per key: 38 us for 80 MB).
 __global__ void k_offsets(const uint32_t* __restrict__ out_keys, const uint32_t* __restrict__ in_keys, int64_t m,
-                          int32_t n, int64_t* __restrict__ out_off, int64_t* __restrict__ in_off) {
+                          int32_t n, int64_t* __restrict__ out_off, int64_t* __restrict__ in_off, const uint32_t* err) {
     const uint32_t* keys = blockIdx.y ? in_keys : out_keys;
     int64_t* off = blockIdx.y ? in_off : out_off;
     const int64_t i0 = 4 * (blockIdx.x * (int64_t)blockDim.x + threadIdx.x);
-    if (i0 > m) return;
+    if (i0 > m || gave_up(err)) return;
     uint32_t k[4];
     if (i0 + 4 <= m) {
         const uint4 q = *reinterpret_cast<const uint4*>(keys + i0);   // the arrays start on 256 bytes
@@ -163,7 +163,8 @@ __device__ __forceinline__ void pair_insert(unsigned long long* slots, uint32_t 
 // every pair into a table of one part (emptied before)
 __global__ void k_pair_insert(const int32_t* __restrict__ src, const int32_t* __restrict__ dst, const int32_t* __restrict__ pair_beg,
                               const int32_t* __restrict__ pair_end, int64_t m, unsigned long long* __restrict__ slots,
-                              uint32_t mask) {
+                              uint32_t mask, const uint32_t* err) {
+    if (gave_up(err)) return;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x)
         if (pair_beg[i] == (int32_t)i) pair_insert(slots, mask, pair_slot_value(src[i], dst[i], i, pair_end[i]));
 }
@@ -287,11 +288,12 @@ constexpr int kPairWords = kPairTile / 32;
 template <bool BUCKETS>
 __global__ void __launch_bounds__(kThreads) k_pairs(const uint32_t* __restrict__ src, const int32_t* __restrict__ dst,
                         const int64_t* __restrict__ out_off, int64_t m, int32_t n, int32_t* __restrict__ pair_beg,
-                        int32_t* __restrict__ pair_end, PairBuckets B, uint32_t* __restrict__ filt, unsigned long long fmask, unsigned long long* __restrict__ P) {
+                        int32_t* __restrict__ pair_end, PairBuckets B, uint32_t* __restrict__ filt, unsigned long long fmask, unsigned long long* __restrict__ P, const uint32_t* err) {
     __shared__ uint32_t s_head[kPairWords];
     __shared__ int s_prev[kPairWords], s_next[kPairWords];   // last start before the word, first after it
     __shared__ int32_t s_beg, s_end;                         // of the segments crossing the tile's borders
     __shared__ uint32_t s_cnt[kBuckets], s_base[kBuckets];   // the tile's records per list, and their place
+    if (gave_up(err)) return;
     if (BUCKETS && threadIdx.x < kBuckets) s_cnt[threadIdx.x] = 0;
     const int64_t tbase = (int64_t)blockIdx.x * kPairTile;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -676,15 +678,15 @@ int build_graph(const int32_t* d_src, const int32_t* d_dst, const int64_t* d_t, 
     if (rc == TM_OK) rc = sort_run(W, &pr, 1, 2, tb, st);
     if (rc == TM_OK) {
         k_offsets<<<dim3((unsigned)((m / 4 + kThreads) / kThreads), 2), kThreads, 0, st>>>(
-            (const uint32_t*)out_src, (const uint32_t*)in_dst, m, n, out_off, in_off);
+            (const uint32_t*)out_src, (const uint32_t*)in_dst, m, n, out_off, in_off, W.err);
         launched();
     }
     if (rc == TM_OK) {
         const unsigned gp = (unsigned)((m + kPairTile - 1) / kPairTile);
         if (parted)
-            k_pairs<true><<<gp, kThreads, 0, st>>>((const uint32_t*)out_src, pair_dst, out_off, m, n, pair_beg, pair_end, B, filt, fw - 1, dP);
+            k_pairs<true><<<gp, kThreads, 0, st>>>((const uint32_t*)out_src, pair_dst, out_off, m, n, pair_beg, pair_end, B, filt, fw - 1, dP, W.err);
         else
-            k_pairs<false><<<gp, kThreads, 0, st>>>((const uint32_t*)out_src, pair_dst, out_off, m, n, pair_beg, pair_end, B, filt, fw - 1, dP);
+            k_pairs<false><<<gp, kThreads, 0, st>>>((const uint32_t*)out_src, pair_dst, out_off, m, n, pair_beg, pair_end, B, filt, fw - 1, dP, W.err);
         launched();
     }
     uint32_t h[24];   // error word, flags, pair count, list-full mark
@@ -701,7 +703,7 @@ int build_graph(const int32_t* d_src, const int32_t* d_dst, const int64_t* d_t, 
         G.hslots = (const unsigned long long*)table;
         G.hparts = 1;
         G.hmask = (uint32_t)(slots - 1);
-        k_pair_insert<<<grid_for(m, 32), kThreads, 0, st>>>(out_src, pair_dst, pair_beg, pair_end, m, (unsigned long long*)table, G.hmask);
+        k_pair_insert<<<grid_for(m, 32), kThreads, 0, st>>>(out_src, pair_dst, pair_beg, pair_end, m, (unsigned long long*)table, G.hmask, W.err);
         launched();
     };
     if (rc == TM_OK && !parted) insert_all(g->hash_block, cap);

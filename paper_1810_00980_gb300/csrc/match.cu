@@ -47,6 +47,7 @@ std::atomic<int64_t>& ride_capacity() {
 namespace {
 
 constexpr int64_t kInf = INT64_MAX;
+constexpr const char* kExpired = "batch: a wait for an earlier tile expired";
 constexpr int64_t kWtabMax = (int64_t)1 << 22;   // largest delta+1 given a weight table
 constexpr double kFullScanP = 0.25;              // keep rate from which windows enumerate by node
 constexpr int64_t kRevMinLen = 8;                // shortest second-edge range worth closing from the other side
@@ -114,6 +115,7 @@ struct MatchArgs {
     const int64_t* hs_a;   // [F] closing pair range start (queries whose last edge is fixed by the first)
     const int64_t* hs_hi;  // [F] closing pair range end
     const int64_t* d_W2;   // total second-edge candidates
+    const uint32_t* err;   // see gave_up
     unsigned long long* counter;
     int64_t chunk;
     int enum_threshold;
@@ -668,7 +670,8 @@ __global__ void k_wtab(const QPlan* __restrict__ plans, const int32_t* __restric
 // offsets and number too, instead of by a scan of their own)
 template <typename TT>
 __global__ void k_windows(GraphDevT<TT> G, const QPlan* __restrict__ plans, int nq, WinDev W, int64_t NW,
-                          int64_t* __restrict__ dF) {
+                          int64_t* __restrict__ dF, const uint32_t* err) {
+    if (gave_up(err)) return;   // (the partition by windows may be missing)
     for (int64_t w = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; w < NW;
          w += (int64_t)gridDim.x * blockDim.x) {
         int lo_q = 0, hi_q = nq;
@@ -735,13 +738,14 @@ __global__ void k_windows(GraphDevT<TT> G, const QPlan* __restrict__ plans, int 
     if (threadIdx.x == NW - 1) *dF = before + inc;
 }
 
-// windows of a batch, and the scan of their first edges' numbers (words: scan_once_words(NW))
+// windows of a batch, and the scan of their first edges' numbers (words: scan_once_words(NW));
+// sorted: some plan's windows come from a partition of a view (k_woff)
 template <typename TT>
 int launch_windows(const GraphDevT<TT>& G, const QPlan* dplans, int nq, const WinDev& W, int64_t NW, int64_t* dF,
-                   unsigned long long* words, uint32_t* err, int nsm, cudaStream_t st) {
+                   unsigned long long* words, uint32_t* err, bool sorted, int nsm, cudaStream_t st) {
     const bool one = NW <= kWindowThreads;
     const unsigned gr = (unsigned)std::min<int64_t>((NW + kWindowThreads - 1) / kWindowThreads, (int64_t)nsm * 16);
-    k_windows<TT><<<gr, kWindowThreads, 0, st>>>(G, dplans, nq, W, NW, one ? dF : nullptr); count_launch();
+    k_windows<TT><<<gr, kWindowThreads, 0, st>>>(G, dplans, nq, W, NW, one ? dF : nullptr, sorted ? err : nullptr); count_launch();
     TM_CUDA(cudaGetLastError());
     return one ? TM_OK : scan_once_i64(W.nfirst, W.fbase, NW, dF, words, err, st);
 }
@@ -757,7 +761,9 @@ __global__ void k_winkey(const TT* __restrict__ tv, int64_t m, int64_t s, int64_
     }
 }
 
-__global__ void k_woff(const uint32_t* __restrict__ keys, int64_t m, int64_t nkeys, int64_t* __restrict__ off) {
+__global__ void k_woff(const uint32_t* __restrict__ keys, int64_t m, int64_t nkeys, int64_t* __restrict__ off,
+                       const uint32_t* err) {
+    if (gave_up(err)) return;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i <= m;
          i += (int64_t)gridDim.x * blockDim.x) {
         int64_t prev = i == 0 ? -1 : (int64_t)keys[i - 1];
@@ -780,9 +786,10 @@ __device__ __forceinline__ int64_t first_thi(const QPlan& Q, const WinDev& W, in
 // window of first edge 32 b for every block b of 32 first edges: one search each,
 // run at full occupancy instead of on the critical path of k_level2's warps
 __global__ void k_blockwin(const int64_t* __restrict__ fbase, int64_t NW, int64_t Fh,
-                           const int64_t* __restrict__ d_F, int32_t* __restrict__ bw) {
+                           const int64_t* __restrict__ d_F, int32_t* __restrict__ bw, const uint32_t* err) {
     grid_wait();
     const int64_t F = d_F ? *d_F : Fh;
+    if (gave_up(err)) return;
     int64_t nb = (F + 31) >> 5;
     for (int64_t b = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; b < nb;
          b += (int64_t)gridDim.x * blockDim.x) {
@@ -811,6 +818,7 @@ __global__ void __launch_bounds__(256, 8) k_level2(MatchArgs<TT> A, FRec<TT>* __
     acc_zero(acc);
     grid_wait();
     const int64_t F = A.d_F ? *A.d_F : A.F;
+    if (gave_up(A.err)) return;
     for (int64_t base = warp * 32; base < F; base += nwarps * 32) {
         int64_t f = base + lane;
         bool valid = f < F;
@@ -1227,6 +1235,7 @@ __global__ void __launch_bounds__(256, OCC) k_match(MatchArgs<TT> A) {
     grid_wait();
     int64_t W2 = *A.d_W2;
     const int64_t F = A.d_F ? *A.d_F : A.F;
+    if (gave_up(A.err)) return;
     // few items: smaller chunks, so that every warp gets some (17,000 items in chunks of 256 kept 67
     // warps busy for eight rounds each: 43 us of a 20,000-edge count)
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -2291,13 +2300,13 @@ int run_batch_t(const tm_graph* g, const tm_query* qs, int nq, tm_result* res, c
             if (rc == TM_OK) rc = radix_sort_pairs(pk_key, vals, pk_ktmp, pk_vtmp, g->m, bits, dserr, st);
             if (rc == TM_OK) {
                 k_woff<<<(unsigned)std::min<int64_t>((g->m + 256) / 256, (int64_t)nsm * 8), 256, 0, st>>>(
-                    pk_key, g->m, P.J, (int64_t*)(P.woff + (size_t)k * (size_t)(P.J + 1)));
+                    pk_key, g->m, P.J, (int64_t*)(P.woff + (size_t)k * (size_t)(P.J + 1)), dserr);
                 count_launch();
                 fail(cudaGetLastError(), "k_woff");
             }
         }
     }
-    if (rc == TM_OK && NW > 0) rc = launch_windows<TT>(G, dplans, nq, W, NW, dF, words_w, dserr, nsm, st);
+    if (rc == TM_OK && NW > 0) rc = launch_windows<TT>(G, dplans, nq, W, NW, dF, words_w, dserr, any_full, nsm, st);
     // The per-first-edge scratch is sized for the bound on F when that fits in
     // kBoundScratchBytes, and the kernels read F on the device: no host round trip
     // between the window partition and the matcher.  Otherwise F is read back first.
@@ -2307,7 +2316,12 @@ int run_batch_t(const tm_graph* g, const tm_query* qs, int nq, tm_result* res, c
     nv.next("tm_sizing");
     if (rc == TM_OK && !bounded) {
         fail(cudaMemcpyAsync(&F, dF, 8, cudaMemcpyDeviceToHost, st), "F readback");
+        fail(cudaMemcpyAsync(&h_serr, dserr, 4, cudaMemcpyDeviceToHost, st), "error word");
         fail(cudaStreamSynchronize(st), "sync F");
+        if (rc == TM_OK && h_serr) {   // F is not known
+            set_error(kExpired);
+            rc = TM_ECUDA;
+        }
     }
     const int64_t Fa = bounded ? F_ub : F;   // first edges the scratch holds
     ScratchLease fb;
@@ -2330,7 +2344,7 @@ int run_batch_t(const tm_graph* g, const tm_query* qs, int nq, tm_result* res, c
             const int64_t* d_Fk = bounded ? dF : nullptr;
             A.G = G; A.plans = dplans; A.nq = nq; A.W = W; A.NW = NW; A.F = Fa; A.d_F = d_Fk;
             A.rec = rec; A.excl = excl; A.hs_a = hs_a; A.hs_hi = hs_hi;
-            A.d_W2 = dW2; A.counter = dctr;
+            A.d_W2 = dW2; A.err = dserr; A.counter = dctr;
             A.enum_threshold = tu.enum_threshold;
             A.chunk = tu.chunk_items;
             A.blockwin = bwin; A.chunkf = cf; A.nchunkf = (int64_t)ncf; A.grain_log = item_grain_log(Fa);
@@ -2340,7 +2354,7 @@ int run_batch_t(const tm_graph* g, const tm_query* qs, int nq, tm_result* res, c
             int64_t gl2 = std::min<int64_t>((Fa + 255) / 256, (int64_t)nsm * 8);
             if (NW > 1) {   // (one window: nothing to search)
                 launch_after(k_blockwin, dim3((unsigned)std::min<int64_t>(((int64_t)nbw + 255) / 256, (int64_t)nsm * 8)), 256, 0, st,
-                             W.fbase, NW, Fa, d_Fk, bwin);
+                             W.fbase, NW, Fa, d_Fk, bwin, dserr);
                 count_launch();
             } else {
                 A.blockwin = nullptr;
@@ -2424,7 +2438,7 @@ int run_batch_t(const tm_graph* g, const tm_query* qs, int nq, tm_result* res, c
         std::memcpy(&h_rcount, h_res.data() + res_bytes, 8);
         std::memcpy(&h_serr, h_res.data() + res_bytes + 8, 4);
         if (h_serr) {
-            set_error("batch: a wait for an earlier tile expired");
+            set_error(kExpired);
             rc = TM_ECUDA;
         }
     }
@@ -2917,14 +2931,14 @@ int count_exact_noalloc_t(const tm_graph* g, const tm_motif* m, int64_t delta, c
     if (e == cudaSuccess) e = cudaMemsetAsync(words, 0, 8 * (size_t)kNaWsElems / 2, st);
     if (e != cudaSuccess) return na_status(e);
     GraphDevT<TT> G = typed<TT>(g->dev);
-    rc = launch_windows<TT>(G, dplan, 1, W, 1, dF, nullptr, nullptr, sm_count(), st);
+    rc = launch_windows<TT>(G, dplan, 1, W, 1, dF, nullptr, derr, false, sm_count(), st);
     if (rc != TM_OK) return TM_ECUDA;
     int64_t F = g->m;   // one window holding every edge
     if (F > 0) {
         const Tuning tu = tuning();
         MatchArgs<TT> A;
         A.G = G; A.plans = dplan; A.nq = 1; A.W = W; A.NW = 1; A.F = F; A.d_F = nullptr;
-        A.rec = rec; A.excl = excl; A.d_W2 = dW2; A.counter = dctr;
+        A.rec = rec; A.excl = excl; A.d_W2 = dW2; A.err = derr; A.counter = dctr;
         A.hs_a = nullptr; A.hs_hi = nullptr;
         A.enum_threshold = tu.enum_threshold;
         A.chunk = tu.chunk_items;
@@ -3147,10 +3161,10 @@ int batch_create_t(const tm_graph* g, const tm_query* qs, int nq, tm_batch** out
     fail(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal), "begin capture");
     fail(cudaMemsetAsync(derr, 0, (size_t)(zero_end - (char*)derr), st), "accumulators");
     if (rc == TM_OK && NW > 0 && (n_words_w || NW <= kWindowThreads)) {
-        rc = launch_windows<TT>(G, dplans, nq, W, NW, dF, words_w, derr, nsm, st);
+        rc = launch_windows<TT>(G, dplans, nq, W, NW, dF, words_w, derr, false, nsm, st);
     } else if (rc == TM_OK && NW > 0) {   // (a scan too long for one launch, in the batch's own workspace)
         unsigned gr = (unsigned)std::min<int64_t>((NW + 255) / 256, (int64_t)nsm * 16);
-        k_windows<TT><<<gr, kWindowThreads, 0, st>>>(G, dplans, nq, W, NW, nullptr); count_launch();
+        k_windows<TT><<<gr, kWindowThreads, 0, st>>>(G, dplans, nq, W, NW, nullptr, nullptr); count_launch();
         fail(cudaGetLastError(), "k_windows");
         if (rc == TM_OK) rc = scan_exclusive_i64_ws(W.nfirst, W.fbase, NW, dF, wsp1, ws1, st);
     }
@@ -3158,13 +3172,13 @@ int batch_create_t(const tm_graph* g, const tm_query* qs, int nq, tm_batch** out
         MatchArgs<TT> A;
         A.G = G; A.plans = dplans; A.nq = nq; A.W = W; A.NW = NW; A.F = Fmax; A.d_F = dF;
         A.rec = rec; A.excl = excl; A.hs_a = hs_a; A.hs_hi = hs_hi;
-        A.d_W2 = dW2; A.counter = dctr;
+        A.d_W2 = dW2; A.err = derr; A.counter = dctr;
         A.enum_threshold = tu.enum_threshold;
         A.chunk = tu.chunk_items;
         A.blockwin = bwin; A.chunkf = cf; A.nchunkf = (int64_t)ncf; A.grain_log = item_grain_log(Fmax);
         int64_t gl2 = std::min<int64_t>((Fmax + 255) / 256, (int64_t)nsm * 8);
         launch_after(k_blockwin, dim3((unsigned)std::min<int64_t>(((int64_t)nbw + 255) / 256, (int64_t)nsm * 8)), 256, 0, st,
-                     W.fbase, NW, Fmax, dF, bwin);
+                     W.fbase, NW, Fmax, dF, bwin, derr);
         count_launch();
         launch_after(k_level2<TT>, dim3((unsigned)std::max<int64_t>(gl2, 1)), 256, match_smem_bytes(A.nq, 256), st, A, rec, len32, hs_a, hs_hi); count_launch();
         fail(cudaGetLastError(), "k_level2");
@@ -3222,7 +3236,7 @@ int tm_batch_launch(tm_batch* b, void* stream) {
 int tm_batch_results(tm_batch* b, void* stream, tm_result* results) {
     if (!b || !results) { tmo::set_error("bad argument"); return TM_EINVAL; }
     TM_CUDA(cudaStreamSynchronize((cudaStream_t)stream));
-    if (*b->h_err) { tmo::set_error("batch: a wait for an earlier tile expired"); return TM_ECUDA; }
+    if (*b->h_err) { tmo::set_error(tmo::kExpired); return TM_ECUDA; }
     int first = b->first_err;
     for (int i = 0; i < b->nq; i++) {
         results[i] = b->h_res[i];

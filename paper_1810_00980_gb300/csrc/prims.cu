@@ -1,7 +1,9 @@
-// Device primitives: exclusive scan of int64 (reduce-then-scan over tiles: no block waits on
-// another) and a stable LSD radix sort of 32-bit keys with up to 12 bytes of payload (a tile
+// Device primitives: exclusive scans into int64 (reduce-then-scan over tiles, where no block waits
+// on another; up to 1,024 tiles in one launch, where a tile waits, with a limit, for the sums of
+// earlier tiles) and a stable LSD radix sort of 32-bit keys with up to 12 bytes of payload (a tile
 // waits, with a limit, for the counts of earlier tiles).
 #include <algorithm>
+#include <atomic>
 #include <mutex>
 #include <vector>
 
@@ -129,7 +131,7 @@ __device__ __forceinline__ void note_big(const BigRanges& B, int64_t* cf, int64_
 // memory so that both the 32-bit loads and the 64-bit stores are coalesced.  cf: as k_scan_once
 __global__ void k_len_scan(const int32_t* __restrict__ in, int64_t* __restrict__ out, int64_t n_max,
                            const int64_t* __restrict__ d_n, const int64_t* __restrict__ offs,
-                           int64_t* __restrict__ cf, int64_t ncf) {
+                           int64_t* __restrict__ cf, int64_t ncf, const uint32_t* err) {
     __shared__ int64_t smem[33];
     __shared__ int64_t tile[kScanTile + kScanTile / 16];   // one pad word per 16: no bank conflicts
     __shared__ BigRanges big;
@@ -137,7 +139,7 @@ __global__ void k_len_scan(const int32_t* __restrict__ in, int64_t* __restrict__
     if (threadIdx.x == 0) big.n = 0;
     int64_t n = d_n ? min(*d_n, n_max) : n_max;
     int64_t t0 = (int64_t)blockIdx.x * kScanTile;
-    if (t0 >= n) return;
+    if (t0 >= n || gave_up(err)) return;   // (the lengths may be missing)
     for (int i = threadIdx.x; i < kScanTile; i += blockDim.x) {
         int64_t idx = t0 + i;
         tile[i + (i >> 4)] = idx < n ? (int64_t)in[idx] : 0;
@@ -228,7 +230,7 @@ __device__ __forceinline__ void st_tile64(unsigned long long* p, unsigned long l
 template <typename TI, bool CF>
 __global__ void __launch_bounds__(kOneThreads) k_scan_once(const TI* __restrict__ in, int64_t* __restrict__ out, int64_t n_max,
                             const int64_t* __restrict__ d_n, int64_t* __restrict__ d_total, unsigned long long* words,
-                            uint32_t* err, int64_t* __restrict__ cf, int64_t ncf) {
+                            uint32_t* err, int limit, int64_t* __restrict__ cf, int64_t ncf) {
     __shared__ int64_t smem[33];
     __shared__ int64_t tile[kOneTile + kOneTile / 16];   // one pad word per 16: no bank conflicts
     __shared__ int64_t s_before;
@@ -238,7 +240,11 @@ __global__ void __launch_bounds__(kOneThreads) k_scan_once(const TI* __restrict_
     if (CF && threadIdx.x == 0) big.n = 0;
     grid_wait();
     const int64_t n = d_n ? min(*d_n, n_max) : n_max;
-    if (threadIdx.x == 0) s_tile = gridDim.x == 1 ? 0u : (uint32_t)atomicAdd(words, 1ull);
+    // (nothing to scan, and no tile, after an expired wait: the total stays at zero)
+    if (threadIdx.x == 0) {
+        const uint32_t ticket = gridDim.x == 1 ? 0u : (uint32_t)atomicAdd(words, 1ull);
+        s_tile = gave_up(err) ? 0xffffffffu : ticket;
+    }
     __syncthreads();
     const int64_t t = s_tile, t0 = t * kOneTile;
     words += 8;
@@ -260,6 +266,7 @@ __global__ void __launch_bounds__(kOneThreads) k_scan_once(const TI* __restrict_
     if (threadIdx.x < 32) {
         const int lane = threadIdx.x;
         int64_t before = 0;
+        bool lost = false;
         if (t > 0) {
             if (lane == 0) st_tile64(words + t, (1ull << 62) | (unsigned long long)total);
             int64_t at = t - 1;
@@ -274,13 +281,20 @@ __global__ void __launch_bounds__(kOneThreads) k_scan_once(const TI* __restrict_
                 before += x;
                 if (first_pre < first_gap) break;
                 at -= first_gap;
-                if (first_gap == 0 && ++spins > kSpinLimit) {
+                if (first_gap > 0) {
+                    spins = 0;
+                } else if (++spins > limit) {
                     if (lane == 0) atomicOr(err, 1u);
-                    break;
+                    lost = true;
+                } else if ((spins & 63) == 0) {
+                    lost = __any_sync(kFull, gave_up(err));
                 }
+                if (lost) break;
             }
         }
-        if (lane == 0) {
+        if (lost) {
+            if (lane == 0) s_before = -1;
+        } else if (lane == 0) {
             if (gridDim.x > 1) st_tile64(words + t, (2ull << 62) | (unsigned long long)(before + total));
             s_before = before;
             if (t0 + kOneTile >= n) {
@@ -293,6 +307,7 @@ __global__ void __launch_bounds__(kOneThreads) k_scan_once(const TI* __restrict_
         }
     }
     __syncthreads();
+    if (s_before < 0) return;   // the wait expired
     int64_t run = s_before + off;
 #pragma unroll
     for (int i = 0; i < kOneItems; i++) {
@@ -408,13 +423,16 @@ __global__ void __launch_bounds__(kSortThreads, TB == 8 ? 2 : 3) k_sort_pass(Sor
     __shared__ uint32_t s_tile, red[kSortWarps];
     const SortJob job = (J.jobs == 2 && (blockIdx.x & 1)) ? J.job[1] : J.job[0];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    if (threadIdx.x == 0) s_tile = atomicAdd(job.ticket, 1u);
+    if (threadIdx.x == 0) {
+        const uint32_t ticket = atomicAdd(job.ticket, 1u);
+        s_tile = gave_up(J.err) ? 0xffffffffu : ticket;
+    }
     for (int i = threadIdx.x; i < kSortWarps * ND / 2; i += kSortThreads) ((uint32_t*)cnt)[i] = 0;
     __syncthreads();
     const int64_t tile = s_tile;
     const int64_t tbase = tile * kSortTile;
+    if (tbase >= n) return;   // (also after an expired wait: an earlier pass may have left its lists unwritten)
     const int tn = (int)min((int64_t)kSortTile, n - tbase);
-    if (tn <= 0) return;
     const int wbase = w * (kSortItems * 32) + lane;
     uint32_t key[kSortItems], rank[kSortItems];
 #pragma unroll
@@ -476,19 +494,23 @@ __global__ void __launch_bounds__(kSortThreads, TB == 8 ? 2 : 3) k_sort_pass(Sor
         }
     }
     // each digit's place in the output
+    bool lost = false;
     if (d0 < ND) {
 #pragma unroll
         for (int x = 0; x < PER; x++) {
             uint32_t before = 0;
             if (tile > 0) {
-                before = look_back(job.words + d0 + x, tile, ND, J.err);
+                if (!look_back(job.words + d0 + x, tile, ND, J.err, J.limit, before)) {
+                    lost = true;
+                    break;
+                }
                 st_tile(words + d0 + x, kTilePrefix | (before + tot[x]));
             }
             gbase[d0 + x] = job.base[d0 + x] + before - tds[d0 + x];
         }
     }
     asm volatile("cp.async.wait_all;" ::: "memory");
-    __syncthreads();
+    if (__syncthreads_or(lost)) return;   // a place is not known: the tile stays unwritten
     for (int i = threadIdx.x; i < tn; i += kSortThreads) {
         const uint32_t k = sk[i], o = slot[i];
         const int64_t pos = TM_CHK_IDX((int64_t)(uint32_t)(gbase[(k >> shift) & (ND - 1)] + (uint32_t)i), n, kChkSort);
@@ -527,8 +549,22 @@ __global__ void __launch_bounds__(kSortThreads) k_digit_base(uint32_t* __restric
         }
 }
 
+// Polls after which a wait of the next launch expires; `ticket` numbers its tiles, zeroed before.
+// The checked build can be told to leave tile 0 of a launch of several to nobody (check_expire): the
+// tickets then start at one, the block with the last one finds no tile, and the others wait for a
+// word that never comes.
+#ifdef TM_CHECKED
+std::atomic<int> g_expire{0};
+int wait_limit(void* ticket, int64_t tiles, cudaStream_t st) {
+    if (tiles < 2 || g_expire.load() <= 0 || g_expire.fetch_sub(1) != 1) return kSpinLimit;
+    return cudaMemsetAsync(ticket, 1, 1, st) == cudaSuccess ? 1 << 10 : kSpinLimit;
+}
+#else
+int wait_limit(void*, int64_t, cudaStream_t) { return kSpinLimit; }
+#endif
+
 template <int TB, int DB>
-int sort_pass(const SortJobs& J, int64_t n, int shift, cudaStream_t st) {
+int sort_pass(SortJobs& J, int64_t n, int shift, cudaStream_t st) {
     {
         // the tile's shared memory exceeds the 48 KB default: allowed once per device
         static std::mutex mu;
@@ -542,7 +578,8 @@ int sort_pass(const SortJobs& J, int64_t n, int shift, cudaStream_t st) {
             if (dev >= 0 && dev < 64) done[dev] = true;
         }
     }
-    const int64_t blocks = J.jobs * ((n + kSortTile - 1) / kSortTile);
+    const int64_t tiles = (n + kSortTile - 1) / kSortTile, blocks = J.jobs * tiles;
+    J.limit = wait_limit(J.job[0].ticket, tiles, st);
     k_sort_pass<TB, DB><<<(unsigned)blocks, kSortThreads, sort_smem_bytes<TB, DB>(), st>>>(J, n, shift);
     count_launch();
     TM_CUDA(cudaGetLastError());
@@ -550,7 +587,7 @@ int sort_pass(const SortJobs& J, int64_t n, int shift, cudaStream_t st) {
 }
 
 template <int TB>
-int sort_pass_db(const SortJobs& J, int64_t n, int shift, int db, cudaStream_t st) {
+int sort_pass_db(SortJobs& J, int64_t n, int shift, int db, cudaStream_t st) {
     switch (db) {
         case 5: return sort_pass<TB, 5>(J, n, shift, st);
         case 6: return sort_pass<TB, 6>(J, n, shift, st);
@@ -562,6 +599,10 @@ int sort_pass_db(const SortJobs& J, int64_t n, int shift, int db, cudaStream_t s
 }
 
 }  // namespace
+
+#ifdef TM_CHECKED
+int check_expire(int nth) { return g_expire.exchange(nth); }
+#endif
 
 int scan_exclusive_i64(const int64_t* in, int64_t* out, int64_t n, int64_t* d_total,
                        cudaStream_t st) {
@@ -629,9 +670,11 @@ int scan_lengths(const int32_t* in, int64_t* out, int64_t n_max, const int64_t* 
         return TM_OK;
     }
     if (scan_once_words(n_max)) {
+        const int64_t tiles = (n_max + kOneTile - 1) / kOneTile;
+        const int limit = wait_limit(words, tiles, st);
         count_launch();
-        TM_CUDA(launch_after(k_scan_once<int32_t, true>, dim3((unsigned)((n_max + kOneTile - 1) / kOneTile)), kOneThreads, 0, st,
-                             in, out, n_max, d_n, d_total, words, err, cf, ncf));
+        TM_CUDA(launch_after(k_scan_once<int32_t, true>, dim3((unsigned)tiles), kOneThreads, 0, st,
+                             in, out, n_max, d_n, d_total, words, err, limit, cf, ncf));
         return TM_OK;
     }
     int64_t ntiles = (n_max + kScanTile - 1) / kScanTile;
@@ -651,7 +694,7 @@ int scan_lengths(const int32_t* in, int64_t* out, int64_t n_max, const int64_t* 
         if (cudaGetLastError() != cudaSuccess) rc = TM_ECUDA;
         if (rc == TM_OK) rc = scan_exclusive_i64_ws(sums, soffs, ntiles, d_total, ws + 2 * ntiles, need - 2 * ntiles, st);
         if (rc == TM_OK) {
-            k_len_scan<<<(unsigned)ntiles, kScanThreads, 0, st>>>(in, out, n_max, d_n, soffs, cf, ncf); count_launch();
+            k_len_scan<<<(unsigned)ntiles, kScanThreads, 0, st>>>(in, out, n_max, d_n, soffs, cf, ncf, err); count_launch();
             if (cudaGetLastError() != cudaSuccess) rc = TM_ECUDA;
         }
     }
@@ -674,9 +717,11 @@ size_t scan_once_words(int64_t n_max) {
 int scan_once_i64(const int64_t* in, int64_t* out, int64_t n, int64_t* d_total, unsigned long long* words, uint32_t* err,
                   cudaStream_t st) {
     if (!scan_once_words(n)) return scan_exclusive_i64(in, out, n, d_total, st);
+    const int64_t tiles = (n + kOneTile - 1) / kOneTile;
+    const int limit = wait_limit(words, tiles, st);
     count_launch();
-    TM_CUDA(launch_after(k_scan_once<int64_t, false>, dim3((unsigned)((n + kOneTile - 1) / kOneTile)), kOneThreads, 0, st,
-                         in, out, n, nullptr, d_total, words, err, nullptr, 0));
+    TM_CUDA(launch_after(k_scan_once<int64_t, false>, dim3((unsigned)tiles), kOneThreads, 0, st,
+                         in, out, n, nullptr, d_total, words, err, limit, nullptr, 0));
     return TM_OK;
 }
 

@@ -66,6 +66,11 @@ int check_word_match(unsigned* w, bool clear);
 int check_word_graph(unsigned* w, bool clear);
 int check_word_prims(unsigned* w, bool clear);
 int check_selftest();
+#ifdef TM_CHECKED
+// tm_check_expire: the nth launch from now of a kernel that waits between tiles runs without its first
+// tile (nobody gets that ticket) and with few polls
+int check_expire(int nth);   // returns what was left of the last one (0: it has happened)
+#endif
 
 // ----------------------------------------------------------------------------
 // error plumbing
@@ -367,7 +372,8 @@ int radix_sort_pairs(uint32_t* keys, uint32_t* vals, uint32_t* keys_tmp, uint32_
 //   sort_bases     counts -> starts of the digits' runs
 //   sort_run       the passes of sorts [first, first + sorts) side by side in one launch per pass
 //                  (SortIo::counts names the counted list with the same keys)
-// Asynchronous; *W.err is non-zero afterwards if a wait between tiles expired.
+// Asynchronous; *W.err is non-zero afterwards if a wait between tiles expired (the lists are then
+// incomplete: gave_up).
 struct SortDigits { int bits, passes, db; };
 struct SortWs {
     SortDigits D;
@@ -400,6 +406,7 @@ constexpr int kMaxSortJobs = 2;
 struct SortJobs {
     SortJob job[kMaxSortJobs];
     int jobs;
+    int limit;   // polls of a wait
     uint32_t* err;
 };
 SortDigits sort_digits(int bits);
@@ -582,15 +589,21 @@ __device__ __forceinline__ void st_tile(uint32_t* p, uint32_t v) {
     asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 
-// Sum of the words of tiles tile-1, tile-2, ... at `stride` apart, back to the first that holds a
+// Whether a wait of this call has expired.  What the waiting kernel should have written is then
+// missing, so every kernel behind it that takes an index, a range or a loop bound from there
+// reads the word first and returns; the host reports it.  (The word is read beside the kernel's
+// other first loads; a kernel that may set it itself lets one thread decide for its block.)
+__device__ __forceinline__ bool gave_up(const uint32_t* err) { return err && ld_tile(err) != 0; }
+
+// sum += the words of tiles tile-1, tile-2, ... at `stride` apart, back to the first that holds a
 // prefix, kLookBack of them read at a time (the reads are a serial chain otherwise: prefixes
 // travel forward at most that many tiles per memory latency).  Tiles are numbered in the order
 // blocks start, so every word waited for belongs to a block that already runs; if one still
-// never comes the error word is set and the sum so far returned (positions stay in range: it is
-// too small, never too large).
+// never comes within `limit` polls the error word is set.  False then, and when another tile has
+// set it: the caller writes nothing more.
 constexpr int kLookBack = 4;
-__device__ __forceinline__ uint32_t look_back(const uint32_t* words, int64_t tile, int64_t stride, uint32_t* err) {
-    uint32_t sum = 0;
+__device__ __forceinline__ bool look_back(const uint32_t* words, int64_t tile, int64_t stride, uint32_t* err, int limit,
+                                          uint32_t& sum) {
     int64_t at = tile - 1;
     int spins = 0;
     while (at >= 0) {
@@ -601,7 +614,10 @@ __device__ __forceinline__ uint32_t look_back(const uint32_t* words, int64_t til
 #pragma unroll
         for (int i = 0; i < kLookBack; i++) {
             if (open) {
-                if (v[i] & kTilePrefix) return sum + (v[i] & ~kTilePrefix);
+                if (v[i] & kTilePrefix) {
+                    sum += v[i] & ~kTilePrefix;
+                    return true;
+                }
                 open = v[i] != 0;
                 if (open) {
                     sum += v[i] - 1;
@@ -609,12 +625,17 @@ __device__ __forceinline__ uint32_t look_back(const uint32_t* words, int64_t til
                 }
             }
         }
-        if (v[0] == 0 && ++spins > kSpinLimit) {
-            atomicOr(err, 1u);
-            return sum;
+        if (v[0] == 0) {
+            if (++spins > limit) {
+                atomicOr(err, 1u);
+                return false;
+            }
+            if ((spins & 63) == 0 && gave_up(err)) return false;
+        } else {
+            spins = 0;
         }
     }
-    return sum;
+    return true;
 }
 
 // upper_bound_i64 on a node's list of times (or the whole graph's): the first probe where v would be if

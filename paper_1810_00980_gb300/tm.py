@@ -112,6 +112,7 @@ _SIGS = {
     "tm_release_cached_memory": (ctypes.c_int, []),
     "tm_check_status": (ctypes.c_int, [_vp, _c_i32]),
     "tm_check_selftest": (ctypes.c_int, []),
+    "tm_check_expire": (ctypes.c_int, [_c_i32, _vp]),
     "tm_serve_create": (ctypes.c_int, [_vp, _vp]),
     "tm_serve_attach_graph": (ctypes.c_int, [_vp, _vp, _vp]),
     "tm_serve_submit": (ctypes.c_int, [_vp, _c_i32, _vp, _vp]),
@@ -149,6 +150,14 @@ def check_status(clear: bool = True) -> int:
 def check_selftest():
     """tm_check_selftest: one deliberately out-of-range index through the checks."""
     _check(lib().tm_check_selftest(), "tm_check_selftest")
+
+
+def check_expire(nth: int) -> int:
+    """tm_check_expire: the nth launch from now that waits between tiles loses its first tile (checked
+    build only); returns what was left of the last one asked for."""
+    left = _c_i32(0)
+    _check(lib().tm_check_expire(int(nth), ctypes.byref(left)), "tm_check_expire")
+    return left.value
 
 
 def _check(status: int, where: str):
