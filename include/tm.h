@@ -283,8 +283,8 @@ void tm_batch_free(tm_batch* b);
  * (tm_autotune) writes these after timing candidates on a graph. */
 typedef struct {
     int32_t block_threads;     /* threads per block of the matcher (multiple of 32) */
-    int32_t blocks_per_sm;     /* persistent blocks per SM (until it is set or found by the
-                                  autotuner, the matcher takes the number that suits its kernel) */
+    int32_t blocks_per_sm;     /* persistent blocks per SM (6 until it is set or found by the
+                                  autotuner) */
     int32_t chunk_items;       /* level-2 items a warp takes per queue grab (multiple of 32) */
     int32_t enum_threshold;    /* last-level ranges longer than this are counted by
                                   subtraction instead of being read entry by entry */

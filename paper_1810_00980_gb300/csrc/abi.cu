@@ -241,10 +241,7 @@ int tm_set_tuning(const tm_tuning* in) {
     std::lock_guard<std::mutex> lk(g_tune_mu);
     Tuning& t = tuning();
     if (in->block_threads) t.block_threads = in->block_threads;
-    if (in->blocks_per_sm) {
-        t.blocks_per_sm = in->blocks_per_sm;
-        t.blocks_set = true;
-    }
+    if (in->blocks_per_sm) t.blocks_per_sm = in->blocks_per_sm;
     if (in->chunk_items) t.chunk_items = in->chunk_items;
     if (in->enum_threshold) t.enum_threshold = in->enum_threshold;
     return TM_OK;
@@ -283,7 +280,6 @@ int tm_autotune(const tm_graph* g, const tm_query* queries, int32_t n_queries, t
                     Tuning t;
                     t.block_threads = bt;
                     t.blocks_per_sm = bps;
-                    t.blocks_set = true;
                     t.chunk_items = ch;
                     t.enum_threshold = thr_matters ? thr_all[ti] : saved.enum_threshold;
                     {

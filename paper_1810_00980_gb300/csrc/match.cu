@@ -1789,8 +1789,10 @@ void launch_match(const MatchArgs<TT>& A, int lmax, int kmax, const Tuning& tu, 
     // beat fewer with more registers and less spilling (k_match, ms, at 6 / 4 / 2 / 1 blocks: the
     // benchmark batch on 1e7 edges 1.35 / 1.56; 192 seeds of the 4-cycle there 3.54 / 4.29 / 5.11 /
     // 9.00; four- and five-edge counts on 1.25e6 edges 1.00 / 1.02 / 1.21 / 2.12, by the deepest
-    // instantiation at 4 / 3 / 2 / 1 blocks 1.17 / 1.27 / 1.53 / 2.17; eight blocks are no better).  A tuning that was set or found picks the one for its blocks per SM.
-    const int bps = tu.blocks_set ? tu.blocks_per_sm : 6, bt = tu.block_threads;
+    // instantiation at 4 / 3 / 2 / 1 blocks 1.17 / 1.27 / 1.53 / 2.17; eight blocks are no better).
+    // Below six blocks per SM three- and four-edge motifs run a variant at 64 registers; five edges,
+    // and four edges with riders, have the one at 40, the deepest motifs the one at 64.
+    const int bps = tu.blocks_per_sm, bt = tu.block_threads;
     const unsigned gm = (unsigned)(nsm * bps);
     const size_t sm = match_smem_bytes(A.nq, bt);
     if (lmax <= 3 && kmax <= 4 && !expand) {

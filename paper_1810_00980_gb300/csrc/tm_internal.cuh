@@ -302,8 +302,7 @@ static_assert(sizeof(QPlan) == 320, "plan stride");
 
 struct Tuning {
     int block_threads = 256;
-    int blocks_per_sm = 4;
-    bool blocks_set = false;   // by tm_set_tuning or tm_autotune (else the matcher chooses)
+    int blocks_per_sm = 6;   // (launch_match gives the times)
     int chunk_items = 256;
     int enum_threshold = 48;
 };
