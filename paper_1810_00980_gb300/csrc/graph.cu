@@ -744,6 +744,7 @@ int build_graph(const int32_t* d_src, const int32_t* d_dst, const int64_t* d_t, 
         while (2 * slots < 3 * P) slots <<= 1;
         pool_free(g->table_block, dev);
         g->table_block = nullptr;
+        g->bytes += 16 * ((int64_t)slots - (int64_t)G.hparts * kPartSlots);
         e = cudaMallocAsync(&g->table_block, 16 * slots, st);
         if (e == cudaSuccess) e = cudaMemsetAsync(g->table_block, 0xff, 16 * slots, st);
         if (e != cudaSuccess) rc = cuda_status(e, "cudaMalloc(pair table)", __FILE__, __LINE__);
