@@ -425,6 +425,7 @@ __global__ void __launch_bounds__(kThreads) k_pairs(const uint32_t* __restrict__
 // (at most 2^22 slots, 64 MB) stays in L2, and one kernel that inserts is quicker than two steps of
 // lists (about 20 us of insertion for 7e5 pairs).
 constexpr int64_t kPartEdges = (int64_t)1 << 21;
+constexpr size_t kSpareBytes = (size_t)4 << 20;   // a table of at most this size stays as it is
 
 int bits_for(int32_t n) {
     int b = 0;
@@ -750,6 +751,29 @@ int build_graph(const int32_t* d_src, const int32_t* d_dst, const int64_t* d_t, 
         if (e != cudaSuccess) rc = cuda_status(e, "cudaMalloc(pair table)", __FILE__, __LINE__);
         if (rc == TM_OK) insert_all(g->table_block, slots);
         if (rc == TM_OK) settle();
+    }
+    // A small graph whose edges repeat few pairs would keep a table sized by its edges (up to 64 MB
+    // where the pairs need kilobytes): beyond kSpareBytes the pairs move to one of their own size.
+    // (Only then: waiting for their number first would cost every small build a round trip.)
+    if (rc == TM_OK && !parted && table_bytes >= kSpareBytes) {
+        uint64_t P = 0, slots = 2;
+        std::memcpy(&P, h + 16, 8);
+        while (2 * slots < 3 * P) slots <<= 1;
+        void* block = nullptr;
+        if (4 * slots <= cap && cudaMallocAsync(&block, 16 * slots + 4 * fw, st) == cudaSuccess) {
+            uint32_t* f = (uint32_t*)((char*)block + 16 * slots);
+            e = cudaMemsetAsync(block, 0xff, 16 * slots, st);
+            if (e == cudaSuccess) e = cudaMemcpyAsync(f, filt, 4 * fw, cudaMemcpyDeviceToDevice, st);
+            if (e != cudaSuccess) rc = cuda_status(e, "pair table", __FILE__, __LINE__);
+            if (rc == TM_OK) insert_all(block, slots);
+            if (rc == TM_OK) settle();
+            else cudaStreamSynchronize(st);
+            std::swap(block, g->hash_block);
+            pool_free(block, dev);
+            G.pfilt = f;
+            g->bytes -= 16 * (int64_t)(cap - slots);
+        }
+        cudaGetLastError();   // no room for a second table: the first stays
     }
     int64_t P = 0;
     if (rc == TM_OK) {

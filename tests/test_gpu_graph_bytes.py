@@ -34,7 +34,7 @@ def _crowd(u, v):
     return np.flatnonzero(((x ^ (x >> np.uint64(31))) >> np.uint64(58)) == 5)
 
 
-@pytest.mark.parametrize("kind", ["inserted", "parts", "crowded"])
+@pytest.mark.parametrize("kind", ["inserted", "parts", "crowded", "few", "few and small"])
 def test_device_bytes_count_the_table_that_is_there(kind):
     import torch
     import __graft_entry__
@@ -42,9 +42,10 @@ def test_device_bytes_count_the_table_that_is_there(kind):
     torch.cuda.set_device(0)
     from paper_1810_00980_gb300 import tm
     rng = np.random.default_rng(8)
-    n, m = 20_000, 100_003 if kind == "inserted" else (1 << 21) + 5
+    n, m = 20_000, {"inserted": 100_003, "few": 1_500_001, "few and small": 50_001}.get(kind, (1 << 21) + 5)
     u, v = rng.integers(0, n, 6_000_000), rng.integers(0, n, 6_000_000)
-    pool = _crowd(u, v) if kind == "crowded" else np.arange(len(u))
+    u[50:100], v[50:100] = v[:50].copy(), u[:50].copy()   # (a few pairs with replies)
+    pool = _crowd(u, v) if kind == "crowded" else np.arange(100 if kind.startswith("few") else len(u))
     pick = pool[rng.integers(0, len(pool), m)]
     src, dst = u[pick].astype(np.int32), v[pick].astype(np.int32)
     t = np.sort(rng.integers(0, 50_000, m)).astype(np.int64)
@@ -52,10 +53,15 @@ def test_device_bytes_count_the_table_that_is_there(kind):
         info = g.info()
         pairs = len(np.unique(src.astype(np.int64) * n + dst))
         assert info.n_pairs == pairs
-        if kind == "inserted":
+        if kind in ("inserted", "few and small"):
             table = 16 * _pow2(m)
-        elif kind == "crowded":
+        elif kind in ("crowded", "few"):   # by the pairs
             table = 16 * _pow2(pairs)
         else:
             table = 64 * -(-pairs // (64 * 1900)) * 4096 * 16
         assert info.device_bytes == _expected(m, n, table), (kind, info.device_bytes)
+        # the table answers: replies within 3 ticks
+        key = np.sort((src.astype(np.int64) * n + dst) * 100_000 + t)
+        rev = ((dst.astype(np.int64) * n + src) * 100_000 + t)[src != dst]
+        want = int((np.searchsorted(key, rev + 3, "right") - np.searchsorted(key, rev, "right")).sum())
+        assert tm.count_exact(g, tm.Motif([0, 1], [1, 0]), 3) == want
