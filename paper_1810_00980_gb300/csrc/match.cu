@@ -2518,10 +2518,48 @@ bool same_motif(const tm_motif* a, const tm_motif* b) {
     return std::memcmp(a->lv, b->lv, sizeof(LevelPlan) * (size_t)a->l) == 0;
 }
 
+// What riding along saves an estimate, in ns per shift (below zero: it stays apart).  Apart, a shift
+// takes p of the graph's edges as first edges, in time order, and what hangs off them; with p = 1
+// all of them in node order.  Riding, k_ride goes over every shift for every record, kept or not
+// (1 us for its chain of loads once there are more than a few dozen, and the records: few per edge
+// unless the first edge fixes the closing pair), for two-node motifs k_level2 does so for every
+// first edge; and a shift with p = 1, one sum when alone, takes a slot of 280 bytes and two searches
+// for every window.  Times in ms, sharing / apart, of seeds with a constant sum of p: 3-cycle on 1e7
+// edges, 64 at p = 1/32 0.96 / 3.5, 512 at 1/256 2.5 / 3.1, 4,000 at 1/2,000 14 / 10; on 1e6 edges 0.44 /
+// 0.53, 1.9 / 1.3, 12.5 / 7.3; out-star on 2e7 edges, 2,000 at 0.0021 21 / 14; ping-pong on 1e7 edges
+// 2.3 / 3.3, 13 / 3.0, 120 / 10; two seeds at p = 1 on 1e7 edges with 63 windows per 100 edges 4.2 /
+// 0.72, with 6.3 0.87 / 0.76 (eight: 1.7 / 2.7), with 1.1 0.64 / 0.94.  The true lines vary by
+// motif, span and graph by a factor of about two (the records are not known before); over 800
+// such batches from 1e5 to 2e7 edges the form chosen takes at most 1.45 times the better one.
+constexpr double kApartEdge = 0.12, kApartEdgeTwoNode = 0.13, kApartAllEdge = 0.035;   // per edge of the graph
+constexpr double kRideEdge = 0.05e-3, kRideEdgeFixed = 0.2e-3, kRideEdgeTwoNode = 2.0e-3;
+constexpr double kRideChain = 1100.0, kRideWindow = 0.2;
+constexpr double kFewShifts = 64;
+constexpr double kSharedEdge = 0.045;     // the enumeration that they share
+
+double keep_rate(const tm_graph* g, const tm_query& q, double& J) {
+    J = 1.0 + (double)g->t_max / ((double)q.c * (double)q.delta);
+    return q.q_mode == TM_Q_UNIFORM ? q.p : std::min(1.0, q.p / J);
+}
+
+// q among `shifts` shifts of its motif
+double ride_gain(const tm_graph* g, const tm_query& q, double shifts) {
+    const double m = (double)g->m;
+    double J;
+    const double p = keep_rate(g, q, J);
+    const bool all = q.q_mode == TM_Q_UNIFORM && q.p >= 1.0;
+    const bool two = q.motif->k == 2;
+    const LevelPlan& L = q.motif->lv[q.motif->l - 1];
+    const double apart = m * (all ? kApartAllEdge : p * (two ? kApartEdgeTwoNode : kApartEdge));
+    const double edge = two ? kRideEdgeTwoNode : std::max(L.su, L.sv) < 2 ? kRideEdgeFixed : kRideEdge;
+    return apart - m * edge - (all ? J * kRideWindow : 0.0) -
+           (shifts > kFewShifts ? kRideChain : 0.0);
+}
+
 // When estimates share an enumeration of their own (run_batch_once).  Both sides, us a call on 1e7
 // edges: the nine calibrated estimates (sums 1.5 to 2.6 first edges per motif, candidates 1.02 to
 // 1.04) 6,362 apart and 3,352 sharing; 192 seeds of the 4-cycle (10.6 of each) 49,200 apart and
-// 6,580 sharing, build included.  The margin over 1 pays for the records and their weighing.
+// 6,580 sharing, build included.  The margin over 1 pays for the records.
 constexpr double kHideFirst = 1.4, kHideCand = 0.9;
 
 int run_batch_once(const tm_graph* g, const tm_query* qs, int nq, tm_result* res, cudaStream_t st,
@@ -2562,13 +2600,14 @@ int run_batch_once(const tm_graph* g, const tm_query* qs, int nq, tm_result* res
     // estimate needs no enumeration of its own (its windows and fold stay its own)
     std::vector<int> host((size_t)nq, -1);    // estimate -> its exact head (nq + h: hidden head h)
     std::vector<int> nrid((size_t)nq, 0);
-    std::vector<int> alone;                   // estimates that could ride and have no head
+    std::vector<int64_t> nshift((size_t)nq, 0);   // shifts riding on a head
     int lmax = 1, kmax = 2;
     for (int i = 0; i < nq; i++)
         if (qs[i].motif) {
             lmax = std::max(lmax, qs[i].motif->l);
             kmax = std::max(kmax, qs[i].motif->k);
         }
+    std::vector<std::vector<int>> kinds;      // the estimates of each motif that could ride
     for (int i = 0; i < nq; i++) {
         const tm_query& q = qs[i];
         std::string why;
@@ -2576,44 +2615,59 @@ int run_batch_once(const tm_graph* g, const tm_query* qs, int nq, tm_result* res
         // (four edges: the matcher's four-edge instantiation emits the records)
         if (!q.motif || (q.motif->l != 3 && !(q.motif->l == 4 && lmax <= 4 && kmax <= 4))) continue;
         if (q.motif->lv[q.motif->l - 1].view != kPair || validate_query(g, q, why) != TM_OK) continue;
-        for (int L : heads)
-            if (nrid[(size_t)L] < kMaxRide && qs[L].delta >= q.delta && same_motif(qs[L].motif, q.motif)) {
-                host[(size_t)i] = L;
-                nrid[(size_t)L]++;
-                any = true;
-                break;
-            }
-        if (host[(size_t)i] < 0) alone.push_back(i);
+        size_t k = 0;
+        while (k < kinds.size() && !same_motif(qs[kinds[k][0]].motif, q.motif)) k++;
+        if (k == kinds.size()) kinds.emplace_back();
+        kinds[k].push_back(i);
+    }
+    for (std::vector<int>& gr : kinds) {
+        double shifts = 0;
+        for (int i : gr) shifts += qs[i].b;
+        gr.erase(std::remove_if(gr.begin(), gr.end(), [&](int i) { return ride_gain(g, qs[i], shifts) < 0.0; }), gr.end());
+        std::vector<int> alone;               // no head for them in the batch
+        for (int i : gr) {
+            const tm_query& q = qs[i];
+            for (int L : heads)
+                if (nrid[(size_t)L] < kMaxRide && nshift[(size_t)L] + q.b <= kMaxRideShifts && qs[L].delta >= q.delta &&
+                    same_motif(qs[L].motif, q.motif)) {
+                    host[(size_t)i] = L;
+                    nrid[(size_t)L]++;
+                    nshift[(size_t)L] += q.b;
+                    any = true;
+                    break;
+                }
+            if (host[(size_t)i] < 0) alone.push_back(i);
+        }
+        gr.swap(alone);
     }
     // Estimates of one motif without such an exact query: when together they keep enough windows,
     // one enumeration of the whole graph for all of them costs less than their own, so they ride
     // along with an exact query that nobody asked for.  Theirs cost, in first edges, sum b p, and in
     // candidates (which grow with the span) sum b p delta; the shared one 1 and its span.  It is
-    // taken for the longest span for which the first sum is at least kHideFirst and the second at
-    // least kHideCand of it (measured: see kHideFirst).
+    // taken for the longest span for which the first sum is at least kHideFirst, the second at
+    // least kHideCand of it (measured: see kHideFirst), and riding saves what it costs.
     std::vector<tm_query> hidden;
     std::vector<int> top;                     // per hidden head, the estimate whose span it has
-    std::vector<std::vector<int>> kinds;      // the estimates of each motif
-    for (int i : alone) {
-        size_t k = 0;
-        while (k < kinds.size() && !same_motif(qs[kinds[k][0]].motif, qs[i].motif)) k++;
-        if (k == kinds.size()) kinds.emplace_back();
-        kinds[k].push_back(i);
-    }
     if (!hide) kinds.clear();
     for (std::vector<int>& gr : kinds) {
         std::stable_sort(gr.begin(), gr.end(), [&](int a, int b) { return qs[a].delta > qs[b].delta; });
-        std::vector<double> first(1, 0.0), cand(1, 0.0);   // sums of b p and of b p delta, longest spans first
+        // sums of b p, of b p delta and of the gains, longest spans first
+        std::vector<double> first(1, 0.0), cand(1, 0.0), gain(1, 0.0);
+        std::vector<int64_t> shifts(1, 0);
+        for (int i : gr) shifts.push_back(shifts.back() + qs[i].b);
         for (int i : gr) {
             const tm_query& q = qs[i];
-            const double J = 1.0 + (double)g->t_max / ((double)q.c * (double)q.delta);
-            const double bp = q.b * (q.q_mode == TM_Q_UNIFORM ? q.p : std::min(1.0, q.p / J));
+            double J;
+            const double bp = q.b * keep_rate(g, q, J);
             first.push_back(first.back() + bp);
             cand.push_back(cand.back() + bp * (double)q.delta);
+            gain.push_back(gain.back() + q.b * ride_gain(g, q, (double)shifts.back()));
         }
         for (size_t y = 0; y < gr.size();) {
-            const size_t e = std::min(gr.size(), y + (size_t)kMaxRide);
-            if (first[e] - first[y] < kHideFirst || cand[e] - cand[y] < kHideCand * (double)qs[gr[y]].delta) {
+            const size_t fit = (size_t)(std::upper_bound(shifts.begin(), shifts.end(), shifts[y] + kMaxRideShifts) - shifts.begin()) - 1;
+            const size_t e = std::min(fit, y + (size_t)kMaxRide);   // (at least y + 1: b <= 2^20)
+            if (first[e] - first[y] < kHideFirst || cand[e] - cand[y] < kHideCand * (double)qs[gr[y]].delta ||
+                gain[e] - gain[y] < kSharedEdge * (double)g->m) {
                 y++;   // the next shorter span
                 continue;
             }

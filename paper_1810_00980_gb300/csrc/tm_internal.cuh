@@ -297,7 +297,8 @@ struct QPlan {
     LevelPlan lv[TM_L_MAX];
 };
 constexpr int kMaxSub = 3;
-constexpr int kMaxRide = 4096;   // riders of one exact query
+constexpr int kMaxRide = 4096;                           // riders of one exact query
+constexpr int64_t kMaxRideShifts = (int64_t)1 << 22;     // and their shifts (64 bytes each)
 static_assert(sizeof(QPlan) == 320, "plan stride");
 
 struct Tuning {
