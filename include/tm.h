@@ -295,8 +295,10 @@ int tm_set_tuning(const tm_tuning* in);
  * estimates riding along with it) and smaller spans to a second kernel, as one record per group
  * of instances, in a device buffer taken from the batch scratch.  `records` (1 .. 2^36) sets how
  * many records the next batches make room for (default 2^23: 192 MB with 32-bit times, 256 MB
- * with 64-bit times).  A batch that needs more runs a second time with room for all of them and
- * raises the capacity to that, so the setting changes only memory and time, never a result.
+ * with 64-bit times).  A batch that produces more goes on in rounds, the matcher stopping while
+ * the second kernel empties the buffer; one that overruns the buffer within a round runs again
+ * with a larger one, whose size the graph keeps for its next batches.  The setting changes only
+ * memory and time, never a result.
  * Returns TM_EINVAL outside that range. */
 int tm_set_ride_capacity(int64_t records);
 /* Time candidate tunings on `queries` over g (results discarded) and keep the

@@ -37,8 +37,7 @@ Tuning& tuning() {
     return t;
 }
 
-// Records the deferred-rider buffer of a batch holds: grows to the largest count a batch has
-// needed (tm_set_ride_capacity sets it)
+// Records the deferred-rider buffer of a batch holds (tm_set_ride_capacity)
 std::atomic<int64_t>& ride_capacity() {
     static std::atomic<int64_t> cap{(int64_t)1 << 23};
     return cap;
@@ -126,6 +125,11 @@ struct MatchArgs {
     RideRec<TT>* rrec = nullptr;        // [rcap] deferred rider / smaller-span work (see RideRec)
     unsigned long long* rcount = nullptr;   // records appended (counts past rcap: the batch reruns)
     int64_t rcap = 0;
+    // From rstop records on the warps finish the chunks they have and take no more (*more = 1 then):
+    // k_ride weighs the records so far and the matcher goes on from the queue's counter (resume).
+    unsigned long long rstop = 0;
+    uint32_t* more = nullptr;
+    int resume = 0;
 };
 
 // ----------------------------------------------------------------- helpers
@@ -1043,6 +1047,12 @@ __global__ void __launch_bounds__(256, 8) k_level2(MatchArgs<TT> A, FRec<TT>* __
     acc_flush_warp(acc, A.W.acc);
 }
 
+// set by the block's warps that have seen rstop records
+__device__ __forceinline__ volatile int& stop_flag() {
+    __shared__ int flag;
+    return flag;
+}
+
 // The warp's deferred rider / smaller-span records (lanes with rn != 0), appended with one atomic
 template <typename TT>
 __device__ __forceinline__ void ride_emit(const MatchArgs<TT>& A, int64_t rx, int32_t rn, int64_t t1, int64_t tc, int32_t q) {
@@ -1050,7 +1060,10 @@ __device__ __forceinline__ void ride_emit(const MatchArgs<TT>& A, int64_t rx, in
     const unsigned rm = __ballot_sync(kFull, rn != 0);
     if (!rm) return;
     unsigned long long rb = 0;
-    if (lane == 0) rb = atomicAdd(A.rcount, (unsigned long long)__popc(rm));
+    if (lane == 0) {
+        rb = atomicAdd(A.rcount, (unsigned long long)__popc(rm));
+        if (rb >= A.rstop) stop_flag() = 1;
+    }
     rb = __shfl_sync(kFull, rb, 0) + __popc(rm & ((1u << lane) - 1u));
     if (rn && (int64_t)rb < A.rcap) {
         RideRec<TT> rr;
@@ -1227,7 +1240,9 @@ template <typename TT, int LMAX, int KMAX, int OCC = 4, bool EXPAND = true, bool
 __global__ void __launch_bounds__(256, OCC) k_match(MatchArgs<TT> A) {
     const GraphDevT<TT>& G = A.G;
     extern __shared__ __align__(16) unsigned char smem_plans[];
+    if (threadIdx.x == 0) stop_flag() = 0;
     const QPlan* PL = stage_plans(A.plans, A.nq, smem_plans);
+    if (A.nq > kSmemPlans) __syncthreads();   // (stage_plans ends with a barrier otherwise)
     int lane = threadIdx.x & 31;
     Acc acc;
     acc_init(acc, smem_plans, A.nq);
@@ -1244,7 +1259,19 @@ __global__ void __launch_bounds__(256, OCC) k_match(MatchArgs<TT> A) {
     const int64_t chunk = min((((A.chunk - 1) >> gl) + 1) << gl, share);
     // a warp's first chunk is its own, the others come from the counter (with few items no warp
     // asks it: 7,000 atomics on one word take longer than such a batch's items)
-    for (int64_t c0 = ((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5) * chunk; c0 < W2;) {
+    auto next_chunk = [&]() -> int64_t {
+        unsigned long long c = 0;
+        if (lane == 0) {
+            if (stop_flag()) {
+                *A.more = 1;
+                c = (unsigned long long)W2;   // past the last item
+            } else {
+                c = atomicAdd(A.counter, (unsigned long long)chunk);
+            }
+        }
+        return nwarps * chunk + (int64_t)__shfl_sync(kFull, c, 0);
+    };
+    for (int64_t c0 = A.resume ? next_chunk() : ((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5) * chunk; c0 < W2;) {
         int64_t c1 = min(c0 + chunk, W2);
         int64_t fb = 0, fe = 0;
         const int64_t ci = c0 >> gl, ce = ((c1 - 1) >> gl) + 1;
@@ -1435,9 +1462,7 @@ __global__ void __launch_bounds__(256, OCC) k_match(MatchArgs<TT> A) {
         }
         acc_flush_warp(acc, A.W.acc);
         if (nwarps * chunk >= W2) break;
-        unsigned long long c0u = 0;
-        if (lane == 0) c0u = atomicAdd(A.counter, (unsigned long long)chunk);
-        c0 = nwarps * chunk + (int64_t)__shfl_sync(kFull, c0u, 0);
+        c0 = next_chunk();
     }
     acc_flush_warp(acc, A.W.acc);
 }
@@ -2170,9 +2195,9 @@ int run_batch_t(const tm_graph* g, const tm_query* qs, int nq, tm_result* res, c
                           a256(8 * (size_t)hp[(size_t)i].b * (size_t)(hp[(size_t)i].J + 1));
         }
     }
-    // exact queries with riders or smaller spans leave that work to k_ride in records; the
-    // record buffer holds as many as the largest batch so far needed (a batch that needs more
-    // runs again with room for all of them)
+    // exact queries with riders or smaller spans leave that work to k_ride in records, in rounds
+    // when the record buffer fills up before the queue is empty; a batch that overruns it within a
+    // round runs again with a larger one, whose size the graph keeps
     // the riders' shifts, one entry each, in their exact query's order
     std::vector<RideEnt> h_rides;
     std::vector<size_t> ride_at0((size_t)nq, 0);
@@ -2188,7 +2213,8 @@ int run_batch_t(const tm_graph* g, const tm_query* qs, int nq, tm_result* res, c
         }
     bool any_share = false;
     for (const QPlan& P : hp) any_share |= P.nsub > 0 || P.nride > 0;
-    const int64_t rcap = any_share ? std::max(ride_capacity().load(), dbg->need_records) : 0;   // (shares come with dbg)
+    // (shares come with dbg)
+    const int64_t rcap = any_share ? std::max({ride_capacity().load(), g->ride_need.load(), dbg->need_records}) : 0;
     const size_t rrec_bytes = any_share ? a256(sizeof(RideRec<TT>) * (size_t)rcap) : 0;
     // ---- scratch layout
     const int64_t n_parts = fold_parts(hp);
@@ -2235,13 +2261,15 @@ int run_batch_t(const tm_graph* g, const tm_query* qs, int nq, tm_result* res, c
     W.k = (int32_t*)take(4 * NWs);
     W.kept = (int32_t*)take(4 * NWs);
     W.qj = (double*)take(8 * NWs);
-    // the results and, right behind them (one copy brings all back), the record count and the
-    // error word of the kernels that wait between blocks; from there on everything starts at zero
+    // the results and, right behind them (one copy brings all back), the record count, the error
+    // word of the kernels that wait between blocks and whether the matcher stopped early; from
+    // there on everything starts at zero
     const size_t res_bytes = sizeof(tm_result) * (size_t)nq;
     static_assert(sizeof(tm_result) % 8 == 0, "the counters follow the results");
     tm_result* dres = (tm_result*)take(res_bytes + 16);
     unsigned long long* drcount = (unsigned long long*)((char*)dres + res_bytes);
     uint32_t* dserr = (uint32_t*)(drcount + 1);
+    uint32_t* dmore = dserr + 1;
     W.acc = (unsigned long long*)take(8 * A_N * NWs);
     int64_t* dF = (int64_t*)take(8);
     int64_t* dW2 = (int64_t*)take(8);
@@ -2273,7 +2301,7 @@ int run_batch_t(const tm_graph* g, const tm_query* qs, int nq, tm_result* res, c
     int ev_w0 = pe.mark(st), ev_w1 = -1, ev_l0 = -1, ev_l1 = -1, ev_l2 = -1, ev_m1 = -1, ev_r1 = -1, ev_f1 = -1;
     int64_t hW2 = 0;
     unsigned long long h_rcount = 0;
-    uint32_t h_serr = 0;
+    uint32_t h_serr = 0, h_more = 0;
     std::vector<char> h_plans;
     fail(copy_plans(hp, wown, h_plans, dplans, st), "plans");
     if (!h_rides.empty())
@@ -2326,6 +2354,13 @@ int run_batch_t(const tm_graph* g, const tm_query* qs, int nq, tm_result* res, c
         }
     }
     const int64_t Fa = bounded ? F_ub : F;   // first edges the scratch holds
+    const bool expands = std::any_of(hp.begin(), hp.end(), [](const QPlan& P) { return plan_expands(P); });
+    MatchArgs<TT> A;
+    auto launch_ride = [&]() {
+        launch_after(k_ride<TT>, dim3((unsigned)(nsm * 8)), 256, match_smem_bytes(A.nq, 256, true), st, A);
+        count_launch();
+        fail(cudaGetLastError(), "k_ride");
+    };
     ScratchLease fb;
     if (rc == TM_OK && Fa > 0) {
         size_t Fs = (size_t)Fa;
@@ -2342,7 +2377,6 @@ int run_batch_t(const tm_graph* g, const tm_query* qs, int nq, tm_result* res, c
             int32_t* bwin = (int32_t*)take2(4 * nbw);
             int64_t* cf = (int64_t*)take2(8 * ncf);
             RideRec<TT>* rrec = any_share ? (RideRec<TT>*)take2(sizeof(RideRec<TT>) * (size_t)rcap) : nullptr;
-            MatchArgs<TT> A;
             const int64_t* d_Fk = bounded ? dF : nullptr;
             A.G = G; A.plans = dplans; A.nq = nq; A.W = W; A.NW = NW; A.F = Fa; A.d_F = d_Fk;
             A.rec = rec; A.excl = excl; A.hs_a = hs_a; A.hs_hi = hs_hi;
@@ -2353,6 +2387,11 @@ int run_batch_t(const tm_graph* g, const tm_query* qs, int nq, tm_result* res, c
             A.rrec = rrec;
             A.rcount = drcount;
             A.rcap = rcap;
+            // room for the chunks in flight (three edges: at most a record per item), or half of it
+            const int64_t held = (int64_t)nsm * tu.blocks_per_sm * (tu.block_threads / 32) *
+                                 std::max<int64_t>(tu.chunk_items, item_grain(Fa));
+            A.rstop = (unsigned long long)std::max(rcap / 2, rcap - held);
+            A.more = dmore;
             int64_t gl2 = std::min<int64_t>((Fa + 255) / 256, (int64_t)nsm * 8);
             if (NW > 1) {   // (one window: nothing to search)
                 launch_after(k_blockwin, dim3((unsigned)std::min<int64_t>(((int64_t)nbw + 255) / 256, (int64_t)nsm * 8)), 256, 0, st,
@@ -2371,15 +2410,12 @@ int run_batch_t(const tm_graph* g, const tm_query* qs, int nq, tm_result* res, c
             ev_l1 = pe.mark(st);
             nv.next("tm_match");
             if (rc == TM_OK) {
-                launch_match<TT>(A, lmax, kmax, tu, nsm, st,
-                                 std::any_of(hp.begin(), hp.end(), [](const QPlan& P) { return plan_expands(P); }));
+                launch_match<TT>(A, lmax, kmax, tu, nsm, st, expands);
                 fail(cudaGetLastError(), "k_match");
                 ev_m1 = pe.mark(st);
                 if (any_share && rc == TM_OK) {
                     nv.next("tm_ride");
-                    launch_after(k_ride<TT>, dim3((unsigned)(nsm * 8)), 256, match_smem_bytes(A.nq, 256, true), st, A);
-                    count_launch();
-                    fail(cudaGetLastError(), "k_ride");
+                    launch_ride();
                     ev_r1 = pe.mark(st);
                 }
                 if (pe.on) fail(cudaMemcpyAsync(&hW2, dW2, 8, cudaMemcpyDeviceToHost, st), "W2");
@@ -2399,10 +2435,18 @@ int run_batch_t(const tm_graph* g, const tm_query* qs, int nq, tm_result* res, c
         if (ev_r1 < 0) ev_r1 = ev_m1;
     }
     std::vector<char> h_res(res_bytes + 16);
-    if (rc == TM_OK) fail(cudaMemcpyAsync(h_res.data(), dres, res_bytes + 16, cudaMemcpyDeviceToHost, st), "results");
-    if (rc == TM_OK && dbg && dbg->sub_count)
-        fail(cudaMemcpyAsync(dbg->sub_count, dsubc, 8 * kMaxSub * (size_t)nq, cudaMemcpyDeviceToHost, st),
-             "span counts");
+    auto copy_results = [&]() {
+        fail(cudaMemcpyAsync(h_res.data(), dres, res_bytes + 16, cudaMemcpyDeviceToHost, st), "results");
+        if (rc == TM_OK && dbg && dbg->sub_count)
+            fail(cudaMemcpyAsync(dbg->sub_count, dsubc, 8 * kMaxSub * (size_t)nq, cudaMemcpyDeviceToHost, st),
+                 "span counts");
+    };
+    auto read_words = [&]() {
+        std::memcpy(&h_rcount, h_res.data() + res_bytes, 8);
+        std::memcpy(&h_serr, h_res.data() + res_bytes + 8, 4);
+        std::memcpy(&h_more, h_res.data() + res_bytes + 12, 4);
+    };
+    if (rc == TM_OK) copy_results();
     if (rc == TM_OK && dbg && dbg->sums && n_sums > 0) {
         std::memset(dbg->sums, 0, sizeof(ShiftSums) * (size_t)n_sums);   // rejected queries write none
         fail(cudaMemcpyAsync(dbg->sums, dsums, sizeof(ShiftSums) * (size_t)n_sums, cudaMemcpyDeviceToHost, st),
@@ -2436,34 +2480,64 @@ int run_batch_t(const tm_graph* g, const tm_query* qs, int nq, tm_result* res, c
     cudaError_t se = cudaStreamSynchronize(st);
     fail(se, "batch sync");
     if (rc == TM_OK) {
-        std::memcpy(res, h_res.data(), res_bytes);
-        std::memcpy(&h_rcount, h_res.data() + res_bytes, 8);
-        std::memcpy(&h_serr, h_res.data() + res_bytes + 8, 4);
+        read_words();
         if (h_serr) {
             set_error(kExpired);
             rc = TM_ECUDA;
         }
     }
+    // further rounds of the matcher and k_ride, then the fold again (the first one saw the sums so far)
+    unsigned long long records = h_rcount;
+    double round_match_ms = 0.0, round_ride_ms = 0.0;
+    bool rounds = false;
+    while (rc == TM_OK && h_more && (int64_t)h_rcount <= rcap) {
+        rounds = true;
+        A.resume = 1;
+        PhaseEvents pr(pe.on);
+        fail(cudaMemsetAsync(drcount, 0, 16, st), "record count");
+        const int e0 = pr.mark(st);
+        if (rc == TM_OK) launch_match<TT>(A, lmax, kmax, tu, nsm, st, expands);
+        fail(cudaGetLastError(), "k_match");
+        const int e1 = pr.mark(st);
+        if (rc == TM_OK) launch_ride();
+        const int e2 = pr.mark(st);
+        fail(cudaMemcpyAsync(h_res.data() + res_bytes, drcount, 16, cudaMemcpyDeviceToHost, st), "records");
+        fail(cudaStreamSynchronize(st), "round sync");
+        if (rc != TM_OK) break;
+        read_words();
+        records += h_rcount;
+        round_match_ms += pr.ms(e0, e1);
+        round_ride_ms += pr.ms(e1, e2);
+    }
+    if (rc == TM_OK && rounds && (int64_t)h_rcount <= rcap) {
+        fail(cudaMemsetAsync(dfolded, 0, 4 * (size_t)nq, st), "fold");
+        if (rc == TM_OK)
+            launch_fold(dplans, nq, n_parts, W, dpart, dfolded, dres, nullptr, dbg && dbg->sub_count ? dsubc : nullptr, st);
+        fail(cudaGetLastError(), "fold");
+        if (rc == TM_OK) copy_results();
+        fail(cudaStreamSynchronize(st), "fold sync");
+    }
+    if (rc == TM_OK) std::memcpy(res, h_res.data(), res_bytes);
     if (pe.on && rc == TM_OK) {
         double wall = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - wall0).count();
-        store_profile_batch(pe.ms(ev_w0, ev_w1), pe.ms(ev_l0, ev_l2), ev_l1 >= 0 ? pe.ms(ev_l1, ev_m1) : 0.0,
+        store_profile_batch(pe.ms(ev_w0, ev_w1), pe.ms(ev_l0, ev_l2), (ev_l1 >= 0 ? pe.ms(ev_l1, ev_m1) : 0.0) + round_match_ms,
                             pe.ms(ev_m1 >= 0 && ev_l1 >= 0 ? ev_r1 : ev_f1, ev_f1), wall, hW2, F,
                             ev_l0 >= 0 ? pe.ms(ev_w1, ev_l0) : 0.0, ev_l1 >= 0 ? pe.ms(ev_l2, ev_l1) : 0.0,
-                            ev_l1 >= 0 ? pe.ms(ev_m1, ev_r1) : 0.0);
+                            (ev_l1 >= 0 ? pe.ms(ev_m1, ev_r1) : 0.0) + round_ride_ms);
     }
-    if (pe.on && rc == TM_OK) store_profile_ride_records((int64_t)h_rcount);
+    if (pe.on && rc == TM_OK) store_profile_ride_records((int64_t)records);
     scratch_release(fb, st);
     cudaFreeAsync(sb, st);
     if (rc != TM_OK) return rc;
     if ((int64_t)h_rcount > rcap) {
-        // more deferred records than the buffer held: run again with room for all of them
-        int64_t want = (int64_t)h_rcount + (int64_t)(h_rcount >> 3) + 1024;
+        // a round left more deferred records than the buffer held: run again with a larger one
+        const int64_t want = std::max(4 * rcap, (int64_t)h_rcount + (int64_t)(h_rcount >> 3) + 1024);
         if (dbg->hidden && want > kHiddenRecords) return TM_ENOMEM;   // run_batch_once runs the estimates apart
         dbg->need_records = want;
         rc = run_batch_t<TT>(g, qs, nq, res, st, dbg);
         if (rc == TM_ENOMEM) return rc;   // (the next batches keep the capacity that fits)
-        int64_t cur = ride_capacity().load();
-        while (cur < want && !ride_capacity().compare_exchange_weak(cur, want)) {}
+        int64_t cur = g->ride_need.load();
+        while (cur < want && !g->ride_need.compare_exchange_weak(cur, want)) {}
         return rc;
     }
     if (dbg && dq_n > 0) {

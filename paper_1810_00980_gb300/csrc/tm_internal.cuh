@@ -193,6 +193,8 @@ struct tm_graph {
     void* table_block;      // a large graph's pair table (or null)
     void* ex_own_block;     // the two-node tables ([m+1] each), built on first use (or null)
     void* ex_rev_block;
+    // records that a round of a batch on this graph has needed room for, beyond the set capacity
+    mutable std::atomic<int64_t> ride_need{0};
     tmo::GraphDev dev;
 };
 
