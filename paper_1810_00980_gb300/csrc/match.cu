@@ -114,7 +114,6 @@ struct MatchArgs {
     const int64_t* hs_a;   // [F] closing pair range start (queries whose last edge is fixed by the first)
     const int64_t* hs_hi;  // [F] closing pair range end
     const int64_t* d_W2;   // total second-edge candidates
-    const uint32_t* err;   // see gave_up
     unsigned long long* counter;
     int64_t chunk;
     int enum_threshold;
@@ -675,7 +674,7 @@ __global__ void k_wtab(const QPlan* __restrict__ plans, const int32_t* __restric
 template <typename TT>
 __global__ void k_windows(GraphDevT<TT> G, const QPlan* __restrict__ plans, int nq, WinDev W, int64_t NW,
                           int64_t* __restrict__ dF, const uint32_t* err) {
-    if (gave_up(err)) return;   // (the partition by windows may be missing)
+    const bool lost = gave_up(err);   // the partition by windows is missing: no first edges
     for (int64_t w = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; w < NW;
          w += (int64_t)gridDim.x * blockDim.x) {
         int lo_q = 0, hi_q = nq;
@@ -729,7 +728,7 @@ __global__ void k_windows(GraphDevT<TT> G, const QPlan* __restrict__ plans, int 
         }
         W.lo[w] = lo; W.hi[w] = hi; W.tend[w] = tend; W.start[w] = start; W.j[w] = j;
         W.q[w] = lo_q; W.k[w] = k; W.kept[w] = kept; W.qj[w] = qj;
-        W.nfirst[w] = (kept && !Q.riding) ? hi - lo : 0;   // riders take no first edges
+        W.nfirst[w] = (kept && !Q.riding && !lost) ? hi - lo : 0;   // riders take no first edges
     }
     if (!dF) return;
     __shared__ int64_t s_warp[kWindowThreads / 32];
@@ -790,10 +789,9 @@ __device__ __forceinline__ int64_t first_thi(const QPlan& Q, const WinDev& W, in
 // window of first edge 32 b for every block b of 32 first edges: one search each,
 // run at full occupancy instead of on the critical path of k_level2's warps
 __global__ void k_blockwin(const int64_t* __restrict__ fbase, int64_t NW, int64_t Fh,
-                           const int64_t* __restrict__ d_F, int32_t* __restrict__ bw, const uint32_t* err) {
+                           const int64_t* __restrict__ d_F, int32_t* __restrict__ bw) {
     grid_wait();
     const int64_t F = d_F ? *d_F : Fh;
-    if (gave_up(err)) return;
     int64_t nb = (F + 31) >> 5;
     for (int64_t b = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; b < nb;
          b += (int64_t)gridDim.x * blockDim.x) {
@@ -821,8 +819,7 @@ __global__ void __launch_bounds__(256, 8) k_level2(MatchArgs<TT> A, FRec<TT>* __
     acc_init(acc, smem_plans, A.nq);
     acc_zero(acc);
     grid_wait();
-    const int64_t F = A.d_F ? *A.d_F : A.F;
-    if (gave_up(A.err)) return;
+    const int64_t F = A.d_F ? *A.d_F : A.F;   // (below zero when a wait of their scan expired)
     for (int64_t base = warp * 32; base < F; base += nwarps * 32) {
         int64_t f = base + lane;
         bool valid = f < F;
@@ -1248,9 +1245,8 @@ __global__ void __launch_bounds__(256, OCC) k_match(MatchArgs<TT> A) {
     acc_init(acc, smem_plans, A.nq);
     acc_zero(acc);
     grid_wait();
-    int64_t W2 = *A.d_W2;
+    int64_t W2 = *A.d_W2;   // (below zero when a wait of their scan expired)
     const int64_t F = A.d_F ? *A.d_F : A.F;
-    if (gave_up(A.err)) return;
     // few items: smaller chunks, so that every warp gets some (17,000 items in chunks of 256 kept 67
     // warps busy for eight rounds each: 43 us of a 20,000-edge count)
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -2380,7 +2376,7 @@ int run_batch_t(const tm_graph* g, const tm_query* qs, int nq, tm_result* res, c
             const int64_t* d_Fk = bounded ? dF : nullptr;
             A.G = G; A.plans = dplans; A.nq = nq; A.W = W; A.NW = NW; A.F = Fa; A.d_F = d_Fk;
             A.rec = rec; A.excl = excl; A.hs_a = hs_a; A.hs_hi = hs_hi;
-            A.d_W2 = dW2; A.err = dserr; A.counter = dctr;
+            A.d_W2 = dW2; A.counter = dctr;
             A.enum_threshold = tu.enum_threshold;
             A.chunk = tu.chunk_items;
             A.blockwin = bwin; A.chunkf = cf; A.nchunkf = (int64_t)ncf; A.grain_log = item_grain_log(Fa);
@@ -2395,7 +2391,7 @@ int run_batch_t(const tm_graph* g, const tm_query* qs, int nq, tm_result* res, c
             int64_t gl2 = std::min<int64_t>((Fa + 255) / 256, (int64_t)nsm * 8);
             if (NW > 1) {   // (one window: nothing to search)
                 launch_after(k_blockwin, dim3((unsigned)std::min<int64_t>(((int64_t)nbw + 255) / 256, (int64_t)nsm * 8)), 256, 0, st,
-                             W.fbase, NW, Fa, d_Fk, bwin, dserr);
+                             W.fbase, NW, Fa, d_Fk, bwin);
                 count_launch();
             } else {
                 A.blockwin = nullptr;
@@ -3068,7 +3064,7 @@ int count_exact_noalloc_t(const tm_graph* g, const tm_motif* m, int64_t delta, c
         const Tuning tu = tuning();
         MatchArgs<TT> A;
         A.G = G; A.plans = dplan; A.nq = 1; A.W = W; A.NW = 1; A.F = F; A.d_F = nullptr;
-        A.rec = rec; A.excl = excl; A.d_W2 = dW2; A.err = derr; A.counter = dctr;
+        A.rec = rec; A.excl = excl; A.d_W2 = dW2; A.counter = dctr;
         A.hs_a = nullptr; A.hs_hi = nullptr;
         A.enum_threshold = tu.enum_threshold;
         A.chunk = tu.chunk_items;
@@ -3302,13 +3298,13 @@ int batch_create_t(const tm_graph* g, const tm_query* qs, int nq, tm_batch** out
         MatchArgs<TT> A;
         A.G = G; A.plans = dplans; A.nq = nq; A.W = W; A.NW = NW; A.F = Fmax; A.d_F = dF;
         A.rec = rec; A.excl = excl; A.hs_a = hs_a; A.hs_hi = hs_hi;
-        A.d_W2 = dW2; A.err = derr; A.counter = dctr;
+        A.d_W2 = dW2; A.counter = dctr;
         A.enum_threshold = tu.enum_threshold;
         A.chunk = tu.chunk_items;
         A.blockwin = bwin; A.chunkf = cf; A.nchunkf = (int64_t)ncf; A.grain_log = item_grain_log(Fmax);
         int64_t gl2 = std::min<int64_t>((Fmax + 255) / 256, (int64_t)nsm * 8);
         launch_after(k_blockwin, dim3((unsigned)std::min<int64_t>(((int64_t)nbw + 255) / 256, (int64_t)nsm * 8)), 256, 0, st,
-                     W.fbase, NW, Fmax, dF, bwin, derr);
+                     W.fbase, NW, Fmax, dF, bwin);
         count_launch();
         launch_after(k_level2<TT>, dim3((unsigned)std::max<int64_t>(gl2, 1)), 256, match_smem_bytes(A.nq, 256), st, A, rec, len32, hs_a, hs_hi); count_launch();
         fail(cudaGetLastError(), "k_level2");

@@ -131,7 +131,7 @@ __device__ __forceinline__ void note_big(const BigRanges& B, int64_t* cf, int64_
 // memory so that both the 32-bit loads and the 64-bit stores are coalesced.  cf: as k_scan_once
 __global__ void k_len_scan(const int32_t* __restrict__ in, int64_t* __restrict__ out, int64_t n_max,
                            const int64_t* __restrict__ d_n, const int64_t* __restrict__ offs,
-                           int64_t* __restrict__ cf, int64_t ncf, const uint32_t* err) {
+                           int64_t* __restrict__ cf, int64_t ncf) {
     __shared__ int64_t smem[33];
     __shared__ int64_t tile[kScanTile + kScanTile / 16];   // one pad word per 16: no bank conflicts
     __shared__ BigRanges big;
@@ -139,7 +139,7 @@ __global__ void k_len_scan(const int32_t* __restrict__ in, int64_t* __restrict__
     if (threadIdx.x == 0) big.n = 0;
     int64_t n = d_n ? min(*d_n, n_max) : n_max;
     int64_t t0 = (int64_t)blockIdx.x * kScanTile;
-    if (t0 >= n || gave_up(err)) return;   // (the lengths may be missing)
+    if (t0 >= n) return;
     for (int i = threadIdx.x; i < kScanTile; i += blockDim.x) {
         int64_t idx = t0 + i;
         tile[i + (i >> 4)] = idx < n ? (int64_t)in[idx] : 0;
@@ -212,6 +212,7 @@ __global__ void k_set_i64(int64_t* p, int64_t v) { *p = v; }
 // 2^62), and a warp looks back over 32 tiles at a time.  Prefixes travel 32 tiles per memory
 // latency, so beyond kOnePassTiles tiles the two-pass form is as quick; below, one launch takes
 // the place of three to five (a 20,000-edge count spent 22 of its 118 us on them).
+// *d_total is zero before and, when a wait expires, below zero afterwards.
 // CF also notes the first edge of every grain-th item (cf[i]: the element whose range holds item
 // i * grain, grain = item_grain(n_max); past the last, n - 1), as far as cf's ncf entries go.
 constexpr int kOneThreads = 256;
@@ -240,18 +241,11 @@ __global__ void __launch_bounds__(kOneThreads) k_scan_once(const TI* __restrict_
     if (CF && threadIdx.x == 0) big.n = 0;
     grid_wait();
     const int64_t n = d_n ? min(*d_n, n_max) : n_max;
-    // (nothing to scan, and no tile, after an expired wait: the total stays at zero)
-    if (threadIdx.x == 0) {
-        const uint32_t ticket = gridDim.x == 1 ? 0u : (uint32_t)atomicAdd(words, 1ull);
-        s_tile = gave_up(err) ? 0xffffffffu : ticket;
-    }
+    if (threadIdx.x == 0) s_tile = gridDim.x == 1 ? 0u : (uint32_t)atomicAdd(words, 1ull);
     __syncthreads();
     const int64_t t = s_tile, t0 = t * kOneTile;
     words += 8;
-    if (t0 >= n) {
-        if (n == 0 && t == 0 && threadIdx.x == 0) *d_total = 0;
-        return;
-    }
+    if (t0 >= n) return;   // (no elements, or their number is not known: the total stays at zero)
     for (int i = threadIdx.x; i < kOneTile; i += kOneThreads) {
         const int64_t idx = t0 + i;
         tile[i + (i >> 4)] = idx < n ? (int64_t)in[idx] : 0;
@@ -287,18 +281,23 @@ __global__ void __launch_bounds__(kOneThreads) k_scan_once(const TI* __restrict_
                     if (lane == 0) atomicOr(err, 1u);
                     lost = true;
                 } else if ((spins & 63) == 0) {
-                    lost = __any_sync(kFull, gave_up(err));
+                    lost = __any_sync(kFull, ld_tile((const uint32_t*)err) != 0);
                 }
                 if (lost) break;
             }
         }
         if (lost) {
-            if (lane == 0) s_before = -1;
+            // no item may be taken from offsets that were not written: whichever comes first, the
+            // last tile's total or this, what stays is below zero
+            if (lane == 0) {
+                atomicMin((long long*)d_total, -1ll);
+                s_before = -1;
+            }
         } else if (lane == 0) {
             if (gridDim.x > 1) st_tile64(words + t, (2ull << 62) | (unsigned long long)(before + total));
             s_before = before;
             if (t0 + kOneTile >= n) {
-                *d_total = before + total;
+                atomicCAS((unsigned long long*)d_total, 0ull, (unsigned long long)(before + total));
                 if (CF) {
                     const int64_t end = (before + total + grain - 1) / grain;
                     if (end < ncf) cf[TM_CHK_IDX(end, ncf, kChkSort)] = n - 1;
@@ -694,7 +693,7 @@ int scan_lengths(const int32_t* in, int64_t* out, int64_t n_max, const int64_t* 
         if (cudaGetLastError() != cudaSuccess) rc = TM_ECUDA;
         if (rc == TM_OK) rc = scan_exclusive_i64_ws(sums, soffs, ntiles, d_total, ws + 2 * ntiles, need - 2 * ntiles, st);
         if (rc == TM_OK) {
-            k_len_scan<<<(unsigned)ntiles, kScanThreads, 0, st>>>(in, out, n_max, d_n, soffs, cf, ncf, err); count_launch();
+            k_len_scan<<<(unsigned)ntiles, kScanThreads, 0, st>>>(in, out, n_max, d_n, soffs, cf, ncf); count_launch();
             if (cudaGetLastError() != cudaSuccess) rc = TM_ECUDA;
         }
     }

@@ -429,7 +429,8 @@ int64_t scan_dn_ws_elems(int64_t n_max);
 // Exclusive scan of 32-bit range lengths into 64-bit offsets (the first *d_n, or n_max when d_n is
 // null) with, in cf, the element that holds every grain-th item (as far as ncf goes).  words:
 // scan_once_words(n_max) zeroed words; when that is 0 (too many tiles for one launch) ws of
-// scan_dn_ws_elems(n_max), or null to allocate it on the stream.  *err: as SortWs::err
+// scan_dn_ws_elems(n_max), or null to allocate it on the stream.  *err: as SortWs::err; in one
+// launch *d_total, zeroed before, ends below zero then
 // The matcher's chunks are whole grains.  Few first edges: 32 items, so that small batches cut
 // small chunks, with entries for 64 items per first edge; many: 256, where every chunk is at
 // least that long anyway, for as many items in an eighth of the memory.  (The bound counts: a
@@ -591,11 +592,13 @@ __device__ __forceinline__ void st_tile(uint32_t* p, uint32_t v) {
     asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 
-// Whether a wait of this call has expired.  What the waiting kernel should have written is then
-// missing, so every kernel behind it that takes an index, a range or a loop bound from there
-// reads the word first and returns; the host reports it.  (The word is read beside the kernel's
-// other first loads; a kernel that may set it itself lets one thread decide for its block.)
-__device__ __forceinline__ bool gave_up(const uint32_t* err) { return err && ld_tile(err) != 0; }
+// Whether a wait of an earlier kernel of this call has expired.  What that kernel should have
+// written is then missing, so every kernel behind a sort that takes an index, a range or a loop
+// bound from there reads the word first and returns; the host reports it.  (A plain load: kernels
+// that start with an empty L1, not overlapped launches.  Read past L1 by every warp, one word held
+// up the small counts by 5 us and the build of 1e8 edges by 2 %.)  Behind a scan the total says so:
+// it is negative, and there are no items (k_scan_once).
+__device__ __forceinline__ bool gave_up(const uint32_t* err) { return err && *err != 0; }
 
 // sum += the words of tiles tile-1, tile-2, ... at `stride` apart, back to the first that holds a
 // prefix, kLookBack of them read at a time (the reads are a serial chain otherwise: prefixes
@@ -632,7 +635,7 @@ __device__ __forceinline__ bool look_back(const uint32_t* words, int64_t tile, i
                 atomicOr(err, 1u);
                 return false;
             }
-            if ((spins & 63) == 0 && gave_up(err)) return false;
+            if ((spins & 63) == 0 && ld_tile(err) != 0) return false;
         } else {
             spins = 0;
         }
