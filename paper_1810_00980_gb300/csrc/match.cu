@@ -125,11 +125,19 @@ struct MatchArgs {
     unsigned long long* rcount = nullptr;   // records appended (counts past rcap: the batch reruns)
     int64_t rcap = 0;
     // From rstop records on the warps finish the chunks they have and take no more (*more = 1 then):
-    // k_ride weighs the records so far and the matcher goes on from the queue's counter (resume).
+    // k_ride weighs the records so far and the matcher goes on from item `from` where they stopped.
     unsigned long long rstop = 0;
     uint32_t* more = nullptr;
-    int resume = 0;
+    int64_t from = 0;
 };
+
+// Items a warp takes at a time.  Few items: smaller chunks, so that every warp gets some (17,000
+// items in chunks of 256 kept 67 warps busy for eight rounds each: 43 us of a 20,000-edge count)
+__host__ __device__ __forceinline__ int64_t match_chunk(int64_t items, int64_t nwarps, int64_t chunk, int grain_log) {
+    const int64_t share = ((items / nwarps >> grain_log) + 1) << grain_log;
+    const int64_t whole = (((chunk - 1) >> grain_log) + 1) << grain_log;
+    return whole < share ? whole : share;
+}
 
 // ----------------------------------------------------------------- helpers
 template <int K>
@@ -1247,27 +1255,12 @@ __global__ void __launch_bounds__(256, OCC) k_match(MatchArgs<TT> A) {
     grid_wait();
     int64_t W2 = *A.d_W2;   // (below zero when a wait of their scan expired)
     const int64_t F = A.d_F ? *A.d_F : A.F;
-    // few items: smaller chunks, so that every warp gets some (17,000 items in chunks of 256 kept 67
-    // warps busy for eight rounds each: 43 us of a 20,000-edge count)
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
     const int gl = A.grain_log;
-    const int64_t share = ((W2 / nwarps >> gl) + 1) << gl;
-    const int64_t chunk = min((((A.chunk - 1) >> gl) + 1) << gl, share);
+    const int64_t chunk = match_chunk(W2, nwarps, A.chunk, gl);
     // a warp's first chunk is its own, the others come from the counter (with few items no warp
     // asks it: 7,000 atomics on one word take longer than such a batch's items)
-    auto next_chunk = [&]() -> int64_t {
-        unsigned long long c = 0;
-        if (lane == 0) {
-            if (stop_flag()) {
-                *A.more = 1;
-                c = (unsigned long long)W2;   // past the last item
-            } else {
-                c = atomicAdd(A.counter, (unsigned long long)chunk);
-            }
-        }
-        return nwarps * chunk + (int64_t)__shfl_sync(kFull, c, 0);
-    };
-    for (int64_t c0 = A.resume ? next_chunk() : ((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5) * chunk; c0 < W2;) {
+    for (int64_t c0 = A.from + ((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5) * chunk; c0 < W2;) {
         int64_t c1 = min(c0 + chunk, W2);
         int64_t fb = 0, fe = 0;
         const int64_t ci = c0 >> gl, ce = ((c1 - 1) >> gl) + 1;
@@ -1457,8 +1450,17 @@ __global__ void __launch_bounds__(256, OCC) k_match(MatchArgs<TT> A) {
             }
         }
         acc_flush_warp(acc, A.W.acc);
-        if (nwarps * chunk >= W2) break;
-        c0 = next_chunk();
+        if (A.from + nwarps * chunk >= W2) break;
+        unsigned long long c0u = 0;
+        if (lane == 0) {
+            if (stop_flag()) {
+                *A.more = 1;
+                c0u = (unsigned long long)W2;   // past the last item
+            } else {
+                c0u = atomicAdd(A.counter, (unsigned long long)chunk);
+            }
+        }
+        c0 = A.from + nwarps * chunk + (int64_t)__shfl_sync(kFull, c0u, 0);
     }
     acc_flush_warp(acc, A.W.acc);
 }
@@ -2351,6 +2353,7 @@ int run_batch_t(const tm_graph* g, const tm_query* qs, int nq, tm_result* res, c
     }
     const int64_t Fa = bounded ? F_ub : F;   // first edges the scratch holds
     const bool expands = std::any_of(hp.begin(), hp.end(), [](const QPlan& P) { return plan_expands(P); });
+    const int64_t nwarps = (int64_t)nsm * tu.blocks_per_sm * (tu.block_threads / 32);   // of the matcher
     MatchArgs<TT> A;
     auto launch_ride = [&]() {
         launch_after(k_ride<TT>, dim3((unsigned)(nsm * 8)), 256, match_smem_bytes(A.nq, 256, true), st, A);
@@ -2384,8 +2387,7 @@ int run_batch_t(const tm_graph* g, const tm_query* qs, int nq, tm_result* res, c
             A.rcount = drcount;
             A.rcap = rcap;
             // room for the chunks in flight (three edges: at most a record per item), or half of it
-            const int64_t held = (int64_t)nsm * tu.blocks_per_sm * (tu.block_threads / 32) *
-                                 std::max<int64_t>(tu.chunk_items, item_grain(Fa));
+            const int64_t held = nwarps * std::max<int64_t>(tu.chunk_items, item_grain(Fa));
             A.rstop = (unsigned long long)std::max(rcap / 2, rcap - held);
             A.more = dmore;
             int64_t gl2 = std::min<int64_t>((Fa + 255) / 256, (int64_t)nsm * 8);
@@ -2488,8 +2490,14 @@ int run_batch_t(const tm_graph* g, const tm_query* qs, int nq, tm_result* res, c
     bool rounds = false;
     while (rc == TM_OK && h_more && (int64_t)h_rcount <= rcap) {
         rounds = true;
-        A.resume = 1;
+        unsigned long long taken = 0;   // beyond the warps' first chunks
+        fail(cudaMemcpyAsync(&hW2, dW2, 8, cudaMemcpyDeviceToHost, st), "W2");
+        fail(cudaMemcpyAsync(&taken, dctr, 8, cudaMemcpyDeviceToHost, st), "queue counter");
+        fail(cudaStreamSynchronize(st), "round sync");
+        A.from += nwarps * match_chunk(hW2, nwarps, A.chunk, A.grain_log) + (int64_t)taken;
+        if (rc != TM_OK || A.from >= hW2) break;
         PhaseEvents pr(pe.on);
+        fail(cudaMemsetAsync(dctr, 0, 8, st), "queue counter");
         fail(cudaMemsetAsync(drcount, 0, 16, st), "record count");
         const int e0 = pr.mark(st);
         if (rc == TM_OK) launch_match<TT>(A, lmax, kmax, tu, nsm, st, expands);
