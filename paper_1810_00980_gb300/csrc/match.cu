@@ -2114,9 +2114,6 @@ RideEnt ride_entry(const QPlan& R, int k, int64_t t_max) {
     return E;
 }
 
-// most deferred records made room for on behalf of estimates that could do without (12.9 GB)
-constexpr int64_t kHiddenRecords = (int64_t)1 << 29;
-
 template <typename TT>
 int run_batch_t(const tm_graph* g, const tm_query* qs, int nq, tm_result* res, cudaStream_t st,
                 BatchOut* dbg) {
@@ -2536,7 +2533,7 @@ int run_batch_t(const tm_graph* g, const tm_query* qs, int nq, tm_result* res, c
     if ((int64_t)h_rcount > rcap) {
         // a round left more deferred records than the buffer held: run again with a larger one
         const int64_t want = std::max(4 * rcap, (int64_t)h_rcount + (int64_t)(h_rcount >> 3) + 1024);
-        if (dbg->hidden && want > kHiddenRecords) return TM_ENOMEM;   // run_batch_once runs the estimates apart
+        if (dbg->hidden && want > dbg->hidden_records) return TM_ENOMEM;   // run_batch_once runs the estimates apart
         dbg->need_records = want;
         rc = run_batch_t<TT>(g, qs, nq, res, st, dbg);
         if (rc == TM_ENOMEM) return rc;   // (the next batches keep the capacity that fits)
@@ -2641,7 +2638,7 @@ double ride_gain(const tm_graph* g, const tm_query& q, double shifts) {
 constexpr double kHideFirst = 1.4, kHideCand = 0.9;
 
 int run_batch_once(const tm_graph* g, const tm_query* qs, int nq, tm_result* res, cudaStream_t st,
-                   BatchOut* dbg, bool hide = true) {
+                   BatchOut* dbg, int64_t hidden_records) {
     if (dbg || !g || !qs || !res || nq < 2) return run_batch_typed(g, qs, nq, res, st, dbg);
     std::vector<int> lead((size_t)nq, -1), slot((size_t)nq, -1);   // span members: their leader
     std::vector<std::vector<int>> groups;
@@ -2726,7 +2723,7 @@ int run_batch_once(const tm_graph* g, const tm_query* qs, int nq, tm_result* res
     // least kHideCand of it (measured: see kHideFirst), and riding saves what it costs.
     std::vector<tm_query> hidden;
     std::vector<int> top;                     // per hidden head, the estimate whose span it has
-    if (!hide) kinds.clear();
+    if (hidden_records <= 0) kinds.clear();
     for (std::vector<int>& gr : kinds) {
         std::stable_sort(gr.begin(), gr.end(), [&](int a, int b) { return qs[a].delta > qs[b].delta; });
         // sums of b p, of b p delta and of the gains, longest spans first
@@ -2785,10 +2782,11 @@ int run_batch_once(const tm_graph* g, const tm_query* qs, int nq, tm_result* res
     bo.sub_count = sc.data();
     bo.riders = &riders;
     bo.hidden = (int)hidden.size();
+    bo.hidden_records = hidden_records;
     int rc = run_batch_typed(g, qc.data(), nc, rc_res.data(), st, &bo);
     // the shared enumeration's records (one per group of instances) may not fit where the
     // estimates' own enumerations, which keep none, do
-    if (rc == TM_ENOMEM && !hidden.empty()) return run_batch_once(g, qs, nq, res, st, dbg, false);
+    if (rc == TM_ENOMEM && !hidden.empty()) return run_batch_once(g, qs, nq, res, st, dbg, 0);
     for (int i = 0; i < nq; i++) {
         if (lead[(size_t)i] < 0) {
             res[i] = rc_res[(size_t)pos[(size_t)i]];
@@ -2828,12 +2826,23 @@ double auto_p(const tm_result& pilot, double target, int32_t b) {
 
 }  // namespace
 
+int64_t share_bytes(const tm_graph* g, const tm_query* qs, int nq) {
+    int n = 0;   // queries that may share
+    for (int i = 0; i < nq; i++) {
+        const tm_motif* m = qs[i].motif;
+        n += m && (m->l == 3 || m->l == 4) && m->lv[m->l - 1].view == kPair;
+    }
+    if (n < 2) return 0;
+    const int64_t records = std::max(ride_capacity().load(), g->ride_need.load());
+    return records * (int64_t)(g->dev.tbytes == 4 ? sizeof(RideRec<int32_t>) : sizeof(RideRec<int64_t>));
+}
+
 int run_batch(const tm_graph* g, const tm_query* qs, int nq, tm_result* res, cudaStream_t st,
-              BatchOut* dbg) {
+              BatchOut* dbg, int64_t hidden_records) {
     bool any_auto = false;
     for (int i = 0; qs && i < nq; i++)
         any_auto |= qs[i].mode == TM_MODE_ESTIMATE && qs[i].q_mode == TM_Q_AUTO;
-    if (!any_auto) return run_batch_once(g, qs, nq, res, st, dbg);
+    if (!any_auto) return run_batch_once(g, qs, nq, res, st, dbg, hidden_records);
     if (!g || !res) { set_error("NULL argument"); return TM_EINVAL; }
     if (dbg && (dbg->seg || dbg->query >= 0)) { set_error("TM_Q_AUTO needs the whole graph"); return TM_EINVAL; }
     // pilot batch: the auto queries at p0 (valid ones only; the rest is checked below)
@@ -2853,7 +2862,7 @@ int run_batch(const tm_graph* g, const tm_query* qs, int nq, tm_result* res, cud
     std::vector<tm_result> pr(pq.size());
     std::vector<tm_query> fq(qs, qs + nq);
     if (!pq.empty()) {
-        int rc = run_batch_once(g, pq.data(), (int)pq.size(), pr.data(), st, nullptr);
+        int rc = run_batch_once(g, pq.data(), (int)pq.size(), pr.data(), st, nullptr, hidden_records);
         if (rc != TM_OK) return rc;
         for (size_t x = 0; x < pq.size(); x++) {
             tm_query& q = fq[(size_t)pidx[x]];
@@ -2861,7 +2870,7 @@ int run_batch(const tm_graph* g, const tm_query* qs, int nq, tm_result* res, cud
             q.q_mode = TM_Q_UNIFORM;
         }
     }
-    return run_batch_once(g, fq.data(), nq, res, st, dbg);
+    return run_batch_once(g, fq.data(), nq, res, st, dbg, hidden_records);
 }
 
 template <typename TT>

@@ -92,7 +92,7 @@ void worker_main(tm_server* S) {
     std::vector<tm_result> rs;
     for (;;) {
         int32_t gid = -1;
-        int64_t fp_total = 0;
+        int64_t fp_total = 0, records = 0;
         double work = 0.0, budget = 0.0;
         ids.clear();
         qs.clear();
@@ -134,10 +134,18 @@ void worker_main(tm_server* S) {
                 S->cv_work.wait_for(lk, std::chrono::milliseconds(50));
             }
             if (ids.empty()) break;  // stopping and drained
+            // Queries that share an enumeration need a record buffer besides their footprints (the
+            // first edges of an enumeration of their own are fewer than those counted for the
+            // estimates in it).  Estimates share one only where the budget has room for the
+            // buffer, and it does not grow for them.
+            const int64_t buffer = tmo::share_bytes(S->graphs[(size_t)gid], qs.data(), (int)qs.size());
+            const bool fits = S->in_use + fp_total + buffer <= S->cfg.mem_budget_bytes;
+            records = fits ? 1 : 0;
+            if (fits) fp_total += buffer;
             S->in_use += fp_total;
         }
         rs.assign(qs.size(), tm_result{});
-        int rc = tmo::run_batch(S->graphs[(size_t)gid], qs.data(), (int)qs.size(), rs.data(), st, nullptr);
+        int rc = tmo::run_batch(S->graphs[(size_t)gid], qs.data(), (int)qs.size(), rs.data(), st, nullptr, records);
         {
             std::lock_guard<std::mutex> lk(S->mu);
             S->in_use -= fp_total;

@@ -346,14 +346,21 @@ struct BatchOut {                 // optional per-window readback for one query
     ShiftSums* sums = nullptr;    // host: per query, per shift (exact: one), or null
     const std::vector<std::vector<int>>* riders = nullptr;   // per query: plan indices of its riders
     int hidden = 0;                           // trailing queries whose results nobody asked for
+    int64_t hidden_records = 0;               // most deferred records made room for on their behalf
     int64_t need_records = 0;                 // deferred records to make room for, past the usual capacity
     const int32_t* nsub = nullptr;            // per query: spans counted alongside (exact)
     const int64_t* sub_delta = nullptr;       // [nq][kMaxSub]
     unsigned long long* sub_count = nullptr;  // host out: [nq][kMaxSub]
 };
 
+// Most deferred records made room for on behalf of estimates that could do without (12.9 GB)
+constexpr int64_t kHiddenRecords = (int64_t)1 << 29;
+// hidden_records: of estimates that share an enumeration nobody asked for; 0: they do not
 int run_batch(const tm_graph* g, const tm_query* qs, int nq, tm_result* res,
-              cudaStream_t st, BatchOut* dbg);
+              cudaStream_t st, BatchOut* dbg, int64_t hidden_records = kHiddenRecords);
+// bytes of the record buffer that a batch of these queries takes when it shares enumerations (0: it
+// does not)
+int64_t share_bytes(const tm_graph* g, const tm_query* qs, int nq);
 int count_plain(const tm_graph* g, const tm_motif* m, int64_t delta, int64_t* count);
 // query checks of tm_run_batch against a graph whose normalised times end at t_max
 int check_query(int64_t t_max, const tm_query& q, std::string& why);
