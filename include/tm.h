@@ -295,7 +295,8 @@ int tm_set_tuning(const tm_tuning* in);
  * estimates riding along with it) and smaller spans to a second kernel, as one record per group
  * of instances, in a device buffer taken from the batch scratch.  `records` (1 .. 2^36) sets how
  * many records the next batches make room for (default 2^23: 192 MB with 32-bit times, 256 MB
- * with 64-bit times).  A batch that produces more goes on in rounds, the matcher stopping while
+ * with 64-bit times; at the default, graphs of more than 2^25 edges get a quarter of a record per
+ * edge, 2^27 at most).  A batch that produces more goes on in rounds, the matcher stopping while
  * the second kernel empties the buffer; one that overruns the buffer within a round runs again
  * with a larger one, whose size the graph keeps for its next batches.  The setting changes only
  * memory and time, never a result.

@@ -39,8 +39,18 @@ Tuning& tuning() {
 
 // Records the deferred-rider buffer of a batch holds (tm_set_ride_capacity)
 std::atomic<int64_t>& ride_capacity() {
-    static std::atomic<int64_t> cap{(int64_t)1 << 23};
+    static std::atomic<int64_t> cap{kRideCapacity};
     return cap;
+}
+
+// Records that a batch on g has room for.  Unless a capacity was set, a quarter of a record per edge
+// of a large graph (6 bytes beside its 90): a round ends with the longest chunk in flight, and 192
+// riders of the 4-cycle on 1e8 edges took 482 ms in 15 rounds of 2^23, 477 in five of these and 476
+// in one.
+static int64_t ride_room(const tm_graph* g) {
+    int64_t cap = ride_capacity().load();
+    if (cap == kRideCapacity) cap = std::max(cap, std::min(g->m / 4, kRideCapacityMost));
+    return std::max(cap, g->ride_need.load());
 }
 
 namespace {
@@ -2209,7 +2219,7 @@ int run_batch_t(const tm_graph* g, const tm_query* qs, int nq, tm_result* res, c
     bool any_share = false;
     for (const QPlan& P : hp) any_share |= P.nsub > 0 || P.nride > 0;
     // (shares come with dbg)
-    const int64_t rcap = any_share ? std::max({ride_capacity().load(), g->ride_need.load(), dbg->need_records}) : 0;
+    const int64_t rcap = any_share ? std::max(ride_room(g), dbg->need_records) : 0;
     const size_t rrec_bytes = any_share ? a256(sizeof(RideRec<TT>) * (size_t)rcap) : 0;
     // ---- scratch layout
     const int64_t n_parts = fold_parts(hp);
@@ -2670,9 +2680,10 @@ int run_batch_once(const tm_graph* g, const tm_query* qs, int nq, tm_result* res
             if (i != L) { lead[(size_t)i] = L; slot[(size_t)i] = k++; }
     }
     // estimates of the same three-edge motif with a span no larger than an exact query's ride
-    // along with it: each instance that query enumerates also adds its weight to the window of
-    // an estimate when it lies inside one of its kept windows and within its span, so the
-    // estimate needs no enumeration of its own (its windows and fold stay its own)
+    // along with it where that costs less (ride_gain): each instance that query enumerates also
+    // adds its weight to the window of an estimate when it lies inside one of its kept windows and
+    // within its span, so the estimate needs no enumeration of its own (its windows and fold stay
+    // its own)
     std::vector<int> host((size_t)nq, -1);    // estimate -> its exact head (nq + h: hidden head h)
     std::vector<int> nrid((size_t)nq, 0);
     std::vector<int64_t> nshift((size_t)nq, 0);   // shifts riding on a head
@@ -2833,8 +2844,7 @@ int64_t share_bytes(const tm_graph* g, const tm_query* qs, int nq) {
         n += m && (m->l == 3 || m->l == 4) && m->lv[m->l - 1].view == kPair;
     }
     if (n < 2) return 0;
-    const int64_t records = std::max(ride_capacity().load(), g->ride_need.load());
-    return records * (int64_t)(g->dev.tbytes == 4 ? sizeof(RideRec<int32_t>) : sizeof(RideRec<int64_t>));
+    return ride_room(g) * (int64_t)(g->dev.tbytes == 4 ? sizeof(RideRec<int32_t>) : sizeof(RideRec<int64_t>));
 }
 
 int run_batch(const tm_graph* g, const tm_query* qs, int nq, tm_result* res, cudaStream_t st,

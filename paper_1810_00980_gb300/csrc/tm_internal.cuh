@@ -310,6 +310,7 @@ struct Tuning {
     int enum_threshold = 48;
 };
 Tuning& tuning();
+constexpr int64_t kRideCapacity = (int64_t)1 << 23, kRideCapacityMost = (int64_t)1 << 27;
 std::atomic<int64_t>& ride_capacity();
 
 // one query's part of a segment of a streamed graph
@@ -490,8 +491,8 @@ void store_profile_ride_records(int64_t n);
 void count_launch(int n = 1);
 
 // NVTX ranges naming the host-side phases of a call (graph build, window partition, second-edge
-// ranges, matcher, fold), one after another, so that a profiler can select them (for example
-// ncu --nvtx --nvtx-include "tm_match/"); without a tool attached each call costs a branch
+// ranges, matcher, fold), one after another, so that a profiler can select them; without a tool
+// attached each call costs a branch
 struct NvtxPhases {
     nvtxRangeId_t id = 0;
     bool open = false;
