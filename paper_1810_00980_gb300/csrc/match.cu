@@ -2612,11 +2612,14 @@ bool same_motif(const tm_motif* a, const tm_motif* b) {
 // for every window.  Times in ms, sharing / apart, of seeds with a constant sum of p: 3-cycle on 1e7
 // edges, 64 at p = 1/32 0.96 / 3.5, 512 at 1/256 2.5 / 3.1, 4,000 at 1/2,000 14 / 10; on 1e6 edges 0.44 /
 // 0.53, 1.9 / 1.3, 12.5 / 7.3; out-star on 2e7 edges, 2,000 at 0.0021 21 / 14; ping-pong on 1e7 edges
-// 2.3 / 3.3, 13 / 3.0, 120 / 10; two seeds at p = 1 on 1e7 edges with 63 windows per 100 edges 4.2 /
-// 0.72, with 6.3 0.87 / 0.76 (eight: 1.7 / 2.7), with 1.1 0.64 / 0.94.  The true lines vary by
-// motif, span and graph by a factor of about two (the records are not known before); over 800
-// such batches from 1e5 to 2e7 edges the form chosen takes at most 1.45 times the better one.
-constexpr double kApartEdge = 0.12, kApartEdgeTwoNode = 0.13, kApartAllEdge = 0.035;   // per edge of the graph
+// 2.3 / 3.3, 13 / 3.0, 120 / 10; 4-cycle on 5e5 skewed edges, 72 at 0.01 beside 72 at 0.1 0.66 / 0.73,
+// on 1e6 edges 2,000 at 0.0021 7.2 / 4.2; two seeds at p = 1 on 1e7 edges with 63 windows per 100
+// edges 4.2 / 0.72, with 6.3 0.87 / 0.76 (eight: 1.7 / 2.7), with 1.1 0.64 / 0.94.  The true lines vary
+// by motif, span and graph by a factor of about two (the records are not known before); of 800
+// such batches from 1e5 to 2e7 edges, those whose sums of p reach kHideFirst take at most 1.45
+// times what the better form does.
+constexpr double kApartEdge = 0.12, kApartEdgeTwoNode = 0.13, kApartEdgeFour = 0.30;   // per edge of the graph
+constexpr double kApartAllEdge = 0.035;
 constexpr double kRideEdge = 0.05e-3, kRideEdgeFixed = 0.2e-3, kRideEdgeTwoNode = 2.0e-3;
 constexpr double kRideChain = 1100.0, kRideWindow = 0.2;
 constexpr double kFewShifts = 64;
@@ -2635,7 +2638,7 @@ double ride_gain(const tm_graph* g, const tm_query& q, double shifts) {
     const bool all = q.q_mode == TM_Q_UNIFORM && q.p >= 1.0;
     const bool two = q.motif->k == 2;
     const LevelPlan& L = q.motif->lv[q.motif->l - 1];
-    const double apart = m * (all ? kApartAllEdge : p * (two ? kApartEdgeTwoNode : kApartEdge));
+    const double apart = m * (all ? kApartAllEdge : p * (two ? kApartEdgeTwoNode : q.motif->l == 4 ? kApartEdgeFour : kApartEdge));
     const double edge = two ? kRideEdgeTwoNode : std::max(L.su, L.sv) < 2 ? kRideEdgeFixed : kRideEdge;
     return apart - m * edge - (all ? J * kRideWindow : 0.0) -
            (shifts > kFewShifts ? kRideChain : 0.0);
